@@ -346,8 +346,9 @@ struct asd_ctx {
     int prefill_mode = ASD_PREFILL_AUTO;
     // tensor maps of the dense prompt path (host copies, passed to the kernels by value): activations with boxes of
     // 64 x 128, and per layer the four matrices with boxes of 64 x 128 ([0..3]) and 64 x 256 ([4..7])
-    CUtensorMap tm_xn{}, tm_a{}, tm_t{};
+    CUtensorMap tm_xn{}, tm_q{}, tm_a{}, tm_t{};
     std::vector<CUtensorMap> tm_w;
+    std::vector<CUtensorMap> tm_kv;  // per layer the K and the V cache (the pass kernel reads its own copy in the workspace)
     asd_stats stats{};
     int32_t* pinned = nullptr;  // small host staging buffer
     uint32_t bar_base = 0;      // value of the grid-barrier counter at the start of the next pass
@@ -461,9 +462,11 @@ static int make_tensor_maps(asd_ctx* x) {
         const Layout& ly = x->lay;
         const size_t d = c.d_model, f = c.d_ffn, kvd = x->kv_dim, R = ly.pf_rows;
         bool ok = encode_operand_map(encode, &x->tm_xn, x->ws + ly.pf_xn, d, R, kGemmBM) &&
+                  encode_operand_map(encode, &x->tm_q, x->ws + ly.pf_q, d, R, kGemmBM) &&
                   encode_operand_map(encode, &x->tm_a, x->ws + ly.pf_a, d, R, kGemmBM) &&
                   encode_operand_map(encode, &x->tm_t, x->ws + ly.pf_t, f, R, kGemmBM);
         x->tm_w.assign((size_t)8 * L, CUtensorMap{});
+        x->tm_kv = maps;
         for (int l = 0; l < L && ok; ++l) {
             unsigned char* rw = x->ws + ly.rm_layers + (size_t)l * ly.rm_layer_stride;
             for (int v = 0; v < 2 && ok; ++v) {
@@ -664,10 +667,10 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
 static int check_device_error(asd_ctx* x, const int32_t* w) {
     if (w[0] == 0) return ASD_OK;
     static const char* names[] = {"", "a ring slot was never filled", "a ring slot was never released", "the grid barrier never completed",
-                                  "a pipeline barrier of the prompt GEMM never completed"};
+                                  "a pipeline barrier of the prompt GEMM never completed", "a pipeline barrier of the prompt attention never completed"};
     char buf[256];
     snprintf(buf, sizeof buf, "a kernel gave up waiting: %s (stage %d, item %d, slot %d, CTA %d, thread %d, tag %d, parity %d)",
-             (w[0] >= 1 && w[0] <= 4) ? names[w[0]] : "unknown", w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+             (w[0] >= 1 && w[0] <= 5) ? names[w[0]] : "unknown", w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
     x->dev_failed = true;
     x->dev_failed_msg = std::string(buf) + " (call asd_reset before going on)";
     return fail(x, ASD_ERR_DEVICE_TIMEOUT, x->dev_failed_msg);
@@ -1048,7 +1051,7 @@ static int prefill_dense(asd_ctx* x, const int32_t* dev_tokens, int n, int pos0)
             e.rope_cos = x->at<float>(ly.rope_cos), e.rope_sin = x->at<float>(ly.rope_sin);
             e.pos0 = p0, e.d_model = d, e.kv_dim = kvd, e.head_dim = c.head_dim;
             if ((rc = dense_gemm(x, x->tm_xn, l, 0, rows, d + 2 * kvd, d, e))) return rc;
-            ASD_CUDA(x, launch_flash_prefill(pq, kc, vc, pa, rows, p0, d, kvd, c.head_dim, c.n_heads, c.n_kv_heads, c.max_seq, scale, s));
+            ASD_CUDA(x, launch_flash_prefill(x->tm_q, x->tm_kv[(size_t)l * 2], x->tm_kv[(size_t)l * 2 + 1], pa, rows, p0, d, c.head_dim, c.n_heads, c.n_kv_heads, scale, err, s));
             GemmEpi o{};
             o.err = err;
             o.mode = kGemmF32;

@@ -3,71 +3,9 @@
 
 #include "common.cuh"
 #include "ring.cuh"
+#include "tcgen05.cuh"
 
 namespace asd {
-
-constexpr int kErrGemmWait = 4;  // a pipeline barrier of the GEMM never completed
-
-// ============================================================================================ tcgen05 helpers
-__device__ __forceinline__ void tmem_alloc(uint32_t* smem_slot, uint32_t n_cols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_slot)), "r"(n_cols) : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() { asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t n_cols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(n_cols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// all tcgen05.mma issued so far by this thread arrive on the barrier when they have finished
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// D (tensor memory, 128 lanes x N columns fp32) (+)= A (smem, 128 x 16 bf16, K-major) * B (smem, N x 16 bf16, K-major)^T
-__device__ __forceinline__ void tc_mma_bf16(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.u32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// 32 consecutive fp32 columns of this thread's lane of tensor memory
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-          "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-          "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// Shared-memory matrix descriptor of a K-major bf16 tile whose rows are 128 bytes (64 elements) stored with the
-// 128-byte swizzle, tile base 1024-byte aligned: groups of 8 rows are 1024 bytes apart (stride byte offset);
-// the leading byte offset is not used by swizzled K-major layouts. Fields: start address >> 4 in bits 0-13,
-// leading offset >> 4 in bits 16-29, stride offset >> 4 in bits 32-45, descriptor version 1 in bits 46-47,
-// swizzle mode (2 = 128 bytes) in bits 61-63.
-__device__ __forceinline__ uint64_t umma_desc_k128(uint32_t smem_addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-// Instruction descriptor of kind::f16: fp32 accumulator (bits 4-5 = 1), bf16 A and B (bits 7-9, 10-12 = 1), both
-// K-major (bits 15, 16 = 0), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
-__host__ __device__ constexpr uint32_t umma_idesc_bf16(int m, int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
 
 // ============================================================================================ GEMM epilogues
 // One call per (row, 32 consecutive columns starting at col0) with the fp32 accumulators in v.
@@ -81,11 +19,6 @@ __device__ __forceinline__ void epi_f32(const GemmEpi& ep, int row, int col0, in
         for (int i = 0; i < 32; ++i)
             if (col0 + i < N) dst[i] = v[i];
     }
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 __device__ __forceinline__ void epi_swiglu(const GemmEpi& ep, int row, int col0, int N, const float (&v)[32]) {
@@ -501,229 +434,6 @@ cudaError_t launch_sumcos(const float* cos_rows, int stride, int n_rows, int n_s
     return cudaGetLastError();
 }
 
-// ============================================================================================ causal attention over the prompt
-// One CTA = 64 query rows of one head (4 warps x 16 rows); keys and values stream through shared memory in tiles of
-// 64 keys (double-buffered cp.async). Scores are bf16 x bf16 products accumulated in fp32 (mma.sync m16n8k16), the
-// softmax is kept on line in fp32 (running maximum and sum per row), and the probabilities enter the P V product as
-// the sum of three bf16 numbers (p = hi + mid + lo, three MMAs), which represents every fp32 probability exactly:
-// with fewer terms the 2^-17 error of P flips bf16 roundings of the attention output in about every second row.
-constexpr int kFaRows = 64, kFaKeys = 64, kFaThreads = 128;
-
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void* smem_src) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_u32(smem_src)));
-}
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t (&r)[4], const void* smem_src) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_u32(smem_src)));
-}
-__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-template <int HD>
-__global__ void __launch_bounds__(kFaThreads, 3)
-flash_prefill_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ kc, const __nv_bfloat16* __restrict__ vc,
-                     __nv_bfloat16* __restrict__ out, int n_rows, int pos0, int d_model, int kv_dim, int group, int max_seq, float scale) {
-    constexpr int LD = HD + 8;  // padded row: rows stay 16-byte aligned and ldmatrix reads are free of bank conflicts
-    constexpr int VPR = HD / 8;  // 16-byte vectors per row
-    extern __shared__ __align__(16) unsigned char fa_smem[];
-    __nv_bfloat16* Ks = reinterpret_cast<__nv_bfloat16*>(fa_smem);  // [2][64][LD]
-    __nv_bfloat16* Vs = Ks + 2 * kFaKeys * LD;                      // [2][64][LD]
-    __nv_bfloat16* Qs = Vs + kFaKeys * LD;  // [64][LD]: the queries are staged in the second V buffer, which is first filled after they are in registers
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q4 = lane & 3;
-    const int qt = gridDim.x - 1 - blockIdx.x;  // the tiles with the most keys start first
-    const int head = blockIdx.y, kvh = head / group;
-    const int r0 = qt * kFaRows;
-    const int last_row = min(r0 + kFaRows - 1, n_rows - 1);
-    const int n_kt = (pos0 + last_row) / kFaKeys + 1;
-
-    auto load_tile = [&](int kt, int buf) {
-        for (int idx = tid; idx < kFaKeys * VPR; idx += kFaThreads) {
-            const int row = idx / VPR, c = idx - row * VPR;
-            const int key = kt * kFaKeys + row;
-            __nv_bfloat16* kd = Ks + (size_t)(buf * kFaKeys + row) * LD + c * 8;
-            __nv_bfloat16* vd = Vs + (size_t)(buf * kFaKeys + row) * LD + c * 8;
-            if (key < max_seq) {
-                const size_t off = (size_t)key * kv_dim + (size_t)kvh * HD + c * 8;
-                cp_async16(kd, kc + off);
-                cp_async16(vd, vc + off);
-            } else {
-                *reinterpret_cast<uint4*>(kd) = make_uint4(0u, 0u, 0u, 0u);
-                *reinterpret_cast<uint4*>(vd) = make_uint4(0u, 0u, 0u, 0u);
-            }
-        }
-        cp_async_commit();
-    };
-    load_tile(0, 0);
-    for (int idx = tid; idx < kFaRows * VPR; idx += kFaThreads) {
-        const int row = idx / VPR, c = idx - row * VPR;
-        const int r = min(r0 + row, n_rows - 1);  // rows past the prompt repeat the last row and are not stored
-        *reinterpret_cast<uint4*>(Qs + (size_t)row * LD + c * 8) =
-            *reinterpret_cast<const uint4*>(q + (size_t)r * d_model + (size_t)head * HD + c * 8);
-    }
-    __syncthreads();
-    uint32_t qf[HD / 16][4];
-#pragma unroll
-    for (int kk = 0; kk < HD / 16; ++kk) ldsm_x4(qf[kk], Qs + (size_t)(warp * 16 + (lane & 15)) * LD + kk * 16 + (lane >> 4) * 8);
-    __syncthreads();  // every warp has its queries: the buffer may now receive values
-
-    const int pos_a = pos0 + min(r0 + warp * 16 + g, n_rows - 1);
-    const int pos_b = pos0 + min(r0 + warp * 16 + g + 8, n_rows - 1);
-    float o[HD / 8][4];
-#pragma unroll
-    for (int i = 0; i < HD / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
-
-    for (int kt = 0; kt < n_kt; ++kt) {
-        const int buf = kt & 1;
-        if (kt + 1 < n_kt) {
-            load_tile(kt + 1, buf ^ 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-        const __nv_bfloat16* Kb = Ks + (size_t)buf * kFaKeys * LD;
-        const __nv_bfloat16* Vb = Vs + (size_t)buf * kFaKeys * LD;
-
-        // ---- scores of 16 rows x 64 keys
-        float sc[8][4];
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
-#pragma unroll
-        for (int k2 = 0; k2 < HD / 32; ++k2) {  // 32 dimensions at a time over all 8 key blocks: consecutive MMAs are independent
-            uint32_t b[8][4];
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt) ldsm_x4(b[nt], Kb + (size_t)(nt * 8 + (lane & 7)) * LD + k2 * 32 + (lane >> 3) * 8);
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt) mma16816(sc[nt], qf[2 * k2], b[nt][0], b[nt][1]);
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt) mma16816(sc[nt], qf[2 * k2 + 1], b[nt][2], b[nt][3]);
-        }
-        // ---- scale, causal mask (the row at position p sees keys <= p), running maximum
-        const int key0 = kt * kFaKeys + 2 * q4;
-        float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int key = key0 + nt * 8 + (e & 1);
-                const int pos = (e < 2) ? pos_a : pos_b;
-                const float s = (key <= pos) ? sc[nt][e] * scale : -INFINITY;
-                sc[nt][e] = s;
-                mx[e >> 1] = fmaxf(mx[e >> 1], s);
-            }
-        float alpha[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
-            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-            const float m_new = fmaxf(m_run[h], mx[h]);  // finite from the first tile on: key 0 is visible to every row
-            alpha[h] = expf(m_run[h] - m_new);
-            m_run[h] = m_new;
-            l_run[h] *= alpha[h];
-        }
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float p = expf(sc[nt][e] - m_run[e >> 1]);
-                sc[nt][e] = p;
-                l_run[e >> 1] += p;  // this lane's share of the row sum; the four lanes of a row are added at the end
-            }
-#pragma unroll
-        for (int i = 0; i < HD / 8; ++i) {
-            o[i][0] *= alpha[0], o[i][1] *= alpha[0];
-            o[i][2] *= alpha[1], o[i][3] *= alpha[1];
-        }
-        // ---- O += P V, P = hi + mid + lo in bf16
-#pragma unroll
-        for (int kk = 0; kk < kFaKeys / 16; ++kk) {
-            uint32_t a_hi[4], a_mid[4], a_lo[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int nt = 2 * kk + (u >> 1), e = (u & 1) * 2;
-                const float p0 = sc[nt][e], p1 = sc[nt][e + 1];
-                const __nv_bfloat162 hi = __floats2bfloat162_rn(p0, p1);
-                const float r0 = p0 - __low2float(hi), r1 = p1 - __high2float(hi);  // exact
-                const __nv_bfloat162 mid = __floats2bfloat162_rn(r0, r1);
-                const __nv_bfloat162 lo = __floats2bfloat162_rn(r0 - __low2float(mid), r1 - __high2float(mid));
-                a_hi[u] = *reinterpret_cast<const uint32_t*>(&hi);
-                a_mid[u] = *reinterpret_cast<const uint32_t*>(&mid);
-                a_lo[u] = *reinterpret_cast<const uint32_t*>(&lo);
-            }
-            // all value fragments of the 16 keys first, then one term of the probabilities after the other (smallest first)
-            // over all output blocks: consecutive MMAs never depend on each other
-            uint32_t b[HD / 16][4];
-#pragma unroll
-            for (int n2 = 0; n2 < HD / 16; ++n2)
-                ldsm_x4_trans(b[n2], Vb + (size_t)(kk * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * LD + n2 * 16 + (lane >> 4) * 8);
-#pragma unroll
-            for (int n2 = 0; n2 < HD / 16; ++n2) {
-                mma16816(o[2 * n2], a_lo, b[n2][0], b[n2][1]);
-                mma16816(o[2 * n2 + 1], a_lo, b[n2][2], b[n2][3]);
-            }
-#pragma unroll
-            for (int n2 = 0; n2 < HD / 16; ++n2) {
-                mma16816(o[2 * n2], a_mid, b[n2][0], b[n2][1]);
-                mma16816(o[2 * n2 + 1], a_mid, b[n2][2], b[n2][3]);
-            }
-#pragma unroll
-            for (int n2 = 0; n2 < HD / 16; ++n2) {
-                mma16816(o[2 * n2], a_hi, b[n2][0], b[n2][1]);
-                mma16816(o[2 * n2 + 1], a_hi, b[n2][2], b[n2][3]);
-            }
-        }
-        __syncthreads();  // this buffer is refilled two iterations from now
-    }
-
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
-        l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
-    }
-    const int ra = r0 + warp * 16 + g, rb = ra + 8;
-    const float inv_a = 1.0f / l_run[0], inv_b = 1.0f / l_run[1];
-#pragma unroll
-    for (int i = 0; i < HD / 8; ++i) {
-        const size_t col = (size_t)head * HD + i * 8 + 2 * q4;
-        if (ra < n_rows) *reinterpret_cast<uint32_t*>(out + (size_t)ra * d_model + col) = pack_bf16(o[i][0] * inv_a, o[i][1] * inv_a);
-        if (rb < n_rows) *reinterpret_cast<uint32_t*>(out + (size_t)rb * d_model + col) = pack_bf16(o[i][2] * inv_b, o[i][3] * inv_b);
-    }
-}
-
-template <int HD>
-static constexpr size_t fa_smem_bytes() { return (size_t)4 * kFaKeys * (HD + 8) * 2; }
-
-cudaError_t launch_flash_prefill(const __nv_bfloat16* q, const __nv_bfloat16* k_cache, const __nv_bfloat16* v_cache, __nv_bfloat16* out,
-                                 int n_rows, int pos0, int d_model, int kv_dim, int head_dim, int n_heads, int n_kv_heads, int max_seq,
-                                 float scale, cudaStream_t s) {
-    if (n_rows <= 0) return cudaErrorInvalidValue;
-    const dim3 grid((n_rows + kFaRows - 1) / kFaRows, n_heads);
-    const int group = n_heads / n_kv_heads;
-    if (head_dim == 128)
-        flash_prefill_kernel<128><<<grid, kFaThreads, fa_smem_bytes<128>(), s>>>(q, k_cache, v_cache, out, n_rows, pos0, d_model, kv_dim, group, max_seq, scale);
-    else if (head_dim == 64)
-        flash_prefill_kernel<64><<<grid, kFaThreads, fa_smem_bytes<64>(), s>>>(q, k_cache, v_cache, out, n_rows, pos0, d_model, kv_dim, group, max_seq, scale);
-    else
-        return cudaErrorInvalidValue;
-    return cudaGetLastError();
-}
-
 cudaError_t configure_prefill(int max_smem) {
     cudaError_t e;
     (void)max_smem;
@@ -733,9 +443,7 @@ cudaError_t configure_prefill(int max_smem) {
     if (sms > 0) g_gemm_ctas = sms;
     if ((e = cudaFuncSetAttribute(gemm_tn_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmCfg<256>::kSmem)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(gemm_tn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmCfg<128>::kSmem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(flash_prefill_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fa_smem_bytes<128>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(flash_prefill_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fa_smem_bytes<64>())) != cudaSuccess) return e;
-    return cudaSuccess;
+    return configure_prefill_attention();
 }
 
 }  // namespace asd

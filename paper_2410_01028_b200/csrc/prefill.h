@@ -5,7 +5,7 @@
 // With hundreds of rows the sublayer products are dense contractions, so they run as tcgen05 GEMMs: operand
 // tiles staged in shared memory by TMA (128-byte swizzle), accumulators in tensor memory, one elected thread
 // issuing tcgen05.mma, four epilogue warps reading the accumulators back with tcgen05.ld. Causal attention
-// over the prompt is a flash-style kernel on mma.sync. Row-wise work (embedding, RMSNorm, residual add with
+// over the prompt is a flash-style tcgen05 kernel (prefill_attn.cu). Row-wise work (embedding, RMSNorm, residual add with
 // the cosine sums) runs one CTA per row.
 #pragma once
 #include <cuda.h>
@@ -62,9 +62,11 @@ cudaError_t launch_resid_norm(int n_rows, int d, float* x, const float* c, const
 // sumcos[b] += sum over rows of cos_rows[b * stride + r], rows in a fixed order, double precision
 cudaError_t launch_sumcos(const float* cos_rows, int stride, int n_rows, int n_sub, double* sumcos, cudaStream_t s);
 
-// causal attention of prompt rows [0, n_rows) at positions pos0 + r over keys 0 .. pos0 + r of the cache
-cudaError_t launch_flash_prefill(const __nv_bfloat16* q, const __nv_bfloat16* k_cache, const __nv_bfloat16* v_cache, __nv_bfloat16* out,
-                                 int n_rows, int pos0, int d_model, int kv_dim, int head_dim, int n_heads, int n_kv_heads, int max_seq,
-                                 float scale, cudaStream_t s);
+// causal attention of prompt rows [0, n_rows) at positions pos0 + r over keys 0 .. pos0 + r of the cache. Tensor maps (bf16,
+// 128-byte swizzle): the queries [rows, d_model] in boxes of 64 columns x 128 rows, the caches [max_seq, kv_dim] in boxes of
+// 64 columns x 64 keys. head_dim 64 or 128.
+cudaError_t launch_flash_prefill(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, __nv_bfloat16* out, int n_rows, int pos0,
+                                 int d_model, int head_dim, int n_heads, int n_kv_heads, float scale, int* err, cudaStream_t s);
+cudaError_t configure_prefill_attention();
 
 }  // namespace asd

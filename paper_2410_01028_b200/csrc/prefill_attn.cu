@@ -1,0 +1,323 @@
+// Causal attention over the prompt on tcgen05 (see prefill.h).
+//
+// One CTA = 128 query rows of one head, two CTAs per SM. Scores S = Q K^T of 128 rows x 64 keys and the output O = P V
+// live in tensor memory; a thread owns one query row, so maximum, sum and mask need no exchange between threads.
+// The probabilities are fp32 and enter the P V product as the sum of three bf16 numbers (p = hi + mid + lo, cut off
+// at 8 mantissa bits each, which represents every fp32 probability exactly); with fewer terms the 2^-17 error of P
+// flips bf16 roundings of the attention output in about every second row.
+//
+// What bounds it: the tensor core. Per 64 keys an S tile takes 384 cycles (N = 64 with both operands in shared memory is
+// bound by the operand reads: 48 KB at 128 B per cycle) and the three P V products take 256 each; the softmax between
+// the two takes about 700-800 cycles of the other units (64 ex2 per row are 512 cycles of the SFUs), which the second
+// CTA of the SM covers. Tiles of 64 keys because O (128 columns) and S / P (128 columns: the three terms take 96)
+// of two CTAs then fill the 512 columns of tensor memory.
+//
+// The running maximum is only moved when it has grown by more than 2^8 (probabilities up to 256 are as exact as those
+// up to 1): moving it means reading, scaling and writing O in tensor memory, which random scores need once or
+// twice per row instead of once per tile.
+//
+// Measured (8192-token prompt, 32 heads of 128, per layer): 3.4 ms with mma.sync and 64-row tiles, 1.22 ms here, the tensor
+// core active half of the time: a CTA's own chain S -> softmax -> P V -> S is longer than the other CTA's share covers.
+#include "common.cuh"
+#include "prefill.h"
+#include "tcgen05.cuh"
+
+namespace asd {
+
+constexpr int kFaRows = 128, kFaKeys = 64, kFaThreads = 192, kFaStages = 2;
+constexpr int kFaTmemCols = 256;                       // O: 0-127; S: 128-191
+constexpr int kFaColS = 128, kFaColHi = 192, kFaColMid = 224, kFaColLo = 128;  // the lo terms take the place of S
+
+template <int HD>
+struct FaCfg {
+    static constexpr int kPanels = HD / 64;                      // panels of 64 columns (128 bytes, one swizzle span)
+    static constexpr uint32_t kQPanel = kFaRows * 128, kKvPanel = kFaKeys * 128;
+    static constexpr uint32_t kQBytes = kPanels * kQPanel, kKvBytes = kPanels * kKvPanel;
+    static constexpr size_t kSmem = kQBytes + 2 * kFaStages * kKvBytes + 1024 /* alignment */ + 128 /* barriers */;
+};
+
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ unsigned long long fadd2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// the upper halves of two words: bf16 pairs cut off from two fp32 numbers (a in the low half)
+__device__ __forceinline__ uint32_t upper_halves(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); }
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};" ::"r"(r[0]),
+        "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]),
+        "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+        : "memory");
+}
+
+// 32 scores of one row -> probabilities 2^(s c - m c), their sum added to sum2, their three bf16 terms to tensor memory
+__device__ __forceinline__ void probabilities32(const uint32_t (&s)[32], unsigned long long c2, unsigned long long nmc2, unsigned long long& sum2,
+                                                uint32_t t_hi, uint32_t t_mid, uint32_t t_lo) {
+    uint32_t p[32], w[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        float a, b;
+        unpack2(ffma2(pack2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), c2, nmc2), a, b);
+        a = ex2(a), b = ex2(b);
+        sum2 = fadd2(sum2, pack2(a, b));
+        p[2 * i] = __float_as_uint(a), p[2 * i + 1] = __float_as_uint(b);
+        w[i] = upper_halves(p[2 * i], p[2 * i + 1]);
+    }
+    tmem_st16(t_hi, w);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) p[i] = __float_as_uint(__uint_as_float(p[i]) - __uint_as_float(p[i] & 0xFFFF0000u));  // exact
+#pragma unroll
+    for (int i = 0; i < 16; ++i) w[i] = upper_halves(p[2 * i], p[2 * i + 1]);
+    tmem_st16(t_mid, w);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) p[i] = __float_as_uint(__uint_as_float(p[i]) - __uint_as_float(p[i] & 0xFFFF0000u));  // exact, 8 bits left
+#pragma unroll
+    for (int i = 0; i < 16; ++i) w[i] = upper_halves(p[2 * i], p[2 * i + 1]);
+    tmem_st16(t_lo, w);
+}
+
+// Warps 0-3: softmax and epilogue, thread = query row. Warp 4: TMA producer (one lane). Warp 5: issues the MMAs (one lane)
+// and owns the tensor-memory allocation. Barriers: q_full, k_full / v_full[s] (bytes landed), k_empty / v_empty[s] (the
+// MMAs reading the stage have finished), s_full (S of tile j is complete, and with it every earlier MMA: O holds the
+// tiles before j and P may be overwritten; phase n_kt: O is complete), p_full (the 128 rows' P of tile j are in tensor
+// memory). The MMAs of one CTA run in issue order: P V of tile j, then S of tile j + 1 over the columns of P's lo terms.
+template <int HD>
+__global__ void __launch_bounds__(kFaThreads, 2)
+flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+                     __nv_bfloat16* __restrict__ out, int n_rows, int pos0, int d_model, int group, float scale_log2, int* err_words) {
+    using Cfg = FaCfg<HD>;
+    extern __shared__ unsigned char fa_smem_raw[];
+    unsigned char* base = fa_smem_raw + ((1024u - (smem_u32(fa_smem_raw) & 1023u)) & 1023u);
+    unsigned char* k_smem = base + Cfg::kQBytes;
+    unsigned char* v_smem = k_smem + kFaStages * Cfg::kKvBytes;
+    uint64_t* q_full = reinterpret_cast<uint64_t*>(v_smem + kFaStages * Cfg::kKvBytes);
+    uint64_t *k_full = q_full + 1, *k_empty = k_full + kFaStages, *v_full = k_empty + kFaStages, *v_empty = v_full + kFaStages;
+    uint64_t *s_full = v_empty + kFaStages, *p_full = s_full + 1, *drained = p_full + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drained + 1);
+    volatile int* err = err_words;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int head = blockIdx.x, kvh = head / group;
+    const int r0 = (gridDim.y - 1 - blockIdx.y) * kFaRows;  // the tiles with the most keys start first
+    const int last_row = min(r0 + kFaRows, n_rows) - 1;
+    const int n_kt = (pos0 + last_row) / kFaKeys + 1;
+
+    if (threadIdx.x == 0) {
+        mbar_init(q_full, 1);
+        for (int s = 0; s < kFaStages; ++s) mbar_init(&k_full[s], 1), mbar_init(&k_empty[s], 1), mbar_init(&v_full[s], 1), mbar_init(&v_empty[s], 1);
+        mbar_init(s_full, 1);
+        mbar_init(p_full, kFaRows);
+        mbar_init(drained, 1);
+        mbar_fence_init();
+    }
+    if (warp == 5) {
+        tmem_alloc(tmem_slot, kFaTmemCols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 4) {
+        if (lane == 0) {
+            mbar_expect_tx(q_full, Cfg::kQBytes);
+            for (int p = 0; p < Cfg::kPanels; ++p) tma_load_2d(base + p * Cfg::kQPanel, &tm_q, head * HD + p * 64, r0, q_full);
+            bool ok = true;
+            int nk = 0, nv = 0;  // K and V tiles requested so far
+            while (nv < n_kt && ok) {
+                // K runs one tile ahead of V: S of tile j + 1 is issued right behind P V of tile j
+                if (nk < n_kt && nk <= nv + 1) {
+                    const int s = nk % kFaStages;
+                    if (nk >= kFaStages) ok = mbar_wait(&k_empty[s], (uint32_t)((nk / kFaStages - 1) & 1), err, kErrAttnWait, 0, nk, s, 1);
+                    if (!ok) break;
+                    mbar_expect_tx(&k_full[s], Cfg::kKvBytes);
+                    for (int p = 0; p < Cfg::kPanels; ++p)
+                        tma_load_2d(k_smem + s * Cfg::kKvBytes + p * Cfg::kKvPanel, &tm_k, kvh * HD + p * 64, nk * kFaKeys, &k_full[s]);
+                    ++nk;
+                    if (nk == 1 && n_kt > 1) continue;
+                }
+                const int s = nv % kFaStages;
+                if (nv >= kFaStages) ok = mbar_wait(&v_empty[s], (uint32_t)((nv / kFaStages - 1) & 1), err, kErrAttnWait, 0, nv, s, 2);
+                if (!ok) break;
+                mbar_expect_tx(&v_full[s], Cfg::kKvBytes);
+                for (int p = 0; p < Cfg::kPanels; ++p)
+                    tma_load_2d(v_smem + s * Cfg::kKvBytes + p * Cfg::kKvPanel, &tm_v, kvh * HD + p * 64, nv * kFaKeys, &v_full[s]);
+                ++nv;
+            }
+            if (!ok || *err != kErrNone) {
+                // abandoned: let the copies still in flight land before the CTA gives its shared memory back
+                const long long t0 = clock64();
+                auto landed = [&](uint64_t* bar, int n) { return n <= 0 || mbar_try_wait(bar, (uint32_t)((n - 1) & 1)); };
+                bool all = false;
+                while (!all && clock64() - t0 < 20000000LL) {
+                    all = landed(q_full, 1);
+                    for (int s = 0; s < kFaStages; ++s)
+                        all = all && landed(&k_full[s], (nk + kFaStages - 1 - s) / kFaStages) && landed(&v_full[s], (nv + kFaStages - 1 - s) / kFaStages);
+                }
+            }
+        }
+    } else if (warp == 5) {
+        if (lane == 0) {
+            constexpr uint32_t idesc_s = umma_idesc_bf16(kFaRows, kFaKeys);
+            constexpr uint32_t idesc_o = umma_idesc_bf16(kFaRows, HD) | (1u << 16);  // V is [key][dimension]: N-major
+            const uint32_t q_addr = smem_u32(base);
+            bool ok = mbar_wait(q_full, 0, err, kErrAttnWait, 1, 0, 0, 3);
+            auto scores = [&](int j) {  // S of tile j
+                const int s = j % kFaStages;
+                ok = ok && mbar_wait(&k_full[s], (uint32_t)((j / kFaStages) & 1), err, kErrAttnWait, 1, j, s, 4);
+                if (!ok) return;
+                tc_fence_after();
+                const uint32_t k_addr = smem_u32(k_smem) + s * Cfg::kKvBytes;
+#pragma unroll
+                for (int k = 0; k < HD / 16; ++k)
+                    tc_mma_bf16(tmem + kFaColS, umma_desc_k128(q_addr + (k / 4) * Cfg::kQPanel) + 2 * (k % 4),
+                                umma_desc_k128(k_addr + (k / 4) * Cfg::kKvPanel) + 2 * (k % 4), idesc_s, k != 0);
+                tc_commit(&k_empty[s]);
+                tc_commit(s_full);
+            };
+            scores(0);
+            for (int j = 0; j < n_kt && ok; ++j) {
+                const int s = j % kFaStages;
+                ok = mbar_wait(&v_full[s], (uint32_t)((j / kFaStages) & 1), err, kErrAttnWait, 1, j, s, 5) &&
+                     mbar_wait(p_full, (uint32_t)(j & 1), err, kErrAttnWait, 1, j, s, 6);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t v_desc = umma_desc_mn128(smem_u32(v_smem) + s * Cfg::kKvBytes, Cfg::kKvPanel);
+#pragma unroll
+                for (int t = 0; t < 3; ++t) {  // lo, mid, hi: the smallest terms first
+                    const uint32_t a = tmem + (t == 0 ? kFaColLo : (t == 1 ? kFaColMid : kFaColHi));
+#pragma unroll
+                    for (int k = 0; k < kFaKeys / 16; ++k)  // 16 keys: 8 columns of P, 2048 bytes of V
+                        tc_mma_bf16_ts(tmem, a + 8 * k, v_desc + (uint64_t)(128 * k), idesc_o, (j | t | k) != 0);
+                }
+                tc_commit(&v_empty[s]);
+                if (j + 1 < n_kt) scores(j + 1);
+                else tc_commit(s_full);  // O is complete
+            }
+            if (!ok) {  // abandoned: the MMAs already issued end before the tensor memory is freed
+                tc_commit(drained);
+                const long long t0 = clock64();
+                while (!mbar_try_wait(drained, 0) && clock64() - t0 < 20000000LL) {
+                }
+            }
+        }
+    } else {
+        const int row = r0 + threadIdx.x;
+        const int pos = pos0 + min(row, n_rows - 1);  // rows past the prompt are computed like the last one and not stored
+        const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+        const unsigned long long c2 = pack2(scale_log2, scale_log2);
+        float m = 0.f;
+        unsigned long long sum2 = pack2(0.f, 0.f);
+        bool ok = true;
+        for (int j = 0; j < n_kt; ++j) {
+            ok = mbar_wait(s_full, (uint32_t)(j & 1), err, kErrAttnWait, 2, j, 0, 7);
+            ok = __all_sync(0xffffffffu, ok);  // tensor-memory accesses are warp-wide
+            if (!ok) break;
+            tc_fence_after();
+            uint32_t s0[32], s1[32];
+            tmem_ld32_async(lane_base + kFaColS, s0);
+            tmem_ld32_async(lane_base + kFaColS + 32, s1);
+            tmem_ld_wait(s0);
+            tmem_ld_wait(s1);
+            const int key0 = j * kFaKeys;
+            if (key0 + kFaKeys - 1 > pos0 + r0) {  // a tile on the diagonal: the row at position p sees keys <= p
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    if (key0 + i > pos) s0[i] = 0xFF800000u;
+                    if (key0 + 32 + i > pos) s1[i] = 0xFF800000u;
+                }
+            }
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) {
+                mx[(i >> 1) & 3] = fmaxf(mx[(i >> 1) & 3], fmaxf(__uint_as_float(s0[i]), __uint_as_float(s0[i + 1])));
+                mx[(i >> 1) & 3] = fmaxf(mx[(i >> 1) & 3], fmaxf(__uint_as_float(s1[i]), __uint_as_float(s1[i + 1])));
+            }
+            const float tile_max = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+            if (j == 0) {
+                m = tile_max;  // finite: key 0 is visible to every row
+            } else if (__any_sync(0xffffffffu, (tile_max - m) * scale_log2 > 8.0f)) {
+                const float m_new = fmaxf(m, tile_max), alpha = ex2((m - m_new) * scale_log2);
+                m = m_new;
+                float a, b;
+                unpack2(sum2, a, b);
+                sum2 = pack2(a * alpha, b * alpha);
+#pragma unroll 1
+                for (int c = 0; c < HD; c += 32) {
+                    uint32_t o[32];
+                    tmem_ld32_async(lane_base + c, o);
+                    tmem_ld_wait(o);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                    tmem_st32(lane_base + c, o);
+                }
+            }
+            const float nmc = -m * scale_log2;
+            const unsigned long long nmc2 = pack2(nmc, nmc);
+            // the lo terms overwrite S: both halves have been read
+            probabilities32(s0, c2, nmc2, sum2, lane_base + kFaColHi, lane_base + kFaColMid, lane_base + kFaColLo);
+            probabilities32(s1, c2, nmc2, sum2, lane_base + kFaColHi + 16, lane_base + kFaColMid + 16, lane_base + kFaColLo + 16);
+            tmem_st_wait();
+            tc_fence_before();
+            mbar_arrive(p_full);
+        }
+        if (ok) ok = mbar_wait(s_full, (uint32_t)(n_kt & 1), err, kErrAttnWait, 2, n_kt, 0, 8);
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok) {
+            tc_fence_after();
+            float a, b;
+            unpack2(sum2, a, b);
+            const float inv = 1.0f / (a + b);
+            __nv_bfloat16* dst = out + (size_t)row * d_model + (size_t)head * HD;
+#pragma unroll
+            for (int c = 0; c < HD; c += 32) {
+                float v[32];
+                tmem_ld32(lane_base + c, v);
+                if (row < n_rows) {
+                    uint32_t w[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) w[i] = pack_bf16(v[2 * i] * inv, v[2 * i + 1] * inv);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        reinterpret_cast<uint4*>(dst + c)[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 5) {
+        tc_fence_after();
+        tmem_dealloc(tmem, kFaTmemCols);
+    }
+}
+
+cudaError_t launch_flash_prefill(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, __nv_bfloat16* out, int n_rows, int pos0,
+                                 int d_model, int head_dim, int n_heads, int n_kv_heads, float scale, int* err, cudaStream_t s) {
+    if (n_rows <= 0) return cudaErrorInvalidValue;
+    const dim3 grid(n_heads, (n_rows + kFaRows - 1) / kFaRows);
+    const int group = n_heads / n_kv_heads;
+    const float scale_log2 = scale * 1.4426950408889634f;
+    if (head_dim == 128)
+        flash_prefill_kernel<128><<<grid, kFaThreads, FaCfg<128>::kSmem, s>>>(tm_q, tm_k, tm_v, out, n_rows, pos0, d_model, group, scale_log2, err);
+    else if (head_dim == 64)
+        flash_prefill_kernel<64><<<grid, kFaThreads, FaCfg<64>::kSmem, s>>>(tm_q, tm_k, tm_v, out, n_rows, pos0, d_model, group, scale_log2, err);
+    else
+        return cudaErrorInvalidValue;
+    return cudaGetLastError();
+}
+
+cudaError_t configure_prefill_attention() {
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(flash_prefill_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FaCfg<128>::kSmem)) != cudaSuccess) return e;
+    return cudaFuncSetAttribute(flash_prefill_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FaCfg<64>::kSmem);
+}
+
+}  // namespace asd

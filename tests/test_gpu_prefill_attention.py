@@ -1,0 +1,45 @@
+"""GPU parity of the prompt attention kernel at the edges of its tiles (128 query rows x 64 keys): prompts that end one
+row before, at and one row behind a tile border, and prompts appended to a cache whose length is not a multiple of a
+tile, against the CPU oracle; with weights large enough that the running maximum has to move between tiles."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from helpers import COS_TOL
+
+pytestmark = pytest.mark.gpu
+
+HD128 = synth.DecoderShape(n_layers=2, d_model=256, n_heads=2, head_dim=128, d_ffn=264, vocab=97, n_kv_heads=1)
+HD64 = synth.DecoderShape(n_layers=2, d_model=256, n_heads=4, head_dim=64, d_ffn=264, vocab=97, n_kv_heads=2)
+
+
+@pytest.mark.parametrize("shape", [HD128, HD64], ids=["hd128", "hd64"])
+@pytest.mark.parametrize("std", [0.02, 0.15])  # 0.15: scores of several units, the maximum of a row grows by more than 2^8
+@pytest.mark.parametrize("parts", [(2,), (63,), (64,), (65,), (127,), (128, 1), (129,), (33, 96), (61, 131), (192, 65), (257, 300)])
+def test_prompt_attention_at_tile_edges(shape, std, parts):
+    import paper_2410_01028_b200 as asd
+    model = synth.make_model(shape, seed=7, std=std)
+    n = sum(parts)
+    dec = asd.Decoder(shape, max_seq=n, max_draft=1)
+    dec.load_weights_host(model)
+    dec.set_prefill_mode(asd.PREFILL_GEMM)
+    orc = oracle.Oracle(model, max_seq=n)
+    prompt = synth.make_prompt(shape.vocab, n, seed=11)
+    at = 0
+    for part in parts:
+        if part == 1:
+            dec.set_prefill_mode(asd.PREFILL_AUTO)  # a single row takes the row passes
+        dec.prefill(prompt[at:at + part])
+        orc.prefill(prompt[at:at + part])
+        at += part
+    ca_g, cm_g, rows = dec.get_similarity()
+    ca_o, cm_o, _ = orc.similarity()
+    assert rows == n
+    assert np.abs(ca_g - ca_o).max() <= COS_TOL and np.abs(cm_g - cm_o).max() <= COS_TOL
+    # the second layer's K and V rows carry the first layer's attention output of the same position. A flipped bf16
+    # rounding upstream moves them by about 1e-3 of their scale; the bound is one ulp plus 1e-2 of the row's scale
+    for p in range(n):
+        for g, o in zip(dec.get_kv(1, p), orc.kv(1, p)):
+            g = synth.bf16_to_f32(g)
+            assert np.all(np.abs(g - o) <= 2 ** -7 * np.abs(o) + 1e-2 * np.abs(o).max()), (p, np.abs(g - o).max(), np.abs(o).max())
