@@ -190,7 +190,8 @@ struct Layout {
     int chunk_stride;
     // dense prompt path: row-major copies of the sublayer matrices (one block per layer) and activations of a chunk
     size_t rm_layers, rm_layer_stride, rm_wqkv, rm_wo, rm_wgu, rm_wd;
-    size_t pf_x, pf_xn, pf_q, pf_a, pf_t, pf_c, pf_cos;  // pf_c: two buffers (the halves of a product cut along its reduction dimension)
+    size_t pf_x, pf_xn, pf_q, pf_a, pf_t, pf_c, pf_cos;
+    size_t pf_c_rows;  // rows of pf_c: the parts of W_o / W_d products of a chunk's rows lie behind one another in it
     int pf_rows;  // prompt rows per chunk of the dense path (0: shape not supported by it)
 };
 
@@ -305,7 +306,8 @@ static Layout make_layout(const asd_config& c) {
         L.pf_q = take(R * d * 2);
         L.pf_a = take(R * d * 2);
         L.pf_t = take(R * f * 2);
-        L.pf_c = take((size_t)2 * R * d * 4);
+        L.pf_c_rows = std::max<size_t>(2 * R, 1024);
+        L.pf_c = take(L.pf_c_rows * d * 4);
         L.pf_cos = take((size_t)2 * c.n_layers * R * 4);
     }
     L.total = o;
@@ -345,7 +347,7 @@ struct asd_ctx {
     int last_n_stages = 0;
     int prefill_mode = ASD_PREFILL_AUTO;
     // tensor maps of the dense prompt path (host copies, passed to the kernels by value): activations with boxes of
-    // 64 x 128, and per layer the four matrices with boxes of 64 x 128 ([0..3]) and 64 x 256 ([4..7])
+    // 64 x 128, and per layer the kWBoxes maps of each of the four matrices
     CUtensorMap tm_xn{}, tm_q{}, tm_a{}, tm_t{};
     std::vector<CUtensorMap> tm_w;
     std::vector<CUtensorMap> tm_kv;  // per layer the K and the V cache (the pass kernel reads its own copy in the workspace)
@@ -422,6 +424,13 @@ static bool encode_operand_map(EncodeTiledFn encode, CUtensorMap* m, void* base,
                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// the tensor maps of one weight matrix, one per box height that the product's tiles need
+static bool encode_weight_maps(EncodeTiledFn encode, CUtensorMap* m, void* base, size_t inner, size_t rows) {
+    for (int i = 0; i < kWBoxes; ++i)
+        if (!encode_operand_map(encode, m + i, base, inner, rows, (uint32_t)kWBoxRows[i])) return false;
+    return true;
+}
+
 static EncodeTiledFn tensor_map_encoder() {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
@@ -465,18 +474,13 @@ static int make_tensor_maps(asd_ctx* x) {
                   encode_operand_map(encode, &x->tm_q, x->ws + ly.pf_q, d, R, kGemmBM) &&
                   encode_operand_map(encode, &x->tm_a, x->ws + ly.pf_a, d, R, kGemmBM) &&
                   encode_operand_map(encode, &x->tm_t, x->ws + ly.pf_t, f, R, kGemmBM);
-        x->tm_w.assign((size_t)8 * L, CUtensorMap{});
         x->tm_kv = maps;
+        x->tm_w.assign((size_t)4 * kWBoxes * L, CUtensorMap{});
         for (int l = 0; l < L && ok; ++l) {
             unsigned char* rw = x->ws + ly.rm_layers + (size_t)l * ly.rm_layer_stride;
-            for (int v = 0; v < 2 && ok; ++v) {
-                const uint32_t bn = v ? 256u : 128u;
-                CUtensorMap* m = &x->tm_w[(size_t)l * 8 + v * 4];
-                ok = encode_operand_map(encode, m + 0, rw + ly.rm_wqkv, d, d + 2 * kvd, bn) &&
-                     encode_operand_map(encode, m + 1, rw + ly.rm_wo, d, d, bn) &&
-                     encode_operand_map(encode, m + 2, rw + ly.rm_wgu, d, 2 * f, bn) &&
-                     encode_operand_map(encode, m + 3, rw + ly.rm_wd, f, d, bn);
-            }
+            CUtensorMap* m = &x->tm_w[(size_t)l * 4 * kWBoxes];
+            ok = encode_weight_maps(encode, m, rw + ly.rm_wqkv, d, d + 2 * kvd) && encode_weight_maps(encode, m + kWBoxes, rw + ly.rm_wo, d, d) &&
+                 encode_weight_maps(encode, m + 2 * kWBoxes, rw + ly.rm_wgu, d, 2 * f) && encode_weight_maps(encode, m + 3 * kWBoxes, rw + ly.rm_wd, f, d);
         }
         if (!ok) return fail(x, ASD_ERR_CUDA, "cuTensorMapEncodeTiled failed for an operand of the dense prompt path");
     }
@@ -997,24 +1001,11 @@ extern "C" int asd_reset(asd_ctx* x) {
 }
 
 // ---------------------------------------------------------------- prefill (Section 3.2)
-// One sublayer product of the dense prompt path: the 64 x 256 weight boxes when that still gives every SM a tile. A
-// product with fp32 output (W_o, W_d) that has fewer such tiles than SMs is cut in two along its reduction dimension
-// instead of taking the 128-column tiles, which run at half the rate per SM (bound by shared-memory bandwidth): the
-// two halves are work items of their own and the row kernel that follows adds them (half 0 + half 1). *split_out
-// tells the caller whether it was.
-static int dense_gemm(asd_ctx* x, const CUtensorMap& tm_a, int layer, int which, int M, int N, int K, GemmEpi ep, bool* split_out = nullptr) {
-    const int m_tiles = (M + kGemmBM - 1) / kGemmBM;
-    const int tiles256 = ((N + 255) / 256) * m_tiles;
-    // cut in two when the 256-column tiles do not fill the SMs, or when twice as many half-length work items take fewer
-    // rounds' worth of time over the SMs (a half item costs a little more than half an item: 0.525)
-    const int sms = x->dev->num_sms;
-    const bool fewer_rounds = 525LL * ((2 * tiles256 + sms - 1) / sms) < 1000LL * ((tiles256 + sms - 1) / sms);
-    const bool split = ep.mode == kGemmF32 && split_out && K >= 2048 && (tiles256 < sms || fewer_rounds);
-    const int bn = (tiles256 >= x->dev->num_sms || split) ? 256 : 128;
-    ep.k_split = split ? 2 : 1;
-    if (split_out) *split_out = split;
-    const CUtensorMap& tm_w = x->tm_w[(size_t)layer * 8 + (bn == 256 ? 4 : 0) + which];
-    ASD_CUDA(x, launch_gemm_tn(tm_a, tm_w, M, N, K, bn, ep, x->stream));
+// One sublayer product of the dense prompt path. W_o and W_d (fp32 output) may come in parts of their reduction
+// dimension, which the row kernel that follows adds: as many as fit the buffer, up to eight.
+static int dense_gemm(asd_ctx* x, const CUtensorMap& tm_a, int layer, int which, int M, int N, int K, const GemmEpi& ep, int* parts = nullptr) {
+    const int max_parts = parts ? (int)std::min<size_t>(8, x->lay.pf_c_rows / M) : 1;
+    ASD_CUDA(x, launch_gemm_tn(tm_a, &x->tm_w[((size_t)layer * 4 + which) * kWBoxes], M, N, K, max_parts, ep, x->stream, parts));
     x->stats.kernel_launches += 1;
     return ASD_OK;
 }
@@ -1056,18 +1047,18 @@ static int prefill_dense(asd_ctx* x, const int32_t* dev_tokens, int n, int pos0)
             o.err = err;
             o.mode = kGemmF32;
             o.c = pc, o.ldc = d;
-            o.c_split_stride = (size_t)R * d;
-            bool split = false;
-            if ((rc = dense_gemm(x, x->tm_a, l, 1, rows, d, d, o, &split))) return rc;
-            ASD_CUDA(x, launch_resid_norm(rows, d, px, pc, split ? pc + (size_t)R * d : nullptr, gain(l, ly.l_mlp_norm), c.rms_eps, pxn,
+            o.c_part_stride = (size_t)rows * d;
+            int parts = 1;
+            if ((rc = dense_gemm(x, x->tm_a, l, 1, rows, d, d, o, &parts))) return rc;
+            ASD_CUDA(x, launch_resid_norm(rows, d, px, pc, parts, o.c_part_stride, gain(l, ly.l_mlp_norm), c.rms_eps, pxn,
                                           pcos + (size_t)l * R, s));
             GemmEpi g{};
             g.err = err;
             g.mode = kGemmSwiglu;
             g.t = pt, g.ldt = f;
             if ((rc = dense_gemm(x, x->tm_xn, l, 2, rows, 2 * f, d, g))) return rc;
-            if ((rc = dense_gemm(x, x->tm_t, l, 3, rows, d, f, o, &split))) return rc;
-            ASD_CUDA(x, launch_resid_norm(rows, d, px, pc, split ? pc + (size_t)R * d : nullptr, l + 1 < L ? gain(l + 1, ly.l_attn_norm) : nullptr, c.rms_eps, pxn,
+            if ((rc = dense_gemm(x, x->tm_t, l, 3, rows, d, f, o, &parts))) return rc;
+            ASD_CUDA(x, launch_resid_norm(rows, d, px, pc, parts, o.c_part_stride, l + 1 < L ? gain(l + 1, ly.l_attn_norm) : nullptr, c.rms_eps, pxn,
                                           pcos + (size_t)(L + l) * R, s));
             x->stats.kernel_launches += 3;
         }
@@ -1583,11 +1574,9 @@ extern "C" int asd_gemm_bf16(void* cuda_stream, int32_t M, int32_t N, int32_t K,
     if (device_info(&dv) != cudaSuccess) return ASD_ERR_CUDA;
     EncodeTiledFn encode = tensor_map_encoder();
     if (!encode) return ASD_ERR_CUDA;
-    const int m_tiles = (M + kGemmBM - 1) / kGemmBM;
-    const int bn = (((N + 255) / 256) * m_tiles >= dv->num_sms) ? 256 : 128;
-    CUtensorMap tm_a, tm_w;
+    CUtensorMap tm_a, tm_w[kWBoxes];
     if (!encode_operand_map(encode, &tm_a, const_cast<uint16_t*>(A), (size_t)K, (size_t)M, kGemmBM) ||
-        !encode_operand_map(encode, &tm_w, const_cast<uint16_t*>(W), (size_t)K, (size_t)N, (uint32_t)bn))
+        !encode_weight_maps(encode, tm_w, const_cast<uint16_t*>(W), (size_t)K, (size_t)N))
         return ASD_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     if (cudaMemsetAsync(dev_status, 0, 32, s) != cudaSuccess) return ASD_ERR_CUDA;
@@ -1595,7 +1584,7 @@ extern "C" int asd_gemm_bf16(void* cuda_stream, int32_t M, int32_t N, int32_t K,
     e.mode = kGemmF32;
     e.err = dev_status;
     e.c = C, e.ldc = N;
-    if (launch_gemm_tn(tm_a, tm_w, M, N, K, bn, e, s) != cudaSuccess) return ASD_ERR_CUDA;
+    if (launch_gemm_tn(tm_a, tm_w, M, N, K, 1, e, s) != cudaSuccess) return ASD_ERR_CUDA;
     return ASD_OK;
 }
 

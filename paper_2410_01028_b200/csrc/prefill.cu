@@ -1,6 +1,8 @@
 // Kernels of the dense prompt path (see prefill.h).
 #include "prefill.h"
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "ring.cuh"
 #include "tcgen05.cuh"
@@ -9,9 +11,15 @@ namespace asd {
 
 // ============================================================================================ GEMM epilogues
 // One call per (row, 32 consecutive columns starting at col0) with the fp32 accumulators in v.
-__device__ __forceinline__ void epi_f32(const GemmEpi& ep, int row, int col0, int N, const float (&v)[32], int half) {
-    float* dst = ep.c + (size_t)half * ep.c_split_stride + (size_t)row * ep.ldc + col0;
-    if (col0 + 32 <= N && (ep.ldc & 3) == 0) {
+__device__ __forceinline__ void epi_f32(const GemmEpi& ep, int row, int col0, int N, const float (&v)[32], int part) {
+    float* dst = ep.c + (size_t)part * ep.c_part_stride + (size_t)row * ep.ldc + col0;
+    if (col0 + 32 <= N && (((ep.ldc | ep.c_part_stride) * 4) | ((uintptr_t)ep.c & 31)) % 32 == 0) {
+        uint32_t w[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) w[i] = __float_as_uint(v[i]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) st_global_v8(dst + 8 * i, w + 8 * i);
+    } else if (col0 + 32 <= N && (ep.ldc & 3) == 0) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) reinterpret_cast<float4*>(dst)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
     } else {
@@ -30,11 +38,15 @@ __device__ __forceinline__ void epi_swiglu(const GemmEpi& ep, int row, int col0,
         t[i] = g / (1.0f + expf(-g)) * u;
     }
     if (col0 + 32 <= N && (ep.ldt & 7) == 0) {
-        uint4 o0, o1;
-        o0.x = pack_bf16(t[0], t[1]), o0.y = pack_bf16(t[2], t[3]), o0.z = pack_bf16(t[4], t[5]), o0.w = pack_bf16(t[6], t[7]);
-        o1.x = pack_bf16(t[8], t[9]), o1.y = pack_bf16(t[10], t[11]), o1.z = pack_bf16(t[12], t[13]), o1.w = pack_bf16(t[14], t[15]);
-        reinterpret_cast<uint4*>(dst)[0] = o0;
-        reinterpret_cast<uint4*>(dst)[1] = o1;
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = pack_bf16(t[2 * i], t[2 * i + 1]);
+        if ((ep.ldt & 15) == 0) {
+            st_global_v8(dst, w);
+        } else {
+            reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            reinterpret_cast<uint4*>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        }
     } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i)
@@ -42,20 +54,19 @@ __device__ __forceinline__ void epi_swiglu(const GemmEpi& ep, int row, int col0,
     }
 }
 
-// head_dim is a multiple of 32 and the q, k and v column ranges start at multiples of head_dim, so the 32 columns
-// belong to one head of one of q, k, v.
+// head_dim is 64 or 128 and the q, k and v column ranges start at multiples of head_dim, so the 32 columns
+// belong to one head of one of q, k, v, and all rows and row parts are 32-byte aligned.
 __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, int N, const float (&v)[32]) {
     if (col0 >= N) return;
     const int pos = ep.pos0 + row;
     const int hd = ep.head_dim, half = hd >> 1;
     if (col0 >= ep.d_model + ep.kv_dim) {  // values: natural order, no rotation
         __nv_bfloat16* dst = ep.v_cache + (size_t)pos * ep.kv_dim + (col0 - ep.d_model - ep.kv_dim);
-        uint4 o[4];
-        uint32_t* w = reinterpret_cast<uint32_t*>(o);
+        uint32_t w[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) w[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) reinterpret_cast<uint4*>(dst)[i] = o[i];
+        st_global_v8(dst, w);
+        st_global_v8(dst + 16, w + 8);
         return;
     }
     const bool is_q = col0 < ep.d_model;
@@ -78,46 +89,83 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
     __nv_bfloat16* base = is_q ? ep.q + (size_t)row * ep.d_model : ep.k_cache + (size_t)pos * ep.kv_dim;
     __nv_bfloat16* dlo = base + (size_t)head * hd + j0;
     __nv_bfloat16* dhi = dlo + half;
-    uint4 o[2];
-    uint32_t* w = reinterpret_cast<uint32_t*>(o);
+    uint32_t w[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) w[i] = pack_bf16(lo[2 * i], lo[2 * i + 1]);
-    reinterpret_cast<uint4*>(dlo)[0] = o[0];
-    reinterpret_cast<uint4*>(dlo)[1] = o[1];
+    st_global_v8(dlo, w);
 #pragma unroll
     for (int i = 0; i < 8; ++i) w[i] = pack_bf16(hi[2 * i], hi[2 * i + 1]);
-    reinterpret_cast<uint4*>(dhi)[0] = o[0];
-    reinterpret_cast<uint4*>(dhi)[1] = o[1];
+    st_global_v8(dhi, w);
 }
 
 // ============================================================================================ the GEMM
-// Persistent CTAs (one per SM) walk the 128 x BN tiles of the product, row tiles fastest. Warp 0 (one lane) is the TMA
-// producer, warp 1 (one lane) issues the MMAs and owns the tensor-memory allocation, warps 2-5 are the epilogue (warp
-// w reads lanes 32 * (w % 4) .. + 31 of tensor memory, the quarter its position in the warp group gives it access
-// to). The accumulator is double-buffered in tensor memory (2 x BN columns), so the epilogue of a tile runs while the
-// MMAs of the next tile are already filling the other buffer. Barriers: full[s] (TMA bytes landed in stage s),
-// empty[s] (the MMAs reading stage s have finished: tcgen05.commit), acc_full[b] (all MMAs of the tile in buffer b
-// have finished), acc_empty[b] (the 128 epilogue threads have read buffer b). Ragged edges: TMA fills out-of-range
+// Persistent units (CG = 1: one SM; CG = 2: a cluster of two SMs) walk the 128 * CG x BN tiles of the product, row tiles
+// fastest. Warp 0 (one lane) is the TMA producer, warp 1 (one lane) issues the MMAs and owns the tensor-memory allocation,
+// warps 2-5 are the epilogue (warp w reads lanes 32 * (w % 4) .. + 31 of tensor memory, the quarter its position in the
+// warp group gives it access to). The accumulator is double-buffered in tensor memory (2 x BN columns), so the epilogue
+// of a tile runs while the MMAs of the next tile are already filling the other buffer. Barriers: full[s] (TMA bytes landed
+// in stage s), empty[s] (the MMAs reading stage s have finished: tcgen05.commit), acc_full[b] (all MMAs of the tile in
+// buffer b have finished), acc_empty[b] (the epilogue warps have read buffer b). Ragged edges: TMA fills out-of-range
 // rows and reduction elements with zeros; the epilogue skips rows >= M and columns >= N. Every wait is bounded; after
 // a failed wait the roles fall through to the common exit, where the producer lets its copies in flight land and
 // the tensor memory is freed.
+//
+// What bounds it: an SM takes in at most 64 bytes per cycle from L2 (measured: 32 KB per 64 elements of the reduction at
+// 0.28 us, whatever the tile does with them). A 128 x 256 tile on one SM wants 48 KB per 512 cycles of MMA and is held
+// at two thirds of the tensor rate (0.37 us per 64 elements); two SMs sharing a 256 x 256 tile (cta_group::2, CG = 2: each
+// stages its 128 rows of A and half of the rows of W and keeps its 128 rows of the accumulator) want 32 KB each and run at
+// 0.285 us, 90 % tensor activity, until the power limit takes the clock down (2048 x 22016 x 4096: 337 us -> 299 us back
+// to back). With CG = 2 the leader (rank 0) issues the MMAs; full[s] lives in the leader and counts both CTAs' bytes;
+// empty[s] and acc_full[b] are signalled in both CTAs by multicast commits; acc_empty[b] lives in the leader and counts
+// the epilogue warps of both.
+//
+// Units and tiles rarely divide evenly, so the host picks the kind of unit, the tile width and, for the products whose
+// consumer adds them up (fp32 output), the number of parts the reduction dimension is cut into by the time they take
+// over the rounds (launch_gemm_tn). Cutting the tiles of a last round with an exchange of the parts through L2 inside the
+// kernel (last arriver adds) was measured: 8-10 us per exchange, more than the part of a round it saves.
 constexpr int kGemmThreads = 192;
 static int g_gemm_ctas = 148;  // persistent CTAs per launch: the SM count of the device (set by configure_prefill)
 
-template <int BN>
+template <int BN, int CG>
 struct GemmCfg {
-    static constexpr int kStages = (BN == 256) ? 4 : 6;
     static constexpr uint32_t kABytes = kGemmBM * kGemmBK * 2;
-    static constexpr uint32_t kBBytes = BN * kGemmBK * 2;
+    static constexpr uint32_t kBBytes = BN / CG * kGemmBK * 2;
     static constexpr uint32_t kStageBytes = kABytes + kBBytes;
+    static constexpr int kStages = kStageBytes > 40000 ? 4 : 6;
+    static constexpr int kTmemCols = BN > 128 ? 512 : 256;  // a power of two
+    // rows of W per copy: the two halves of a 256-row tile on one SM come in two boxes, so that one tensor map serves
+    // every kind with boxes of this height
+    static constexpr int kWBox = CG == 1 && BN == 256 ? 128 : BN / CG;
     static constexpr size_t kSmem = (size_t)kStages * kStageBytes + 1024 /* alignment */ + 256 /* barriers */;
 };
 
-template <int BN>
+// The work of one launch: items (tile, part of the reduction dimension), tiles fastest, dealt round robin to the units.
+struct GemmWork {
+    int m_tiles, tiles, parts;
+};
+struct GemmItem {
+    int tile, part, kb0, kb1;
+};
+// item `local` of unit `unit`; false when there is none
+__device__ __forceinline__ bool gemm_item(const GemmWork& w, int num_kb, int unit, int n_units, int local, GemmItem& it) {
+    const int item = unit + local * n_units;
+    if (item >= w.tiles * w.parts) return false;
+    it.tile = item % w.tiles, it.part = item / w.tiles;
+    it.kb0 = it.part * num_kb / w.parts, it.kb1 = (it.part + 1) * num_kb / w.parts;
+    return true;
+}
+
+__device__ __forceinline__ void gemm_epilogue(const GemmEpi& ep, int row, int col0, int N, const float (&v)[32], int part) {
+    if (ep.mode == kGemmF32) epi_f32(ep, row, col0, N, v, part);
+    else if (ep.mode == kGemmSwiglu) epi_swiglu(ep, row, col0, N, v);
+    else epi_qkv(ep, row, col0, N, v);
+}
+
+template <int BN, int CG>
 __global__ void __launch_bounds__(kGemmThreads, 1)
-gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w, int M, int N, int K, int m_tiles,
-               int n_tiles_total, const GemmEpi ep) {
-    using Cfg = GemmCfg<BN>;
+gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w, int M, int N, int K, const GemmWork work,
+               const GemmEpi ep) {
+    using Cfg = GemmCfg<BN, CG>;
     constexpr int kStages = Cfg::kStages;
     extern __shared__ unsigned char gemm_smem_raw[];
     unsigned char* base = gemm_smem_raw + ((1024u - (smem_u32(gemm_smem_raw) & 1023u)) & 1023u);
@@ -128,12 +176,8 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = CG == 2 ? (int)cluster_rank() : 0, unit = blockIdx.x / CG, n_units = gridDim.x / CG;
     const int num_kb = (K + kGemmBK - 1) / kGemmBK;
-    // Work item = (tile, half of the reduction dimension); without a split there is one half. Items of half 0 come
-    // first, so CTAs that run together still share their weight tile.
-    const int k_split = (ep.mode == kGemmF32 && ep.k_split == 2) ? 2 : 1;
-    const int kb_per = (num_kb + k_split - 1) / k_split;
-    const int n_items = n_tiles_total * k_split;
     volatile int* err = ep.err;
 
     if (threadIdx.x == 0) {
@@ -143,40 +187,50 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 128);
+            mbar_init(&acc_empty[b], 4 * CG);
         }
         mbar_fence_init();
     }
     if (warp == 1) {
-        tmem_alloc(tmem_slot, 2 * BN);
-        tmem_relinquish();
+        if (CG == 2) tmem_alloc_pair(tmem_slot, Cfg::kTmemCols), tmem_relinquish_pair();
+        else tmem_alloc(tmem_slot, Cfg::kTmemCols), tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
+    if (CG == 2) cluster_sync_all();  // both CTAs' barriers exist before either signals the other's
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
         if (lane == 0) {
-            int issued = 0;  // k-blocks requested so far, over all tiles of this CTA
+            int issued = 0;  // k-blocks requested so far, over all items of this unit
             bool ok = true;
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                // row tiles vary fastest: CTAs that run together share their weight tile (read once from HBM, then from L2)
-                const int tile = item % n_tiles_total, half = item / n_tiles_total;
-                const int m0 = (tile % m_tiles) * kGemmBM, n0 = (tile / m_tiles) * BN;
-                for (int kb = half * kb_per; kb < min(num_kb, (half + 1) * kb_per); ++kb) {
+            GemmItem it;
+            for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
+                // row tiles vary fastest: units that run together share their weight tile (read once from HBM, then from L2)
+                const int m0 = (it.tile % work.m_tiles * CG + rank) * kGemmBM, n0 = it.tile / work.m_tiles * BN + rank * (BN / CG);
+                for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     const int s = issued % kStages;
                     if (issued >= kStages) ok = mbar_wait(&empty[s], (uint32_t)((issued / kStages - 1) & 1), err, kErrGemmWait, 0, issued, s, 1);
                     if (!ok) break;
                     unsigned char* a_dst = base + (size_t)s * Cfg::kStageBytes;
-                    mbar_expect_tx(&full[s], Cfg::kStageBytes);
-                    tma_load_2d(a_dst, &tm_a, kb * kGemmBK, m0, &full[s]);
-                    tma_load_2d(a_dst + Cfg::kABytes, &tm_w, kb * kGemmBK, n0, &full[s]);
+                    if (rank == 0) mbar_expect_tx(&full[s], CG * Cfg::kStageBytes);  // the bytes of both CTAs
+                    if (CG == 2) {
+                        const uint32_t bar = cluster_addr(&full[s], 0);
+                        tma_load_2d_pair(a_dst, &tm_a, kb * kGemmBK, m0, bar);
+                        tma_load_2d_pair(a_dst + Cfg::kABytes, &tm_w, kb * kGemmBK, n0, bar);
+                    } else {
+                        tma_load_2d(a_dst, &tm_a, kb * kGemmBK, m0, &full[s]);
+#pragma unroll
+                        for (int h = 0; h < BN / Cfg::kWBox; ++h)
+                            tma_load_2d(a_dst + Cfg::kABytes + h * (Cfg::kWBox * kGemmBK * 2), &tm_w, kb * kGemmBK, n0 + h * Cfg::kWBox, &full[s]);
+                    }
                     ++issued;
                 }
             }
-            if (!ok || *err != kErrNone) {
-                // abandoned: let the copies still in flight land before the CTA gives its shared memory back
+            if (rank == 0 && (!ok || *err != kErrNone)) {
+                // abandoned: let the copies still in flight (with CG = 2 those of both CTAs, which the cluster barrier below
+                // holds back) land before the shared memory is given back
                 for (int i = max(0, issued - kStages); i < issued; ++i) {
                     const long long t0 = clock64();
                     while (!mbar_try_wait(&full[i % kStages], (uint32_t)((i / kStages) & 1)) && clock64() - t0 < 20000000LL) {
@@ -185,19 +239,19 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(kGemmBM, BN);
-            int done = 0, local = 0;  // k-blocks consumed so far; tiles of this CTA started so far
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc = umma_idesc_bf16(kGemmBM * CG, BN);
+            int done = 0;  // k-blocks consumed so far
             bool ok = true;
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++local) {
+            GemmItem it;
+            for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
                 const int buf = local & 1;
-                const int kb0 = (item / n_tiles_total) * kb_per, kb1 = min(num_kb, kb0 + kb_per);
-                // the epilogue must have read this buffer's previous tile (tile local - 2) before it is overwritten
+                // the epilogue must have read this buffer's previous tile (item local - 2) before it is overwritten
                 if (local >= 2) ok = mbar_wait(&acc_empty[buf], (uint32_t)((local / 2 - 1) & 1), err, kErrGemmWait, 3, local, buf, 4);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t tmem_d = tmem + (uint32_t)(buf * BN);
-                for (int kb = kb0; kb < kb1; ++kb) {
+                for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     const int s = done % kStages;
                     ok = mbar_wait(&full[s], (uint32_t)((done / kStages) & 1), err, kErrGemmWait, 1, done, s, 2);
                     if (!ok) break;
@@ -205,64 +259,112 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     const uint32_t a_addr = smem_u32(base + (size_t)s * Cfg::kStageBytes);
                     const uint64_t a_desc = umma_desc_k128(a_addr), b_desc = umma_desc_k128(a_addr + Cfg::kABytes);
 #pragma unroll
-                    for (int k = 0; k < kGemmBK / 16; ++k)  // 16 elements = 32 bytes further along the swizzled row: +2 in the address field
-                        tc_mma_bf16(tmem_d, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, ((kb - kb0) | k) != 0 ? 1u : 0u);
-                    tc_commit(&empty[s]);  // the stage may be refilled once these MMAs have read it
+                    for (int k = 0; k < kGemmBK / 16; ++k) {  // 16 elements = 32 bytes further along the swizzled row: +2 in the address field
+                        const uint32_t acc = ((kb - it.kb0) | k) != 0 ? 1u : 0u;
+                        if (CG == 2) tc_mma_bf16_pair(tmem_d, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc);
+                        else tc_mma_bf16(tmem_d, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc);
+                    }
+                    if (CG == 2) tc_commit_pair(&empty[s]);  // the stage may be refilled once these MMAs have read it
+                    else tc_commit(&empty[s]);
                     ++done;
                 }
-                tc_commit(&acc_full[buf]);  // arrives when every MMA issued above has finished
+                if (CG == 2) tc_commit_pair(&acc_full[buf]);  // arrives when every MMA issued above has finished
+                else tc_commit(&acc_full[buf]);
             }
         }
     } else {
         const int quarter = warp & 3;
         bool ok = true;
-        int local = 0;
-        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++local) {
+        GemmItem it;
+        for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
             const int buf = local & 1;
-            const int tile = item % n_tiles_total, half = item / n_tiles_total;
-            const int m0 = (tile % m_tiles) * kGemmBM, n0 = (tile / m_tiles) * BN;
+            const int m0 = (it.tile % work.m_tiles * CG + rank) * kGemmBM, n0 = it.tile / work.m_tiles * BN;
             const int row = m0 + quarter * 32 + lane;
             ok = mbar_wait(&acc_full[buf], (uint32_t)((local / 2) & 1), err, kErrGemmWait, 2, local, buf, 3) && *err == kErrNone;
+            ok = __all_sync(0xffffffffu, ok);  // tensor-memory loads are warp-wide
             tc_fence_after();
             if (!ok) break;
-            for (int cb = 0; cb < BN / 32; ++cb) {
-                const int col0 = n0 + cb * 32;
-                if (col0 >= N) break;  // uniform across the warp
+            const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN);
+            const int n_cols = min(BN, N - n0);
+            for (int c = 0; c < n_cols; c += 32) {
                 float v[32];
-                tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cb * 32), v);
-                if (row < M) {
-                    if (ep.mode == kGemmF32) epi_f32(ep, row, col0, N, v, half);
-                    else if (ep.mode == kGemmSwiglu) epi_swiglu(ep, row, col0, N, v);
-                    else epi_qkv(ep, row, col0, N, v);
-                }
+                tmem_ld32(acc + c, v);
+                if (row < M) gemm_epilogue(ep, row, n0 + c, N, v, it.part);
             }
             tc_fence_before();
-            mbar_arrive(&acc_empty[buf]);  // this thread has read its lanes of the buffer
+            __syncwarp();
+            if (lane == 0) {  // this warp has read its lanes of the buffer
+                if (CG == 2) mbar_arrive_cluster(cluster_addr(&acc_empty[buf], 0));
+                else mbar_arrive(&acc_empty[buf]);
+            }
         }
     }
     tc_fence_before();
     __syncthreads();
+    if (CG == 2) cluster_sync_all();  // no CTA leaves while the other's copies, commits or arrivals may still reach it
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, 2 * BN);
+        if (CG == 2) tmem_dealloc_pair(tmem, Cfg::kTmemCols);
+        else tmem_dealloc(tmem, Cfg::kTmemCols);
     }
 }
 
-template <int BN>
-static cudaError_t launch_gemm_bn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmEpi& ep, cudaStream_t s) {
-    const int m_tiles = (M + kGemmBM - 1) / kGemmBM, n_tiles = (N + BN - 1) / BN;
-    const int total = m_tiles * n_tiles;
-    const int items = total * ((ep.mode == kGemmF32 && ep.k_split == 2) ? 2 : 1);
-    gemm_tn_kernel<BN><<<items < g_gemm_ctas ? items : g_gemm_ctas, kGemmThreads, GemmCfg<BN>::kSmem, s>>>(tm_a, tm_w, M, N, K, m_tiles, total, ep);
-    return cudaGetLastError();
+// The kinds of unit and what a k-block (64 elements of the reduction) of one of their tiles takes, in ns: measured as the
+// slope between K = 4096 and 11008 with one round of tiles; the two narrower pair tiles by the bytes an SM takes in.
+struct GemmKind {
+    int bn, cg, ns, w_map;
+};
+constexpr GemmKind kGemmKinds[] = {{256, 2, 285, kWBox128}, {224, 2, 267, kWBox112}, {192, 2, 250, kWBox96}, {128, 1, 280, kWBox128}, {256, 1, 370, kWBox128}};
+
+template <int BN, int CG>
+static cudaError_t launch_gemm(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmWork& w, const GemmEpi& ep,
+                               cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(std::min(g_gemm_ctas / CG, w.tiles * w.parts) * CG));
+    cfg.blockDim = dim3(kGemmThreads);
+    cfg.dynamicSmemBytes = GemmCfg<BN, CG>::kSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CG, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
+    cfg.attrs = at, cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, gemm_tn_kernel<BN, CG>, tm_a, tm_w, M, N, K, w, ep);
 }
 
-cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, int bn, const GemmEpi& ep,
-                           cudaStream_t s) {
+// The rule: the kind and the number of parts with the least time over their rounds, rounds x k-blocks of a part x the time
+// of a k-block, plus writing and reading the further parts (8 bytes per element at about 4 TB/s). It picks pairs of SMs
+// for nearly every prompt of more than 128 rows (511 x 12288 x 4096: 192-column pair tiles, two rounds as with 256 columns
+// but shorter ones), single SMs where those waste half a row tile (257 rows: one round of 144 tiles, 39.5 us, against
+// two rounds of 96 pair tiles, 52.2 us) and for up to 128 rows (22016 x 4096: 86 tiles of 256 columns 44.9 us, 172 of 128
+// in two rounds 56.3 us).
+cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap* tm_w, int M, int N, int K, int max_parts, const GemmEpi& ep, cudaStream_t s,
+                           int* parts_out) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
-    if (bn == 256) return launch_gemm_bn<256>(tm_a, tm_w, M, N, K, ep, s);
-    if (bn == 128) return launch_gemm_bn<128>(tm_a, tm_w, M, N, K, ep, s);
-    return cudaErrorInvalidValue;
+    const int num_kb = (K + kGemmBK - 1) / kGemmBK;
+    int best = 0;
+    long long best_ns = -1;
+    GemmWork best_work{};
+    for (int i = 0; i < (int)(sizeof(kGemmKinds) / sizeof(kGemmKinds[0])); ++i) {
+        const GemmKind& k = kGemmKinds[i];
+        GemmWork w{};
+        w.m_tiles = (M + kGemmBM * k.cg - 1) / (kGemmBM * k.cg);
+        w.tiles = w.m_tiles * ((N + k.bn - 1) / k.bn);
+        const int units = g_gemm_ctas / k.cg;
+        for (w.parts = 1; w.parts == 1 || (w.parts <= max_parts && num_kb / w.parts >= 8); ++w.parts) {
+            const long long rounds = ((long long)w.tiles * w.parts + units - 1) / units;
+            const long long ns = rounds * ((num_kb + w.parts - 1) / w.parts) * k.ns + (long long)(w.parts - 1) * M * N / 500;
+            if (best_ns < 0 || ns < best_ns) best = i, best_ns = ns, best_work = w;
+        }
+    }
+    if (parts_out) *parts_out = best_work.parts;
+    const CUtensorMap& wm = tm_w[kGemmKinds[best].w_map];
+    switch (best) {
+        case 0: return launch_gemm<256, 2>(tm_a, wm, M, N, K, best_work, ep, s);
+        case 1: return launch_gemm<224, 2>(tm_a, wm, M, N, K, best_work, ep, s);
+        case 2: return launch_gemm<192, 2>(tm_a, wm, M, N, K, best_work, ep, s);
+        case 3: return launch_gemm<128, 1>(tm_a, wm, M, N, K, best_work, ep, s);
+        default: return launch_gemm<256, 1>(tm_a, wm, M, N, K, best_work, ep, s);
+    }
 }
 
 // ============================================================================================ row kernels
@@ -309,17 +411,18 @@ __global__ void __launch_bounds__(kRowThreads) embed_norm_kernel(const int* toke
 
 // The residual add with the cosine similarity of the hidden state before and after the sublayer (Section 3.2), and
 // the RMSNorm that feeds the next sublayer (its statistic is the |y|^2 just computed).
-__global__ void __launch_bounds__(kRowThreads) resid_norm_kernel(int d, float* x, const float* c, const float* c2, const __nv_bfloat16* gain, float eps,
+__global__ void __launch_bounds__(kRowThreads) resid_norm_kernel(int d, float* x, const float* c, int parts, size_t part_stride, const __nv_bfloat16* gain, float eps,
                                                                 __nv_bfloat16* xn, float* cos_out) {
     __shared__ float red[24];
     const int r = blockIdx.x;
     float* xr = x + (size_t)r * d;
     const float* cr = c + (size_t)r * d;
-    const float* cr2 = c2 ? c2 + (size_t)r * d : nullptr;  // second half of a product whose reduction dimension was cut in two
     float s[3] = {0.f, 0.f, 0.f};
     for (int i = threadIdx.x; i < d; i += kRowThreads) {
         const float xv = xr[i];
-        const float y = xv + (cr2 ? cr[i] + cr2[i] : cr[i]);
+        float o = cr[i];
+        for (int p = 1; p < parts; ++p) o += cr[p * part_stride + i];  // a product that came in parts of its reduction dimension
+        const float y = xv + o;
         xr[i] = y;
         s[0] = fmaf(xv, y, s[0]);
         s[1] = fmaf(xv, xv, s[1]);
@@ -341,7 +444,7 @@ __global__ void __launch_bounds__(kRowThreads) resid_norm_kernel(int d, float* x
 // sublayer output are read once, 16 bytes per load, and the sums, the new hidden state and the normalised row all
 // come from those registers.
 template <int NV>
-__global__ void __launch_bounds__(kRowThreads) resid_norm_vec_kernel(int d, float* x, const float* c, const float* c2, const __nv_bfloat16* gain, float eps,
+__global__ void __launch_bounds__(kRowThreads) resid_norm_vec_kernel(int d, float* x, const float* c, int parts, size_t part_stride, const __nv_bfloat16* gain, float eps,
                                                                     __nv_bfloat16* xn, float* cos_out) {
     __shared__ float red[24];
     const int r = blockIdx.x, nvec = d >> 2;
@@ -354,13 +457,13 @@ __global__ void __launch_bounds__(kRowThreads) resid_norm_vec_kernel(int d, floa
         y[v] = cv[v] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (i < nvec) y[v] = xr[i], cv[v] = cr[i];
     }
-    if (c2) {  // the product came in two halves of its reduction dimension: half 0 + half 1
-        const float4* cr2 = reinterpret_cast<const float4*>(c2 + (size_t)r * d);
+    for (int p = 1; p < parts; ++p) {  // a product that came in parts of its reduction dimension: added in order
+        const float4* cp = reinterpret_cast<const float4*>(c + p * part_stride + (size_t)r * d);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             const int i = threadIdx.x + v * kRowThreads;
             if (i < nvec) {
-                const float4 o = cr2[i];
+                const float4 o = cp[i];
                 cv[v].x += o.x, cv[v].y += o.y, cv[v].z += o.z, cv[v].w += o.w;
             }
         }
@@ -418,15 +521,15 @@ cudaError_t launch_embed_norm(const int* tokens, int n_rows, int d, int vocab, c
     embed_norm_kernel<<<n_rows, kRowThreads, 0, s>>>(tokens, d, vocab, embed, gain, eps, x, xn);
     return cudaGetLastError();
 }
-cudaError_t launch_resid_norm(int n_rows, int d, float* x, const float* c, const float* c2, const __nv_bfloat16* gain, float eps, __nv_bfloat16* xn,
+cudaError_t launch_resid_norm(int n_rows, int d, float* x, const float* c, int parts, size_t part_stride, const __nv_bfloat16* gain, float eps, __nv_bfloat16* xn,
                               float* cos_out, cudaStream_t s) {
     const int nv = (d + kRowThreads * 4 - 1) / (kRowThreads * 4);
-    if (d % 4 != 0 || nv > 8) resid_norm_kernel<<<n_rows, kRowThreads, 0, s>>>(d, x, c, c2, gain, eps, xn, cos_out);
-    else if (nv <= 1) resid_norm_vec_kernel<1><<<n_rows, kRowThreads, 0, s>>>(d, x, c, c2, gain, eps, xn, cos_out);
-    else if (nv <= 2) resid_norm_vec_kernel<2><<<n_rows, kRowThreads, 0, s>>>(d, x, c, c2, gain, eps, xn, cos_out);
-    else if (nv <= 4) resid_norm_vec_kernel<4><<<n_rows, kRowThreads, 0, s>>>(d, x, c, c2, gain, eps, xn, cos_out);
-    else if (nv <= 5) resid_norm_vec_kernel<5><<<n_rows, kRowThreads, 0, s>>>(d, x, c, c2, gain, eps, xn, cos_out);
-    else resid_norm_vec_kernel<8><<<n_rows, kRowThreads, 0, s>>>(d, x, c, c2, gain, eps, xn, cos_out);
+    if (d % 4 != 0 || nv > 8) resid_norm_kernel<<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
+    else if (nv <= 1) resid_norm_vec_kernel<1><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
+    else if (nv <= 2) resid_norm_vec_kernel<2><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
+    else if (nv <= 4) resid_norm_vec_kernel<4><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
+    else if (nv <= 5) resid_norm_vec_kernel<5><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
+    else resid_norm_vec_kernel<8><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
     return cudaGetLastError();
 }
 cudaError_t launch_sumcos(const float* cos_rows, int stride, int n_rows, int n_sub, double* sumcos, cudaStream_t s) {
@@ -441,8 +544,14 @@ cudaError_t configure_prefill(int max_smem) {
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if (sms > 0) g_gemm_ctas = sms;
-    if ((e = cudaFuncSetAttribute(gemm_tn_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmCfg<256>::kSmem)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(gemm_tn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmCfg<128>::kSmem)) != cudaSuccess) return e;
+#define ASD_SET_GEMM(BN, CG) \
+    if ((e = cudaFuncSetAttribute(gemm_tn_kernel<BN, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmCfg<BN, CG>::kSmem)) != cudaSuccess) return e
+    ASD_SET_GEMM(256, 2);
+    ASD_SET_GEMM(224, 2);
+    ASD_SET_GEMM(192, 2);
+    ASD_SET_GEMM(128, 1);
+    ASD_SET_GEMM(256, 1);
+#undef ASD_SET_GEMM
     return configure_prefill_attention();
 }
 

@@ -31,8 +31,7 @@ struct GemmEpi {
     // kGemmF32
     float* c;
     int ldc;
-    int k_split;            // 1, or 2: the reduction dimension is cut in two halves, each a work item of its own
-    size_t c_split_stride;  // floats between the partial results of the halves (the caller adds them: half 0 + half 1)
+    size_t c_part_stride;  // floats between the parts of a product whose reduction dimension is cut (the caller adds them in order)
     // kGemmQkv: columns are [q | k | v]; inside every q and k head the rotary partners (j, j + head_dim/2) are
     // neighbours (2j, 2j+1); v columns are in natural order. Row r sits at position pos0 + r.
     __nv_bfloat16 *q, *k_cache, *v_cache;
@@ -45,18 +44,23 @@ struct GemmEpi {
 
 cudaError_t configure_prefill(int max_smem);
 
-// C[M, N] = A[M, K] * W[N, K]^T, bf16 operands described by 2-D tensor maps (boxes of 64 x 128 for A, 64 x bn for W,
-// 128-byte swizzle), fp32 accumulation. bn is 128 or 256.
-cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, int bn, const GemmEpi& ep,
-                           cudaStream_t s);
+// tensor maps of one weight matrix [N, K] with 128-byte swizzle: boxes of 64 elements x 128, 112 or 96 rows
+enum GemmWeightMap : int { kWBox128 = 0, kWBox112 = 1, kWBox96 = 2, kWBoxes = 3 };
+constexpr int kWBoxRows[kWBoxes] = {128, 112, 96};
+
+// C[M, N] = A[M, K] * W[N, K]^T, bf16 operands described by 2-D tensor maps (A in boxes of 64 x 128, 128-byte swizzle; tm_w:
+// the kWBoxes maps of W), fp32 accumulation. With max_parts > 1 (kGemmF32 only) the reduction dimension may be cut into
+// up to that many parts, *parts_out products of their own c_part_stride apart.
+cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap* tm_w, int M, int N, int K, int max_parts, const GemmEpi& ep, cudaStream_t s,
+                           int* parts_out = nullptr);
 
 // x[r, :] = embedding row of tokens[r] (fp32); xn[r, :] = bf16(RMSNorm(x[r]) * gain)
 cudaError_t launch_embed_norm(const int* tokens, int n_rows, int d, int vocab, const __nv_bfloat16* embed, const __nv_bfloat16* gain,
                               float eps, float* x, __nv_bfloat16* xn, cudaStream_t s);
 
-// y = x + c (in place in x), cos_out[r] = <x, y> / (|x| |y|) (Section 3.2), and, when gain is given,
+// y = x + c (in place in x; c is the sum of `parts` buffers, added in order), cos_out[r] = <x, y> / (|x| |y|) (Section 3.2), and, when gain is given,
 // xn[r, :] = bf16(RMSNorm(y) * gain) for the next sublayer
-cudaError_t launch_resid_norm(int n_rows, int d, float* x, const float* c, const float* c2, const __nv_bfloat16* gain, float eps, __nv_bfloat16* xn,
+cudaError_t launch_resid_norm(int n_rows, int d, float* x, const float* c, int parts, size_t part_stride, const __nv_bfloat16* gain, float eps, __nv_bfloat16* xn,
                               float* cos_out, cudaStream_t s);
 
 // sumcos[b] += sum over rows of cos_rows[b * stride + r], rows in a fixed order, double precision

@@ -284,9 +284,8 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     uint32_t w[16];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) w[i] = pack_bf16(v[2 * i] * inv, v[2 * i + 1] * inv);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        reinterpret_cast<uint4*>(dst + c)[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                    st_global_v8(dst + c, w);
+                    st_global_v8(dst + c + 16, w + 8);
                 }
             }
         }
