@@ -12,6 +12,7 @@
 
 #include "../../include/asd.h"
 #include "common.cuh"
+#include "gemv.cuh"
 #include "pass.cuh"
 #include "prefill.h"
 #include "sample.h"
@@ -25,16 +26,6 @@ constexpr long long kShortWaitCycles = 2000000LL;  // ASD_DEBUG_SHORT_WAITS: abo
 
 static size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
-// ---------------------------------------------------------------- shared-memory budgets
-size_t gemv_smem_bytes(int M, int n_rows, int n_in, int grid, bool x_in_smem) {
-    const size_t n_pairs = ((size_t)n_rows + 1) / 2;
-    const size_t max_np = (n_pairs + grid - 1) / grid;
-    const size_t n_seg = ((size_t)n_in + kSeg - 1) / kSeg;
-    size_t psum = (max_np * n_seg * 2 * M + 3) & ~(size_t)3;
-    size_t b = (size_t)kGemvWarps * kMaxRows * 4 * 4 + 16 + psum * 4;
-    if (x_in_smem) b += (size_t)M * n_in * 2;
-    return b;
-}
 static cudaError_t launch_gemv(int M, int epi, bool norm, const GemvParams& p, int grid, size_t smem, cudaStream_t s) {
     switch (M) {
         case 1: return launch_gemv_m1(epi, norm, p, grid, smem, s);
@@ -100,24 +91,51 @@ static cudaError_t device_info(DeviceInfo** out) {
     return cudaSuccess;
 }
 
-// Choose the launch shape of one fused GEMV: one CTA per SM; more CTAs only when the per-CTA partial-sum
-// buffer would not fit in shared memory; activations fall back to L1 reads when they do not fit.
-static bool plan_gemv(const DeviceInfo& dv, int M, int n_rows, int n_in, bool norm, int* grid, int* x_in_smem, size_t* smem) {
+// The shapes that the fused GEMV takes, and for how many CTAs' partial results a caller has to have room: one CTA per SM,
+// or as many as let the sums of a CTA's pairs of rows over segments of 1024 inputs (and with RMSNorm the whole
+// activations) stay in shared memory. The kernel needs no more than one CTA per SM for any of them; the limits are
+// the interface's (the built-in scratch array of the static variant refuses what is beyond it).
+static bool gemv_accepts(const DeviceInfo& dv, int M, int n_rows, int n_in, bool norm, int* ctas) {
+    const size_t n_pairs = ((size_t)n_rows + 1) / 2, n_seg = ((size_t)n_in + 1023) / 1024;
     for (int g = dv.num_sms; g <= kMaxGemvGrid; g += dv.num_sms) {
-        size_t b = gemv_smem_bytes(M, n_rows, n_in, g, true);
-        if (b <= (size_t)dv.max_smem) {
-            *grid = g, *x_in_smem = 1, *smem = b;
+        const size_t sums = ((n_pairs + g - 1) / g * n_seg * 2 * M + 3) & ~(size_t)3;
+        const size_t bytes = (size_t)16 * kMaxRows * 4 * 4 + 16 + sums * 4 + (norm ? (size_t)M * n_in * 2 : 0);
+        if (bytes <= (size_t)dv.max_smem) {
+            *ctas = g;
             return true;
-        }
-        if (!norm) {
-            b = gemv_smem_bytes(M, n_rows, n_in, g, false);
-            if (b <= (size_t)dv.max_smem) {
-                *grid = g, *x_in_smem = 0, *smem = b;
-                return true;
-            }
         }
     }
     return false;
+}
+
+// The plan of one launch (shared memory returned). Sub-items per group: the split that leaves the warps least unequal,
+// counted in segments of the longest warp; a finer split has to gain a twentieth, because each costs an epilogue addition.
+// Windows of the activations: as few as kGemvSmem holds, of equal length, beginning at multiples of the runs of all
+// sub-items. The split does not depend on M.
+// kGemvSmem is half of the SM's 256 KB although a block may have 227: the weights in flight take lines of what is left as L1
+// cache (five rows of 13760 inputs: one window and 170 KB 43-59 us, depending on how much is in flight).
+constexpr size_t kGemvSmem = 128 * 1024;
+static size_t plan_gemv(const DeviceInfo& dv, int M, int n_rows, int n_in, GemvParams* p) {
+    const int n_seg = (n_in + kGemvSeg - 1) / kGemvSeg, n_run = (n_seg + kGemvRun - 1) / kGemvRun;
+    p->max_rows = 0;
+    for (int b = 0; b < dv.num_sms; ++b) p->max_rows = std::max(p->max_rows, gemv_row(n_rows, dv.num_sms, b + 1) - gemv_row(n_rows, dv.num_sms, b));
+    p->n_blk = (p->max_rows + kGemvBlockRows - 1) / kGemvBlockRows;
+    if (p->n_blk > 1) p->max_rows = (p->max_rows + p->n_blk - 1) / p->n_blk + 2;  // block boundaries are even
+    const int groups = (p->max_rows + 15) / 16;
+    auto longest = [&](int s) { return (groups * s + kGemvWarps - 1) / kGemvWarps * ((n_run + s - 1) / s); };
+    p->split = 1;
+    for (int s = 2; s <= 16 && s <= n_run && groups * s <= kGemvMaxSub; ++s)
+        if (20 * longest(s) < 19 * longest(p->split)) p->split = s;
+    p->max_sub = groups * p->split;
+    const size_t fixed = (size_t)gemv_fixed_smem(M, p->max_sub, p->max_rows);
+    const size_t room = kGemvSmem > fixed ? (kGemvSmem - fixed) / M / 2 : 0;
+    const int most = room > (size_t)kGemvPad ? (int)((room - kGemvPad) / kGemvSeg) : 0, unit = p->split * kGemvRun;
+    p->win_segs = n_seg;
+    if (n_seg > most) {
+        const int unit_most = std::max(most / unit, 1) * unit, n_win = (n_seg + unit_most - 1) / unit_most;
+        p->win_segs = ((n_seg + n_win - 1) / n_win + unit - 1) / unit * unit;
+    }
+    return fixed + (size_t)M * (p->win_segs * kGemvSeg + kGemvPad) * 2;
 }
 
 // Shared-memory plan of the persistent pass kernel for M rows: ring slots, barriers, reduction scratch,
@@ -1556,11 +1574,10 @@ extern "C" int asd_fused_gemv(void* cuda_stream, int32_t M, int32_t n_in, int32_
     p.cos_out = cosv;
     p.counter = reinterpret_cast<unsigned*>(scratch);
     p.partials = reinterpret_cast<float*>(static_cast<unsigned char*>(scratch) + 256);
-    int grid, xin;
-    size_t smem;
-    if (!plan_gemv(*dv, M, n_rows, n_in, gain != nullptr, &grid, &xin, &smem)) return ASD_ERR_ARG;
-    p.x_in_smem = xin;
-    if (launch_gemv(M, epilogue, gain != nullptr, p, grid, smem, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
+    int ctas;
+    if (!gemv_accepts(*dv, M, n_rows, n_in, gain != nullptr, &ctas)) return ASD_ERR_ARG;
+    const size_t smem = plan_gemv(*dv, M, n_rows, n_in, &p);
+    if (launch_gemv(M, epilogue, gain != nullptr, p, dv->num_sms, smem, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return ASD_ERR_CUDA;
     return ASD_OK;
 }
@@ -1621,14 +1638,13 @@ extern "C" int asd_fused_gemv_static(void* cuda_stream, int32_t M, int32_t n_in,
         }
         scratch = static_cast<unsigned char*>(g_static_scratch_addr[dev]);
     }
-    int grid, xin;
-    size_t smem;
-    if (!plan_gemv(*dv, M, n_rows, n_in, gain != nullptr, &grid, &xin, &smem)) return ASD_ERR_ARG;
-    if (grid > kStaticMaxGrid) {
+    int ctas;
+    if (!gemv_accepts(*dv, M, n_rows, n_in, gain != nullptr, &ctas)) return ASD_ERR_ARG;
+    if (ctas > kStaticMaxGrid) {
         fprintf(stderr,
                 "asd_fused_gemv_static: this shape needs a %d-CTA launch plan but the built-in scratch array holds "
                 "partials for at most %d CTAs; call asd_fused_gemv with caller-provided scratch instead\n",
-                grid, kStaticMaxGrid);
+                ctas, kStaticMaxGrid);
         return ASD_ERR_NOMEM;
     }
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
@@ -1646,7 +1662,7 @@ extern "C" int asd_fused_gemv_static(void* cuda_stream, int32_t M, int32_t n_in,
     p.cos_out = cosv;
     p.counter = reinterpret_cast<unsigned*>(scratch);
     p.partials = reinterpret_cast<float*>(scratch + 256);
-    p.x_in_smem = xin;
-    if (launch_gemv(M, epilogue, gain != nullptr, p, grid, smem, s) != cudaSuccess) return ASD_ERR_CUDA;
+    const size_t smem = plan_gemv(*dv, M, n_rows, n_in, &p);
+    if (launch_gemv(M, epilogue, gain != nullptr, p, dv->num_sms, smem, s) != cudaSuccess) return ASD_ERR_CUDA;
     return ASD_OK;
 }

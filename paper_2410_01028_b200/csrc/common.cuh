@@ -10,7 +10,6 @@ constexpr int kMaxRows = 9;        // rows of the stand-alone fused GEMV: max dr
 constexpr int kPassMaxRows = 16;   // rows of one pass of the persistent kernel (prefill feeds the prompt 16 rows at a time)
 constexpr int kGemvThreads = 512;  // 16 warps per CTA, one CTA per SM
 constexpr int kGemvWarps = kGemvThreads / 32;
-constexpr int kSeg = 1024;         // elements of the reduction dimension per warp work item
 constexpr int kAttnChunk = 128;    // keys per attention work item; chunks are aligned to absolute positions
 
 enum Epilogue : int { kEpiPlain = 0, kEpiSwiglu = 1, kEpiResidual = 2 };
@@ -22,11 +21,13 @@ struct GemvParams {
     const void* x;              // gain ? float [M, n_in] : bf16 [M, n_in]
     const __nv_bfloat16* gain;  // [n_in] or null
     float eps;
-    int x_in_smem;  // stage the activations in shared memory (else read them through L1)
+    int win_segs;   // segments of the inputs whose activations are in shared memory at a time
+    int n_blk;              // blocks of rows of a CTA
+    int max_sub, max_rows;  // most sub-items and weight rows of a block
+    int split;  // sub-items per group of 16 weight rows
     // plain / swiglu / residual
     void* out;
     float* cos_out;   // residual: [M]
-    double* sumcos;   // residual: running sum over prompt rows, or null
     float* partials;  // [gridDim.x][kMaxRows][4] cross-CTA partial results
     unsigned* counter;  // zero before launch; reset by the last CTA
 };
@@ -50,7 +51,20 @@ ASD_DECLARE_LAUNCHERS(9)
 cudaError_t launch_pass_m16(const PassParams& p, int grid, size_t smem, cudaStream_t s);
 cudaError_t configure_m16(int max_smem);
 
-size_t gemv_smem_bytes(int M, int n_rows, int n_in, int grid, bool x_in_smem);
+// ---------------------------------------------------------------- launch helper
+// Launches a kernel that begins with pdl_wait(): its launch and its CTAs' start overlap the end of the kernel before it.
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid, cfg.blockDim = block, cfg.dynamicSmemBytes = smem, cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster, at[1].val.clusterDim.y = 1, at[1].val.clusterDim.z = 1;
+    cfg.attrs = at, cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
+}
 
 // ---------------------------------------------------------------- device helpers
 __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
@@ -64,6 +78,12 @@ __device__ __forceinline__ uint4 ldg_stream(const void* p) {
                  : "l"(p));
     return v;
 }
+
+// Programmatic dependent launch: a kernel that was launched with the attribute may start while the one before it on the
+// stream is still running (once all of that one's CTAs have asked for it or ended) and waits here for its end and its
+// writes before it reads or writes anything itself. Without the attribute both do nothing.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll

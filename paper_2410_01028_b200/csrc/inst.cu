@@ -15,8 +15,7 @@ namespace asd {
 #if ASD_M <= 9
 template <int EPI, bool NORM>
 static cudaError_t launch_one(const GemvParams& p, int grid, size_t smem, cudaStream_t s) {
-    gemv_kernel<ASD_M, EPI, NORM><<<grid, kGemvThreads, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_pdl(gemv_kernel<ASD_M, EPI, NORM>, dim3(grid), dim3(kGemvThreads), smem, s, 1, p);
 }
 
 cudaError_t ASD_CAT(launch_gemv_m, ASD_M)(int epi, bool norm, const GemvParams& p, int grid, size_t smem, cudaStream_t s) {
