@@ -1054,7 +1054,7 @@ static int prefill_dense(asd_ctx* x, const int32_t* dev_tokens, int n, int pos0)
             __nv_bfloat16* kc = reinterpret_cast<__nv_bfloat16*>(x->ws + ly.kcache + (size_t)l * ly.kv_layer_stride);
             __nv_bfloat16* vc = reinterpret_cast<__nv_bfloat16*>(x->ws + ly.vcache + (size_t)l * ly.kv_layer_stride);
             GemmEpi e{};
-            e.err = err;
+            e.err = err, e.w_static = 1;
             e.mode = kGemmQkv;
             e.q = pq, e.k_cache = kc, e.v_cache = vc;
             e.rope_cos = x->at<float>(ly.rope_cos), e.rope_sin = x->at<float>(ly.rope_sin);
@@ -1062,7 +1062,7 @@ static int prefill_dense(asd_ctx* x, const int32_t* dev_tokens, int n, int pos0)
             if ((rc = dense_gemm(x, x->tm_xn, l, 0, rows, d + 2 * kvd, d, e))) return rc;
             ASD_CUDA(x, launch_flash_prefill(x->tm_q, x->tm_kv[(size_t)l * 2], x->tm_kv[(size_t)l * 2 + 1], pa, rows, p0, d, c.head_dim, c.n_heads, c.n_kv_heads, scale, err, s));
             GemmEpi o{};
-            o.err = err;
+            o.err = err, o.w_static = 1;
             o.mode = kGemmF32;
             o.c = pc, o.ldc = d;
             o.c_part_stride = (size_t)rows * d;
@@ -1071,7 +1071,7 @@ static int prefill_dense(asd_ctx* x, const int32_t* dev_tokens, int n, int pos0)
             ASD_CUDA(x, launch_resid_norm(rows, d, px, pc, parts, o.c_part_stride, gain(l, ly.l_mlp_norm), c.rms_eps, pxn,
                                           pcos + (size_t)l * R, s));
             GemmEpi g{};
-            g.err = err;
+            g.err = err, g.w_static = 1;
             g.mode = kGemmSwiglu;
             g.t = pt, g.ldt = f;
             if ((rc = dense_gemm(x, x->tm_xn, l, 2, rows, 2 * f, d, g))) return rc;

@@ -200,6 +200,25 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (CG == 2) cluster_sync_all();  // both CTAs' barriers exist before either signals the other's
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_launch_dependents();
+    auto load_w = [&](int s, int kb, int n0) {  // announces the bytes of a stage and requests its weights
+        if (rank == 0) mbar_expect_tx(&full[s], CG * Cfg::kStageBytes);  // the bytes of both CTAs
+        unsigned char* b_dst = base + (size_t)s * Cfg::kStageBytes + Cfg::kABytes;
+        if (CG == 2) {
+            tma_load_2d_pair(b_dst, &tm_w, kb * kGemmBK, n0, cluster_addr(&full[s], 0));
+        } else {
+#pragma unroll
+            for (int h = 0; h < BN / Cfg::kWBox; ++h)
+                tma_load_2d(b_dst + h * (Cfg::kWBox * kGemmBK * 2), &tm_w, kb * kGemmBK, n0 + h * Cfg::kWBox, &full[s]);
+        }
+    };
+    int ahead = 0;  // k-blocks of the first item whose weights are requested before the kernel in front has ended
+    if (warp == 0 && lane == 0 && ep.w_static) {
+        GemmItem it;
+        if (gemm_item(work, num_kb, unit, n_units, 0, it))
+            for (; ahead < kStages && it.kb0 + ahead < it.kb1; ++ahead) load_w(ahead, it.kb0 + ahead, it.tile / work.m_tiles * BN + rank * (BN / CG));
+    }
+    pdl_wait();  // everything above overlaps the end of the kernel in front
 
     if (warp == 0) {
         if (lane == 0) {
@@ -213,18 +232,10 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     const int s = issued % kStages;
                     if (issued >= kStages) ok = mbar_wait(&empty[s], (uint32_t)((issued / kStages - 1) & 1), err, kErrGemmWait, 0, issued, s, 1);
                     if (!ok) break;
+                    if (issued >= ahead) load_w(s, kb, n0);
                     unsigned char* a_dst = base + (size_t)s * Cfg::kStageBytes;
-                    if (rank == 0) mbar_expect_tx(&full[s], CG * Cfg::kStageBytes);  // the bytes of both CTAs
-                    if (CG == 2) {
-                        const uint32_t bar = cluster_addr(&full[s], 0);
-                        tma_load_2d_pair(a_dst, &tm_a, kb * kGemmBK, m0, bar);
-                        tma_load_2d_pair(a_dst + Cfg::kABytes, &tm_w, kb * kGemmBK, n0, bar);
-                    } else {
-                        tma_load_2d(a_dst, &tm_a, kb * kGemmBK, m0, &full[s]);
-#pragma unroll
-                        for (int h = 0; h < BN / Cfg::kWBox; ++h)
-                            tma_load_2d(a_dst + Cfg::kABytes + h * (Cfg::kWBox * kGemmBK * 2), &tm_w, kb * kGemmBK, n0 + h * Cfg::kWBox, &full[s]);
-                    }
+                    if (CG == 2) tma_load_2d_pair(a_dst, &tm_a, kb * kGemmBK, m0, cluster_addr(&full[s], 0));
+                    else tma_load_2d(a_dst, &tm_a, kb * kGemmBK, m0, &full[s]);
                     ++issued;
                 }
             }
@@ -319,16 +330,8 @@ constexpr GemmKind kGemmKinds[] = {{256, 2, 285, kWBox128}, {224, 2, 267, kWBox1
 template <int BN, int CG>
 static cudaError_t launch_gemm(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmWork& w, const GemmEpi& ep,
                                cudaStream_t s) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(std::min(g_gemm_ctas / CG, w.tiles * w.parts) * CG));
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = GemmCfg<BN, CG>::kSmem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CG, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
-    cfg.attrs = at, cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_tn_kernel<BN, CG>, tm_a, tm_w, M, N, K, w, ep);
+    const dim3 grid((unsigned)(std::min(g_gemm_ctas / CG, w.tiles * w.parts) * CG));
+    return launch_pdl(gemm_tn_kernel<BN, CG>, grid, dim3(kGemmThreads), GemmCfg<BN, CG>::kSmem, s, CG, tm_a, tm_w, M, N, K, w, ep);
 }
 
 // The rule: the kind and the number of parts with the least time over their rounds, rounds x k-blocks of a part x the time
@@ -393,20 +396,32 @@ __device__ __forceinline__ void block_sum(float (&v)[NV], float* red /* [NV][8] 
 __global__ void __launch_bounds__(kRowThreads) embed_norm_kernel(const int* tokens, int d, int vocab, const __nv_bfloat16* embed,
                                                                 const __nv_bfloat16* gain, float eps, float* x, __nv_bfloat16* xn) {
     __shared__ float red[8];
+    pdl_launch_dependents();
     const int r = blockIdx.x;
     int t = tokens[r];
     t = min(max(t, 0), vocab - 1);
-    const __nv_bfloat16* e = embed + (size_t)t * d;
+    const uint4* e = reinterpret_cast<const uint4*>(embed + (size_t)t * d);  // d is a multiple of 8
     float s[1] = {0.f};
-    for (int i = threadIdx.x; i < d; i += kRowThreads) {
-        const float v = __bfloat162float(e[i]);
-        x[(size_t)r * d + i] = v;
-        s[0] = fmaf(v, v, s[0]);
+    for (int i = threadIdx.x; i < d / 8; i += kRowThreads) {
+        const uint4 v = e[i];
+        const float f[8] = {bf_lo(v.x), bf_hi(v.x), bf_lo(v.y), bf_hi(v.y), bf_lo(v.z), bf_hi(v.z), bf_lo(v.w), bf_hi(v.w)};
+        float4* dst = reinterpret_cast<float4*>(x + (size_t)r * d + 8 * i);
+        dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+        dst[1] = make_float4(f[4], f[5], f[6], f[7]);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[0] = fmaf(f[k], f[k], s[0]);
     }
     block_sum<1>(s, red);
     const float inv = 1.0f / sqrtf(s[0] / (float)d + eps);
-    for (int i = threadIdx.x; i < d; i += kRowThreads)
-        xn[(size_t)r * d + i] = __float2bfloat16_rn(__bfloat162float(e[i]) * inv * __bfloat162float(gain[i]));
+    for (int i = threadIdx.x; i < d / 8; i += kRowThreads) {
+        const uint4 v = e[i], g = reinterpret_cast<const uint4*>(gain)[i];
+        uint4 o;
+        o.x = pack_bf16(bf_lo(v.x) * inv * bf_lo(g.x), bf_hi(v.x) * inv * bf_hi(g.x));
+        o.y = pack_bf16(bf_lo(v.y) * inv * bf_lo(g.y), bf_hi(v.y) * inv * bf_hi(g.y));
+        o.z = pack_bf16(bf_lo(v.z) * inv * bf_lo(g.z), bf_hi(v.z) * inv * bf_hi(g.z));
+        o.w = pack_bf16(bf_lo(v.w) * inv * bf_lo(g.w), bf_hi(v.w) * inv * bf_hi(g.w));
+        reinterpret_cast<uint4*>(xn + (size_t)r * d)[i] = o;
+    }
 }
 
 // The residual add with the cosine similarity of the hidden state before and after the sublayer (Section 3.2), and
@@ -414,6 +429,8 @@ __global__ void __launch_bounds__(kRowThreads) embed_norm_kernel(const int* toke
 __global__ void __launch_bounds__(kRowThreads) resid_norm_kernel(int d, float* x, const float* c, int parts, size_t part_stride, const __nv_bfloat16* gain, float eps,
                                                                 __nv_bfloat16* xn, float* cos_out) {
     __shared__ float red[24];
+    pdl_launch_dependents();
+    pdl_wait();
     const int r = blockIdx.x;
     float* xr = x + (size_t)r * d;
     const float* cr = c + (size_t)r * d;
@@ -447,6 +464,8 @@ template <int NV>
 __global__ void __launch_bounds__(kRowThreads) resid_norm_vec_kernel(int d, float* x, const float* c, int parts, size_t part_stride, const __nv_bfloat16* gain, float eps,
                                                                     __nv_bfloat16* xn, float* cos_out) {
     __shared__ float red[24];
+    pdl_launch_dependents();
+    pdl_wait();
     const int r = blockIdx.x, nvec = d >> 2;
     float4* xr = reinterpret_cast<float4*>(x + (size_t)r * d);
     const float4* cr = reinterpret_cast<const float4*>(c + (size_t)r * d);
@@ -524,13 +543,13 @@ cudaError_t launch_embed_norm(const int* tokens, int n_rows, int d, int vocab, c
 cudaError_t launch_resid_norm(int n_rows, int d, float* x, const float* c, int parts, size_t part_stride, const __nv_bfloat16* gain, float eps, __nv_bfloat16* xn,
                               float* cos_out, cudaStream_t s) {
     const int nv = (d + kRowThreads * 4 - 1) / (kRowThreads * 4);
-    if (d % 4 != 0 || nv > 8) resid_norm_kernel<<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
-    else if (nv <= 1) resid_norm_vec_kernel<1><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
-    else if (nv <= 2) resid_norm_vec_kernel<2><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
-    else if (nv <= 4) resid_norm_vec_kernel<4><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
-    else if (nv <= 5) resid_norm_vec_kernel<5><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
-    else resid_norm_vec_kernel<8><<<n_rows, kRowThreads, 0, s>>>(d, x, c, parts, part_stride, gain, eps, xn, cos_out);
-    return cudaGetLastError();
+    void (*kernel)(int, float*, const float*, int, size_t, const __nv_bfloat16*, float, __nv_bfloat16*, float*) = resid_norm_vec_kernel<8>;
+    if (d % 4 != 0 || nv > 8) kernel = resid_norm_kernel;
+    else if (nv <= 1) kernel = resid_norm_vec_kernel<1>;
+    else if (nv <= 2) kernel = resid_norm_vec_kernel<2>;
+    else if (nv <= 4) kernel = resid_norm_vec_kernel<4>;
+    else if (nv <= 5) kernel = resid_norm_vec_kernel<5>;
+    return launch_pdl(kernel, dim3(n_rows), dim3(kRowThreads), 0, s, 1, d, x, c, parts, part_stride, gain, eps, xn, cos_out);
 }
 cudaError_t launch_sumcos(const float* cos_rows, int stride, int n_rows, int n_sub, double* sumcos, cudaStream_t s) {
     sumcos_kernel<<<n_sub, 32, 0, s>>>(cos_rows, stride, n_rows, sumcos);

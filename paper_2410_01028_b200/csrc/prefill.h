@@ -28,6 +28,7 @@ enum GemmEpilogue : int {
 struct GemmEpi {
     int mode;
     int* err;  // device error words shared with the pass kernel (word 0 = code)
+    int w_static;  // no kernel in flight writes W: its first tiles may be requested before the kernel in front has ended
     // kGemmF32
     float* c;
     int ldc;

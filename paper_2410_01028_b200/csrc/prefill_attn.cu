@@ -124,6 +124,8 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_launch_dependents();
+    pdl_wait();  // everything above overlaps the end of the kernel before
 
     if (warp == 4) {
         if (lane == 0) {
@@ -305,12 +307,10 @@ cudaError_t launch_flash_prefill(const CUtensorMap& tm_q, const CUtensorMap& tm_
     const int group = n_heads / n_kv_heads;
     const float scale_log2 = scale * 1.4426950408889634f;
     if (head_dim == 128)
-        flash_prefill_kernel<128><<<grid, kFaThreads, FaCfg<128>::kSmem, s>>>(tm_q, tm_k, tm_v, out, n_rows, pos0, d_model, group, scale_log2, err);
-    else if (head_dim == 64)
-        flash_prefill_kernel<64><<<grid, kFaThreads, FaCfg<64>::kSmem, s>>>(tm_q, tm_k, tm_v, out, n_rows, pos0, d_model, group, scale_log2, err);
-    else
-        return cudaErrorInvalidValue;
-    return cudaGetLastError();
+        return launch_pdl(flash_prefill_kernel<128>, grid, dim3(kFaThreads), FaCfg<128>::kSmem, s, 1, tm_q, tm_k, tm_v, out, n_rows, pos0, d_model, group, scale_log2, err);
+    if (head_dim == 64)
+        return launch_pdl(flash_prefill_kernel<64>, grid, dim3(kFaThreads), FaCfg<64>::kSmem, s, 1, tm_q, tm_k, tm_v, out, n_rows, pos0, d_model, group, scale_log2, err);
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t configure_prefill_attention() {
