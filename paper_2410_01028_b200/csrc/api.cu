@@ -1022,8 +1022,11 @@ extern "C" int asd_reset(asd_ctx* x) {
 // One sublayer product of the dense prompt path. W_o and W_d (fp32 output) may come in parts of their reduction
 // dimension, which the row kernel that follows adds: as many as fit the buffer, up to eight.
 static int dense_gemm(asd_ctx* x, const CUtensorMap& tm_a, int layer, int which, int M, int N, int K, const GemmEpi& ep, int* parts = nullptr) {
-    const int max_parts = parts ? (int)std::min<size_t>(8, x->lay.pf_c_rows / M) : 1;
-    ASD_CUDA(x, launch_gemm_tn(tm_a, &x->tm_w[((size_t)layer * 4 + which) * kWBoxes], M, N, K, max_parts, ep, x->stream, parts));
+    const GemmPlan plan = plan_gemm(M, N, K, parts ? (int)std::min<size_t>(8, x->lay.pf_c_rows / M) : 1);
+    if (parts) *parts = plan.parts;
+    int box = 0;
+    while (box + 1 < kWBoxes && kWBoxRows[box] != plan.w_box()) ++box;
+    ASD_CUDA(x, launch_gemm_tn(tm_a, x->tm_w[((size_t)layer * 4 + which) * kWBoxes + box], M, N, K, plan, ep, x->stream));
     x->stats.kernel_launches += 1;
     return ASD_OK;
 }
@@ -1591,9 +1594,10 @@ extern "C" int asd_gemm_bf16(void* cuda_stream, int32_t M, int32_t N, int32_t K,
     if (device_info(&dv) != cudaSuccess) return ASD_ERR_CUDA;
     EncodeTiledFn encode = tensor_map_encoder();
     if (!encode) return ASD_ERR_CUDA;
-    CUtensorMap tm_a, tm_w[kWBoxes];
+    const GemmPlan plan = plan_gemm(M, N, K, 1);
+    CUtensorMap tm_a, tm_w;
     if (!encode_operand_map(encode, &tm_a, const_cast<uint16_t*>(A), (size_t)K, (size_t)M, kGemmBM) ||
-        !encode_weight_maps(encode, tm_w, const_cast<uint16_t*>(W), (size_t)K, (size_t)N))
+        !encode_operand_map(encode, &tm_w, const_cast<uint16_t*>(W), (size_t)K, (size_t)N, (uint32_t)plan.w_box()))
         return ASD_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     if (cudaMemsetAsync(dev_status, 0, 32, s) != cudaSuccess) return ASD_ERR_CUDA;
@@ -1601,7 +1605,7 @@ extern "C" int asd_gemm_bf16(void* cuda_stream, int32_t M, int32_t N, int32_t K,
     e.mode = kGemmF32;
     e.err = dev_status;
     e.c = C, e.ldc = N;
-    if (launch_gemm_tn(tm_a, tm_w, M, N, K, 1, e, s) != cudaSuccess) return ASD_ERR_CUDA;
+    if (launch_gemm_tn(tm_a, tm_w, M, N, K, plan, e, s) != cudaSuccess) return ASD_ERR_CUDA;
     return ASD_OK;
 }
 

@@ -100,7 +100,7 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 
 // ============================================================================================ the GEMM
 // Persistent units (CG = 1: one SM; CG = 2: a cluster of two SMs) walk the 128 * CG x BN tiles of the product, row tiles
-// fastest. Warp 0 (one lane) is the TMA producer, warp 1 (one lane) issues the MMAs and owns the tensor-memory allocation,
+// fastest. Warp 0 is the TMA producer, warp 1 issues the MMAs and owns the tensor-memory allocation,
 // warps 2-5 are the epilogue (warp w reads lanes 32 * (w % 4) .. + 31 of tensor memory, the quarter its position in the
 // warp group gives it access to). The accumulator is double-buffered in tensor memory (2 x BN columns), so the epilogue
 // of a tile runs while the MMAs of the next tile are already filling the other buffer. Barriers: full[s] (TMA bytes landed
@@ -110,12 +110,13 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 // a failed wait the roles fall through to the common exit, where the producer lets its copies in flight land and
 // the tensor memory is freed.
 //
-// What bounds it: an SM takes in at most 64 bytes per cycle from L2 (measured: 32 KB per 64 elements of the reduction at
-// 0.28 us, whatever the tile does with them). A 128 x 256 tile on one SM wants 48 KB per 512 cycles of MMA and is held
-// at two thirds of the tensor rate (0.37 us per 64 elements); two SMs sharing a 256 x 256 tile (cta_group::2, CG = 2: each
-// stages its 128 rows of A and half of the rows of W and keeps its 128 rows of the accumulator) want 32 KB each and run at
-// 0.285 us, 90 % tensor activity, until the power limit takes the clock down (2048 x 22016 x 4096: 337 us -> 299 us back
-// to back). With CG = 2 the leader (rank 0) issues the MMAs; full[s] lives in the leader and counts both CTAs' bytes;
+// What bounds it: an SM takes in at most about 115 bytes per ns (60 per cycle) from L2. A 128 x 256 tile on one SM wants 48 KB
+// per 64 elements of the reduction, 0.35 us where the MMAs take 0.27; two SMs sharing a 256 x 256 tile (cta_group::2, CG =
+// 2: each stages its 128 rows of A and half of the rows of W and keeps its 128 rows of the accumulator) want 32 KB each.
+// Products that fill the chip for rounds are bound by that and by the power limit, which takes the clock down (2048 x
+// 22016 x 4096: 337 us on single SMs at first, 299 us back to back on pairs, 90 % tensor activity); tiles of up to 64
+// columns by the issue of a k-block (0.14 us: wait, four MMAs, commit; 0.28 us when one lane of a divergent warp issued
+// them). With CG = 2 the leader (rank 0) issues the MMAs; full[s] lives in the leader and counts both CTAs' bytes;
 // empty[s] and acc_full[b] are signalled in both CTAs by multicast commits; acc_empty[b] lives in the leader and counts
 // the epilogue warps of both.
 //
@@ -126,22 +127,20 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 constexpr int kGemmThreads = 192;
 static int g_gemm_ctas = 148;  // persistent CTAs per launch: the SM count of the device (set by configure_prefill)
 
+// BN = 0: the width is a parameter of the launch (a multiple of 32).
 template <int BN, int CG>
 struct GemmCfg {
     static constexpr uint32_t kABytes = kGemmBM * kGemmBK * 2;
-    static constexpr uint32_t kBBytes = BN / CG * kGemmBK * 2;
-    static constexpr uint32_t kStageBytes = kABytes + kBBytes;
-    static constexpr int kStages = kStageBytes > 40000 ? 4 : 6;
-    static constexpr int kTmemCols = BN > 128 ? 512 : 256;  // a power of two
-    // rows of W per copy: the two halves of a 256-row tile on one SM come in two boxes, so that one tensor map serves
-    // every kind with boxes of this height
-    static constexpr int kWBox = CG == 1 && BN == 256 ? 128 : BN / CG;
-    static constexpr size_t kSmem = (size_t)kStages * kStageBytes + 1024 /* alignment */ + 256 /* barriers */;
+    static constexpr uint32_t kWRowBytes = kGemmBK * 2;
+    static constexpr size_t kRing = BN ? 6 * (kABytes + BN / CG * kWRowBytes) : 196608;  // bytes of all stages (BN = 0: at most)
+    static constexpr size_t kSmem = kRing + 1024 /* alignment */ + 256 /* barriers */;
+    static constexpr int kMaxStages = BN ? 6 : 8;
+    static constexpr int kAccStride = BN ? BN : 256;  // columns from one accumulator to the next
 };
 
 // The work of one launch: items (tile, part of the reduction dimension), tiles fastest, dealt round robin to the units.
 struct GemmWork {
-    int m_tiles, tiles, parts;
+    int m_tiles, tiles, parts, bn;
 };
 struct GemmItem {
     int tile, part, kb0, kb1;
@@ -166,12 +165,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w, int M, int N, int K, const GemmWork work,
                const GemmEpi ep) {
     using Cfg = GemmCfg<BN, CG>;
-    constexpr int kStages = Cfg::kStages;
+    const int bn = BN ? BN : work.bn;
+    const uint32_t stage_bytes = Cfg::kABytes + (uint32_t)(bn / CG) * Cfg::kWRowBytes;
+    const int kStages = BN ? Cfg::kMaxStages : min(Cfg::kMaxStages, (int)(Cfg::kRing / stage_bytes));
     extern __shared__ unsigned char gemm_smem_raw[];
     unsigned char* base = gemm_smem_raw + ((1024u - (smem_u32(gemm_smem_raw) & 1023u)) & 1023u);
-    uint64_t* full = reinterpret_cast<uint64_t*>(base + (size_t)kStages * Cfg::kStageBytes);
-    uint64_t* empty = full + kStages;
-    uint64_t* acc_full = empty + kStages;   // [2]
+    uint64_t* full = reinterpret_cast<uint64_t*>(base + Cfg::kRing);
+    uint64_t* empty = full + Cfg::kMaxStages;
+    uint64_t* acc_full = empty + Cfg::kMaxStages;   // [2]
     uint64_t* acc_empty = acc_full + 2;     // [2]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
 
@@ -192,8 +193,8 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         mbar_fence_init();
     }
     if (warp == 1) {
-        if (CG == 2) tmem_alloc_pair(tmem_slot, Cfg::kTmemCols), tmem_relinquish_pair();
-        else tmem_alloc(tmem_slot, Cfg::kTmemCols), tmem_relinquish();
+        if (CG == 2) tmem_alloc_pair(tmem_slot, 512), tmem_relinquish_pair();
+        else tmem_alloc(tmem_slot, 512), tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
@@ -201,86 +202,81 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     pdl_launch_dependents();
+    const uint32_t on = elect_one();
     auto load_w = [&](int s, int kb, int n0) {  // announces the bytes of a stage and requests its weights
-        if (rank == 0) mbar_expect_tx(&full[s], CG * Cfg::kStageBytes);  // the bytes of both CTAs
-        unsigned char* b_dst = base + (size_t)s * Cfg::kStageBytes + Cfg::kABytes;
-        if (CG == 2) {
-            tma_load_2d_pair(b_dst, &tm_w, kb * kGemmBK, n0, cluster_addr(&full[s], 0));
-        } else {
-#pragma unroll
-            for (int h = 0; h < BN / Cfg::kWBox; ++h)
-                tma_load_2d(b_dst + h * (Cfg::kWBox * kGemmBK * 2), &tm_w, kb * kGemmBK, n0 + h * Cfg::kWBox, &full[s]);
-        }
+        mbar_expect_tx_on(&full[s], CG * stage_bytes, CG == 2 ? on & (uint32_t)(rank == 0) : on);  // the bytes of both CTAs
+        unsigned char* b_dst = base + (size_t)s * stage_bytes + Cfg::kABytes;
+        if (CG == 2) tma_load_2d_pair(b_dst, &tm_w, kb * kGemmBK, n0, cluster_addr(&full[s], 0), on);
+        else tma_load_2d_on(b_dst, &tm_w, kb * kGemmBK, n0, &full[s], on);
     };
     int ahead = 0;  // k-blocks of the first item whose weights are requested before the kernel in front has ended
-    if (warp == 0 && lane == 0 && ep.w_static) {
+    if (warp == 0 && ep.w_static) {
         GemmItem it;
         if (gemm_item(work, num_kb, unit, n_units, 0, it))
-            for (; ahead < kStages && it.kb0 + ahead < it.kb1; ++ahead) load_w(ahead, it.kb0 + ahead, it.tile / work.m_tiles * BN + rank * (BN / CG));
+            for (; ahead < kStages && it.kb0 + ahead < it.kb1; ++ahead) load_w(ahead, it.kb0 + ahead, it.tile / work.m_tiles * bn + rank * (bn / CG));
     }
     pdl_wait();  // everything above overlaps the end of the kernel in front
 
     if (warp == 0) {
-        if (lane == 0) {
-            int issued = 0;  // k-blocks requested so far, over all items of this unit
-            bool ok = true;
-            GemmItem it;
-            for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
-                // row tiles vary fastest: units that run together share their weight tile (read once from HBM, then from L2)
-                const int m0 = (it.tile % work.m_tiles * CG + rank) * kGemmBM, n0 = it.tile / work.m_tiles * BN + rank * (BN / CG);
-                for (int kb = it.kb0; kb < it.kb1; ++kb) {
-                    const int s = issued % kStages;
-                    if (issued >= kStages) ok = mbar_wait(&empty[s], (uint32_t)((issued / kStages - 1) & 1), err, kErrGemmWait, 0, issued, s, 1);
-                    if (!ok) break;
-                    if (issued >= ahead) load_w(s, kb, n0);
-                    unsigned char* a_dst = base + (size_t)s * Cfg::kStageBytes;
-                    if (CG == 2) tma_load_2d_pair(a_dst, &tm_a, kb * kGemmBK, m0, cluster_addr(&full[s], 0));
-                    else tma_load_2d(a_dst, &tm_a, kb * kGemmBK, m0, &full[s]);
-                    ++issued;
-                }
+        int issued = 0;      // k-blocks requested so far, over all items of this unit
+        int s = 0, lap = 0;  // their ring position: issued = lap * kStages + s
+        bool ok = true;
+        GemmItem it;
+        for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
+            // row tiles vary fastest: units that run together share their weight tile (read once from HBM, then from L2)
+            const int m0 = (it.tile % work.m_tiles * CG + rank) * kGemmBM, n0 = it.tile / work.m_tiles * bn + rank * (bn / CG);
+            for (int kb = it.kb0; kb < it.kb1; ++kb) {
+                if (lap > 0) ok = mbar_wait_warp(&empty[s], (uint32_t)((lap - 1) & 1), err, kErrGemmWait, 0, issued, s, 1);
+                if (!ok) break;
+                if (issued >= ahead) load_w(s, kb, n0);
+                unsigned char* a_dst = base + (size_t)s * stage_bytes;
+                if (CG == 2) tma_load_2d_pair(a_dst, &tm_a, kb * kGemmBK, m0, cluster_addr(&full[s], 0), on);
+                else tma_load_2d_on(a_dst, &tm_a, kb * kGemmBK, m0, &full[s], on);
+                ++issued;
+                if (++s == kStages) s = 0, ++lap;
             }
-            if (rank == 0 && (!ok || *err != kErrNone)) {
-                // abandoned: let the copies still in flight (with CG = 2 those of both CTAs, which the cluster barrier below
-                // holds back) land before the shared memory is given back
-                for (int i = max(0, issued - kStages); i < issued; ++i) {
-                    const long long t0 = clock64();
-                    while (!mbar_try_wait(&full[i % kStages], (uint32_t)((i / kStages) & 1)) && clock64() - t0 < 20000000LL) {
-                    }
+        }
+        if (lane == 0 && rank == 0 && (!ok || *err != kErrNone)) {
+            // abandoned: let the copies still in flight (with CG = 2 those of both CTAs, which the cluster barrier below
+            // holds back) land before the shared memory is given back
+            for (int i = max(0, issued - kStages); i < issued; ++i) {
+                const long long t0 = clock64();
+                while (!mbar_try_wait(&full[i % kStages], (uint32_t)((i / kStages) & 1)) && clock64() - t0 < 20000000LL) {
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(kGemmBM * CG, BN);
-            int done = 0;  // k-blocks consumed so far
+        if (rank == 0) {
+            const uint32_t idesc = umma_idesc_bf16(kGemmBM * CG, bn);
+            const uint32_t base_addr = smem_u32(base);
+            int s = 0, lap = 0;  // ring position of the next k-block
             bool ok = true;
             GemmItem it;
             for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
                 const int buf = local & 1;
                 // the epilogue must have read this buffer's previous tile (item local - 2) before it is overwritten
-                if (local >= 2) ok = mbar_wait(&acc_empty[buf], (uint32_t)((local / 2 - 1) & 1), err, kErrGemmWait, 3, local, buf, 4);
+                if (local >= 2) ok = mbar_wait_warp(&acc_empty[buf], (uint32_t)((local / 2 - 1) & 1), err, kErrGemmWait, 3, local, buf, 4);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t tmem_d = tmem + (uint32_t)(buf * BN);
+                const uint32_t tmem_d = tmem + (uint32_t)(buf * Cfg::kAccStride);
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
-                    const int s = done % kStages;
-                    ok = mbar_wait(&full[s], (uint32_t)((done / kStages) & 1), err, kErrGemmWait, 1, done, s, 2);
+                    ok = mbar_wait_warp(&full[s], (uint32_t)(lap & 1), err, kErrGemmWait, 1, kb, s, 2);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t a_addr = smem_u32(base + (size_t)s * Cfg::kStageBytes);
+                    const uint32_t a_addr = base_addr + (uint32_t)s * stage_bytes;
                     const uint64_t a_desc = umma_desc_k128(a_addr), b_desc = umma_desc_k128(a_addr + Cfg::kABytes);
 #pragma unroll
                     for (int k = 0; k < kGemmBK / 16; ++k) {  // 16 elements = 32 bytes further along the swizzled row: +2 in the address field
                         const uint32_t acc = ((kb - it.kb0) | k) != 0 ? 1u : 0u;
-                        if (CG == 2) tc_mma_bf16_pair(tmem_d, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc);
-                        else tc_mma_bf16(tmem_d, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc);
+                        if (CG == 2) tc_mma_bf16_pair(tmem_d, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc, on);
+                        else tc_mma_bf16(tmem_d, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, acc, on);
                     }
-                    if (CG == 2) tc_commit_pair(&empty[s]);  // the stage may be refilled once these MMAs have read it
-                    else tc_commit(&empty[s]);
-                    ++done;
+                    if (CG == 2) tc_commit_pair(&empty[s], on);  // the stage may be refilled once these MMAs have read it
+                    else tc_commit(&empty[s], on);
+                    if (++s == kStages) s = 0, ++lap;
                 }
-                if (CG == 2) tc_commit_pair(&acc_full[buf]);  // arrives when every MMA issued above has finished
-                else tc_commit(&acc_full[buf]);
+                if (CG == 2) tc_commit_pair(&acc_full[buf], on);  // arrives when every MMA issued above has finished
+                else tc_commit(&acc_full[buf], on);
             }
         }
     } else {
@@ -289,14 +285,14 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         GemmItem it;
         for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
             const int buf = local & 1;
-            const int m0 = (it.tile % work.m_tiles * CG + rank) * kGemmBM, n0 = it.tile / work.m_tiles * BN;
+            const int m0 = (it.tile % work.m_tiles * CG + rank) * kGemmBM, n0 = it.tile / work.m_tiles * bn;
             const int row = m0 + quarter * 32 + lane;
             ok = mbar_wait(&acc_full[buf], (uint32_t)((local / 2) & 1), err, kErrGemmWait, 2, local, buf, 3) && *err == kErrNone;
             ok = __all_sync(0xffffffffu, ok);  // tensor-memory loads are warp-wide
             tc_fence_after();
             if (!ok) break;
-            const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN);
-            const int n_cols = min(BN, N - n0);
+            const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * Cfg::kAccStride);
+            const int n_cols = min(bn, N - n0);
             for (int c = 0; c < n_cols; c += 32) {
                 float v[32];
                 tmem_ld32(acc + c, v);
@@ -315,17 +311,10 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (CG == 2) cluster_sync_all();  // no CTA leaves while the other's copies, commits or arrivals may still reach it
     if (warp == 1) {
         tc_fence_after();
-        if (CG == 2) tmem_dealloc_pair(tmem, Cfg::kTmemCols);
-        else tmem_dealloc(tmem, Cfg::kTmemCols);
+        if (CG == 2) tmem_dealloc_pair(tmem, 512);
+        else tmem_dealloc(tmem, 512);
     }
 }
-
-// The kinds of unit and what a k-block (64 elements of the reduction) of one of their tiles takes, in ns: measured as the
-// slope between K = 4096 and 11008 with one round of tiles; the two narrower pair tiles by the bytes an SM takes in.
-struct GemmKind {
-    int bn, cg, ns, w_map;
-};
-constexpr GemmKind kGemmKinds[] = {{256, 2, 285, kWBox128}, {224, 2, 267, kWBox112}, {192, 2, 250, kWBox96}, {128, 1, 280, kWBox128}, {256, 1, 370, kWBox128}};
 
 template <int BN, int CG>
 static cudaError_t launch_gemm(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmWork& w, const GemmEpi& ep,
@@ -334,40 +323,50 @@ static cudaError_t launch_gemm(const CUtensorMap& tm_a, const CUtensorMap& tm_w,
     return launch_pdl(gemm_tn_kernel<BN, CG>, grid, dim3(kGemmThreads), GemmCfg<BN, CG>::kSmem, s, CG, tm_a, tm_w, M, N, K, w, ep);
 }
 
-// The rule: the kind and the number of parts with the least time over their rounds, rounds x k-blocks of a part x the time
-// of a k-block, plus writing and reading the further parts (8 bytes per element at about 4 TB/s). It picks pairs of SMs
-// for nearly every prompt of more than 128 rows (511 x 12288 x 4096: 192-column pair tiles, two rounds as with 256 columns
-// but shorter ones), single SMs where those waste half a row tile (257 rows: one round of 144 tiles, 39.5 us, against
-// two rounds of 96 pair tiles, 52.2 us) and for up to 128 rows (22016 x 4096: 86 tiles of 256 columns 44.9 us, 172 of 128
-// in two rounds 56.3 us).
-cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap* tm_w, int M, int N, int K, int max_parts, const GemmEpi& ep, cudaStream_t s,
-                           int* parts_out) {
-    if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
+// The rule: the tile and the number of parts with the least time over their rounds: rounds x k-blocks of a part x the time
+// of a k-block (64 elements of the reduction), plus writing and reading the further parts (8 bytes per element at about 4
+// TB/s). The times of a k-block in the table are the slopes of one round of tiles; with every SM busy and several rounds all
+// of them grow by about a quarter. Over 48 products of 64 to 2048 rows and 3072 to 22016 columns, each timed with all ten
+// tiles, the rule's choice was within 0.2 % of the best on average and 5 % at worst. Pairs of SMs win where the tiles fill
+// the chip for rounds (2048 x 22016 x 4096: pairs 249-256 us, single SMs 302-334), 128 columns on single SMs where one round is
+// enough (511 x 4096 x 11008: 45.5 us against 63.7 with 256-column pair tiles), narrow tiles for short prompts (64 x 4096 x
+// 11008: 33 us against 60).
+GemmPlan plan_gemm(int M, int N, int K, int max_parts) {
     const int num_kb = (K + kGemmBK - 1) / kGemmBK;
-    int best = 0;
     long long best_ns = -1;
-    GemmWork best_work{};
-    for (int i = 0; i < (int)(sizeof(kGemmKinds) / sizeof(kGemmKinds[0])); ++i) {
-        const GemmKind& k = kGemmKinds[i];
-        GemmWork w{};
-        w.m_tiles = (M + kGemmBM * k.cg - 1) / (kGemmBM * k.cg);
-        w.tiles = w.m_tiles * ((N + k.bn - 1) / k.bn);
-        const int units = g_gemm_ctas / k.cg;
-        for (w.parts = 1; w.parts == 1 || (w.parts <= max_parts && num_kb / w.parts >= 8); ++w.parts) {
-            const long long rounds = ((long long)w.tiles * w.parts + units - 1) / units;
-            const long long ns = rounds * ((num_kb + w.parts - 1) / w.parts) * k.ns + (long long)(w.parts - 1) * M * N / 500;
-            if (best_ns < 0 || ns < best_ns) best = i, best_ns = ns, best_work = w;
+    GemmPlan best{};
+    auto consider = [&](int bn, int cg, int ns_kb) {
+        GemmPlan p{};
+        p.bn = bn, p.cg = cg;
+        p.m_tiles = (M + kGemmBM * cg - 1) / (kGemmBM * cg);
+        p.tiles = p.m_tiles * ((N + bn - 1) / bn);
+        const int units = g_gemm_ctas / cg;
+        for (p.parts = 1; p.parts == 1 || (p.parts <= max_parts && num_kb / p.parts >= 8); ++p.parts) {
+            const long long rounds = ((long long)p.tiles * p.parts + units - 1) / units;
+            const long long ns = rounds * ((num_kb + p.parts - 1) / p.parts) * ns_kb + (long long)(p.parts - 1) * M * N / 500;
+            if (best_ns < 0 || ns < best_ns) best_ns = ns, best = p;
         }
-    }
-    if (parts_out) *parts_out = best_work.parts;
-    const CUtensorMap& wm = tm_w[kGemmKinds[best].w_map];
-    switch (best) {
-        case 0: return launch_gemm<256, 2>(tm_a, wm, M, N, K, best_work, ep, s);
-        case 1: return launch_gemm<224, 2>(tm_a, wm, M, N, K, best_work, ep, s);
-        case 2: return launch_gemm<192, 2>(tm_a, wm, M, N, K, best_work, ep, s);
-        case 3: return launch_gemm<128, 1>(tm_a, wm, M, N, K, best_work, ep, s);
-        default: return launch_gemm<256, 1>(tm_a, wm, M, N, K, best_work, ep, s);
-    }
+    };
+    consider(256, 2, 315);
+    consider(224, 2, 281);
+    consider(192, 2, 247);
+    consider(256, 1, 354);
+    consider(192, 1, 316);
+    consider(160, 1, 244);
+    consider(128, 1, 209);
+    consider(96, 1, 195);
+    consider(64, 1, 145);
+    consider(32, 1, 138);
+    return best;
+}
+
+cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmPlan& p, const GemmEpi& ep, cudaStream_t s) {
+    if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
+    const GemmWork w{p.m_tiles, p.tiles, p.parts, p.bn};
+    if (p.cg == 1) return launch_gemm<0, 1>(tm_a, tm_w, M, N, K, w, ep, s);
+    if (p.bn == 256) return launch_gemm<256, 2>(tm_a, tm_w, M, N, K, w, ep, s);
+    if (p.bn == 224) return launch_gemm<224, 2>(tm_a, tm_w, M, N, K, w, ep, s);
+    return launch_gemm<192, 2>(tm_a, tm_w, M, N, K, w, ep, s);
 }
 
 // ============================================================================================ row kernels
@@ -568,8 +567,7 @@ cudaError_t configure_prefill(int max_smem) {
     ASD_SET_GEMM(256, 2);
     ASD_SET_GEMM(224, 2);
     ASD_SET_GEMM(192, 2);
-    ASD_SET_GEMM(128, 1);
-    ASD_SET_GEMM(256, 1);
+    ASD_SET_GEMM(0, 1);
 #undef ASD_SET_GEMM
     return configure_prefill_attention();
 }

@@ -45,15 +45,21 @@ struct GemmEpi {
 
 cudaError_t configure_prefill(int max_smem);
 
-// tensor maps of one weight matrix [N, K] with 128-byte swizzle: boxes of 64 elements x 128, 112 or 96 rows
-enum GemmWeightMap : int { kWBox128 = 0, kWBox112 = 1, kWBox96 = 2, kWBoxes = 3 };
-constexpr int kWBoxRows[kWBoxes] = {128, 112, 96};
+// How a product runs: tiles of 128 * cg rows x bn columns on units of cg SMs, the reduction dimension in `parts` parts.
+struct GemmPlan {
+    int bn, cg, m_tiles, tiles, parts;
+    int w_box() const { return bn / cg; }  // rows of a box of W's tensor map
+};
+// the heights that w_box() can have; a weight matrix has one tensor map for each
+constexpr int kWBoxRows[] = {32, 64, 96, 112, 128, 160, 192, 256};
+constexpr int kWBoxes = sizeof(kWBoxRows) / sizeof(kWBoxRows[0]);
 
-// C[M, N] = A[M, K] * W[N, K]^T, bf16 operands described by 2-D tensor maps (A in boxes of 64 x 128, 128-byte swizzle; tm_w:
-// the kWBoxes maps of W), fp32 accumulation. With max_parts > 1 (kGemmF32 only) the reduction dimension may be cut into
-// up to that many parts, *parts_out products of their own c_part_stride apart.
-cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap* tm_w, int M, int N, int K, int max_parts, const GemmEpi& ep, cudaStream_t s,
-                           int* parts_out = nullptr);
+// The plan of C[M, N] = A[M, K] * W[N, K]^T. With max_parts > 1 (kGemmF32 only) the reduction dimension may be cut into up to that
+// many parts, products of their own c_part_stride apart.
+GemmPlan plan_gemm(int M, int N, int K, int max_parts);
+// bf16 operands described by 2-D tensor maps (128-byte swizzle, A in boxes of 64 elements x 128 rows, W in boxes of 64 x
+// w_box()), fp32 accumulation
+cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmPlan& plan, const GemmEpi& ep, cudaStream_t s);
 
 // x[r, :] = embedding row of tokens[r] (fp32); xn[r, :] = bf16(RMSNorm(x[r]) * gain)
 cudaError_t launch_embed_norm(const int* tokens, int n_rows, int d, int vocab, const __nv_bfloat16* embed, const __nv_bfloat16* gain,

@@ -82,7 +82,7 @@ __device__ __forceinline__ void probabilities32(const uint32_t (&s)[32], unsigne
     tmem_st16(t_lo, w);
 }
 
-// Warps 0-3: softmax and epilogue, thread = query row. Warp 4: TMA producer (one lane). Warp 5: issues the MMAs (one lane)
+// Warps 0-3: softmax and epilogue, thread = query row. Warp 4: TMA producer. Warp 5: issues the MMAs
 // and owns the tensor-memory allocation. Barriers: q_full, k_full / v_full[s] (bytes landed), k_empty / v_empty[s] (the
 // MMAs reading the stage have finished), s_full (S of tile j is complete, and with it every earlier MMA: O holds the
 // tiles before j and P may be overwritten; phase n_kt: O is complete), p_full (the 128 rows' P of tile j are in tensor
@@ -127,87 +127,84 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     pdl_launch_dependents();
     pdl_wait();  // everything above overlaps the end of the kernel before
 
+    const uint32_t on = elect_one();
     if (warp == 4) {
-        if (lane == 0) {
-            mbar_expect_tx(q_full, Cfg::kQBytes);
-            for (int p = 0; p < Cfg::kPanels; ++p) tma_load_2d(base + p * Cfg::kQPanel, &tm_q, head * HD + p * 64, r0, q_full);
-            bool ok = true;
-            int nk = 0, nv = 0;  // K and V tiles requested so far
-            while (nv < n_kt && ok) {
-                // K runs one tile ahead of V: S of tile j + 1 is issued right behind P V of tile j
-                if (nk < n_kt && nk <= nv + 1) {
-                    const int s = nk % kFaStages;
-                    if (nk >= kFaStages) ok = mbar_wait(&k_empty[s], (uint32_t)((nk / kFaStages - 1) & 1), err, kErrAttnWait, 0, nk, s, 1);
-                    if (!ok) break;
-                    mbar_expect_tx(&k_full[s], Cfg::kKvBytes);
-                    for (int p = 0; p < Cfg::kPanels; ++p)
-                        tma_load_2d(k_smem + s * Cfg::kKvBytes + p * Cfg::kKvPanel, &tm_k, kvh * HD + p * 64, nk * kFaKeys, &k_full[s]);
-                    ++nk;
-                    if (nk == 1 && n_kt > 1) continue;
-                }
-                const int s = nv % kFaStages;
-                if (nv >= kFaStages) ok = mbar_wait(&v_empty[s], (uint32_t)((nv / kFaStages - 1) & 1), err, kErrAttnWait, 0, nv, s, 2);
+        mbar_expect_tx_on(q_full, Cfg::kQBytes, on);
+        for (int p = 0; p < Cfg::kPanels; ++p) tma_load_2d_on(base + p * Cfg::kQPanel, &tm_q, head * HD + p * 64, r0, q_full, on);
+        bool ok = true;
+        int nk = 0, nv = 0;  // K and V tiles requested so far
+        while (nv < n_kt && ok) {
+            // K runs one tile ahead of V: S of tile j + 1 is issued right behind P V of tile j
+            if (nk < n_kt && nk <= nv + 1) {
+                const int s = nk % kFaStages;
+                if (nk >= kFaStages) ok = mbar_wait_warp(&k_empty[s], (uint32_t)((nk / kFaStages - 1) & 1), err, kErrAttnWait, 0, nk, s, 1);
                 if (!ok) break;
-                mbar_expect_tx(&v_full[s], Cfg::kKvBytes);
+                mbar_expect_tx_on(&k_full[s], Cfg::kKvBytes, on);
                 for (int p = 0; p < Cfg::kPanels; ++p)
-                    tma_load_2d(v_smem + s * Cfg::kKvBytes + p * Cfg::kKvPanel, &tm_v, kvh * HD + p * 64, nv * kFaKeys, &v_full[s]);
-                ++nv;
+                    tma_load_2d_on(k_smem + s * Cfg::kKvBytes + p * Cfg::kKvPanel, &tm_k, kvh * HD + p * 64, nk * kFaKeys, &k_full[s], on);
+                ++nk;
+                if (nk == 1 && n_kt > 1) continue;
             }
-            if (!ok || *err != kErrNone) {
-                // abandoned: let the copies still in flight land before the CTA gives its shared memory back
-                const long long t0 = clock64();
-                auto landed = [&](uint64_t* bar, int n) { return n <= 0 || mbar_try_wait(bar, (uint32_t)((n - 1) & 1)); };
-                bool all = false;
-                while (!all && clock64() - t0 < 20000000LL) {
-                    all = landed(q_full, 1);
-                    for (int s = 0; s < kFaStages; ++s)
-                        all = all && landed(&k_full[s], (nk + kFaStages - 1 - s) / kFaStages) && landed(&v_full[s], (nv + kFaStages - 1 - s) / kFaStages);
-                }
+            const int s = nv % kFaStages;
+            if (nv >= kFaStages) ok = mbar_wait_warp(&v_empty[s], (uint32_t)((nv / kFaStages - 1) & 1), err, kErrAttnWait, 0, nv, s, 2);
+            if (!ok) break;
+            mbar_expect_tx_on(&v_full[s], Cfg::kKvBytes, on);
+            for (int p = 0; p < Cfg::kPanels; ++p)
+                tma_load_2d_on(v_smem + s * Cfg::kKvBytes + p * Cfg::kKvPanel, &tm_v, kvh * HD + p * 64, nv * kFaKeys, &v_full[s], on);
+            ++nv;
+        }
+        if (lane == 0 && (!ok || *err != kErrNone)) {
+            // abandoned: let the copies still in flight land before the CTA gives its shared memory back
+            const long long t0 = clock64();
+            auto landed = [&](uint64_t* bar, int n) { return n <= 0 || mbar_try_wait(bar, (uint32_t)((n - 1) & 1)); };
+            bool all = false;
+            while (!all && clock64() - t0 < 20000000LL) {
+                all = landed(q_full, 1);
+                for (int s = 0; s < kFaStages; ++s)
+                    all = all && landed(&k_full[s], (nk + kFaStages - 1 - s) / kFaStages) && landed(&v_full[s], (nv + kFaStages - 1 - s) / kFaStages);
             }
         }
     } else if (warp == 5) {
-        if (lane == 0) {
-            constexpr uint32_t idesc_s = umma_idesc_bf16(kFaRows, kFaKeys);
-            constexpr uint32_t idesc_o = umma_idesc_bf16(kFaRows, HD) | (1u << 16);  // V is [key][dimension]: N-major
-            const uint32_t q_addr = smem_u32(base);
-            bool ok = mbar_wait(q_full, 0, err, kErrAttnWait, 1, 0, 0, 3);
-            auto scores = [&](int j) {  // S of tile j
-                const int s = j % kFaStages;
-                ok = ok && mbar_wait(&k_full[s], (uint32_t)((j / kFaStages) & 1), err, kErrAttnWait, 1, j, s, 4);
-                if (!ok) return;
-                tc_fence_after();
-                const uint32_t k_addr = smem_u32(k_smem) + s * Cfg::kKvBytes;
+        constexpr uint32_t idesc_s = umma_idesc_bf16(kFaRows, kFaKeys);
+        constexpr uint32_t idesc_o = umma_idesc_bf16(kFaRows, HD) | (1u << 16);  // V is [key][dimension]: N-major
+        const uint32_t q_addr = smem_u32(base);
+        bool ok = mbar_wait_warp(q_full, 0, err, kErrAttnWait, 1, 0, 0, 3);
+        auto scores = [&](int j) {  // S of tile j
+            const int s = j % kFaStages;
+            ok = ok && mbar_wait_warp(&k_full[s], (uint32_t)((j / kFaStages) & 1), err, kErrAttnWait, 1, j, s, 4);
+            if (!ok) return;
+            tc_fence_after();
+            const uint32_t k_addr = smem_u32(k_smem) + s * Cfg::kKvBytes;
 #pragma unroll
-                for (int k = 0; k < HD / 16; ++k)
-                    tc_mma_bf16(tmem + kFaColS, umma_desc_k128(q_addr + (k / 4) * Cfg::kQPanel) + 2 * (k % 4),
-                                umma_desc_k128(k_addr + (k / 4) * Cfg::kKvPanel) + 2 * (k % 4), idesc_s, k != 0);
-                tc_commit(&k_empty[s]);
-                tc_commit(s_full);
-            };
-            scores(0);
-            for (int j = 0; j < n_kt && ok; ++j) {
-                const int s = j % kFaStages;
-                ok = mbar_wait(&v_full[s], (uint32_t)((j / kFaStages) & 1), err, kErrAttnWait, 1, j, s, 5) &&
-                     mbar_wait(p_full, (uint32_t)(j & 1), err, kErrAttnWait, 1, j, s, 6);
-                if (!ok) break;
-                tc_fence_after();
-                const uint64_t v_desc = umma_desc_mn128(smem_u32(v_smem) + s * Cfg::kKvBytes, Cfg::kKvPanel);
+            for (int k = 0; k < HD / 16; ++k)
+                tc_mma_bf16(tmem + kFaColS, umma_desc_k128(q_addr + (k / 4) * Cfg::kQPanel) + 2 * (k % 4),
+                            umma_desc_k128(k_addr + (k / 4) * Cfg::kKvPanel) + 2 * (k % 4), idesc_s, k != 0, on);
+            tc_commit(&k_empty[s], on);
+            tc_commit(s_full, on);
+        };
+        scores(0);
+        for (int j = 0; j < n_kt && ok; ++j) {
+            const int s = j % kFaStages;
+            ok = mbar_wait_warp(&v_full[s], (uint32_t)((j / kFaStages) & 1), err, kErrAttnWait, 1, j, s, 5) &&
+                 mbar_wait_warp(p_full, (uint32_t)(j & 1), err, kErrAttnWait, 1, j, s, 6);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t v_desc = umma_desc_mn128(smem_u32(v_smem) + s * Cfg::kKvBytes, Cfg::kKvPanel);
 #pragma unroll
-                for (int t = 0; t < 3; ++t) {  // lo, mid, hi: the smallest terms first
-                    const uint32_t a = tmem + (t == 0 ? kFaColLo : (t == 1 ? kFaColMid : kFaColHi));
+            for (int t = 0; t < 3; ++t) {  // lo, mid, hi: the smallest terms first
+                const uint32_t a = tmem + (t == 0 ? kFaColLo : (t == 1 ? kFaColMid : kFaColHi));
 #pragma unroll
-                    for (int k = 0; k < kFaKeys / 16; ++k)  // 16 keys: 8 columns of P, 2048 bytes of V
-                        tc_mma_bf16_ts(tmem, a + 8 * k, v_desc + (uint64_t)(128 * k), idesc_o, (j | t | k) != 0);
-                }
-                tc_commit(&v_empty[s]);
-                if (j + 1 < n_kt) scores(j + 1);
-                else tc_commit(s_full);  // O is complete
+                for (int k = 0; k < kFaKeys / 16; ++k)  // 16 keys: 8 columns of P, 2048 bytes of V
+                    tc_mma_bf16_ts(tmem, a + 8 * k, v_desc + (uint64_t)(128 * k), idesc_o, (j | t | k) != 0, on);
             }
-            if (!ok) {  // abandoned: the MMAs already issued end before the tensor memory is freed
-                tc_commit(drained);
-                const long long t0 = clock64();
-                while (!mbar_try_wait(drained, 0) && clock64() - t0 < 20000000LL) {
-                }
+            tc_commit(&v_empty[s], on);
+            if (j + 1 < n_kt) scores(j + 1);
+            else tc_commit(s_full, on);  // O is complete
+        }
+        if (!ok) {  // abandoned: the MMAs already issued end before the tensor memory is freed
+            tc_commit(drained, on);
+            const long long t0 = clock64();
+            while (!mbar_try_wait(drained, 0) && clock64() - t0 < 20000000LL) {
             }
         }
     } else {

@@ -1,5 +1,5 @@
 """GPU parity of the prompt products for every kind of tile (pairs of SMs on 256-, 224- and 192-column tiles, single SMs on
-256- and 128-column tiles) at ragged edges, and for products cut into parts of their reduction dimension."""
+tiles of 32 to 256 columns) at ragged edges, and for products cut into parts of their reduction dimension."""
 import numpy as np
 import pytest
 
@@ -11,10 +11,12 @@ pytestmark = pytest.mark.gpu
 
 
 # fp32 sums of K <= 136 products: an error of at most K 2^-24 of the sum of magnitudes, below 1e-5 of the largest output
-@pytest.mark.parametrize("M,N,K", [(3, 40, 72), (129, 1000, 136), (255, 2100, 72),  # 192-column pair tiles
+@pytest.mark.parametrize("M,N,K", [(129, 12289, 72), (1300, 2100, 136),             # 192-column pair tiles
                                    (257, 9401, 136), (640, 6001, 72),               # 256-column pair tiles, several rounds
                                    (640, 5000, 136), (640, 9473, 72),               # 224-column pair tiles
-                                   (3, 18945, 136), (383, 12289, 72)])              # 256-column tiles on single SMs
+                                   (3, 40, 72), (129, 1000, 136), (1, 6001, 72),    # single SMs: 32, 64,
+                                   (3, 9473, 136), (130, 9401, 72), (3, 18945, 136),  # 96, 128, 160,
+                                   (383, 12289, 72)])                               # 256 columns
 def test_every_kind_of_tile(M, N, K):
     import torch
     import paper_2410_01028_b200 as asd
