@@ -22,6 +22,7 @@ namespace asd {
 constexpr int kPrefillRows = kPassMaxRows;  // prompt rows per pass of the chunked prefill
 constexpr size_t kAlign = 256;
 constexpr int kMaxGemvGrid = 1024;
+constexpr size_t kPinnedOut = 256 * 1024;  // larger results of inspection calls go straight to the caller's memory
 constexpr long long kShortWaitCycles = 2000000LL;  // ASD_DEBUG_SHORT_WAITS: about a millisecond per wait
 
 static size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -370,7 +371,14 @@ struct asd_ctx {
     std::vector<CUtensorMap> tm_w;
     std::vector<CUtensorMap> tm_kv;  // per layer the K and the V cache (the pass kernel reads its own copy in the workspace)
     asd_stats stats{};
-    int32_t* pinned = nullptr;  // small host staging buffer
+    // pinned host memory: 4 KB of token / status words, the per-row cosines of one pass, the tokens of a call on their way to
+    // the device, and what the inspection calls bring back (a copy between pinned memory and the device is one transfer;
+    // from and to pageable memory the runtime stages it and waits)
+    int32_t* pinned = nullptr;
+    int32_t* pinned_tokens = nullptr;
+    unsigned char* pinned_out = nullptr;
+    bool tables_current = false;   // the stage tables on the device are those of skip_attn / skip_mlp
+    bool skipped_cos_nan = false;  // the cosines of the sublayers in the mask are NaN: no pass of the full model since they were set
     uint32_t bar_base = 0;      // value of the grid-barrier counter at the start of the next pass
     uint32_t pass_tag = 0x1000; // tag of stage 0 of the next pass in the tagged handoff buffers (never 0: the workspace starts zeroed)
     int n_stages_full = 0, n_stages_draft = 0, n_resid_full = 0, n_resid_draft = 0;
@@ -509,6 +517,7 @@ static int make_tensor_maps(asd_ctx* x) {
 // without the sublayers in the skip mask: they get no stage, so nothing is streamed or touched for them),
 // table 2 = the LM head alone on a hidden state that is already in place (last row of a dense prompt pass).
 static int build_stage_tables(asd_ctx* x) {
+    if (x->tables_current) return ASD_OK;
     const asd_config& c = x->c;
     const Layout& ly = x->lay;
     const int d = c.d_model, f = c.d_ffn, kvd = x->kv_dim, L = c.n_layers;
@@ -587,6 +596,7 @@ static int build_stage_tables(asd_ctx* x) {
     }
     ASD_CUDA(x, cudaMemcpyAsync(x->ws + ly.stage_tab, tab.data(), tab.size() * sizeof(StageDesc), cudaMemcpyHostToDevice, x->stream));
     ASD_CUDA(x, cudaMemcpyAsync(x->ws + ly.resid_tab, resid.data(), resid.size() * sizeof(ResidOut), cudaMemcpyHostToDevice, x->stream));
+    x->tables_current = true;
     return ASD_OK;
 }
 
@@ -606,7 +616,10 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     if (!plan_pass(*x->dev, c, M, &pl)) return fail(x, ASD_ERR_ARG, "decoder shape does not fit the pass kernel's shared-memory plan");
 
     float* cosv = x->at<float>(ly.cosv);
-    ASD_CUDA(x, cudaMemsetAsync(cosv, 0xFF, (size_t)2 * std::max(L, 1) * kPassMaxRows * 4, s));  // NaN = skipped
+    // NaN = skipped. A pass of the full model writes every sublayer's entry of its rows, a draft pass those of the kept
+    // sublayers, so the others have to be set only in front of the first draft pass behind a full one.
+    if (use_mask && !x->skipped_cos_nan) ASD_CUDA(x, cudaMemsetAsync(cosv, 0xFF, (size_t)2 * std::max(L, 1) * kPassMaxRows * 4, s));
+    x->skipped_cos_nan = use_mask;
 
     unsigned* words = x->at<unsigned>(ly.sync_words);
     PassParams p{};
@@ -704,6 +717,18 @@ static int read_back(asd_ctx* x, const int* dev_src, int n) {
     ASD_CUDA(x, cudaMemcpyAsync(x->pinned + 32, x->at<unsigned>(x->lay.sync_words) + 32, 32, cudaMemcpyDeviceToHost, x->stream));
     ASD_CUDA(x, cudaStreamSynchronize(x->stream));
     return check_device_error(x, x->pinned + 32);
+}
+
+// copies device results to the caller's memory (up to two pieces) and waits for the stream
+static int copy_out(asd_ctx* x, void* dst0, const void* src0, size_t bytes0, void* dst1 = nullptr, const void* src1 = nullptr, size_t bytes1 = 0) {
+    const size_t n0 = dst0 ? bytes0 : 0, n1 = dst1 ? bytes1 : 0;
+    const bool staged = n0 + n1 <= kPinnedOut;
+    if (n0) ASD_CUDA(x, cudaMemcpyAsync(staged ? x->pinned_out : dst0, src0, n0, cudaMemcpyDeviceToHost, x->stream));
+    if (n1) ASD_CUDA(x, cudaMemcpyAsync(staged ? x->pinned_out + n0 : dst1, src1, n1, cudaMemcpyDeviceToHost, x->stream));
+    ASD_CUDA(x, cudaStreamSynchronize(x->stream));
+    if (staged && n0) memcpy(dst0, x->pinned_out, n0);
+    if (staged && n1) memcpy(dst1, x->pinned_out + n0, n1);
+    return ASD_OK;
 }
 
 // Sampling: row `row` of the pass that has just been launched chooses the token at `position`. Its distribution
@@ -808,8 +833,15 @@ extern "C" int asd_create(const asd_config* cfg, void* dev_workspace, size_t byt
             return ASD_ERR_ARG;
         }
     }
-    // 4 KB of token / status words, then room for the per-row cosines of one pass ([2][L][kPassMaxRows] floats)
-    if ((e = cudaHostAlloc((void**)&x->pinned, 4096 + (size_t)2 * std::max(cfg->n_layers, 1) * kPassMaxRows * 4, cudaHostAllocDefault)) != cudaSuccess) return bail(e);
+    {
+        const size_t cos_bytes = align_up((size_t)2 * std::max(cfg->n_layers, 1) * kPassMaxRows * 4);
+        const size_t tok_bytes = align_up(((size_t)cfg->max_seq + 64) * 4);
+        unsigned char* h = nullptr;
+        if ((e = cudaHostAlloc((void**)&h, 4096 + cos_bytes + tok_bytes + kPinnedOut, cudaHostAllocDefault)) != cudaSuccess) return bail(e);
+        x->pinned = reinterpret_cast<int32_t*>(h);
+        x->pinned_tokens = reinterpret_cast<int32_t*>(h + 4096 + cos_bytes);
+        x->pinned_out = h + 4096 + cos_bytes + tok_bytes;
+    }
     // rotary table: angle(p, j) = p * theta^(-2j/head_dim), evaluated in double, stored as float
     {
         const int half = cfg->head_dim / 2;
@@ -997,12 +1029,20 @@ extern "C" int asd_load_weights_file(asd_ctx* x, const char* path) {
     return upload_weights(x, w);
 }
 
+// the draft model's mask (null = nothing skipped); the stage tables are built again only when it changes
+static void set_masks(asd_ctx* x, const uint8_t* skip_attn, const uint8_t* skip_mlp) {
+    for (int l = 0; l < x->c.n_layers; ++l) {
+        const uint8_t a = skip_attn && skip_attn[l] ? 1 : 0, m = skip_mlp && skip_mlp[l] ? 1 : 0;
+        if (a != x->skip_attn[l] || m != x->skip_mlp[l]) x->tables_current = x->skipped_cos_nan = false;
+        x->skip_attn[l] = a, x->skip_mlp[l] = m;
+    }
+}
+
 extern "C" int asd_reset(asd_ctx* x) {
     if (!x) return ASD_ERR_ARG;
     ASD_CUDA(x, cudaStreamSynchronize(x->stream));
     x->n_committed = x->draft_cursor = 0;
-    std::fill(x->skip_attn.begin(), x->skip_attn.end(), 0);
-    std::fill(x->skip_mlp.begin(), x->skip_mlp.end(), 0);
+    set_masks(x, nullptr, nullptr);
     x->n_sim_rows = 0;
     std::fill(x->run_attn.begin(), x->run_attn.end(), 0.0);
     std::fill(x->run_mlp.begin(), x->run_mlp.end(), 0.0);
@@ -1156,8 +1196,9 @@ extern "C" int asd_prefill_device(asd_ctx* x, const int32_t* dev_tokens, int32_t
 static int stage_tokens(asd_ctx* x, const int32_t* tokens, int32_t n, int32_t* dev_dst) {
     for (int i = 0; i < n; ++i)
         if (tokens[i] < 0 || tokens[i] >= x->c.vocab) return fail(x, ASD_ERR_ARG, "token id out of range");
-    ASD_CUDA(x, cudaMemcpyAsync(dev_dst, tokens, (size_t)n * 4, cudaMemcpyHostToDevice, x->stream));
-    ASD_CUDA(x, cudaStreamSynchronize(x->stream));  // the host array is only borrowed for the call
+    // the host array is only borrowed for the call; its pinned copy is free again when the call returns, behind its read-back
+    memcpy(x->pinned_tokens, tokens, (size_t)n * 4);
+    ASD_CUDA(x, cudaMemcpyAsync(dev_dst, x->pinned_tokens, (size_t)n * 4, cudaMemcpyHostToDevice, x->stream));
     return ASD_OK;
 }
 
@@ -1178,8 +1219,8 @@ extern "C" int asd_get_similarity(asd_ctx* x, float* c_attn, float* c_mlp, int32
     if (x->n_sim_rows == 0) return fail(x, ASD_ERR_STATE, "no prompt row has been processed");
     const int L = x->c.n_layers;
     std::vector<double> h(2 * (size_t)std::max(L, 1));
-    ASD_CUDA(x, cudaMemcpyAsync(h.data(), x->ws + x->lay.sumcos, h.size() * 8, cudaMemcpyDeviceToHost, x->stream));
-    ASD_CUDA(x, cudaStreamSynchronize(x->stream));
+    const int rc = copy_out(x, h.data(), x->ws + x->lay.sumcos, h.size() * 8);
+    if (rc) return rc;
     for (int l = 0; l < L; ++l) {
         if (c_attn) c_attn[l] = (float)((h[l] + x->run_attn[l]) / (double)rows);
         if (c_mlp) c_mlp[l] = (float)((h[L + l] + x->run_mlp[l]) / (double)rows);
@@ -1189,10 +1230,7 @@ extern "C" int asd_get_similarity(asd_ctx* x, float* c_attn, float* c_mlp, int32
 
 extern "C" int asd_set_skip_mask(asd_ctx* x, const uint8_t* skip_attn, const uint8_t* skip_mlp) {
     if (!x || !skip_attn || !skip_mlp) return ASD_ERR_ARG;
-    for (int l = 0; l < x->c.n_layers; ++l) {
-        x->skip_attn[l] = skip_attn[l] ? 1 : 0;
-        x->skip_mlp[l] = skip_mlp[l] ? 1 : 0;
-    }
+    set_masks(x, skip_attn, skip_mlp);
     x->draft_cursor = x->n_committed;
     x->drafted.clear();
     return build_stage_tables(x);
@@ -1461,8 +1499,8 @@ extern "C" int asd_get_last_cosines(asd_ctx* x, int32_t* M, float* cos_attn, flo
     const int L = x->c.n_layers, m = x->last_M;
     if (M) *M = m;
     std::vector<float> h((size_t)2 * std::max(L, 1) * kPassMaxRows);
-    ASD_CUDA(x, cudaMemcpyAsync(h.data(), x->ws + x->lay.cosv, h.size() * 4, cudaMemcpyDeviceToHost, x->stream));
-    ASD_CUDA(x, cudaStreamSynchronize(x->stream));
+    const int rc = copy_out(x, h.data(), x->ws + x->lay.cosv, h.size() * 4);
+    if (rc) return rc;
     for (int l = 0; l < L; ++l)
         for (int r = 0; r < m; ++r) {
             if (cos_attn) cos_attn[(size_t)l * m + r] = h[((size_t)0 * L + l) * kPassMaxRows + r];
@@ -1513,31 +1551,21 @@ extern "C" int asd_get_last_logits(asd_ctx* x, int32_t* M, float* logits) {
     if (!x) return ASD_ERR_ARG;
     if (x->last_M == 0 || !x->last_has_logits) return fail(x, ASD_ERR_STATE, "no logits recorded (asd_set_debug)");
     if (M) *M = x->last_M;
-    if (logits) {
-        ASD_CUDA(x, cudaMemcpyAsync(logits, x->ws + x->lay.logits, (size_t)x->last_M * x->c.vocab * 4, cudaMemcpyDeviceToHost, x->stream));
-        ASD_CUDA(x, cudaStreamSynchronize(x->stream));
-    }
-    return ASD_OK;
+    return logits ? copy_out(x, logits, x->ws + x->lay.logits, (size_t)x->last_M * x->c.vocab * 4) : ASD_OK;
 }
 
 extern "C" int asd_get_last_margins(asd_ctx* x, int32_t* M, float* margins) {
     if (!x) return ASD_ERR_ARG;
     if (x->last_M == 0 || !x->last_had_lm_head) return fail(x, ASD_ERR_STATE, "no pass with an LM head has run");
     if (M) *M = x->last_M;
-    if (margins) {
-        ASD_CUDA(x, cudaMemcpyAsync(margins, x->at<int>(x->lay.argmax) + 32, (size_t)x->last_M * 4, cudaMemcpyDeviceToHost, x->stream));
-        ASD_CUDA(x, cudaStreamSynchronize(x->stream));
-    }
-    return ASD_OK;
+    return margins ? copy_out(x, margins, x->at<int>(x->lay.argmax) + 32, (size_t)x->last_M * 4) : ASD_OK;
 }
 
 extern "C" int asd_get_kv(asd_ctx* x, int32_t layer, int32_t pos, uint16_t* k, uint16_t* v) {
     if (!x || layer < 0 || layer >= x->c.n_layers || pos < 0 || pos >= x->c.max_seq) return ASD_ERR_ARG;
     const size_t off = (size_t)layer * x->lay.kv_layer_stride + (size_t)pos * x->kv_dim * 2;
-    if (k) ASD_CUDA(x, cudaMemcpyAsync(k, x->ws + x->lay.kcache + off, (size_t)x->kv_dim * 2, cudaMemcpyDeviceToHost, x->stream));
-    if (v) ASD_CUDA(x, cudaMemcpyAsync(v, x->ws + x->lay.vcache + off, (size_t)x->kv_dim * 2, cudaMemcpyDeviceToHost, x->stream));
-    ASD_CUDA(x, cudaStreamSynchronize(x->stream));
-    return ASD_OK;
+    const size_t row = (size_t)x->kv_dim * 2;
+    return copy_out(x, k, x->ws + x->lay.kcache + off, row, v, x->ws + x->lay.vcache + off, row);
 }
 
 extern "C" int asd_get_positions(asd_ctx* x, int32_t* n_committed, int32_t* draft_cursor) {
