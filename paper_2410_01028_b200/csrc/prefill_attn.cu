@@ -86,7 +86,10 @@ __device__ __forceinline__ void probabilities32(const uint32_t (&s)[32], unsigne
 // and owns the tensor-memory allocation. Barriers: q_full, k_full / v_full[s] (bytes landed), k_empty / v_empty[s] (the
 // MMAs reading the stage have finished), s_full (S of tile j is complete, and with it every earlier MMA: O holds the
 // tiles before j and P may be overwritten; phase n_kt: O is complete), p_full (the 128 rows' P of tile j are in tensor
-// memory). The MMAs of one CTA run in issue order: P V of tile j, then S of tile j + 1 over the columns of P's lo terms.
+// memory), lo_read (the products with the lo terms of tile j have finished). S of tile j + 1 goes over the columns of those lo
+// terms. PTX orders a pair of tcgen05.mma by their issue only when they share accumulator and shape (memory consistency model
+// of tcgen05, "pipelined instructions"), which P V and S do not, so its issue waits for lo_read: the lo products come first
+// and the wait passes while the mid and hi products, 512 cycles, still run.
 template <int HD>
 __global__ void __launch_bounds__(kFaThreads, 2)
 flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -98,7 +101,7 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     unsigned char* v_smem = k_smem + kFaStages * Cfg::kKvBytes;
     uint64_t* q_full = reinterpret_cast<uint64_t*>(v_smem + kFaStages * Cfg::kKvBytes);
     uint64_t *k_full = q_full + 1, *k_empty = k_full + kFaStages, *v_full = k_empty + kFaStages, *v_empty = v_full + kFaStages;
-    uint64_t *s_full = v_empty + kFaStages, *p_full = s_full + 1, *drained = p_full + 1;
+    uint64_t *s_full = v_empty + kFaStages, *p_full = s_full + 1, *lo_read = p_full + 1, *drained = lo_read + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drained + 1);
     volatile int* err = err_words;
 
@@ -113,6 +116,7 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         for (int s = 0; s < kFaStages; ++s) mbar_init(&k_full[s], 1), mbar_init(&k_empty[s], 1), mbar_init(&v_full[s], 1), mbar_init(&v_empty[s], 1);
         mbar_init(s_full, 1);
         mbar_init(p_full, kFaRows);
+        mbar_init(lo_read, 1);
         mbar_init(drained, 1);
         mbar_fence_init();
     }
@@ -196,10 +200,15 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 #pragma unroll
                 for (int k = 0; k < kFaKeys / 16; ++k)  // 16 keys: 8 columns of P, 2048 bytes of V
                     tc_mma_bf16_ts(tmem, a + 8 * k, v_desc + (uint64_t)(128 * k), idesc_o, (j | t | k) != 0, on);
+                if (t == 0) tc_commit(lo_read, on);
             }
             tc_commit(&v_empty[s], on);
-            if (j + 1 < n_kt) scores(j + 1);
-            else tc_commit(s_full, on);  // O is complete
+            if (j + 1 < n_kt) {
+                ok = mbar_wait_warp(lo_read, (uint32_t)(j & 1), err, kErrAttnWait, 1, j, s, 9);
+                scores(j + 1);
+            } else {
+                tc_commit(s_full, on);  // O is complete
+            }
         }
         if (!ok) {  // abandoned: the MMAs already issued end before the tensor memory is freed
             tc_commit(drained, on);

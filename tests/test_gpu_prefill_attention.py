@@ -43,3 +43,26 @@ def test_prompt_attention_at_tile_edges(shape, std, parts):
         for g, o in zip(dec.get_kv(1, p), orc.kv(1, p)):
             g = synth.bf16_to_f32(g)
             assert np.all(np.abs(g - o) <= 2 ** -7 * np.abs(o) + 1e-2 * np.abs(o).max()), (p, np.abs(g - o).max(), np.abs(o).max())
+
+
+# nothing in the kernel may depend on when its products, copies and warps get their turn: many blocks per SM over many
+# key tiles, and every repetition gives the same bits
+@pytest.mark.parametrize("shape", [HD128, HD64], ids=["hd128", "hd64"])
+def test_repeated_prompts_give_the_same_bits(shape):
+    import paper_2410_01028_b200 as asd
+    n = 2500  # two chunks; up to 40 key tiles per block
+    dec = asd.Decoder(shape, max_seq=n, max_draft=1)
+    dec.load_weights_host(synth.make_model(shape, seed=7, std=0.15))
+    dec.set_prefill_mode(asd.PREFILL_GEMM)
+    dec.set_debug(True)
+    prompt = synth.make_prompt(shape.vocab, n, seed=11)
+
+    def outputs():
+        dec.reset()
+        dec.prefill(prompt)
+        kv = [a.copy() for p in range(0, n, 7) for a in dec.get_kv(1, p)]
+        return kv + [dec.get_last_logits().copy(), *(c.copy() for c in dec.get_similarity()[:2])]
+
+    first = outputs()
+    for _ in range(5):
+        assert all(np.array_equal(a, b) for a, b in zip(first, outputs()))
