@@ -107,8 +107,9 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 // in stage s), empty[s] (the MMAs reading stage s have finished: tcgen05.commit), acc_full[b] (all MMAs of the tile in
 // buffer b have finished), acc_empty[b] (the epilogue warps have read buffer b). Ragged edges: TMA fills out-of-range
 // rows and reduction elements with zeros; the epilogue skips rows >= M and columns >= N. Every wait is bounded; after
-// a failed wait the roles fall through to the common exit, where the producer lets its copies in flight land and
-// the tensor memory is freed.
+// a failed wait the roles fall through to the common exit. Nothing outlives the kernel there: the MMA warp waits for its
+// last MMA (drained), whatever the other roles do, and when a producer or the MMA warp has given up (abandoned, set in both
+// CTAs of a pair) the copies that are still in flight land before shared and tensor memory are given back.
 //
 // What bounds it: an SM takes in at most about 115 bytes per ns (60 per cycle) from L2. A 128 x 256 tile on one SM wants 48 KB
 // per 64 elements of the reduction, 0.35 us where the MMAs take 0.27; two SMs sharing a 256 x 256 tile (cta_group::2, CG =
@@ -174,7 +175,10 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     uint64_t* empty = full + Cfg::kMaxStages;
     uint64_t* acc_full = empty + Cfg::kMaxStages;   // [2]
     uint64_t* acc_empty = acc_full + 2;     // [2]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+    uint64_t* drained = acc_empty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drained + 1);
+    int* abandoned = reinterpret_cast<int*>(tmem_slot + 1);  // a producer or the MMA warp of this unit has given up
+    int* requested = abandoned + 1;                          // [CG], in the leader: k-blocks that each CTA has requested
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = CG == 2 ? (int)cluster_rank() : 0, unit = blockIdx.x / CG, n_units = gridDim.x / CG;
@@ -190,6 +194,8 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], 4 * CG);
         }
+        mbar_init(drained, 1);
+        *abandoned = 0;
         mbar_fence_init();
     }
     if (warp == 1) {
@@ -203,6 +209,10 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     const uint32_t tmem = *tmem_slot;
     pdl_launch_dependents();
     const uint32_t on = elect_one();
+    auto give_up = [&]() {  // one lane; the other CTA's word as well
+        *abandoned = 1;
+        if (CG == 2) st_cluster(cluster_addr(abandoned, rank ^ 1), 1);
+    };
     auto load_w = [&](int s, int kb, int n0) {  // announces the bytes of a stage and requests its weights
         mbar_expect_tx_on(&full[s], CG * stage_bytes, CG == 2 ? on & (uint32_t)(rank == 0) : on);  // the bytes of both CTAs
         unsigned char* b_dst = base + (size_t)s * stage_bytes + Cfg::kABytes;
@@ -236,14 +246,12 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 if (++s == kStages) s = 0, ++lap;
             }
         }
-        if (lane == 0 && rank == 0 && (!ok || *err != kErrNone)) {
-            // abandoned: let the copies still in flight (with CG = 2 those of both CTAs, which the cluster barrier below
-            // holds back) land before the shared memory is given back
-            for (int i = max(0, issued - kStages); i < issued; ++i) {
-                const long long t0 = clock64();
-                while (!mbar_try_wait(&full[i % kStages], (uint32_t)((i / kStages) & 1)) && clock64() - t0 < 20000000LL) {
-                }
-            }
+        if (lane == 0) {
+            if (!ok) give_up();
+            else if (CG == 2)  // the leader's last multicast arrivals at this CTA's barriers come before it leaves
+                for (int i = max(0, issued - kStages); i < issued; ++i) mbar_drain(&empty[i % kStages], (uint32_t)((i / kStages) & 1));
+            if (CG == 2) st_cluster(cluster_addr(requested + rank, 0), issued);
+            else *requested = issued;
         }
     } else if (warp == 1) {
         if (rank == 0) {
@@ -278,6 +286,10 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 if (CG == 2) tc_commit_pair(&acc_full[buf], on);  // arrives when every MMA issued above has finished
                 else tc_commit(&acc_full[buf], on);
             }
+            if (CG == 2) tc_commit_pair_here(drained, on);
+            else tc_commit(drained, on);
+            mbar_drain(drained, 0);
+            if (!ok && lane == 0) give_up();
         }
     } else {
         const int quarter = warp & 3;
@@ -309,6 +321,20 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     tc_fence_before();
     __syncthreads();
     if (CG == 2) cluster_sync_all();  // no CTA leaves while the other's copies, commits or arrivals may still reach it
+    if (*abandoned) {  // the same in both CTAs of a pair
+        if (threadIdx.x == 0 && rank == 0) {
+            const int mine = requested[0], other = requested[CG - 1], last = max(mine, other);
+            for (int i = max(0, last - kStages); i < last; ++i) {  // the last filling of each stage
+                uint64_t* bar = &full[i % kStages];
+                // the leader announces the bytes of both CTAs: make up for a k-block that only one of them has requested
+                if (i >= mine) mbar_expect_tx(bar, stage_bytes);
+                else if (i >= other) mbar_complete_tx(bar, stage_bytes);
+                mbar_drain(bar, (uint32_t)((i / kStages) & 1));
+            }
+        }
+        __syncthreads();
+        if (CG == 2) cluster_sync_all();
+    }
     if (warp == 1) {
         tc_fence_after();
         if (CG == 2) tmem_dealloc_pair(tmem, 512);

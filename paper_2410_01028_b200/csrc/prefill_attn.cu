@@ -157,17 +157,12 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 tma_load_2d_on(v_smem + s * Cfg::kKvBytes + p * Cfg::kKvPanel, &tm_v, kvh * HD + p * 64, nv * kFaKeys, &v_full[s], on);
             ++nv;
         }
-        if (lane == 0 && (!ok || *err != kErrNone)) {
-            // abandoned: let the copies still in flight land before the CTA gives its shared memory back
-            const long long t0 = clock64();
-            auto landed = [&](uint64_t* bar, int n) { return n <= 0 || mbar_try_wait(bar, (uint32_t)((n - 1) & 1)); };
-            bool all = false;
-            while (!all && clock64() - t0 < 20000000LL) {
-                all = landed(q_full, 1);
-                for (int s = 0; s < kFaStages; ++s)
-                    all = all && landed(&k_full[s], (nk + kFaStages - 1 - s) / kFaStages) && landed(&v_full[s], (nv + kFaStages - 1 - s) / kFaStages);
-            }
-        }
+        // the copies land before the CTA gives its shared memory back, also when a role of the CTA gives up
+        auto landed = [&](uint64_t* bar, int n) {
+            if (n > 0) mbar_drain(bar, (uint32_t)((n - 1) & 1));
+        };
+        landed(q_full, 1);
+        for (int s = 0; s < kFaStages; ++s) landed(&k_full[s], (nk + kFaStages - 1 - s) / kFaStages), landed(&v_full[s], (nv + kFaStages - 1 - s) / kFaStages);
     } else if (warp == 5) {
         constexpr uint32_t idesc_s = umma_idesc_bf16(kFaRows, kFaKeys);
         constexpr uint32_t idesc_o = umma_idesc_bf16(kFaRows, HD) | (1u << 16);  // V is [key][dimension]: N-major
@@ -210,12 +205,9 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 tc_commit(s_full, on);  // O is complete
             }
         }
-        if (!ok) {  // abandoned: the MMAs already issued end before the tensor memory is freed
-            tc_commit(drained, on);
-            const long long t0 = clock64();
-            while (!mbar_try_wait(drained, 0) && clock64() - t0 < 20000000LL) {
-            }
-        }
+        // the MMAs end before the tensor memory is freed, also when a role of the CTA gives up
+        tc_commit(drained, on);
+        mbar_drain(drained, 0);
     } else {
         const int row = r0 + threadIdx.x;
         const int pos = pos0 + min(row, n_rows - 1);  // rows past the prompt are computed like the last one and not stored

@@ -71,6 +71,14 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code, stage, item, slot, tag));
 }
 
+// Waits for copies or MMAs in flight before their shared or tensor memory is given back. They end by themselves whatever the
+// error word says, so it is not looked at; the bound (about 10 ms) only guards against a barrier that nothing signals.
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+    const long long t0 = clock64();
+    while (!mbar_try_wait(bar, parity) && clock64() - t0 < 20000000LL) {
+    }
+}
+
 // 1-D bulk copy global -> shared, completion counted on an mbarrier. Both addresses 16-byte aligned, size % 16 == 0.
 __device__ __forceinline__ void tma_load_1d(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(

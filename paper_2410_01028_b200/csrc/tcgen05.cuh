@@ -96,6 +96,14 @@ __device__ __forceinline__ void tc_commit_pair(uint64_t* bar, uint32_t on) {
         "h"((uint16_t)3), "r"(on)
         : "memory");
 }
+// the same, reported to a barrier of this CTA alone
+__device__ __forceinline__ void tc_commit_pair_here(uint64_t* bar, uint32_t on) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)), "r"(on)
+        : "memory");
+}
 // D (256 rows: 128 lanes of each CTA) (+)= A (256 x 16, 128 rows of each CTA) * B (N x 16, N / 2 rows of each CTA)^T
 __device__ __forceinline__ void tc_mma_bf16_pair(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate, uint32_t on) {
     asm volatile(
@@ -129,6 +137,14 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+// a word of the shared memory of either CTA (a shared::cluster address)
+__device__ __forceinline__ void st_cluster(uint32_t cluster_dst, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_dst), "r"(v) : "memory");
+}
+// counts bytes as landed that nobody will copy
+__device__ __forceinline__ void mbar_complete_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(cluster_addr(bar, cluster_rank())), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
