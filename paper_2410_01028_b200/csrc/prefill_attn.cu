@@ -12,9 +12,9 @@
 // CTA of the SM covers. Tiles of 64 keys because O (128 columns) and S / P (128 columns: the three terms take 96)
 // of two CTAs then fill the 512 columns of tensor memory.
 //
-// The running maximum is only moved when it has grown by more than 2^8 (probabilities up to 256 are as exact as those
-// up to 1): moving it means reading, scaling and writing O in tensor memory, which random scores need once or
-// twice per row instead of once per tile.
+// The running maximum of a row is only moved when it has grown by more than 2^8 (the conditional rescaling of FlashAttention-4;
+// probabilities up to 256 are as exact as those up to 1): moving it means reading, scaling and writing O in tensor memory,
+// which random scores need once or twice per row instead of once per tile. Whether a row moves depends on its own scores alone.
 //
 // Measured (8192-token prompt, 32 heads of 128, per layer): 3.4 ms with mma.sync and 64-row tiles, 1.22 ms here, the tensor
 // core active half of the time: a CTA's own chain S -> softmax -> P V -> S is longer than the other CTA's share covers.
@@ -210,7 +210,7 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         mbar_drain(drained, 0);
     } else {
         const int row = r0 + threadIdx.x;
-        const int pos = pos0 + min(row, n_rows - 1);  // rows past the prompt are computed like the last one and not stored
+        const int pos = pos0 + min(row, n_rows - 1);  // rows past the prompt (queries of an earlier one) are computed and not stored
         const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
         const unsigned long long c2 = pack2(scale_log2, scale_log2);
         float m = 0.f;
@@ -243,9 +243,12 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             const float tile_max = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
             if (j == 0) {
                 m = tile_max;  // finite: key 0 is visible to every row
-            } else if (__any_sync(0xffffffffu, (tile_max - m) * scale_log2 > 8.0f)) {
-                const float m_new = fmaxf(m, tile_max), alpha = ex2((m - m_new) * scale_log2);
-                m = m_new;
+            }
+            // each row decides by its own scores: the others in the warp, rows past the prompt among them, scale by exactly 1
+            const bool move = j > 0 && (tile_max - m) * scale_log2 > 8.0f;
+            if (__any_sync(0xffffffffu, move)) {
+                const float alpha = move ? ex2((m - tile_max) * scale_log2) : 1.0f;
+                m = move ? tile_max : m;
                 float a, b;
                 unpack2(sum2, a, b);
                 sum2 = pack2(a * alpha, b * alpha);
