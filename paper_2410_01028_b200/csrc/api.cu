@@ -1103,7 +1103,8 @@ static int prefill_dense(asd_ctx* x, const int32_t* dev_tokens, int n, int pos0)
             e.rope_cos = x->at<float>(ly.rope_cos), e.rope_sin = x->at<float>(ly.rope_sin);
             e.pos0 = p0, e.d_model = d, e.kv_dim = kvd, e.head_dim = c.head_dim;
             if ((rc = dense_gemm(x, x->tm_xn, l, 0, rows, d + 2 * kvd, d, e))) return rc;
-            ASD_CUDA(x, launch_flash_prefill(x->tm_q, x->tm_kv[(size_t)l * 2], x->tm_kv[(size_t)l * 2 + 1], pa, rows, p0, d, c.head_dim, c.n_heads, c.n_kv_heads, scale, err, s));
+            ASD_CUDA(x, launch_flash_prefill(x->tm_q, x->tm_kv[(size_t)l * 2], x->tm_kv[(size_t)l * 2 + 1], pa, pc, rows, p0, d,
+                                             c.head_dim, c.n_heads, c.n_kv_heads, scale, err, s));
             GemmEpi o{};
             o.err = err, o.w_static = 1;
             o.mode = kGemmF32;

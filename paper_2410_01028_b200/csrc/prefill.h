@@ -75,9 +75,10 @@ cudaError_t launch_sumcos(const float* cos_rows, int stride, int n_rows, int n_s
 
 // causal attention of prompt rows [0, n_rows) at positions pos0 + r over keys 0 .. pos0 + r of the cache. Tensor maps (bf16,
 // 128-byte swizzle): the queries [rows, d_model] in boxes of 64 columns x 128 rows, the caches [max_seq, kv_dim] in boxes of
-// 64 columns x 64 keys. head_dim 64 or 128.
-cudaError_t launch_flash_prefill(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, __nv_bfloat16* out, int n_rows, int pos0,
-                                 int d_model, int head_dim, int n_heads, int n_kv_heads, float scale, int* err, cudaStream_t s);
+// 64 columns x 64 keys. head_dim 64 or 128. totals: scratch of n_rows (rounded up to
+// whole tiles of 128) x d_model floats, 32-byte aligned.
+cudaError_t launch_flash_prefill(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, __nv_bfloat16* out, float* totals,
+                                 int n_rows, int pos0, int d_model, int head_dim, int n_heads, int n_kv_heads, float scale, int* err, cudaStream_t s);
 cudaError_t configure_prefill_attention();
 
 }  // namespace asd

@@ -16,6 +16,13 @@
 // probabilities up to 256 are as exact as those up to 1): moving it means reading, scaling and writing O in tensor memory,
 // which random scores need once or twice per row instead of once per tile. Whether a row moves depends on its own scores alone.
 //
+// An MMA cuts its sum with the accumulator off towards zero, so a chain of them loses about half an ulp of O at every step:
+// 12 steps per key tile, and twice the loss per step that mma.sync has. Before the key tiles 1, 2, 4, 8, ... O and the row
+// sums are therefore added to fp32 totals in scratch memory (rounded to nearest; L2 holds them) and start anew. No
+// chain is then longer than half of a row's keys, and what is lost in it counts by its share of the sum. Error
+// against 64 bits over the attention kernel on mma.sync, 64 to 8192 keys: 0.3-0.8 of it (without the totals 0.7-2.4); a bias of
+// values with a mean of one 1.8e-5 after 8192 keys instead of 6.0e-5 (mma.sync: 3.1e-5).
+//
 // Measured (8192-token prompt, 32 heads of 128, per layer): 3.4 ms with mma.sync and 64-row tiles, 1.22 ms here, the tensor
 // core active half of the time: a CTA's own chain S -> softmax -> P V -> S is longer than the other CTA's share covers.
 #include "common.cuh"
@@ -27,6 +34,10 @@ namespace asd {
 constexpr int kFaRows = 128, kFaKeys = 64, kFaThreads = 192, kFaStages = 2;
 constexpr int kFaTmemCols = 256;                       // O: 0-127; S: 128-191
 constexpr int kFaColS = 128, kFaColHi = 192, kFaColMid = 224, kFaColLo = 128;  // the lo terms take the place of S
+
+// tiles before which O and the row sums are folded into the totals: 1, 2, 4, 8, ... (absolute key tiles: the same for every row)
+constexpr int kFaFirstFold = 1;
+__device__ __forceinline__ bool fa_folds(int j) { return j >= kFaFirstFold && (j & (j - 1)) == 0; }
 
 template <int HD>
 struct FaCfg {
@@ -93,7 +104,7 @@ __device__ __forceinline__ void probabilities32(const uint32_t (&s)[32], unsigne
 template <int HD>
 __global__ void __launch_bounds__(kFaThreads, 2)
 flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                     __nv_bfloat16* __restrict__ out, int n_rows, int pos0, int d_model, int group, float scale_log2, int* err_words) {
+                     __nv_bfloat16* __restrict__ out, float* totals, int n_rows, int pos0, int d_model, int group, float scale_log2, int* err_words) {
     using Cfg = FaCfg<HD>;
     extern __shared__ unsigned char fa_smem_raw[];
     unsigned char* base = fa_smem_raw + ((1024u - (smem_u32(fa_smem_raw) & 1023u)) & 1023u);
@@ -194,7 +205,7 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 const uint32_t a = tmem + (t == 0 ? kFaColLo : (t == 1 ? kFaColMid : kFaColHi));
 #pragma unroll
                 for (int k = 0; k < kFaKeys / 16; ++k)  // 16 keys: 8 columns of P, 2048 bytes of V
-                    tc_mma_bf16_ts(tmem, a + 8 * k, v_desc + (uint64_t)(128 * k), idesc_o, (j | t | k) != 0, on);
+                    tc_mma_bf16_ts(tmem, a + 8 * k, v_desc + (uint64_t)(128 * k), idesc_o, (t | k) != 0 || !(j == 0 || fa_folds(j)), on);
                 if (t == 0) tc_commit(lo_read, on);
             }
             tc_commit(&v_empty[s], on);
@@ -214,6 +225,23 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
         const unsigned long long c2 = pack2(scale_log2, scale_log2);
         float m = 0.f;
+        // what has been folded: the columns in totals, the sum of probabilities here; both still want the factor since. The
+        // block's part of totals is [HD / 8][128 rows][8], so that the 32 bytes of neighbouring lanes are neighbours.
+        float* total = totals + (size_t)r0 * d_model + (size_t)head * (kFaRows * HD) + threadIdx.x * 8;
+        float sum_total = 0.f, since = 1.f;
+        auto fold = [&](int c, bool first, float (&v)[32]) {  // columns c .. c + 31: total * since + O
+            uint32_t o[32], w[32];
+            tmem_ld32_async(lane_base + c, o);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) w[i] = 0u;
+            if (!first) {
+#pragma unroll
+                for (int i = 0; i < 32; i += 8) ld_global_v8(total + (c + i) * kFaRows, w + i);
+            }
+            tmem_ld_wait(o);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = fmaf(__uint_as_float(w[i]), since, __uint_as_float(o[i]));
+        };
         unsigned long long sum2 = pack2(0.f, 0.f);
         bool ok = true;
         for (int j = 0; j < n_kt; ++j) {
@@ -221,6 +249,20 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             ok = __all_sync(0xffffffffu, ok);  // tensor-memory accesses are warp-wide
             if (!ok) break;
             tc_fence_after();
+            const bool fresh = fa_folds(j);
+            if (fresh) {  // (32 columns at a time: 64, or loads in front of the wait, spill registers of the tile loop)
+#pragma unroll
+                for (int c = 0; c < HD; c += 32) {
+                    float v[32];
+                    fold(c, j == kFaFirstFold, v);
+#pragma unroll
+                    for (int i = 0; i < 32; i += 8) st_global_v8(total + (c + i) * kFaRows, reinterpret_cast<const uint32_t*>(v) + i);
+                }
+                float a, b;
+                unpack2(sum2, a, b);
+                sum_total = fmaf(sum_total, since, a + b);
+                sum2 = pack2(0.f, 0.f), since = 1.f;
+            }
             uint32_t s0[32], s1[32];
             tmem_ld32_async(lane_base + kFaColS, s0);
             tmem_ld32_async(lane_base + kFaColS + 32, s1);
@@ -252,8 +294,9 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 float a, b;
                 unpack2(sum2, a, b);
                 sum2 = pack2(a * alpha, b * alpha);
+                since *= alpha;
 #pragma unroll 1
-                for (int c = 0; c < HD; c += 32) {
+                for (int c = fresh ? HD : 0; c < HD; c += 32) {
                     uint32_t o[32];
                     tmem_ld32_async(lane_base + c, o);
                     tmem_ld_wait(o);
@@ -277,12 +320,12 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             tc_fence_after();
             float a, b;
             unpack2(sum2, a, b);
-            const float inv = 1.0f / (a + b);
+            const float inv = 1.0f / fmaf(sum_total, since, a + b);
             __nv_bfloat16* dst = out + (size_t)row * d_model + (size_t)head * HD;
 #pragma unroll
             for (int c = 0; c < HD; c += 32) {
                 float v[32];
-                tmem_ld32(lane_base + c, v);
+                fold(c, n_kt <= kFaFirstFold, v);
                 if (row < n_rows) {
                     uint32_t w[16];
 #pragma unroll
@@ -301,16 +344,16 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     }
 }
 
-cudaError_t launch_flash_prefill(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, __nv_bfloat16* out, int n_rows, int pos0,
-                                 int d_model, int head_dim, int n_heads, int n_kv_heads, float scale, int* err, cudaStream_t s) {
+cudaError_t launch_flash_prefill(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, __nv_bfloat16* out, float* totals,
+                                 int n_rows, int pos0, int d_model, int head_dim, int n_heads, int n_kv_heads, float scale, int* err, cudaStream_t s) {
     if (n_rows <= 0) return cudaErrorInvalidValue;
     const dim3 grid(n_heads, (n_rows + kFaRows - 1) / kFaRows);
     const int group = n_heads / n_kv_heads;
     const float scale_log2 = scale * 1.4426950408889634f;
     if (head_dim == 128)
-        return launch_pdl(flash_prefill_kernel<128>, grid, dim3(kFaThreads), FaCfg<128>::kSmem, s, 1, tm_q, tm_k, tm_v, out, n_rows, pos0, d_model, group, scale_log2, err);
+        return launch_pdl(flash_prefill_kernel<128>, grid, dim3(kFaThreads), FaCfg<128>::kSmem, s, 1, tm_q, tm_k, tm_v, out, totals, n_rows, pos0, d_model, group, scale_log2, err);
     if (head_dim == 64)
-        return launch_pdl(flash_prefill_kernel<64>, grid, dim3(kFaThreads), FaCfg<64>::kSmem, s, 1, tm_q, tm_k, tm_v, out, n_rows, pos0, d_model, group, scale_log2, err);
+        return launch_pdl(flash_prefill_kernel<64>, grid, dim3(kFaThreads), FaCfg<64>::kSmem, s, 1, tm_q, tm_k, tm_v, out, totals, n_rows, pos0, d_model, group, scale_log2, err);
     return cudaErrorInvalidValue;
 }
 

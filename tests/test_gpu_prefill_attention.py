@@ -45,6 +45,54 @@ def test_prompt_attention_at_tile_edges(shape, std, parts):
             assert np.all(np.abs(g - o) <= 2 ** -7 * np.abs(o) + 1e-2 * np.abs(o).max()), (p, np.abs(g - o).max(), np.abs(o).max())
 
 
+# Long chains of products must not lose what they add up. Tokens share most of their embedding, so that the values of a head
+# have a mean and the rows' sums grow with every key; the attention output is as large as the hidden state it is added to.
+# A sum that has lost the share e of itself moves the mean cosine before and after by about e / 2. Rounded to nearest, the
+# sums of 8192 keys lose far below 1e-6. An MMA cuts every sum off by half an ulp on average: a chain over half of the keys
+# of a row (768 steps on the longest row, counted by half of the sum, at a mean size of half) loses up to 768 * 2^-24 / 4 = 1.1e-5
+# and the shorter ones before it as much again over all rows: a cosine off by at most 6e-6. Left to grow over
+# all keys, a chain loses up to 4.6e-5 (measured: 1e-5 in the mean cosine).
+@pytest.mark.parametrize("head_dim", [128, 64])
+def test_attention_over_many_keys_keeps_its_sums(head_dim):
+    import torch
+    import paper_2410_01028_b200 as asd
+    d, S, H = 256, 8192, 256 // head_dim
+    shape = synth.DecoderShape(n_layers=1, d_model=d, n_heads=H, head_dim=head_dim, d_ffn=64, vocab=499)
+    model = synth.make_model(shape, seed=3, std=0.0625, scale_lo=1.0)
+    base, noise = synth.make_array_f32((1, d), seed=5, stream=1), synth.make_array_f32((499, d), seed=5, stream=2)
+    model.embed = synth.f32_to_bf16(base + 0.5 * noise)
+    prompt = synth.make_prompt(shape.vocab, S, seed=11)
+    dec = asd.Decoder(shape, max_seq=S, max_draft=1)
+    dec.load_weights_host(model)
+    dec.prefill(prompt)
+    got = float(dec.get_similarity()[0][0])
+
+    def w(a):
+        return torch.from_numpy(synth.bf16_to_f32(a)).cuda().double()
+
+    def bf(t):
+        return t.float().to(torch.bfloat16).double()
+
+    x = w(model.embed)[torch.from_numpy(prompt).cuda().long()]
+    xn = bf(x * torch.rsqrt((x * x).mean(-1, keepdim=True) + dec.cfg.rms_eps) * w(model.attn_norm[0]))
+    ang = torch.arange(S, device="cuda").double()[:, None] * torch.exp(
+        -np.log(dec.cfg.rope_theta) * 2.0 * torch.arange(head_dim // 2, device="cuda").double() / head_dim)
+    cos, sin = torch.cos(ang).float().double()[:, None], torch.sin(ang).float().double()[:, None]
+
+    def rope(t):
+        a, b = t.view(S, H, head_dim).chunk(2, -1)
+        return bf(torch.cat([a * cos - b * sin, b * cos + a * sin], -1))
+
+    q, k, v = rope(xn @ w(model.wq[0]).T), rope(xn @ w(model.wk[0]).T), bf(xn @ w(model.wv[0]).T).view(S, H, head_dim)
+    o = torch.empty(S, H, head_dim, dtype=torch.float64, device="cuda")
+    later = torch.ones(S, S, dtype=torch.bool, device="cuda").triu_(1)
+    for h in range(H):
+        o[:, h] = torch.softmax((q[:, h] @ k[:, h].T / head_dim ** 0.5).masked_fill_(later, -np.inf), -1) @ v[:, h]
+    y = x + bf(o).view(S, d) @ w(model.wo[0]).T
+    ref = float(((x * y).sum(-1) / (x.norm(dim=-1) * y.norm(dim=-1))).mean())
+    assert abs(got - ref) <= 6e-6, (got, ref, got - ref)
+
+
 # A row's arithmetic depends on the keys it sees alone: not on later rows, and not on what an earlier prompt left in the
 # buffers behind the last row. A changed order of fp32 operations flips a bf16 rounding in about 3e-5 of the elements of the
 # attention output, of which the rows that share a warp with the changed ones have 40000 per prompt.
