@@ -1,0 +1,58 @@
+// How a dense product of the prompt path is cut into tiles and dealt to the SMs: plain C++, shared by the kernel's launcher
+// and the host code that picks tensor maps and buffers.
+#pragma once
+
+namespace asd {
+
+constexpr int kGemmBM = 128;  // rows of the activation tile of one CTA (the M of tcgen05.mma)
+constexpr int kGemmBK = 64;   // reduction elements per pipeline stage: 128 bytes, one swizzle span
+
+// How a product runs: tiles of 128 * cg rows x bn columns on units of cg SMs, the reduction dimension in `parts` parts.
+struct GemmPlan {
+    int bn, cg, m_tiles, tiles, parts;
+    int w_box() const { return bn / cg; }  // rows of a box of W's tensor map
+};
+// the heights that w_box() can have; a weight matrix has one tensor map for each
+constexpr int kWBoxRows[] = {32, 64, 96, 112, 128, 160, 256};
+constexpr int kWBoxes = sizeof(kWBoxRows) / sizeof(kWBoxRows[0]);
+
+// The plan of C[M, N] = A[M, K] * W[N, K]^T on `sms` SMs. With max_parts > 1 the reduction dimension may be cut into up to that
+// many parts, products of their own.
+//
+// The rule: the tile and the number of parts with the least time over their rounds: rounds x k-blocks of a part x the time
+// of a k-block (64 elements of the reduction), plus writing and reading the further parts (8 bytes per element at about 4
+// TB/s). The times of a k-block in the table are the slopes of one round of tiles; with every SM busy and several rounds all
+// of them grow by about a quarter. Over 48 products of 64 to 2048 rows and 3072 to 22016 columns, each timed with all
+// tiles, the rule's choice was within 0.2 % of the best on average and 5 % at worst. Pairs of SMs win where the tiles fill
+// the chip for rounds, 128 columns on single SMs where one round is enough (511 x 4096 x 11008: 45.5 us against 63.7 with
+// 256-column pair tiles), narrow tiles for short prompts (64 x 4096 x 11008: 33 us against 60). (A 192-column tile on
+// single SMs, 316 ns, was the choice for none of 80000 products.)
+inline GemmPlan plan_gemm(int M, int N, int K, int max_parts, int sms) {
+    const int num_kb = (K + kGemmBK - 1) / kGemmBK;
+    long long best_ns = -1;
+    GemmPlan best{};
+    auto consider = [&](int bn, int cg, int ns_kb) {
+        GemmPlan p{};
+        p.bn = bn, p.cg = cg;
+        p.m_tiles = (M + kGemmBM * cg - 1) / (kGemmBM * cg);
+        p.tiles = p.m_tiles * ((N + bn - 1) / bn);
+        const int units = sms / cg;
+        for (p.parts = 1; p.parts == 1 || (p.parts <= max_parts && num_kb / p.parts >= 8); ++p.parts) {
+            const long long rounds = ((long long)p.tiles * p.parts + units - 1) / units;
+            const long long ns = rounds * ((num_kb + p.parts - 1) / p.parts) * ns_kb + (long long)(p.parts - 1) * M * N / 500;
+            if (best_ns < 0 || ns < best_ns) best_ns = ns, best = p;
+        }
+    };
+    consider(256, 2, 315);
+    consider(224, 2, 281);
+    consider(192, 2, 247);
+    consider(256, 1, 354);
+    consider(160, 1, 244);
+    consider(128, 1, 209);
+    consider(96, 1, 195);
+    consider(64, 1, 145);
+    consider(32, 1, 138);
+    return best;
+}
+
+}  // namespace asd

@@ -123,7 +123,7 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 //
 // Units and tiles rarely divide evenly, so the host picks the kind of unit, the tile width and, for the products whose
 // consumer adds them up (fp32 output), the number of parts the reduction dimension is cut into by the time they take
-// over the rounds (launch_gemm_tn). Cutting the tiles of a last round with an exchange of the parts through L2 inside the
+// over the rounds (gemm_plan.h). Cutting the tiles of a last round with an exchange of the parts through L2 inside the
 // kernel (last arriver adds) was measured: 8-10 us per exchange, more than the part of a round it saves.
 constexpr int kGemmThreads = 192;
 static int g_gemm_ctas = 148;  // persistent CTAs per launch: the SM count of the device (set by configure_prefill)
@@ -349,42 +349,7 @@ static cudaError_t launch_gemm(const CUtensorMap& tm_a, const CUtensorMap& tm_w,
     return launch_pdl(gemm_tn_kernel<BN, CG>, grid, dim3(kGemmThreads), GemmCfg<BN, CG>::kSmem, s, CG, tm_a, tm_w, M, N, K, w, ep);
 }
 
-// The rule: the tile and the number of parts with the least time over their rounds: rounds x k-blocks of a part x the time
-// of a k-block (64 elements of the reduction), plus writing and reading the further parts (8 bytes per element at about 4
-// TB/s). The times of a k-block in the table are the slopes of one round of tiles; with every SM busy and several rounds all
-// of them grow by about a quarter. Over 48 products of 64 to 2048 rows and 3072 to 22016 columns, each timed with all ten
-// tiles, the rule's choice was within 0.2 % of the best on average and 5 % at worst. Pairs of SMs win where the tiles fill
-// the chip for rounds (2048 x 22016 x 4096: pairs 249-256 us, single SMs 302-334), 128 columns on single SMs where one round is
-// enough (511 x 4096 x 11008: 45.5 us against 63.7 with 256-column pair tiles), narrow tiles for short prompts (64 x 4096 x
-// 11008: 33 us against 60).
-GemmPlan plan_gemm(int M, int N, int K, int max_parts) {
-    const int num_kb = (K + kGemmBK - 1) / kGemmBK;
-    long long best_ns = -1;
-    GemmPlan best{};
-    auto consider = [&](int bn, int cg, int ns_kb) {
-        GemmPlan p{};
-        p.bn = bn, p.cg = cg;
-        p.m_tiles = (M + kGemmBM * cg - 1) / (kGemmBM * cg);
-        p.tiles = p.m_tiles * ((N + bn - 1) / bn);
-        const int units = g_gemm_ctas / cg;
-        for (p.parts = 1; p.parts == 1 || (p.parts <= max_parts && num_kb / p.parts >= 8); ++p.parts) {
-            const long long rounds = ((long long)p.tiles * p.parts + units - 1) / units;
-            const long long ns = rounds * ((num_kb + p.parts - 1) / p.parts) * ns_kb + (long long)(p.parts - 1) * M * N / 500;
-            if (best_ns < 0 || ns < best_ns) best_ns = ns, best = p;
-        }
-    };
-    consider(256, 2, 315);
-    consider(224, 2, 281);
-    consider(192, 2, 247);
-    consider(256, 1, 354);
-    consider(192, 1, 316);
-    consider(160, 1, 244);
-    consider(128, 1, 209);
-    consider(96, 1, 195);
-    consider(64, 1, 145);
-    consider(32, 1, 138);
-    return best;
-}
+GemmPlan plan_gemm(int M, int N, int K, int max_parts) { return plan_gemm(M, N, K, max_parts, g_gemm_ctas); }
 
 cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmPlan& p, const GemmEpi& ep, cudaStream_t s) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;

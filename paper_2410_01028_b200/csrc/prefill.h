@@ -13,10 +13,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-namespace asd {
+#include "gemm_plan.h"
 
-constexpr int kGemmBM = 128;  // rows of the activation tile of one CTA (the M of tcgen05.mma)
-constexpr int kGemmBK = 64;   // reduction elements per pipeline stage: 128 bytes, one swizzle span
+namespace asd {
 
 enum GemmEpilogue : int {
     kGemmF32 = 0,     // C[r, n] fp32
@@ -45,17 +44,7 @@ struct GemmEpi {
 
 cudaError_t configure_prefill(int max_smem);
 
-// How a product runs: tiles of 128 * cg rows x bn columns on units of cg SMs, the reduction dimension in `parts` parts.
-struct GemmPlan {
-    int bn, cg, m_tiles, tiles, parts;
-    int w_box() const { return bn / cg; }  // rows of a box of W's tensor map
-};
-// the heights that w_box() can have; a weight matrix has one tensor map for each
-constexpr int kWBoxRows[] = {32, 64, 96, 112, 128, 160, 192, 256};
-constexpr int kWBoxes = sizeof(kWBoxRows) / sizeof(kWBoxRows[0]);
-
-// The plan of C[M, N] = A[M, K] * W[N, K]^T. With max_parts > 1 (kGemmF32 only) the reduction dimension may be cut into up to that
-// many parts, products of their own c_part_stride apart.
+// the plan of C[M, N] = A[M, K] * W[N, K]^T on this device; max_parts > 1 for kGemmF32 only (parts c_part_stride apart)
 GemmPlan plan_gemm(int M, int N, int K, int max_parts);
 // bf16 operands described by 2-D tensor maps (128-byte swizzle, A in boxes of 64 elements x 128 rows, W in boxes of 64 x
 // w_box()), fp32 accumulation

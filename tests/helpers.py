@@ -1,5 +1,10 @@
 """Comparison helpers shared by the GPU parity tests (tolerances of the parity contract)."""
 import collections
+import ctypes
+import functools
+import os
+import subprocess
+import tempfile
 
 import numpy as np
 
@@ -11,6 +16,29 @@ LOGIT_TOL = 2e-2     # |l_gpu - l_orc| <= LOGIT_TOL * max|l_orc| per row
 COS_TOL = 1e-3       # absolute, per sublayer and row
 MARGIN = 1e-2        # token ids must agree wherever the oracle's top-2 logit gap exceeds this
 MASK_MARGIN = 1e-3   # skip masks must agree wherever |C_l - alpha| exceeds this
+
+
+GemmPlan = collections.namedtuple("GemmPlan", "bn cg m_tiles tiles parts")
+
+
+@functools.lru_cache(None)
+def _plan_lib():
+    csrc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2410_01028_b200", "csrc")
+    with tempfile.TemporaryDirectory() as tmp:
+        src, lib = os.path.join(tmp, "plan.cpp"), os.path.join(tmp, "plan.so")
+        with open(src, "w") as f:
+            f.write('#include "gemm_plan.h"\nextern "C" void plan(int m, int n, int k, int parts, int sms, int* o) {\n'
+                    "    const asd::GemmPlan p = asd::plan_gemm(m, n, k, parts, sms);\n"
+                    "    o[0] = p.bn, o[1] = p.cg, o[2] = p.m_tiles, o[3] = p.tiles, o[4] = p.parts;\n}\n")
+        subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", csrc, "-o", lib, src], check=True)
+        return ctypes.CDLL(lib)
+
+
+def gemm_plan(M, N, K, max_parts=1, sms=148):
+    """The library's own rule for the tiles and parts of a dense product, built from its header."""
+    out = (ctypes.c_int * 5)()
+    _plan_lib().plan(M, N, K, max_parts, sms, out)
+    return GemmPlan(*out)
 
 
 def assert_logits_close(gpu, orc):
