@@ -136,8 +136,8 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                 }
             };
             if (sub < n_sub) open(), settle();
-            // the weights do not depend on the activations: get the first ones moving before the prologue (as many as leave the
-            // RMSNorm of M rows its registers), the others before the wait at its end
+            // the weights do not depend on the activations: get the first ones moving before the prologue (one segment beside an
+            // RMSNorm of several rows, which needs registers as well), the others before the wait at its end
             constexpr int kEarly = !NORM || M == 1 ? kGemvDepth : 1;
 #pragma unroll
             for (int d = 0; d < kEarly; ++d) fetch(buf[d], at_sub[d], at_k[d]);
@@ -148,80 +148,92 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                 const int k0 = seg0 * kGemvSeg, k1 = min(n_in, win_end * kGemvSeg), k_pad = (win_end - seg0) * kGemvSeg;
                 if (NORM) {
                     const float* xf = reinterpret_cast<const float*>(p.x);
-                    constexpr int U = M == 1 ? 4 : (M == 2 ? 2 : 1);  // loads of a row in flight together
-                    const bool in_regs = n_in <= kGemvThreads * 4 * U && n_win == 1;  // the whole row: read it once
-                    float4 v[U][M];
+                    // Up to five rows: all of them at a time, several loads of a row in flight together for one and two, and rows that
+                    // fit the registers are read once. More rows go through the registers three at a time and are read again
+                    // from L1 and L2 for their normalisation: beside the weights of a segment there is no room for all of them (seven
+                    // and nine rows of 64 shapes 9 and 10 % faster, five rows 1 % slower that way).
+                    constexpr int U = M == 1 ? 4 : (M == 2 ? 2 : 1), R = M <= 5 ? M : 3;
+                    const bool in_regs = M <= 5 && n_in <= kGemvThreads * 4 * U && n_win == 1;
+                    float4 v[U][R];
 #pragma unroll
                     for (int u = 0; u < U; ++u)  // threads behind the end of the row store zeros
 #pragma unroll
-                        for (int m = 0; m < M; ++m) v[u][m] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int m = 0; m < R; ++m) v[u][m] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (win == 0 && blk == 0) {
-                        float ss[M];
 #pragma unroll
-                        for (int m = 0; m < M; ++m) ss[m] = 0.f;
-                        for (int i0 = tid * 4; i0 < n_in; i0 += kGemvThreads * 4 * U) {
+                        for (int m0 = 0; m0 < M; m0 += R) {
+                            float ss[R];
 #pragma unroll
-                            for (int u = 0; u < U; ++u)
+                            for (int m = 0; m < R; ++m) ss[m] = 0.f;
+                            for (int i0 = tid * 4; i0 < n_in; i0 += kGemvThreads * 4 * U) {
 #pragma unroll
-                                for (int m = 0; m < M; ++m) {
-                                    const int i = i0 + u * kGemvThreads * 4;
-                                    v[u][m] = make_float4(0.f, 0.f, 0.f, 0.f);
-                                    if (i < n_in) v[u][m] = *reinterpret_cast<const float4*>(xf + (size_t)m * n_in + i);
-                                }
+                                for (int u = 0; u < U; ++u)
 #pragma unroll
-                            for (int u = 0; u < U; ++u)
+                                    for (int m = 0; m < R; ++m) {
+                                        const int i = i0 + u * kGemvThreads * 4;
+                                        v[u][m] = make_float4(0.f, 0.f, 0.f, 0.f);
+                                        if (i < n_in && m0 + m < M) v[u][m] = *reinterpret_cast<const float4*>(xf + (size_t)(m0 + m) * n_in + i);
+                                    }
 #pragma unroll
-                                for (int m = 0; m < M; ++m) {
-                                    ss[m] = fmaf(v[u][m].x, v[u][m].x, ss[m]);
-                                    ss[m] = fmaf(v[u][m].y, v[u][m].y, ss[m]);
-                                    ss[m] = fmaf(v[u][m].z, v[u][m].z, ss[m]);
-                                    ss[m] = fmaf(v[u][m].w, v[u][m].w, ss[m]);
-                                }
-                        }
+                                for (int u = 0; u < U; ++u)
 #pragma unroll
-                        for (int m = 0; m < M; ++m) {
-                            ss[m] = warp_sum(ss[m]);
-                            if (lane == 0) red[warp * (kMaxRows * 4) + m] = ss[m];
+                                    for (int m = 0; m < R; ++m) {
+                                        ss[m] = fmaf(v[u][m].x, v[u][m].x, ss[m]);
+                                        ss[m] = fmaf(v[u][m].y, v[u][m].y, ss[m]);
+                                        ss[m] = fmaf(v[u][m].z, v[u][m].z, ss[m]);
+                                        ss[m] = fmaf(v[u][m].w, v[u][m].w, ss[m]);
+                                    }
+                            }
+#pragma unroll
+                            for (int m = 0; m < R; ++m) {
+                                if (m0 + m >= M) continue;
+                                ss[m] = warp_sum(ss[m]);
+                                if (lane == 0) red[warp * (kMaxRows * 4) + m0 + m] = ss[m];
+                            }
                         }
                         __syncthreads();
                     }
-                    float inv_m[M];
 #pragma unroll
-                    for (int m = 0; m < M; ++m) {
-                        float s = 0.f;
+                    for (int m0 = 0; m0 < M; m0 += R) {
+                        float inv_m[R];
 #pragma unroll
-                        for (int w = 0; w < kGemvWarps; ++w) s += red[w * (kMaxRows * 4) + m];
-                        inv_m[m] = 1.0f / sqrtf(s / (float)n_in + p.eps);
-                    }
-                    auto put = [&](int i, const float4* row_v) {  // inputs i .. i + 3 of all rows
-                        uint2 gv = make_uint2(0u, 0u);
-                        if (i < k1) gv = *reinterpret_cast<const uint2*>(p.gain + i);
-                        const float g0 = bf_lo(gv.x), g1 = bf_hi(gv.x), g2 = bf_lo(gv.y), g3 = bf_hi(gv.y);
+                        for (int m = 0; m < R; ++m) {
+                            float s = 0.f;
 #pragma unroll
-                        for (int m = 0; m < M; ++m) {
-                            const __nv_bfloat162 lo = __floats2bfloat162_rn(row_v[m].x * inv_m[m] * g0, row_v[m].y * inv_m[m] * g1);
-                            const __nv_bfloat162 hi = __floats2bfloat162_rn(row_v[m].z * inv_m[m] * g2, row_v[m].w * inv_m[m] * g3);
-                            uint2 o;
-                            o.x = *reinterpret_cast<const uint32_t*>(&lo);
-                            o.y = *reinterpret_cast<const uint32_t*>(&hi);
-                            *reinterpret_cast<uint2*>(xs + (size_t)m * ld + (i - k0)) = o;
+                            for (int w = 0; w < kGemvWarps; ++w) s += red[w * (kMaxRows * 4) + min(m0 + m, M - 1)];
+                            inv_m[m] = 1.0f / sqrtf(s / (float)n_in + p.eps);
                         }
-                    };
-                    if (in_regs) {
+                        auto put = [&](int i, const float4* row_v) {  // inputs i .. i + 3 of these rows
+                            uint2 gv = make_uint2(0u, 0u);
+                            if (i < k1) gv = *reinterpret_cast<const uint2*>(p.gain + i);
+                            const float g0 = bf_lo(gv.x), g1 = bf_hi(gv.x), g2 = bf_lo(gv.y), g3 = bf_hi(gv.y);
 #pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            const int i = tid * 4 + u * kGemvThreads * 4;
-                            if (i < k_pad) put(i, v[u]);
-                        }
-                    } else {
-                        for (int i = k0 + tid * 4; i < k0 + k_pad; i += kGemvThreads * 4) {
-                            float4 r[M];
-#pragma unroll
-                            for (int m = 0; m < M; ++m) {
-                                r[m] = make_float4(0.f, 0.f, 0.f, 0.f);
-                                if (i < k1) r[m] = *reinterpret_cast<const float4*>(xf + (size_t)m * n_in + i);
+                            for (int m = 0; m < R; ++m) {
+                                if (m0 + m >= M) continue;
+                                const __nv_bfloat162 lo = __floats2bfloat162_rn(row_v[m].x * inv_m[m] * g0, row_v[m].y * inv_m[m] * g1);
+                                const __nv_bfloat162 hi = __floats2bfloat162_rn(row_v[m].z * inv_m[m] * g2, row_v[m].w * inv_m[m] * g3);
+                                uint2 o;
+                                o.x = *reinterpret_cast<const uint32_t*>(&lo);
+                                o.y = *reinterpret_cast<const uint32_t*>(&hi);
+                                *reinterpret_cast<uint2*>(xs + (size_t)(m0 + m) * ld + (i - k0)) = o;
                             }
-                            put(i, r);
+                        };
+                        if (in_regs) {
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                const int i = tid * 4 + u * kGemvThreads * 4;
+                                if (i < k_pad) put(i, v[u]);
+                            }
+                        } else {
+                            for (int i = k0 + tid * 4; i < k0 + k_pad; i += kGemvThreads * 4) {
+                                float4 r[R];
+#pragma unroll
+                                for (int m = 0; m < R; ++m) {
+                                    r[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+                                    if (i < k1 && m0 + m < M) r[m] = *reinterpret_cast<const float4*>(xf + (size_t)(m0 + m) * n_in + i);
+                                }
+                                put(i, r);
+                            }
                         }
                     }
                 } else {

@@ -57,3 +57,16 @@ def test_plans_match_oracle_and_rows_do_not_depend_on_M(n_in, n_rows, epi, norm)
         assert np.array_equal(part, full[:M]), M
         if epi == 2:
             assert np.array_equal(part_cos, full_cos[:M]), M
+
+
+# the RMSNorm of more than five rows takes them three at a time: whole and partial groups of three, activations in one window
+# and in several
+@pytest.mark.parametrize("M", [3, 4, 6, 7])
+@pytest.mark.parametrize("n_in,n_rows", [(136, 295), (2056, 4737), (8200, 296)])
+def test_rows_of_partial_groups_equal_those_of_nine_rows(M, n_in, n_rows):
+    x = synth.make_array_f32((9, n_in), seed=n_in, stream=1)
+    W = synth.make_matrix_bf16((n_rows, n_in), seed=n_rows, stream=2, std=0.05)
+    gain = synth.make_matrix_bf16((n_in,), seed=3, stream=3, mean=1.0)
+    full, _ = _run(9, n_in, n_rows, 0, True, x, W, gain, None)  # compared with the oracle above
+    part, _ = _run(M, n_in, n_rows, 0, True, x, W, gain, None)
+    assert np.array_equal(part, full[:M])
