@@ -275,6 +275,9 @@ int asd_gemm_bf16(void* cuda_stream, int32_t M, int32_t N, int32_t K, const uint
  *                               cos[m] = cosine(out before, out after)  -- the summand of C_l, Section 3.2
  *   scratch  : >= asd_fused_gemv_scratch_bytes() bytes, 256-byte aligned; its first 256 bytes must be zero
  *              before the first use and are left zero by every call.
+ *   limit    : a shape counts as the work of c CTAs, c the least multiple of the SM count for which
+ *              2 * M * ceil(ceil(n_rows / 2) / c) * ceil(n_in / 1024) floats (and with a gain M * n_in bf16
+ *              values) fit a block's shared memory; shapes without such a c of at most 1024 are refused (ARG)
  * Errors: ARG, NOMEM (scratch too small), CUDA. Asynchronous on the stream.
  */
 #define ASD_EPI_PLAIN 0
@@ -292,9 +295,9 @@ int asd_fused_gemv(void* cuda_stream, int32_t M, int32_t n_in, int32_t n_rows, c
  * device. For them the cross-CTA scratch of asd_fused_gemv lives in a fixed array inside the library image
  * (about 42 KB of device memory per GPU that loads the library, held until the process exits), so the caller
  * passes only inputs and outputs. Arguments and results are exactly those of asd_fused_gemv.
- *   - Limit: the array covers launch plans of up to 296 CTAs. A shape whose plan needs more (very many rows
- *     with a long reduction dimension and many activation rows) is rejected with ASD_ERR_NOMEM and a message on
- *     stderr; use asd_fused_gemv with your own scratch for those.
+ *   - Limit: shapes that count as the work of up to 296 CTAs (see asd_fused_gemv). One that counts as more (very
+ *     many rows with a long reduction dimension and many activation rows) is rejected with ASD_ERR_NOMEM and a
+ *     message on stderr; use asd_fused_gemv with your own scratch for those.
  *   - The first call on each device looks up the array's device address (that device must be current) and
  *     configures the kernels; make that first call outside any stream capture. The address is kept per device
  *     ordinal for the life of the process: it does not survive a cudaDeviceReset, after which this entry point
@@ -302,7 +305,7 @@ int asd_fused_gemv(void* cuda_stream, int32_t M, int32_t n_in, int32_t n_rows, c
  *   - All calls on a device share the one array: two calls whose kernels can overlap on the GPU (different
  *     streams without ordering, or several host threads) race on it. Order them on one stream.
  *   - The call itself allocates nothing: no cudaMalloc, cudaFree or allocating library routine.
- * Errors: ARG, NOMEM (plan larger than the built-in array), CUDA. Asynchronous on the stream. */
+ * Errors: ARG, NOMEM (beyond the limit), CUDA. Asynchronous on the stream. */
 int asd_fused_gemv_static(void* cuda_stream, int32_t M, int32_t n_in, int32_t n_rows, const void* x,
                           const uint16_t* gain, float eps, const uint16_t* W, int32_t epilogue, void* out, float* cos);
 

@@ -92,10 +92,10 @@ static cudaError_t device_info(DeviceInfo** out) {
     return cudaSuccess;
 }
 
-// The shapes that the fused GEMV takes, and for how many CTAs' partial results a caller has to have room: one CTA per SM,
-// or as many as let the sums of a CTA's pairs of rows over segments of 1024 inputs (and with RMSNorm the whole
-// activations) stay in shared memory. The kernel needs no more than one CTA per SM for any of them; the limits are
-// the interface's (the built-in scratch array of the static variant refuses what is beyond it).
+// The shapes that the fused GEMV takes (the limits that asd.h states). A shape counts as the work of *ctas CTAs: one per SM, or
+// as many times that as let the sums of a CTA's pairs of rows over segments of 1024 inputs (and with RMSNorm the
+// whole activations) fit a block's shared memory. The kernel itself always runs one CTA per SM and would take more; what the
+// entry points refuse stays refused.
 static bool gemv_accepts(const DeviceInfo& dv, int M, int n_rows, int n_in, bool norm, int* ctas) {
     const size_t n_pairs = ((size_t)n_rows + 1) / 2, n_seg = ((size_t)n_in + 1023) / 1024;
     for (int g = dv.num_sms; g <= kMaxGemvGrid; g += dv.num_sms) {
@@ -1675,8 +1675,8 @@ extern "C" int asd_fused_gemv_static(void* cuda_stream, int32_t M, int32_t n_in,
     if (!gemv_accepts(*dv, M, n_rows, n_in, gain != nullptr, &ctas)) return ASD_ERR_ARG;
     if (ctas > kStaticMaxGrid) {
         fprintf(stderr,
-                "asd_fused_gemv_static: this shape needs a %d-CTA launch plan but the built-in scratch array holds "
-                "partials for at most %d CTAs; call asd_fused_gemv with caller-provided scratch instead\n",
+                "asd_fused_gemv_static: this shape counts as the work of %d CTAs and this entry point takes at most %d; "
+                "call asd_fused_gemv with caller-provided scratch instead\n",
                 ctas, kStaticMaxGrid);
         return ASD_ERR_NOMEM;
     }
