@@ -71,15 +71,17 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
 __device__ __forceinline__ void probabilities32(const uint32_t (&s)[32], unsigned long long c2, unsigned long long nmc2, unsigned long long& sum2,
                                                 uint32_t t_hi, uint32_t t_mid, uint32_t t_lo) {
     uint32_t p[32], w[16];
+    unsigned long long part = pack2(0.f, 0.f);  // a sum of its own, so that no chain of additions runs over all keys of a row
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         float a, b;
         unpack2(ffma2(pack2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), c2, nmc2), a, b);
         a = ex2(a), b = ex2(b);
-        sum2 = fadd2(sum2, pack2(a, b));
+        part = fadd2(part, pack2(a, b));
         p[2 * i] = __float_as_uint(a), p[2 * i + 1] = __float_as_uint(b);
         w[i] = upper_halves(p[2 * i], p[2 * i + 1]);
     }
+    sum2 = fadd2(sum2, part);
     tmem_st16(t_hi, w);
 #pragma unroll
     for (int i = 0; i < 32; ++i) p[i] = __float_as_uint(__uint_as_float(p[i]) - __uint_as_float(p[i] & 0xFFFF0000u));  // exact

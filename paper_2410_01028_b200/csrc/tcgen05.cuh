@@ -22,9 +22,8 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t n_cols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // The functions below that take `on` are called by a whole converged warp and issued by the one lane in which `on` is
-// set (elect_one). A branch around them for a single lane would keep descriptors and addresses out of the uniform
-// registers, from which these instructions take their operands: moving them there one by one takes 63 cycles per MMA
-// and 190 per pair of tile copies (measured), more than the tensor core needs for tiles of up to 256 columns.
+// set (elect_one). Behind a branch for a single lane an MMA took 63 cycles to issue and a pair of tile copies 190 (measured),
+// more than the tensor core needs for tiles of up to 256 columns.
 __device__ __forceinline__ uint32_t elect_one() {
     uint32_t on;
     asm volatile(
