@@ -111,12 +111,12 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 // last MMA (drained), whatever the other roles do, and when a producer or the MMA warp has given up (abandoned, set in both
 // CTAs of a pair) the copies that are still in flight land before shared and tensor memory are given back.
 //
-// What bounds it: an SM takes in at most about 115 bytes per ns (60 per cycle) from L2. A 128 x 256 tile on one SM wants 48 KB
-// per 64 elements of the reduction, 0.35 us where the MMAs take 0.27; two SMs sharing a 256 x 256 tile (cta_group::2, CG =
-// 2: each stages its 128 rows of A and half of the rows of W and keeps its 128 rows of the accumulator) want 32 KB each.
-// Products that fill the chip for rounds are bound by that and by the power limit, which takes the clock down (2048 x
-// 22016 x 4096: 337 us on single SMs at first, 299 us back to back on pairs, 90 % tensor activity); tiles of up to 64
-// columns by the issue of a k-block (0.14 us: wait, four MMAs, commit; 0.28 us when one lane of a divergent warp issued
+// What bounds it: on single SMs the operands' way from L2: a 128 x 256 tile wants 48 KB per 64 elements of the reduction and
+// takes 0.35 us for them (139 bytes per ns and SM) where its MMAs take 0.27. Two SMs sharing a 256 x 256 tile (cta_group::2,
+// CG = 2: each stages its 128 rows of A and half of the rows of W and keeps its 128 rows of the accumulator) want 32 KB each
+// and take 0.315 us. Pairs that fill the chip for rounds are bound by the tensor core (93 % of active cycles at 2048 rows)
+// and by the power limit, which takes the clock down (2048 x 22016 x 4096: 251 us alone on a cool chip, 294-302 us back to
+// back; on single SMs 337 us); tiles of up to 64 columns by the issue of a k-block (0.14 us: wait, four MMAs, commit; 0.28 us when one lane of a divergent warp issued
 // them). With CG = 2 the leader (rank 0) issues the MMAs; full[s] lives in the leader and counts both CTAs' bytes;
 // empty[s] and acc_full[b] are signalled in both CTAs by multicast commits; acc_empty[b] lives in the leader and counts
 // the epilogue warps of both.

@@ -6,10 +6,9 @@
 // at 8 mantissa bits each, which represents every fp32 probability exactly); with fewer terms the 2^-17 error of P
 // flips bf16 roundings of the attention output in about every second row.
 //
-// What bounds it: the tensor core. Per 64 keys an S tile takes 384 cycles (N = 64 with both operands in shared memory is
+// What bounds it: the chain S -> softmax -> P V -> S of a CTA, of which the SM's second CTA covers a part. Per 64 keys an S tile takes 384 cycles (N = 64 with both operands in shared memory is
 // bound by the operand reads: 48 KB at 128 B per cycle) and the three P V products take 256 each; the softmax between
-// the two takes about 700-800 cycles of the other units (64 ex2 per row are 512 cycles of the SFUs), which the second
-// CTA of the SM covers. Tiles of 64 keys because O (128 columns) and S / P (128 columns: the three terms take 96)
+// the two takes about 700-800 cycles of the other units (64 ex2 per row are 512 cycles of the SFUs). Tiles of 64 keys because O (128 columns) and S / P (128 columns: the three terms take 96)
 // of two CTAs then fill the 512 columns of tensor memory.
 //
 // The running maximum of a row is only moved when it has grown by more than 2^8 (the conditional rescaling of FlashAttention-4;
@@ -23,8 +22,9 @@
 // against 64 bits over the attention kernel on mma.sync, 64 to 8192 keys: 0.3-0.8 of it (without the totals 0.7-2.4); a bias of
 // values with a mean of one 1.8e-5 after 8192 keys instead of 6.0e-5 (mma.sync: 3.1e-5).
 //
-// Measured (8192-token prompt, 32 heads of 128, per layer): 3.4 ms with mma.sync and 64-row tiles, 1.22 ms here, the tensor
-// core active half of the time: a CTA's own chain S -> softmax -> P V -> S is longer than the other CTA's share covers.
+// Measured (8192-token prompt, 32 heads of 128, per layer, launch to end): 3.4 ms with mma.sync and 64-row tiles, 1.3 ms here,
+// about 0.15 of it for the totals (a fold is a round trip to L2 in the chain of its tile: 4-5 % of a prompt pass of 512 to
+// 8192 tokens). The tensor core is active in 39 % of the cycles over the first 2048 keys.
 #include "common.cuh"
 #include "prefill.h"
 #include "tcgen05.cuh"
