@@ -201,7 +201,7 @@ struct Layout {
     size_t embed, lm_head, final_norm, layers, layer_stride;
     size_t l_attn_norm, l_wqkv, l_wo, l_mlp_norm, l_wgu, l_wd;  // offsets inside one layer block
     size_t rope_cos, rope_sin, kcache, vcache, kv_layer_stride;
-    size_t x, q, a, t, xl, al, tl, ql, kl, vl, pl_acc, pl_ml, part_acc, part_ml, partials, counters, cosv, sumcos;
+    size_t x, q, a, t, xl, al, tl, ql, kl, vl, pl_acc, pl_ml, part_acc, part_ml, partials, cosv, sumcos;
     size_t tok_in, draft_toks, gen_toks, prompt_toks, argmax, accept, logits, probs_p, probs_q;
     size_t stage_tab, tmaps, sync_words, trace, resid_tab;
     int max_stages;
@@ -286,7 +286,6 @@ static Layout make_layout(const asd_config& c) {
     L.part_acc = take((size_t)c.n_heads * L.chunk_stride * kPassMaxRows * c.head_dim * 4);
     L.part_ml = take((size_t)c.n_heads * L.chunk_stride * kPassMaxRows * 2 * 4);
     L.partials = take((size_t)(2 * c.n_layers + 1) * kMaxGemvGrid * kPassMaxRows * 4 * 4);
-    L.counters = take((size_t)(c.n_kv_heads + 64) * 4);
     L.cosv = take((size_t)2 * std::max(c.n_layers, 1) * kPassMaxRows * 4);
     L.sumcos = take((size_t)2 * std::max(c.n_layers, 1) * 8);
     L.tok_in = take(64 * 4);
@@ -380,6 +379,7 @@ struct asd_ctx {
     bool tables_current = false;   // the stage tables on the device are those of skip_attn / skip_mlp
     bool skipped_cos_nan = false;  // the cosines of the sublayers in the mask are NaN: no pass of the full model since they were set
     uint32_t bar_base = 0;      // value of the grid-barrier counter at the start of the next pass
+    uint32_t merge_base = 0;    // the same of the barrier in front of the merges of attention stages
     uint32_t pass_tag = 0x1000; // tag of stage 0 of the next pass in the tagged handoff buffers (never 0: the workspace starts zeroed)
     int n_stages_full = 0, n_stages_draft = 0, n_resid_full = 0, n_resid_draft = 0;
     std::vector<cudaEvent_t> events;
@@ -645,7 +645,6 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     p.pass_tag = x->pass_tag;
     p.part_acc = x->at<float>(ly.part_acc);
     p.part_ml = x->at<float>(ly.part_ml);
-    p.attn_counters = x->at<unsigned>(ly.counters) + 64;
     p.chunk_stride = ly.chunk_stride;
     p.partials = x->at<float>(ly.partials);
     p.resid = x->at<ResidOut>(ly.resid_tab) + (size_t)(use_mask ? 1 : 0) * (2 * std::max(L, 1));
@@ -654,6 +653,8 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     p.grid_bar = words + 16;
     p.err = reinterpret_cast<int*>(words + 32);
     p.bar_base = x->bar_base;
+    p.merge_bar = words + 48;
+    p.merge_base = x->merge_base;
     p.wait_cycles = x->short_waits ? kShortWaitCycles : kWaitCycles;
     p.bar_extra_last = x->inject_missing_arrival ? 1u : 0u;
     const int table = head_only ? 2 : (use_mask ? 1 : 0);
@@ -679,6 +680,8 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     const int grid = x->dev->num_sms;
     ASD_CUDA(x, launch_pass(M, p, grid, pl.smem, s));
     x->bar_base += (uint32_t)p.n_stages * (uint32_t)grid;
+    if (!p.use_ll && !head_only)  // one arrival per CTA and attention stage
+        for (int l = 0; l < L; ++l) x->merge_base += (use_mask && x->skip_attn[l]) ? 0u : (uint32_t)grid;
     x->pass_tag += (uint32_t)ly.max_stages + 1u;
     if (x->pass_tag < 0x1000u) x->pass_tag = 0x1000u;  // wrapped around
     x->stats.kernel_launches += 1;

@@ -84,7 +84,6 @@ struct PassParams {
     uint32_t pass_tag;     // tag of stage 0 of this pass; stage s writes pass_tag + s
     int use_ll;            // 1: launch the kernel variant that hands activations over through the tagged buffers (host: one row, d_model <= 5760)
     float *part_acc, *part_ml;
-    unsigned* attn_counters;
     int chunk_stride;
     float* partials;        // [n_resid + 1][gridDim.x][kPassMaxRows][4] per-CTA partial sums (last block: LM head)
     const ResidOut* resid;  // [n_resid] outputs of the residual stages of this pass, in stage order
@@ -92,6 +91,8 @@ struct PassParams {
     unsigned* fin_counter;
     unsigned* grid_bar;
     unsigned bar_base;
+    unsigned* merge_bar;    // grid barrier in front of the merge of an attention stage (passes without tags), and its value before the pass
+    unsigned merge_base;
     unsigned bar_extra_last;  // test hook: arrivals the finish stage's barrier waits for beyond the grid size (0 in normal use)
     long long wait_cycles;    // cycle budget of every bounded wait of the pass
     int* err;
@@ -181,7 +182,7 @@ __device__ __forceinline__ void cta_pairs(int n_rows, int type, int& pair0, int&
 }
 
 // Attention work items (kv head, 128-key chunk), head-major; CTA b takes the contiguous range
-// [b*T/G, (b+1)*T/G): mostly chunks of one head, so queries, tickets and DRAM pages are reused.
+// [b*T/G, (b+1)*T/G): mostly chunks of one head, so queries and DRAM pages are reused.
 __device__ __forceinline__ int attn_local_items(const PassParams& p, int M, int& n_chunks, int& first) {
     n_chunks = (p.pos0 + M - 1) / kAttnChunk + 1;
     const unsigned total = (unsigned)(p.n_kv_heads * n_chunks);  // heads * chunks * CTAs stays far below 2^32
@@ -434,25 +435,25 @@ __device__ __forceinline__ void consumers_sync() { bar_sync(1, kPassConsumers); 
 
 // release = false: the arrival only counts (nobody will wait for this stage before a later, releasing arrival of the
 // same CTA, whose release is cumulative); the CTA does not wait for its stores to be acknowledged.
-__device__ __forceinline__ void grid_arrive(const PassParams& p, bool release = true) {
+__device__ __forceinline__ void grid_arrive(unsigned* counter, bool release = true) {
     consumers_sync();
     // one release at GPU scope: cumulative over the writes of the whole CTA, which the barrier above ordered before it
     if (threadIdx.x == 0) {
-        if (release) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.grid_bar), "r"(1u) : "memory");
-        else asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p.grid_bar), "r"(1u) : "memory");
+        if (release) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(1u) : "memory");
+        else asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(1u) : "memory");
     }
 }
-__device__ __forceinline__ void grid_wait(const PassParams& p, unsigned target) {
+__device__ __forceinline__ void grid_wait(const PassParams& p, const unsigned* counter, unsigned target) {
     if (threadIdx.x == 0) {
         volatile int* err = p.err;
         const long long t0 = clock64();
         // every poll is a round trip to L2; the error word and the clock are looked at only now and then
-        for (unsigned spin = 1; (int)(ld_acquire_gpu(p.grid_bar) - target) < 0; ++spin) {
+        for (unsigned spin = 1; (int)(ld_acquire_gpu(counter) - target) < 0; ++spin) {
             if ((spin & 63u) != 0) continue;
             if (*err != kErrNone) break;
             if (clock64() - t0 > p.wait_cycles) {
                 if (atomicCAS(p.err, kErrNone, kErrGridWait) == kErrNone) {
-                    p.err[1] = (int)((target - p.bar_base) / gridDim.x), p.err[2] = (int)ld_acquire_gpu(p.grid_bar);
+                    p.err[1] = counter == p.grid_bar ? (int)((target - p.bar_base) / gridDim.x) : -1, p.err[2] = (int)ld_acquire_gpu(counter);
                     p.err[3] = (int)target, p.err[4] = blockIdx.x;
                 }
                 break;
@@ -479,7 +480,7 @@ __device__ __forceinline__ bool last_cta_consumers(unsigned* counter, int* flag_
 // Every stage starts by waiting for the previous stage of all CTAs. Whatever does not depend on activations (the
 // stage descriptor, index arithmetic, zeroing of partial sums, RMSNorm gains) is done before this wait.
 __device__ __forceinline__ void stage_begin(const PassParams& p, int s, unsigned extra = 0u) {
-    if (s > 0) grid_wait(p, p.bar_base + (unsigned)s * gridDim.x + extra);
+    if (s > 0) grid_wait(p, p.grid_bar, p.bar_base + (unsigned)s * gridDim.x + extra);
     trace_mark(p, s, 1);
 }
 
@@ -1534,26 +1535,43 @@ struct TileAddr {
     }
 };
 
-template <int M, bool LL>
-__device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassSmem& sm, uint32_t& gi, int stage) {
+// Merging the chunks of a head: a chunk with maximum m_c moves the running maximum to max(m, m_c), scales what has been added so
+// far by exp(old - new maximum) and comes in with exp(m_c - new). These factors are the same for every output dimension: lane i
+// works out those of chunk i of 32 (the running maximum by a scan over the lanes) and hands them round.
+struct MergeFactors {
+    float s_old, s_new, sum;
+    // ml: (maximum, sum of weights) of this lane's chunk, -inf past the last one; mx: the running maximum, moved on
+    __device__ __forceinline__ MergeFactors(float2 ml, float& mx) : sum(ml.y) {
+        const int lane = threadIdx.x & 31;
+        float m = ml.x;
+#pragma unroll
+        for (int o = 1; o < 32; o *= 2) {
+            const float t = __shfl_up_sync(0xffffffffu, m, o);
+            if (lane >= o) m = fmaxf(m, t);
+        }
+        m = fmaxf(m, mx);
+        float before = __shfl_up_sync(0xffffffffu, m, 1);
+        if (lane == 0) before = mx;
+        s_old = expf(before - m), s_new = expf(ml.x - m);
+        mx = __shfl_sync(0xffffffffu, m, 31);
+    }
+    __device__ __forceinline__ void of(int i, float& so, float& sn, float& s) const {
+        so = __shfl_sync(0xffffffffu, s_old, i), sn = __shfl_sync(0xffffffffu, s_new, i), s = __shfl_sync(0xffffffffu, sum, i);
+    }
+};
+
+// HD: the head size when the code is compiled for it (loops and divisions by it are then fixed), 0: p.head_dim.
+template <int M, bool LL, int HD>
+__device__ void attn_items(const PassParams& p, const StageDesc& st, const PassSmem& sm, uint32_t gi0, int stage, int n_chunks, int first, int n_local) {
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int hd = p.head_dim;
+    const int hd = HD ? HD : p.head_dim;
     const int nhb = hd > 64 ? hd / 64 : 1;
     const int box_cols = hd > 64 ? 64 : hd;
     const int tile_slots = (kAttnChunk / kBoxKeys) * nhb;
-    int n_chunks, first;
-    const int n_local = attn_local_items(p, M, n_chunks, first);
-    const uint32_t gi0 = gi;
-    gi += (uint32_t)(n_local * 2 * tile_slots);
-    if (LL) trace_mark(p, stage, 1);  // tagged handoff: every item waits for exactly the words it needs
-    else stage_begin(p, stage);      // all consumer warps, also those without attention work
     const uint32_t tag_in = p.pass_tag + (uint32_t)(stage - 1), tag_out = p.pass_tag + (uint32_t)stage;  // W_qkv's stage precedes this one
     unsigned ll_spins = 0;
     long long ll_t0 = 0;
     const int grp = warp >> 2;
-    if (grp >= p.attn_groups) return;
-
-    
     const int gt = tid & 127, glane = gt & 31, gwarp = gt >> 5;
     const int bar_id = 2 + grp;
     const int group = p.n_heads / p.n_kv_heads;
@@ -1566,10 +1584,8 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
     float* qs = reinterpret_cast<float*>(base);   // [M][hd]
     float* Ps = qs + M * hd;                       // [M][128]
     float* red = Ps + M * kAttnChunk;              // [4][kPassMaxRows]
-    int* flag = reinterpret_cast<int*>(red + 4 * kPassMaxRows);
 
     int q_head = -1;   // head whose queries are in qs
-    unsigned run_cnt = 0;  // chunks of the current head finished by this group and not yet reported
     for (int j = grp; j < n_local; j += p.attn_groups) {
         const int idx = first + j;
         const int kvh = idx / n_chunks, chunk = idx - kvh * n_chunks;
@@ -1583,17 +1599,33 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
             ring_locate(p, g, slot, gen);
             return sm.ring + (size_t)slot * kSlotBytes;
         };
+        // the boxes of a tile: every warp waits for all of them, a lane each
+        auto wait_tile = [&](uint32_t g0, int tag) {
+            if (glane < tile_slots) ring_wait_full(p, sm, g0 + (uint32_t)glane, stage, tag);
+            __syncwarp();
+        };
+        auto release_tile = [&](uint32_t g0) {  // behind a barrier of the group
+            if (gt < tile_slots) {
+                fence_proxy_async_smem();
+                ring_release(p, sm, g0 + (uint32_t)gt);
+            }
+        };
 
         // ---- K tile: wait for the boxes, then overwrite the rows this pass has just written (the producer may
         //      have copied the tile before the QKV stage of this pass stored them)
-        constexpr int kQPerThread = (M * 256 + 127) / 128;  // head_dim <= 256
-        unsigned short qreg[kQPerThread];
+        constexpr int kQPer = LL ? 1 : (M * 64 + 127) / 128;  // four elements per load, head_dim <= 256
+        uint2 qreg[kQPer];
+        if (!LL) {
 #pragma unroll
-        for (int u = 0; u < kQPerThread; ++u) {  // the first head's queries are requested before waiting for the tile
-            const int i = gt + u * 128;
-            const int m = i / hd, e = i - m * hd;
-            qreg[u] = (!LL && i < M * hd && q_head != kvh * group) ? __ldcg(reinterpret_cast<const unsigned short*>(p.q) + (size_t)m * p.d_model + (size_t)(kvh * group) * hd + e) : 0;
+            for (int u = 0; u < kQPer; ++u) {  // the first head's queries are requested before waiting for the tile
+                const int i = (gt + u * 128) * 4;
+                const int m = i / hd, e = i - m * hd;
+                qreg[u] = make_uint2(0u, 0u);
+                if (i < M * hd && q_head != kvh * group)
+                    qreg[u] = __ldcg(reinterpret_cast<const uint2*>(p.q + (size_t)m * p.d_model + (size_t)(kvh * group) * hd + e));
+            }
         }
+        auto put_q = [&](int i, const uint2& v) { *reinterpret_cast<float4*>(qs + i) = make_float4(bf_lo(v.x), bf_hi(v.x), bf_lo(v.y), bf_hi(v.y)); };
         // tagged handoff (one row): first look at this thread's words of q and of the fresh k and v; stale ones are asked for again where they are used
         constexpr int kLLPer = LL ? 2 : 1;  // head_dim <= 256: at most two elements per thread
         unsigned long long qraw[kLLPer] = {}, kraw[kLLPer] = {}, vraw[kLLPer] = {};
@@ -1610,45 +1642,50 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
         }
         const int fresh0 = max(p.pos0, key0), fresh1 = min(last_pos, key0 + kAttnChunk - 1);
         const int n_fresh = fresh1 - fresh0 + 1;
-        // one or two rows: the fresh V rows are requested here too, so patching the V tile later costs no round trip
-        constexpr bool kVEarly = (M <= 2);
-        constexpr int kVPre = kVEarly ? (M * 32 + 127) / 128 : 1;  // head_dim <= 256: at most 32 vectors per row
-        uint4 vpre[kVPre];
-        if (kVEarly && !LL) {
+        // the fresh K and V rows are requested here too, so patching the tiles later costs no round trip
+        constexpr int kFreshPer = LL ? 1 : (M * 32 + 127) / 128;  // head_dim <= 256: at most 32 vectors per row
+        uint4 kpre[kFreshPer], vpre[kFreshPer];
+        if (!LL) {
 #pragma unroll
-            for (int u = 0; u < kVPre; ++u) {
+            for (int u = 0; u < kFreshPer; ++u) {
                 const int i = gt + u * 128;
-                vpre[u] = make_uint4(0u, 0u, 0u, 0u);
+                kpre[u] = vpre[u] = make_uint4(0u, 0u, 0u, 0u);
                 if (i < n_fresh * vec_per_row) {
                     const int fr = i / vec_per_row, c = i - fr * vec_per_row;
-                    vpre[u] = __ldcg(reinterpret_cast<const uint4*>(st.v_cache + (size_t)(fresh0 + fr) * p.kv_dim + (size_t)kvh * hd + c * 8));
+                    const size_t at = (size_t)(fresh0 + fr) * p.kv_dim + (size_t)kvh * hd + c * 8;
+                    kpre[u] = __ldcg(reinterpret_cast<const uint4*>(st.k_cache + at));
+                    vpre[u] = __ldcg(reinterpret_cast<const uint4*>(st.v_cache + at));
                 }
             }
         }
-        for (int t = 0; t < tile_slots; ++t) ring_wait_full(p, sm, gk + t, stage, M * 1000 + j);
-        if (LL) {
-            if (has_fresh) {  // this pass's key (element by element from the tagged words) over whatever the producer copied
+        auto patch = [&](uint32_t g0, const uint4 (&rows)[kFreshPer]) {  // over whatever the producer copied
 #pragma unroll
-                for (int u = 0; u < kLLPer; ++u) {
-                    const int e = gt + u * 128;
-                    if (e < hd) {
-                        while (!ll_ready(kraw[u], tag_in) && ll_keep_waiting(p, ll_spins, ll_t0, stage)) kraw[u] = ll_load1(p.kl + (size_t)kvh * hd + e);
-                        int sit, off;
-                        ta.locate(p.pos0 - key0, e >> 3, sit, off);
-                        *reinterpret_cast<unsigned short*>(slot_ptr(gk + sit) + off + (e & 7) * 2) = (unsigned short)kraw[u];
-                    }
+            for (int u = 0; u < kFreshPer; ++u) {
+                const int i = gt + u * 128;
+                if (i < n_fresh * vec_per_row) {
+                    const int fr = i / vec_per_row, c = i - fr * vec_per_row;
+                    int sit, off;
+                    ta.locate(fresh0 + fr - key0, c, sit, off);
+                    *reinterpret_cast<uint4*>(slot_ptr(g0 + sit) + off) = rows[u];
                 }
             }
-        } else if (n_fresh > 0) {
-            for (int i = gt; i < n_fresh * vec_per_row; i += 128) {
-                const int fr = i / vec_per_row, c = i - fr * vec_per_row;
-                const int r = fresh0 + fr - key0;
-                int sit, off;
-                ta.locate(r, c, sit, off);
-                *reinterpret_cast<uint4*>(slot_ptr(gk + sit) + off) =
-                    __ldcg(reinterpret_cast<const uint4*>(st.k_cache + (size_t)(fresh0 + fr) * p.kv_dim + (size_t)kvh * hd + c * 8));
+        };
+        // tagged handoff: this pass's key or value, element by element from the tagged words
+        auto patch_tagged = [&](uint32_t g0, const uint2* src, unsigned long long (&raw)[kLLPer]) {
+#pragma unroll
+            for (int u = 0; u < kLLPer; ++u) {
+                const int e = gt + u * 128;
+                if (e < hd) {
+                    while (!ll_ready(raw[u], tag_in) && ll_keep_waiting(p, ll_spins, ll_t0, stage)) raw[u] = ll_load1(src + (size_t)kvh * hd + e);
+                    int sit, off;
+                    ta.locate(p.pos0 - key0, e >> 3, sit, off);
+                    *reinterpret_cast<unsigned short*>(slot_ptr(g0 + sit) + off + (e & 7) * 2) = (unsigned short)raw[u];
+                }
             }
-        }
+        };
+        wait_tile(gk, M * 1000 + j);
+        if (!LL) patch(gk, kpre);
+        else if (has_fresh) patch_tagged(gk, p.kl, kraw);
         for (int g = 0; g < group; ++g) {
             const int head = kvh * group + g;
             bar_sync(bar_id, 128);  // patched tile visible; previous head's Ps / qs consumed
@@ -1664,60 +1701,68 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
                         }
                     }
                 }
-            } else if (g == 0) {
-                if (q_head != head) {
+            } else if (q_head != head) {
 #pragma unroll
-                    for (int u = 0; u < kQPerThread; ++u)
-                        if (gt + u * 128 < M * hd) qs[gt + u * 128] = __uint_as_float((uint32_t)qreg[u] << 16);
-                }
-            } else {
-                for (int i = gt; i < M * hd; i += 128) {
+                for (int u = 0; u < kQPer; ++u) {
+                    const int i = (gt + u * 128) * 4;
                     const int m = i / hd, e = i - m * hd;
-                    qs[i] = __uint_as_float((uint32_t)__ldcg(reinterpret_cast<const unsigned short*>(p.q) + (size_t)m * p.d_model + (size_t)head * hd + e) << 16);
+                    if (i < M * hd) put_q(i, g == 0 ? qreg[u] : __ldcg(reinterpret_cast<const uint2*>(p.q + (size_t)m * p.d_model + (size_t)head * hd + e)));
                 }
             }
             q_head = head;
             bar_sync(bar_id, 128);
 
-            if (j == 0 && g == 0) trace_mark(p, stage, 2);  // attention timeline: 2 = inputs staged, 4 = softmax done, 5 = P V done, 6 = ticket taken / value tile released, 7 = merged
-            // ---- scores: thread t owns key key0 + t. Four independent partial sums per row (16-byte chunk parity x half
-            //      of the chunk) keep the chains of dependent FMAs short; they are added in a fixed order.
+            if (j == 0 && g == 0) trace_mark(p, stage, 2);  // attention timeline: 2 = inputs staged, 4 = softmax done, 5 = P V done, 6 = value tile released, 7 = merged
+            // ---- scores: thread t owns key key0 + t in the end. A score is the sum of four partial sums (16-byte chunk parity x
+            //      half of the chunk), added in a fixed order. The four lanes of a quad take one of them each, for four keys
+            //      (keys 8 apart, so that the eight quads of a warp read rows of eight different swizzles), and exchange them
+            //      afterwards: a query element that comes from shared memory then serves four keys instead of one.
             float sc[M];
             {
-                float s4[M][4];
+                float sp[M][4];  // [row][key of the quad]
 #pragma unroll
-                for (int m = 0; m < M; ++m) s4[m][0] = s4[m][1] = s4[m][2] = s4[m][3] = 0.f;
-                const int rg = gt / kBoxKeys, rr = gt % kBoxKeys;
-                const int chunks_per_box = box_cols / 8;  // even: head_dim >= 16
-                for (int hb = 0; hb < nhb; ++hb) {
-                    const unsigned char* krow = slot_ptr(gk + rg * nhb + hb) + rr * ta.row_bytes;
-                    for (int cc0 = 0; cc0 < chunks_per_box; cc0 += 2) {
+                for (int m = 0; m < M; ++m) sp[m][0] = sp[m][1] = sp[m][2] = sp[m][3] = 0.f;
+                const int par = (glane >> 1) & 1, half = glane & 1, kq = glane >> 2;  // key of the quad: 32 gwarp + 8 i + kq
+                const int rg = (gwarp * 32) / kBoxKeys, rr = (gwarp * 32) % kBoxKeys + kq;  // (rr + 8 i) & 7 == kq
+                auto chunk_pair = [&](const unsigned char* krow, const float* qrow, int cc0) {
+                    const int cc = cc0 + par;
+                    const unsigned char* kp = krow + ((ta.swz ? (cc ^ kq) : cc) << 4);
+                    uint2 kv[4];
 #pragma unroll
-                        for (int par = 0; par < 2; ++par) {
-                            const int cc = cc0 + par, c = hb * 8 + cc;
-                            const uint4 kv = *reinterpret_cast<const uint4*>(krow + ((ta.swz ? (cc ^ (rr & 7)) : cc) << 4));
-                            const float kf[8] = {bf_lo(kv.x), bf_hi(kv.x), bf_lo(kv.y), bf_hi(kv.y),
-                                                 bf_lo(kv.z), bf_hi(kv.z), bf_lo(kv.w), bf_hi(kv.w)};
+                    for (int i = 0; i < 4; ++i) kv[i] = *reinterpret_cast<const uint2*>(kp + i * 8 * ta.row_bytes);
 #pragma unroll
-                            for (int m = 0; m < M; ++m) {
-                                const float4 q0 = *reinterpret_cast<const float4*>(qs + m * hd + c * 8);
-                                const float4 q1 = *reinterpret_cast<const float4*>(qs + m * hd + c * 8 + 4);
-                                float a0 = s4[m][2 * par], a1 = s4[m][2 * par + 1];
-                                a0 = fmaf(q0.x, kf[0], a0);
-                                a1 = fmaf(q1.x, kf[4], a1);
-                                a0 = fmaf(q0.y, kf[1], a0);
-                                a1 = fmaf(q1.y, kf[5], a1);
-                                a0 = fmaf(q0.z, kf[2], a0);
-                                a1 = fmaf(q1.z, kf[6], a1);
-                                a0 = fmaf(q0.w, kf[3], a0);
-                                a1 = fmaf(q1.w, kf[7], a1);
-                                s4[m][2 * par] = a0, s4[m][2 * par + 1] = a1;
-                            }
+                    for (int m = 0; m < M; ++m) {
+                        const float4 qv = *reinterpret_cast<const float4*>(qrow + m * hd + cc0 * 8);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            float a = sp[m][i];
+                            a = fmaf(qv.x, bf_lo(kv[i].x), a);
+                            a = fmaf(qv.y, bf_hi(kv[i].x), a);
+                            a = fmaf(qv.z, bf_lo(kv[i].y), a);
+                            a = fmaf(qv.w, bf_hi(kv[i].y), a);
+                            sp[m][i] = a;
                         }
                     }
-                }
+                };
+#pragma unroll 1
+                for (int hb = 0; hb < nhb; ++hb) {
+                    const unsigned char* krow = slot_ptr(gk + rg * nhb + hb) + rr * ta.row_bytes + half * 8;
+                    const float* qrow = qs + (hb * 8 + par) * 8 + half * 4;
+                    if (HD >= 64) {
 #pragma unroll
-                for (int m = 0; m < M; ++m) sc[m] = (s4[m][0] + s4[m][1]) + (s4[m][2] + s4[m][3]);
+                        for (int cc0 = 0; cc0 < 8; cc0 += 2) chunk_pair(krow, qrow, cc0);
+                    } else {
+                        for (int cc0 = 0; cc0 < box_cols / 8; cc0 += 2) chunk_pair(krow, qrow, cc0);  // an even number: head_dim >= 16
+                    }
+                }
+                const int home = ((glane & 7) << 2) | (glane >> 3);  // the lane that ends up with this lane's key
+#pragma unroll
+                for (int m = 0; m < M; ++m) {
+                    const float b0 = __shfl_xor_sync(0xffffffffu, half ? sp[m][0] : sp[m][1], 1), b1 = __shfl_xor_sync(0xffffffffu, half ? sp[m][2] : sp[m][3], 1);
+                    const float t0 = (half ? sp[m][1] : sp[m][0]) + b0, t1 = (half ? sp[m][3] : sp[m][2]) + b1;  // keys half, half + 2
+                    const float c = __shfl_xor_sync(0xffffffffu, par ? t0 : t1, 2);
+                    sc[m] = __shfl_sync(0xffffffffu, (par ? t1 : t0) + c, home);
+                }
             }
             // ---- chunk-local softmax statistics; the row at position pos0+m sees keys <= pos0+m
             const int key = key0 + gt;
@@ -1730,12 +1775,7 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
                 if (glane == 0) red[gwarp * kPassMaxRows + m] = v;
             }
             bar_sync(bar_id, 128);
-            if (g == group - 1) {  // K tile no longer needed: hand its slots back to the producer
-                if (gt == 0) {
-                    fence_proxy_async_smem();
-                    for (int t = 0; t < tile_slots; ++t) ring_release(p, sm, gk + t);
-                }
-            }
+            if (g == group - 1) release_tile(gk);  // K tile no longer needed: hand its slots back to the producer
 #pragma unroll
             for (int m = 0; m < M; ++m)
                 cmax[m] = fmaxf(fmaxf(red[0 * kPassMaxRows + m], red[1 * kPassMaxRows + m]),
@@ -1749,41 +1789,9 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
                 if (glane == 0) red[gwarp * kPassMaxRows + m] = v;
             }
             if (g == 0) {  // V tile: wait and patch once per item
-                for (int t = 0; t < tile_slots; ++t) ring_wait_full(p, sm, gv + t, stage, M * 1000 + 500 + j);
-                if (LL) {
-                    if (has_fresh) {
-#pragma unroll
-                        for (int u = 0; u < kLLPer; ++u) {
-                            const int e = gt + u * 128;
-                            if (e < hd) {
-                                while (!ll_ready(vraw[u], tag_in) && ll_keep_waiting(p, ll_spins, ll_t0, stage)) vraw[u] = ll_load1(p.vl + (size_t)kvh * hd + e);
-                                int sit, off;
-                                ta.locate(p.pos0 - key0, e >> 3, sit, off);
-                                *reinterpret_cast<unsigned short*>(slot_ptr(gv + sit) + off + (e & 7) * 2) = (unsigned short)vraw[u];
-                            }
-                        }
-                    }
-                } else if (kVEarly) {
-#pragma unroll
-                    for (int u = 0; u < kVPre; ++u) {
-                        const int i = gt + u * 128;
-                        if (i < n_fresh * vec_per_row) {
-                            const int fr = i / vec_per_row, c = i - fr * vec_per_row;
-                            int sit, off;
-                            ta.locate(fresh0 + fr - key0, c, sit, off);
-                            *reinterpret_cast<uint4*>(slot_ptr(gv + sit) + off) = vpre[u];
-                        }
-                    }
-                } else if (n_fresh > 0) {
-                    for (int i = gt; i < n_fresh * vec_per_row; i += 128) {
-                        const int fr = i / vec_per_row, c = i - fr * vec_per_row;
-                        const int r = fresh0 + fr - key0;
-                        int sit, off;
-                        ta.locate(r, c, sit, off);
-                        *reinterpret_cast<uint4*>(slot_ptr(gv + sit) + off) =
-                            __ldcg(reinterpret_cast<const uint4*>(st.v_cache + (size_t)(fresh0 + fr) * p.kv_dim + (size_t)kvh * hd + c * 8));
-                    }
-                }
+                wait_tile(gv, M * 1000 + 500 + j);
+                if (!LL) patch(gv, vpre);
+                else if (has_fresh) patch_tagged(gv, p.vl, vraw);
             }
             bar_sync(bar_id, 128);
             if (gt < M) {
@@ -1800,14 +1808,14 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
             }
             if (j == 0 && g == 0) trace_mark(p, stage, 4);
             // ---- P V: thread (c, kg) owns the 8 output dimensions of 16-byte chunk c for the keys kg, kg + 8, ... (one
-            //      16-byte read per key); the eight key groups of a chunk sit in neighbouring lanes and are added by an
-            //      xor butterfly. Up to six rows share one sweep over the keys (more rows: two or more sweeps).
+            //      16-byte read per key); the eight key groups of a chunk sit in neighbouring lanes and are added in pairs
+            //      (lanes 1, 2, 4 apart). Up to six rows share one sweep over the keys (more rows: two or more sweeps).
             //      Probabilities past n_valid are zero and the tile rows behind them hold finite cache contents.
             {
                 constexpr int kRowBatch = M <= 6 ? M : (M <= 12 ? (M + 1) / 2 : 4);
                 const int kg = gt & 7;
                 const int n_steps = (n_valid + 7) >> 3;  // keys kg + 8 i, i < n_steps
-                for (int c0 = 0; c0 < (hd >> 3); c0 += 16) {  // every lane runs the loop (the butterfly below is warp-wide)
+                for (int c0 = 0; c0 < (hd >> 3); c0 += 16) {  // every lane runs the loop (the sums below are warp-wide)
                     const bool active = c0 + (gt >> 3) < (hd >> 3);
                     const int c = active ? c0 + (gt >> 3) : 0;
                     const int hb = (nhb > 1) ? (c >> 3) : 0, cc = (nhb > 1) ? (c & 7) : c;
@@ -1819,40 +1827,50 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
                         for (int u = 0; u < kRowBatch; ++u)
 #pragma unroll
                             for (int d8 = 0; d8 < 8; ++d8) acc[u][d8] = 0.f;
-                        for (int i = 0; i < n_steps; ++i) {
-                            const int key = kg + 8 * i;
-                            const unsigned char* vrow = slot_ptr(gv + (key / kBoxKeys) * nhb + hb) + (key % kBoxKeys) * ta.row_bytes + coff;
-                            const uint4 vv = *reinterpret_cast<const uint4*>(vrow);
-                            const float vf[8] = {bf_lo(vv.x), bf_hi(vv.x), bf_lo(vv.y), bf_hi(vv.y), bf_lo(vv.z), bf_hi(vv.z), bf_lo(vv.w), bf_hi(vv.w)};
+#pragma unroll 1
+                        for (int b = 0; b < kAttnChunk / kBoxKeys; ++b) {  // the two boxes of 64 keys
+                            const unsigned char* vb = slot_ptr(gv + b * nhb + hb) + kg * ta.row_bytes + coff;
+                            const float* pb = Ps + m0 * kAttnChunk + b * kBoxKeys + kg;
+                            auto step = [&](int i) {
+                                const uint4 vv = *reinterpret_cast<const uint4*>(vb + i * 8 * ta.row_bytes);
+                                const float vf[8] = {bf_lo(vv.x), bf_hi(vv.x), bf_lo(vv.y), bf_hi(vv.y), bf_lo(vv.z), bf_hi(vv.z), bf_lo(vv.w), bf_hi(vv.w)};
 #pragma unroll
-                            for (int u = 0; u < kRowBatch; ++u)
-                                if (m0 + u < M) {
-                                    const float pw = Ps[(m0 + u) * kAttnChunk + key];
+                                for (int u = 0; u < kRowBatch; ++u)
+                                    if (m0 + u < M) {
+                                        const float pw = pb[u * kAttnChunk + i * 8];
 #pragma unroll
-                                    for (int d8 = 0; d8 < 8; ++d8) acc[u][d8] = fmaf(pw, vf[d8], acc[u][d8]);
-                                }
+                                        for (int d8 = 0; d8 < 8; ++d8) acc[u][d8] = fmaf(pw, vf[d8], acc[u][d8]);
+                                    }
+                            };
+                            const int n = n_steps - b * (kBoxKeys / 8);
+                            if (n >= kBoxKeys / 8) {
+#pragma unroll (M <= 4 ? 4 : 2)
+                                for (int i = 0; i < kBoxKeys / 8; ++i) step(i);
+                            } else {
+#pragma unroll 1
+                                for (int i = 0; i < n; ++i) step(i);
+                            }
                         }
 #pragma unroll
                         for (int u = 0; u < kRowBatch; ++u)
                             if (m0 + u < M) {
+                                // sums over the eight lanes, every lane left with the dimension of its number
+                                float r4[4], r2[2];
 #pragma unroll
-                                for (int d8 = 0; d8 < 8; ++d8) {
-                                    float v = acc[u][d8];
-                                    v += __shfl_xor_sync(0xffffffffu, v, 1);
-                                    v += __shfl_xor_sync(0xffffffffu, v, 2);
-                                    v += __shfl_xor_sync(0xffffffffu, v, 4);
-                                    acc[u][d8] = v;
+                                for (int i = 0; i < 4; ++i) {
+                                    const float b = __shfl_xor_sync(0xffffffffu, (kg & 1) ? acc[u][2 * i] : acc[u][2 * i + 1], 1);
+                                    r4[i] = ((kg & 1) ? acc[u][2 * i + 1] : acc[u][2 * i]) + b;
                                 }
-                                if (kg == 0 && active) {
-                                    if (LL) {
-                                        uint2* dst = p.pl_acc + ((size_t)head * p.chunk_stride + chunk) * hd + c * 8;
 #pragma unroll
-                                        for (int d8 = 0; d8 < 8; ++d8) ll_store(dst + d8, __float_as_uint(acc[u][d8]), tag_out);
-                                    } else {
-                                        float* dst = p.part_acc + (((size_t)head * p.chunk_stride + chunk) * kPassMaxRows + m0 + u) * hd + c * 8;
-                                        reinterpret_cast<float4*>(dst)[0] = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-                                        reinterpret_cast<float4*>(dst)[1] = make_float4(acc[u][4], acc[u][5], acc[u][6], acc[u][7]);
-                                    }
+                                for (int i = 0; i < 2; ++i) {
+                                    const float b = __shfl_xor_sync(0xffffffffu, (kg & 2) ? r4[2 * i] : r4[2 * i + 1], 2);
+                                    r2[i] = ((kg & 2) ? r4[2 * i + 1] : r4[2 * i]) + b;
+                                }
+                                const float b = __shfl_xor_sync(0xffffffffu, (kg & 4) ? r2[0] : r2[1], 4);
+                                const float sum = ((kg & 4) ? r2[1] : r2[0]) + b;
+                                if (active) {
+                                    if (LL) ll_store(p.pl_acc + ((size_t)head * p.chunk_stride + chunk) * hd + c * 8 + kg, __float_as_uint(sum), tag_out);
+                                    else p.part_acc[(((size_t)head * p.chunk_stride + chunk) * kPassMaxRows + m0 + u) * hd + c * 8 + kg] = sum;
                                 }
                             }
                     }
@@ -1860,151 +1878,152 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
             }
         }
         if (j == 0) trace_mark(p, stage, 5);
-        // ---- release the V tile. Finished chunks are reported once per run of chunks of the same head; the group
-        //      whose report completes the head merges its chunks in order.
-        ++run_cnt;
-        const int jn = j + p.attn_groups;
-        const bool report = (jn >= n_local) || ((first + jn) / n_chunks != kvh);
         bar_sync(bar_id, 128);
-        if (LL) {
-            // Tagged handoff: no ticket (the heads are merged in a second sweep below)
-            if (gt == 0) {
-                fence_proxy_async_smem();
-                for (int t = 0; t < tile_slots; ++t) ring_release(p, sm, gv + t);
-            }
-            if (j == 0) trace_mark(p, stage, 6);
-            continue;
-        }
-        if (gt == 0) {
-            fence_proxy_async_smem();
-            for (int t = 0; t < tile_slots; ++t) ring_release(p, sm, gv + t);
-            if (report) {
-                // release: the group's partial results (ordered before this thread by the barrier above) are visible
-                // to whoever reads the count; acquire: so are those of the groups that reported earlier
-                unsigned tk;
-                asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(tk) : "l"(p.attn_counters + kvh), "r"(run_cnt) : "memory");
-                *flag = (tk + run_cnt == (unsigned)n_chunks) ? 1 : 0;
-            } else {
-                *flag = 0;
-            }
-        }
-        if (report) run_cnt = 0;
-        bar_sync(bar_id, 128);
+        release_tile(gv);
         if (j == 0) trace_mark(p, stage, 6);
-        if (*flag) {
-            if (gt == 0) p.attn_counters[kvh] = 0u;
-            // warp w of the group merges rows w, w+4, ...; a lane owns four neighbouring output dimensions. The chunks
-            // are merged in ascending order, eight loads of a batch in flight together; explicit roundings keep the
-            // arithmetic identical in every instantiation of the kernel.
-            for (int g = 0; g < group; ++g) {
-                const int head = kvh * group + g;
-                for (int e4 = glane * 4; e4 < hd; e4 += 128) {
-                    for (int m = gwarp; m < M; m += 4) {
-                        const int nc = (p.pos0 + m) / kAttnChunk + 1;
-                        float mx = -INFINITY, l = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
-                        for (int c0 = 0; c0 < nc; c0 += 8) {
-                            float2 ml[8];
-                            float4 pa[8];
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const int c = min(c0 + i, nc - 1);
-                                const size_t b = ((size_t)head * p.chunk_stride + c) * kPassMaxRows + m;
-                                ml[i] = __ldcg(reinterpret_cast<const float2*>(p.part_ml + b * 2));
-                                pa[i] = __ldcg(reinterpret_cast<const float4*>(p.part_acc + b * hd + e4));
-                            }
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                if (c0 + i < nc) {
-                                    const float mn = fmaxf(mx, ml[i].x);
-                                    const float s_old = expf(mx - mn), s_new = expf(ml[i].x - mn);
-                                    acc[0] = __fmaf_rn(acc[0], s_old, __fmul_rn(pa[i].x, s_new));
-                                    acc[1] = __fmaf_rn(acc[1], s_old, __fmul_rn(pa[i].y, s_new));
-                                    acc[2] = __fmaf_rn(acc[2], s_old, __fmul_rn(pa[i].z, s_new));
-                                    acc[3] = __fmaf_rn(acc[3], s_old, __fmul_rn(pa[i].w, s_new));
-                                    l = __fmaf_rn(l, s_old, __fmul_rn(ml[i].y, s_new));
-                                    mx = mn;
-                                }
-                            }
-                        }
-                        const __nv_bfloat162 o01 = __floats2bfloat162_rn(__fdiv_rn(acc[0], l), __fdiv_rn(acc[1], l));
-                        const __nv_bfloat162 o23 = __floats2bfloat162_rn(__fdiv_rn(acc[2], l), __fdiv_rn(acc[3], l));
-                        uint2 o;
-                        o.x = *reinterpret_cast<const uint32_t*>(&o01);
-                        o.y = *reinterpret_cast<const uint32_t*>(&o23);
-                        if (LL) {
-                            uint2* dst = p.al + (((size_t)m * p.d_model + (size_t)head * hd + e4) >> 1);
-                            ll_store(dst, o.x, p.pass_tag + (uint32_t)stage);
-                            ll_store(dst + 1, o.y, p.pass_tag + (uint32_t)stage);
-                        } else {
-                            *reinterpret_cast<uint2*>(p.a + (size_t)m * p.d_model + (size_t)head * hd + e4) = o;
-                        }
-                    }
-                }
-            }
-        }
-        if (j == 0) trace_mark(p, stage, 7);
     }
-    if (LL) {
-        // Tagged handoff, second sweep: the group that took a head's last chunk (the one with this pass's key) merges the
-        // head, after ALL its items: it asks for the chunks' partial results until their tags are this stage's. Nobody who
-        // produces a partial result ever waits for a merge, so the wait ends; merging inside the first sweep would hold
-        // this CTA's later items (and through the ring its other groups) behind chunks that other CTAs reach last.
-        for (int j = grp; j < n_local; j += p.attn_groups) {
-            const int idx = first + j;
-            const int kvh = idx / n_chunks, chunk = idx - kvh * n_chunks;
-            if (chunk != n_chunks - 1) continue;
-            for (int g = 0; g < group; ++g) {
-                const int head = kvh * group + g;
-                for (int e0 = 0; e0 < hd; e0 += 128) {  // one output dimension per thread (every lane runs the loop: shuffle below)
-                    const int e = e0 + gt;
-                    const bool act = e < hd;
-                    float mx = -INFINITY, l = 0.f, acc = 0.f;
-                    // Lane i of every warp fetches (maximum, sum of weights) of chunk c0 + i, 32 chunks per memory round trip,
-                    // and hands them round by shuffle; every thread fetches its own dimension's sums 16 chunks at a time
-                    for (int c0 = 0; c0 < n_chunks; c0 += 32) {
-                        unsigned long long rm = 0, rl = 0;
-                        bool ml_stale = c0 + glane < n_chunks;
+}
+
+// Merging the chunks of a head, 32 output dimensions (a lane each) and one row at a time: `unit` of n_heads * rows * parts. The
+// chunks are merged in ascending order with explicit roundings, so the arithmetic is the same in every instantiation.
+struct MergeUnit {
+    int head, m, e;
+    bool act;
+    __device__ __forceinline__ MergeUnit(int unit, int rows, int hd) {
+        const int parts = (hd + 31) >> 5, lane = threadIdx.x & 31;
+        const int hm = unit / parts;
+        head = hm / rows, m = hm - head * rows, e = (unit - hm * parts) * 32 + lane;
+        act = e < hd;
+    }
+};
+// two neighbouring lanes' results as one word of two bf16, in the even lane
+__device__ __forceinline__ uint32_t merged_pair(float acc, float l) {
+    const uint32_t ob = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(__fdiv_rn(acc, l)));
+    return ob | (__shfl_down_sync(0xffffffffu, ob, 1) << 16);
+}
+
+// Tagged handoff: the warps without attention items merge. They ask for the chunks' (maximum, sum of weights) until the tags are
+// this stage's, then for the sums of 16 chunks at a time. Nobody who produces a partial result ever waits for a merge, so the
+// wait ends. (Merged by the group that took a head's last chunk after its items, a head cost 2-3 us behind the last item at
+// five chunks and 11 us at 65; here the chunks before the last one are merged while that one is still being worked on: attention
+// stage 7.9 -> 4.9 us at 512 positions of the 7B shape, 36.9 -> 25.3 us at 8192.)
+__device__ __forceinline__ void merge_tagged(const PassParams& p, int stage, int n_chunks, int warp0, int n_warps) {
+    const int lane = threadIdx.x & 31, hd = p.head_dim, warp = (threadIdx.x >> 5) - warp0;
+    const uint32_t tag_out = p.pass_tag + (uint32_t)stage;
+    const int units = p.n_heads * ((hd + 31) >> 5);
+    unsigned spins = 0;
+    long long t0 = 0;
+    for (int u = blockIdx.x + warp * gridDim.x; u < units; u += n_warps * gridDim.x) {
+        const MergeUnit mu(u, 1, hd);
+        const size_t chunk0 = (size_t)mu.head * p.chunk_stride;
+        float mx = -INFINITY, l = 0.f, acc = 0.f;
+        for (int c0 = 0; c0 < n_chunks; c0 += 32) {
+            unsigned long long rm = 0, rl = 0;
+            bool stale_ml = c0 + lane < n_chunks;
+            for (;;) {
+                if (stale_ml) {
+                    ll_load2(p.pl_ml + (chunk0 + c0 + lane) * 2, rm, rl);
+                    stale_ml = !(ll_ready(rm, tag_out) && ll_ready(rl, tag_out));
+                }
+                if (!__any_sync(0xffffffffu, stale_ml)) break;
+                if (!__all_sync(0xffffffffu, ll_keep_waiting(p, spins, t0, stage))) break;
+                __nanosleep(100u);
+            }
+            const MergeFactors mf(c0 + lane < n_chunks ? make_float2(__uint_as_float((uint32_t)rm), __uint_as_float((uint32_t)rl)) : make_float2(-INFINITY, 0.f), mx);
 #pragma unroll 1
-                        for (int c1 = c0; c1 < c0 + 32 && c1 < n_chunks; c1 += 16) {
-                            unsigned long long ra[16] = {};
-                            unsigned stale = 0u;
+            for (int c1 = 0; c1 < 32 && c0 + c1 < n_chunks; c1 += 16) {
+                unsigned long long ra[16] = {};
+                unsigned stale = 0u;
 #pragma unroll
-                            for (int i = 0; i < 16; ++i)
-                                if (act && c1 + i < n_chunks) stale |= 1u << i;
-                            for (;;) {
-                                if (ml_stale) ll_load2(p.pl_ml + ((size_t)head * p.chunk_stride + c0 + glane) * 2, rm, rl);
+                for (int i = 0; i < 16; ++i)
+                    if (mu.act && c0 + c1 + i < n_chunks) stale |= 1u << i;
+                for (;;) {
 #pragma unroll
-                                for (int i = 0; i < 16; ++i)
-                                    if (stale & (1u << i)) ra[i] = ll_load1(p.pl_acc + ((size_t)head * p.chunk_stride + c1 + i) * hd + e);
-                                if (ml_stale && ll_ready(rm, tag_out) && ll_ready(rl, tag_out)) ml_stale = false;
+                    for (int i = 0; i < 16; ++i)
+                        if (stale & (1u << i)) ra[i] = ll_load1(p.pl_acc + (chunk0 + c0 + c1 + i) * hd + mu.e);
 #pragma unroll
-                                for (int i = 0; i < 16; ++i)
-                                    if ((stale & (1u << i)) && ll_ready(ra[i], tag_out)) stale &= ~(1u << i);
-                                if ((stale == 0u && !ml_stale) || !ll_keep_waiting(p, ll_spins, ll_t0, stage)) break;
-                                __nanosleep(100u);
-                            }
-                            __syncwarp();
+                    for (int i = 0; i < 16; ++i)
+                        if ((stale & (1u << i)) && ll_ready(ra[i], tag_out)) stale &= ~(1u << i);
+                    if (!__any_sync(0xffffffffu, stale != 0u)) break;
+                    if (!__all_sync(0xffffffffu, ll_keep_waiting(p, spins, t0, stage))) break;
+                    __nanosleep(100u);
+                }
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                if (c1 + i < n_chunks) {  // (uniform) same arithmetic as the merge of the other instantiations
-                                    const float cm = __uint_as_float(__shfl_sync(0xffffffffu, (uint32_t)rm, (c1 - c0) + i));
-                                    const float cl = __uint_as_float(__shfl_sync(0xffffffffu, (uint32_t)rl, (c1 - c0) + i));
-                                    const float mn = fmaxf(mx, cm);
-                                    const float s_old = expf(mx - mn), s_new = expf(cm - mn);
-                                    acc = __fmaf_rn(acc, s_old, __fmul_rn(__uint_as_float((uint32_t)ra[i]), s_new));
-                                    l = __fmaf_rn(l, s_old, __fmul_rn(cl, s_new));
-                                    mx = mn;
-                                }
-                            }
-                        }
+                for (int i = 0; i < 16; ++i) {
+                    if (c0 + c1 + i < n_chunks) {
+                        float s_old, s_new, cl;
+                        mf.of(c1 + i, s_old, s_new, cl);
+                        acc = __fmaf_rn(acc, s_old, __fmul_rn(__uint_as_float((uint32_t)ra[i]), s_new));
+                        l = __fmaf_rn(l, s_old, __fmul_rn(cl, s_new));
                     }
-                    const uint32_t ob = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(__fdiv_rn(acc, l)));
-                    const uint32_t up = __shfl_down_sync(0xffffffffu, ob, 1);
-                    if (act && (gt & 1) == 0) ll_store(p.al + (((size_t)head * hd + e) >> 1), ob | (up << 16), tag_out);
                 }
             }
         }
-        if (grp == 0) trace_mark(p, stage, 7);
+        const uint32_t pair = merged_pair(acc, l);
+        if (mu.act && (lane & 1) == 0) ll_store(p.al + (((size_t)mu.head * hd + mu.e) >> 1), pair, tag_out);
+    }
+}
+
+// Without tags: behind a grid barrier of its own the heads and rows are dealt to all warps of the grid. (Merged by the group whose
+// report completed a head, five rows cost 4 us behind the last item at five chunks and 29 us at 65: 32 of the 148 CTAs, and
+// in each a chain of 18 trips to L2. Attention stage of five rows 17.2 -> 13.3 us at 512 positions of the 7B shape, 91 -> 58 us at 8192,
+// where the shorter items below have a share; two and three rows at 512 positions cost the same either way.)
+template <int M>
+__device__ __forceinline__ void merge_all(const PassParams& p) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, hd = p.head_dim;
+    const int units = p.n_heads * M * ((hd + 31) >> 5);
+    for (int u = blockIdx.x + warp * gridDim.x; u < units; u += kPassConsumerWarps * gridDim.x) {
+        const MergeUnit mu(u, M, hd);
+        const int nc = (p.pos0 + mu.m) / kAttnChunk + 1, e = mu.act ? mu.e : 0;
+        float mx = -INFINITY, l = 0.f, acc = 0.f;
+        for (int c0 = 0; c0 < nc; c0 += 32) {
+            const size_t row0 = ((size_t)mu.head * p.chunk_stride + c0) * kPassMaxRows + mu.m;
+            float pa[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                pa[i] = 0.f;
+                if ((i < 16 || c0 + 16 < nc) && c0 + i < nc) pa[i] = __ldcg(p.part_acc + (row0 + (size_t)i * kPassMaxRows) * hd + e);
+            }
+            const MergeFactors mf(c0 + lane < nc ? __ldcg(reinterpret_cast<const float2*>(p.part_ml + (row0 + (size_t)lane * kPassMaxRows) * 2))
+                                                 : make_float2(-INFINITY, 0.f), mx);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                if (c0 + i < nc) {
+                    float s_old, s_new, cl;
+                    mf.of(i, s_old, s_new, cl);
+                    acc = __fmaf_rn(acc, s_old, __fmul_rn(pa[i], s_new));
+                    l = __fmaf_rn(l, s_old, __fmul_rn(cl, s_new));
+                }
+            }
+        }
+        const uint32_t pair = merged_pair(acc, l);
+        if (mu.act && (lane & 1) == 0) *reinterpret_cast<uint32_t*>(p.a + (size_t)mu.m * p.d_model + (size_t)mu.head * hd + mu.e) = pair;
+    }
+}
+
+template <int M, bool LL>
+__device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassSmem& sm, uint32_t& gi, unsigned& merge_target, int stage) {
+    const int warp = threadIdx.x >> 5;
+    int n_chunks, first;
+    const int n_local = attn_local_items(p, M, n_chunks, first);
+    const uint32_t gi0 = gi;
+    gi += (uint32_t)(n_local * 2 * (kAttnChunk / kBoxKeys) * (p.head_dim > 64 ? p.head_dim / 64 : 1));
+    if (LL) trace_mark(p, stage, 1);  // tagged handoff: every item waits for exactly the words it needs
+    else stage_begin(p, stage);      // all consumer warps, also those without attention work
+    const int item_warps = 4 * p.attn_groups;
+    if (warp < item_warps) {
+        if (p.head_dim == 128) attn_items<M, LL, 128>(p, st, sm, gi0, stage, n_chunks, first, n_local);
+        else if (p.head_dim == 64) attn_items<M, LL, 64>(p, st, sm, gi0, stage, n_chunks, first, n_local);
+        else attn_items<M, LL, 0>(p, st, sm, gi0, stage, n_chunks, first, n_local);
+    } else if (LL) {
+        merge_tagged(p, stage, n_chunks, item_warps, kPassConsumerWarps - item_warps);
+    }
+    if (!LL) {
+        grid_arrive(p.merge_bar);
+        merge_target += gridDim.x;
+        grid_wait(p, p.merge_bar, merge_target);
+        merge_all<M>(p);
+        trace_mark(p, stage, 7);
     }
 }
 
@@ -2054,6 +2073,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
     }
 
     uint32_t gi = 0;
+    unsigned merge_target = p.merge_base;
     if (p.trace && threadIdx.x == 0) {  // which SM runs this CTA (entry 4 of the embedding stage, which streams nothing)
         unsigned smid;
         asm volatile("mov.u32 %0, %smid;" : "=r"(smid));
@@ -2082,7 +2102,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
             stage_begin(p, s, p.bar_extra_last);  // (test hook: extra arrivals that never come)
             finish_stage<M>(p, sm);
         } else if (st.type == kStAttn) {
-            attn_stage<M, LL>(p, st, sm, gi, s);
+            attn_stage<M, LL>(p, st, sm, gi, merge_target, s);
         } else {
             gemv_stage<M, LL>(p, st, sm, gi, s);
         }
@@ -2091,7 +2111,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
         // publishes everything this CTA has written so far, the others just count.
         bool release = true;
         if (LL && next_type >= 0) release = (next_type == kStFinish);
-        grid_arrive(p, release);
+        grid_arrive(p.grid_bar, release);
     }
 }
 
