@@ -6,34 +6,41 @@
 // at 8 mantissa bits each, which represents every fp32 probability exactly); with fewer terms the 2^-17 error of P
 // flips bf16 roundings of the attention output in about every second row.
 //
-// What bounds it: the chain S -> softmax -> P V -> S of a CTA, of which the SM's second CTA covers a part. Per 64 keys an S tile takes 384 cycles (N = 64 with both operands in shared memory is
-// bound by the operand reads: 48 KB at 128 B per cycle) and the three P V products take 256 each; the softmax between
-// the two takes about 700-800 cycles of the other units (64 ex2 per row are 512 cycles of the SFUs). Tiles of 64 keys because O (128 columns) and S / P (128 columns: the three terms take 96)
-// of two CTAs then fill the 512 columns of tensor memory.
+// What bounds it: the tensor core, once two CTAs share an SM. Per 64 keys an S tile takes 384 cycles (N = 64 with both operands
+// in shared memory is bound by the operand reads: 48 KB at 128 B per cycle) and the three P V products take 256 each; the
+// softmax of a row takes about 1400 cycles (450 for S and its maximum, 480 for the exponentials and terms of either half). P is
+// handed over in halves of 32 keys, so that the exponentials of one half run while the products of the other do, and S of the
+// next tile is ready before the softmax wants it: per tile and CTA 2500 cycles and the fold below, 1500 per SM with two CTAs (2700 when
+// a tile was one chain S -> softmax -> P V). Tiles of 64 keys because O (128 columns), S (64) and half a tile's P (64: hi of
+// both halves, mid, lo) of two CTAs then fill the 512 columns of tensor memory.
 //
 // The running maximum of a row is only moved when it has grown by more than 2^8 (the conditional rescaling of FlashAttention-4;
 // probabilities up to 256 are as exact as those up to 1): moving it means reading, scaling and writing O in tensor memory,
 // which random scores need once or twice per row instead of once per tile. Whether a row moves depends on its own scores alone.
 //
 // An MMA cuts its sum with the accumulator off towards zero, so a chain of them loses about half an ulp of O at every step:
-// 12 steps per key tile, and twice the loss per step that mma.sync has. Before the key tiles 1, 2, 4, 8, ... O and the row
-// sums are therefore added to fp32 totals in scratch memory (rounded to nearest; L2 holds them) and start anew. No
-// chain is then longer than half of a row's keys, and what is lost in it counts by its share of the sum. Error
-// against 64 bits over the attention kernel on mma.sync, 64 to 8192 keys: 0.3-0.8 of it (without the totals 0.7-2.4); a bias of
-// values with a mean of one 1.8e-5 after 8192 keys instead of 6.0e-5 (mma.sync: 3.1e-5).
+// 12 steps per key tile, and twice the loss per step that mma.sync has. The terms of a tile are therefore added smallest first (lo and
+// mid of both halves, then hi), and before the key tiles 1, 2, 4, 8, ... O and the row
+// sums are added to fp32 totals (rounded to nearest) and start anew. No chain is then longer than half of a row's keys, and what is
+// lost in it counts by its share of the sum. Error against 64 bits over the attention kernel on mma.sync, 64 to 8192 keys:
+// 0.3-0.8 of it (without the totals 0.7-2.4); a bias of values with a mean of one 1.8e-5 after 8192 keys instead of 6.0e-5
+// (mma.sync: 3.1e-5). Head size 64 leaves tensor memory for the totals; at 128 they are in scratch memory, and a fold is 64 KB
+// each way of L2 traffic that all CTAs make at the same tiles. (Adding in memory, red.add.v4.f32, was slower: 2048 keys 0.127 -> 0.140 ms.)
 //
-// Measured (8192-token prompt, 32 heads of 128, per layer, launch to end): 3.4 ms with mma.sync and 64-row tiles, 1.3 ms here,
-// about 0.15 of it for the totals (a fold is a round trip to L2 in the chain of its tile: 4-5 % of a prompt pass of 512 to
-// 8192 tokens). The tensor core is active in 39 % of the cycles over the first 2048 keys.
+// Measured, 2048 rows of 32 heads of 128, launch to end, against a tile as one chain S -> softmax -> P V with S over the lo terms:
+// 0.139 -> 0.123 ms over their own keys, 0.268 -> 0.222 ms on top of 2048 others, 0.521 -> 0.419 ms on top of 6144; heads of 64
+// 0.085 -> 0.072, 0.181 -> 0.150, 0.368 -> 0.298 ms. What is left over the tensor core's 0.26 ms (6144) is the second round of CTAs (512 on
+// 296 places) and the folds.
 #include "common.cuh"
 #include "prefill.h"
 #include "tcgen05.cuh"
 
 namespace asd {
 
-constexpr int kFaRows = 128, kFaKeys = 64, kFaThreads = 192, kFaStages = 2;
-constexpr int kFaTmemCols = 256;                       // O: 0-127; S: 128-191
-constexpr int kFaColS = 128, kFaColHi = 192, kFaColMid = 224, kFaColLo = 128;  // the lo terms take the place of S
+constexpr int kFaRows = 128, kFaKeys = 64, kFaHalf = kFaKeys / 2, kFaThreads = 192, kFaStages = 2;
+constexpr int kFaTmemCols = 256;                       // O: 0-127; S: 128-191; P of half a key tile: 192-255
+constexpr int kFaColS = 128, kFaColHi = 192, kFaColMid = 224, kFaColLo = 240;  // hi terms of either half
+constexpr int kFaColTotals = 64;                       // head size 64: the totals, behind O
 
 // tiles before which O and the row sums are folded into the totals: 1, 2, 4, 8, ... (absolute key tiles: the same for every row)
 constexpr int kFaFirstFold = 1;
@@ -67,58 +74,62 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
         : "memory");
 }
 
-// 32 scores of one row -> probabilities 2^(s c - m c), their sum added to sum2, their three bf16 terms to tensor memory
+__device__ __forceinline__ unsigned long long fsub2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+// 32 scores of one row -> probabilities 2^(s c - m c), their sum added to sum2, their three bf16 terms (pairs of keys)
 __device__ __forceinline__ void probabilities32(const uint32_t (&s)[32], unsigned long long c2, unsigned long long nmc2, unsigned long long& sum2,
-                                                uint32_t t_hi, uint32_t t_mid, uint32_t t_lo) {
-    uint32_t p[32], w[16];
+                                                uint32_t (&hi)[16], uint32_t (&mid)[16], uint32_t (&lo)[16]) {
     unsigned long long part = pack2(0.f, 0.f);  // a sum of its own, so that no chain of additions runs over all keys of a row
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         float a, b;
         unpack2(ffma2(pack2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), c2, nmc2), a, b);
-        a = ex2(a), b = ex2(b);
-        part = fadd2(part, pack2(a, b));
-        p[2 * i] = __float_as_uint(a), p[2 * i + 1] = __float_as_uint(b);
-        w[i] = upper_halves(p[2 * i], p[2 * i + 1]);
+        unsigned long long p = pack2(ex2(a), ex2(b));
+        part = fadd2(part, p);
+        auto term = [&](uint32_t& w) {  // the upper 8 bits of what is left of both
+            unpack2(p, a, b);
+            w = upper_halves(__float_as_uint(a), __float_as_uint(b));
+            return pack2(__uint_as_float(__float_as_uint(a) & 0xFFFF0000u), __uint_as_float(__float_as_uint(b) & 0xFFFF0000u));
+        };
+        p = fsub2(p, term(hi[i]));  // exact
+        p = fsub2(p, term(mid[i]));  // exact, 8 bits left
+        unpack2(p, a, b);
+        lo[i] = upper_halves(__float_as_uint(a), __float_as_uint(b));
     }
     sum2 = fadd2(sum2, part);
-    tmem_st16(t_hi, w);
-#pragma unroll
-    for (int i = 0; i < 32; ++i) p[i] = __float_as_uint(__uint_as_float(p[i]) - __uint_as_float(p[i] & 0xFFFF0000u));  // exact
-#pragma unroll
-    for (int i = 0; i < 16; ++i) w[i] = upper_halves(p[2 * i], p[2 * i + 1]);
-    tmem_st16(t_mid, w);
-#pragma unroll
-    for (int i = 0; i < 32; ++i) p[i] = __float_as_uint(__uint_as_float(p[i]) - __uint_as_float(p[i] & 0xFFFF0000u));  // exact, 8 bits left
-#pragma unroll
-    for (int i = 0; i < 16; ++i) w[i] = upper_halves(p[2 * i], p[2 * i + 1]);
-    tmem_st16(t_lo, w);
 }
 
 // Warps 0-3: softmax and epilogue, thread = query row. Warp 4: TMA producer. Warp 5: issues the MMAs
 // and owns the tensor-memory allocation. Barriers: q_full, k_full / v_full[s] (bytes landed), k_empty / v_empty[s] (the
-// MMAs reading the stage have finished), s_full (S of tile j is complete, and with it every earlier MMA: O holds the
-// tiles before j and P may be overwritten; phase n_kt: O is complete), p_full (the 128 rows' P of tile j are in tensor
-// memory), lo_read (the products with the lo terms of tile j have finished). S of tile j + 1 goes over the columns of those lo
-// terms. PTX orders a pair of tcgen05.mma by their issue only when they share accumulator and shape (memory consistency model
-// of tcgen05, "pipelined instructions"), which P V and S do not, so its issue waits for lo_read: the lo products come first
-// and the wait passes while the mid and hi products, 512 cycles, still run.
+// MMAs reading the stage have finished), s_full (S of tile j is complete), p_full (the 128 rows' P of half a tile is in tensor
+// memory), pv_done (the products with it have finished, and with them every earlier one: O holds the halves so far and P may be
+// overwritten). S of tile j + 1 goes over S of tile j, which every thread has read before it reports the first half of P.
 template <int HD>
 __global__ void __launch_bounds__(kFaThreads, 2)
 flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                      __nv_bfloat16* __restrict__ out, float* totals, int n_rows, int pos0, int d_model, int group, float scale_log2, int* err_words) {
     using Cfg = FaCfg<HD>;
+    constexpr bool kTmemTotals = HD == 64;
     extern __shared__ unsigned char fa_smem_raw[];
     unsigned char* base = fa_smem_raw + ((1024u - (smem_u32(fa_smem_raw) & 1023u)) & 1023u);
     unsigned char* k_smem = base + Cfg::kQBytes;
     unsigned char* v_smem = k_smem + kFaStages * Cfg::kKvBytes;
     uint64_t* q_full = reinterpret_cast<uint64_t*>(v_smem + kFaStages * Cfg::kKvBytes);
     uint64_t *k_full = q_full + 1, *k_empty = k_full + kFaStages, *v_full = k_empty + kFaStages, *v_empty = v_full + kFaStages;
-    uint64_t *s_full = v_empty + kFaStages, *p_full = s_full + 1, *lo_read = p_full + 1, *drained = lo_read + 1;
+    uint64_t *s_full = v_empty + kFaStages, *p_full = s_full + 1, *pv_done = p_full + 1, *drained = pv_done + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drained + 1);
     volatile int* err = err_words;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
     const int head = blockIdx.x, kvh = head / group;
     const int r0 = (gridDim.y - 1 - blockIdx.y) * kFaRows;  // the tiles with the most keys start first
     const int last_row = min(r0 + kFaRows, n_rows) - 1;
@@ -129,7 +140,7 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         for (int s = 0; s < kFaStages; ++s) mbar_init(&k_full[s], 1), mbar_init(&k_empty[s], 1), mbar_init(&v_full[s], 1), mbar_init(&v_empty[s], 1);
         mbar_init(s_full, 1);
         mbar_init(p_full, kFaRows);
-        mbar_init(lo_read, 1);
+        mbar_init(pv_done, 1);
         mbar_init(drained, 1);
         mbar_fence_init();
     }
@@ -197,26 +208,26 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         scores(0);
         for (int j = 0; j < n_kt && ok; ++j) {
             const int s = j % kFaStages;
-            ok = mbar_wait_warp(&v_full[s], (uint32_t)((j / kFaStages) & 1), err, kErrAttnWait, 1, j, s, 5) &&
-                 mbar_wait_warp(p_full, (uint32_t)(j & 1), err, kErrAttnWait, 1, j, s, 6);
-            if (!ok) break;
-            tc_fence_after();
+            ok = mbar_wait_warp(&v_full[s], (uint32_t)((j / kFaStages) & 1), err, kErrAttnWait, 1, j, s, 5);
+            const bool fresh = j == 0 || fa_folds(j);  // O starts anew
             const uint64_t v_desc = umma_desc_mn128(smem_u32(v_smem) + s * Cfg::kKvBytes, Cfg::kKvPanel);
+#pragma unroll 1
+            for (int h = 0; h < 2 && ok; ++h) {
+                ok = mbar_wait_warp(p_full, (uint32_t)h, err, kErrAttnWait, 1, j, s, 6);
+                if (!ok) break;
+                tc_fence_after();
+                auto products = [&](uint32_t a, int half, bool anew) {  // O (+)= one term of the half's P
 #pragma unroll
-            for (int t = 0; t < 3; ++t) {  // lo, mid, hi: the smallest terms first
-                const uint32_t a = tmem + (t == 0 ? kFaColLo : (t == 1 ? kFaColMid : kFaColHi));
-#pragma unroll
-                for (int k = 0; k < kFaKeys / 16; ++k)  // 16 keys: 8 columns of P, 2048 bytes of V
-                    tc_mma_bf16_ts(tmem, a + 8 * k, v_desc + (uint64_t)(128 * k), idesc_o, (t | k) != 0 || !(j == 0 || fa_folds(j)), on);
-                if (t == 0) tc_commit(lo_read, on);
+                    for (int k = 0; k < kFaHalf / 16; ++k)  // 16 keys: 8 columns of P, 2048 bytes of V
+                        tc_mma_bf16_ts(tmem, tmem + a + 8 * k, v_desc + (uint64_t)(128 * (half * (kFaHalf / 16) + k)), idesc_o, !(anew && k == 0), on);
+                };
+                products(kFaColLo, h, fresh && h == 0);
+                products(kFaColMid, h, false);
+                if (h == 1) products(kFaColHi, 0, false), products(kFaColHi + 16, 1, false);  // the largest terms last
+                tc_commit(pv_done, on);
+                if (h == 0 && j + 1 < n_kt) scores(j + 1);
             }
             tc_commit(&v_empty[s], on);
-            if (j + 1 < n_kt) {
-                ok = mbar_wait_warp(lo_read, (uint32_t)(j & 1), err, kErrAttnWait, 1, j, s, 9);
-                scores(j + 1);
-            } else {
-                tc_commit(s_full, on);  // O is complete
-            }
         }
         // the MMAs end before the tensor memory is freed, also when a role of the CTA gives up
         tc_commit(drained, on);
@@ -231,40 +242,81 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         // block's part of totals is [HD / 8][128 rows][8], so that the 32 bytes of neighbouring lanes are neighbours.
         float* total = totals + (size_t)r0 * d_model + (size_t)head * (kFaRows * HD) + threadIdx.x * 8;
         float sum_total = 0.f, since = 1.f;
-        auto fold = [&](int c, bool first, float (&v)[32]) {  // columns c .. c + 31: total * since + O
-            uint32_t o[32], w[32];
-            tmem_ld32_async(lane_base + c, o);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) w[i] = 0u;
-            if (!first) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 8) ld_global_v8(total + (c + i) * kFaRows, w + i);
-            }
-            tmem_ld_wait(o);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = fmaf(__uint_as_float(w[i]), since, __uint_as_float(o[i]));
-        };
         unsigned long long sum2 = pack2(0.f, 0.f);
         bool ok = true;
-        for (int j = 0; j < n_kt; ++j) {
-            ok = mbar_wait(s_full, (uint32_t)(j & 1), err, kErrAttnWait, 2, j, 0, 7);
+        int halves = 0;  // halves of P reported so far
+        auto products_done = [&]() {  // of every half reported so far
+            if (halves > 0) ok = mbar_wait(pv_done, (uint32_t)((halves - 1) & 1), err, kErrAttnWait, 2, halves, 0, 9) && ok;
             ok = __all_sync(0xffffffffu, ok);  // tensor-memory accesses are warp-wide
-            if (!ok) break;
             tc_fence_after();
-            const bool fresh = fa_folds(j);
-            if (fresh) {  // (32 columns at a time: 64, or loads in front of the wait, spill registers of the tile loop)
+        };
+        // total * since + O, 32 columns at a time, to `take`. In scratch memory the totals of 64 columns are requested at a time, the
+        // first ones while the products still run; in tensor memory (HD = 64 leaves it 64 columns) they are at hand.
+        auto fold = [&](bool first, auto&& take) {
 #pragma unroll
-                for (int c = 0; c < HD; c += 32) {
-                    float v[32];
-                    fold(c, j == kFaFirstFold, v);
+            for (int c = 0; c < HD; c += 64) {
+                uint32_t w[64], o[32];
+                if (!kTmemTotals) {
 #pragma unroll
-                    for (int i = 0; i < 32; i += 8) st_global_v8(total + (c + i) * kFaRows, reinterpret_cast<const uint32_t*>(v) + i);
+                    for (int i = 0; i < 64; ++i) w[i] = 0u;
+                    if (!first) {
+#pragma unroll
+                        for (int i = 0; i < 64; i += 8) ld_global_v8(total + (c + i) * kFaRows, w + i);
+                    }
                 }
+                if (c == 0) products_done();
+                if (!ok) return;
+#pragma unroll
+                for (int h = 0; h < 64; h += 32) {
+                    uint32_t t[32];
+                    tmem_ld32_async(lane_base + c + h, o);
+                    if (kTmemTotals && !first) tmem_ld32_async(lane_base + kFaColTotals + h, t);
+                    tmem_ld_wait(o);
+                    if (kTmemTotals && !first) tmem_ld_wait(t);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        const float before = first ? 0.f : __uint_as_float(kTmemTotals ? t[i] : w[h + i]);
+                        o[i] = __float_as_uint(fmaf(before, since, __uint_as_float(o[i])));
+                    }
+                    take(c + h, o);
+                }
+            }
+        };
+        // the exponentials of half a tile run while the products of the half before do; then its P takes the place that those have left
+        auto report_half = [&](int h, const uint32_t (&s)[32], unsigned long long nmc2) {
+            uint32_t hi[16], mid[16], lo[16];
+            probabilities32(s, c2, nmc2, sum2, hi, mid, lo);
+            products_done();
+            if (!ok) return;
+            tmem_st16(lane_base + kFaColHi + 16 * h, hi);
+            tmem_st16(lane_base + kFaColMid, mid);
+            tmem_st16(lane_base + kFaColLo, lo);
+            tmem_st_wait();
+            tc_fence_before();
+            mbar_arrive(p_full);
+            ++halves;
+        };
+        for (int j = 0; j < n_kt; ++j) {
+            const bool fresh = fa_folds(j);
+            if (fresh) {
+                fold(j == kFaFirstFold, [&](int c, const uint32_t (&v)[32]) {
+                    if (kTmemTotals) {
+                        tmem_st32(lane_base + kFaColTotals + c, v);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 32; i += 8) st_global_v8(total + (c + i) * kFaRows, v + i);
+                    }
+                });
+                if (!ok) break;
                 float a, b;
                 unpack2(sum2, a, b);
                 sum_total = fmaf(sum_total, since, a + b);
                 sum2 = pack2(0.f, 0.f), since = 1.f;
             }
+            ok = mbar_wait(s_full, (uint32_t)(j & 1), err, kErrAttnWait, 2, j, 0, 7);
+            ok = __all_sync(0xffffffffu, ok);  // tensor-memory accesses are warp-wide
+            if (!ok) break;
+            tc_fence_after();
             uint32_t s0[32], s1[32];
             tmem_ld32_async(lane_base + kFaColS, s0);
             tmem_ld32_async(lane_base + kFaColS + 32, s1);
@@ -281,8 +333,8 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
             for (int i = 0; i < 32; i += 2) {
-                mx[(i >> 1) & 3] = fmaxf(mx[(i >> 1) & 3], fmaxf(__uint_as_float(s0[i]), __uint_as_float(s0[i + 1])));
-                mx[(i >> 1) & 3] = fmaxf(mx[(i >> 1) & 3], fmaxf(__uint_as_float(s1[i]), __uint_as_float(s1[i + 1])));
+                mx[(i >> 1) & 1] = max3(mx[(i >> 1) & 1], __uint_as_float(s0[i]), __uint_as_float(s0[i + 1]));
+                mx[2 + ((i >> 1) & 1)] = max3(mx[2 + ((i >> 1) & 1)], __uint_as_float(s1[i]), __uint_as_float(s1[i + 1]));
             }
             const float tile_max = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
             if (j == 0) {
@@ -297,6 +349,8 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 unpack2(sum2, a, b);
                 sum2 = pack2(a * alpha, b * alpha);
                 since *= alpha;
+                if (!fresh) products_done();
+                if (!ok) break;
 #pragma unroll 1
                 for (int c = fresh ? HD : 0; c < HD; c += 32) {
                     uint32_t o[32];
@@ -309,33 +363,24 @@ flash_prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             }
             const float nmc = -m * scale_log2;
             const unsigned long long nmc2 = pack2(nmc, nmc);
-            // the lo terms overwrite S: both halves have been read
-            probabilities32(s0, c2, nmc2, sum2, lane_base + kFaColHi, lane_base + kFaColMid, lane_base + kFaColLo);
-            probabilities32(s1, c2, nmc2, sum2, lane_base + kFaColHi + 16, lane_base + kFaColMid + 16, lane_base + kFaColLo + 16);
-            tmem_st_wait();
-            tc_fence_before();
-            mbar_arrive(p_full);
+            report_half(0, s0, nmc2);
+            if (ok) report_half(1, s1, nmc2);
+            if (!ok) break;
         }
-        if (ok) ok = mbar_wait(s_full, (uint32_t)(n_kt & 1), err, kErrAttnWait, 2, n_kt, 0, 8);
-        ok = __all_sync(0xffffffffu, ok);
         if (ok) {
-            tc_fence_after();
             float a, b;
             unpack2(sum2, a, b);
             const float inv = 1.0f / fmaf(sum_total, since, a + b);
             __nv_bfloat16* dst = out + (size_t)row * d_model + (size_t)head * HD;
-#pragma unroll
-            for (int c = 0; c < HD; c += 32) {
-                float v[32];
-                fold(c, n_kt <= kFaFirstFold, v);
+            fold(n_kt <= kFaFirstFold, [&](int c, const uint32_t (&v)[32]) {
                 if (row < n_rows) {
                     uint32_t w[16];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) w[i] = pack_bf16(v[2 * i] * inv, v[2 * i + 1] * inv);
+                    for (int i = 0; i < 16; ++i) w[i] = pack_bf16(__uint_as_float(v[2 * i]) * inv, __uint_as_float(v[2 * i + 1]) * inv);
                     st_global_v8(dst + c, w);
                     st_global_v8(dst + c + 16, w + 8);
                 }
-            }
+            });
         }
     }
     tc_fence_before();
