@@ -1632,7 +1632,7 @@ extern "C" int asd_gemm_bf16(void* cuda_stream, int32_t M, int32_t N, int32_t K,
         !encode_operand_map(encode, &tm_w, const_cast<uint16_t*>(W), (size_t)K, (size_t)N, (uint32_t)plan.w_box()))
         return ASD_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    if (cudaMemsetAsync(dev_status, 0, 32, s) != cudaSuccess) return ASD_ERR_CUDA;
+    if (launch_clear_status(dev_status, s) != cudaSuccess) return ASD_ERR_CUDA;
     GemmEpi e{};
     e.mode = kGemmF32;
     e.err = dev_status;

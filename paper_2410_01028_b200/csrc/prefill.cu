@@ -360,6 +360,16 @@ cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int
     return launch_gemm<192, 2>(tm_a, tm_w, M, N, K, w, ep, s);
 }
 
+// The status words of a product on its own, cleared by a kernel whose launch overlaps the end of the kernel in front and under
+// which the product's own launch and set-up run (a memset between two products costs both overlaps: 511 x 12288 x 4096
+// 54.5 -> 52.6 us a call, 2048 x 22016 x 4096 300 -> 294 us).
+__global__ void __launch_bounds__(32) clear_status_kernel(int* status) {
+    pdl_launch_dependents();
+    pdl_wait();
+    if (threadIdx.x < 8) status[threadIdx.x] = 0;
+}
+cudaError_t launch_clear_status(int* status, cudaStream_t s) { return launch_pdl(clear_status_kernel, dim3(1), dim3(32), 0, s, 1, status); }
+
 // ============================================================================================ row kernels
 constexpr int kRowThreads = 256;
 

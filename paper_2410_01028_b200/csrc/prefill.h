@@ -50,6 +50,8 @@ GemmPlan plan_gemm(int M, int N, int K, int max_parts);
 // w_box()), fp32 accumulation
 cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmPlan& plan, const GemmEpi& ep, cudaStream_t s);
 
+cudaError_t launch_clear_status(int* status /* 8 words */, cudaStream_t s);
+
 // x[r, :] = embedding row of tokens[r] (fp32); xn[r, :] = bf16(RMSNorm(x[r]) * gain)
 cudaError_t launch_embed_norm(const int* tokens, int n_rows, int d, int vocab, const __nv_bfloat16* embed, const __nv_bfloat16* gain,
                               float eps, float* x, __nv_bfloat16* xn, cudaStream_t s);
