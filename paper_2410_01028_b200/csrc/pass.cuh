@@ -70,7 +70,8 @@ struct ResidOut {
 
 struct PassParams {
     int pos0;
-    const int* tokens;
+    const int* tokens;                // the rows' tokens in device memory, or null:
+    int inline_tokens[kMaxRows];      // a single-step call's tokens come with the launch
     const __nv_bfloat16* embed;
     int d_model, vocab, kv_dim, head_dim, n_heads, n_kv_heads, d_ffn;
     int hd_shift;  // log2(head_dim) when head_dim is a power of two, else 0 (divisions instead of shifts)
@@ -98,10 +99,11 @@ struct PassParams {
     int* err;
     const StageDesc* stages;
     int n_stages;
-    const int* row_tokens;
     int* argmax_out;
     float* margin_out;  // [M] top-1 minus top-2 logit of every row (the confidence that ends a draft run early), or null
-    int* accept_out;
+    int* accept_out;   // greedy verification: accepted drafts, then the tokens (null: none)
+    int* host_out;     // pinned host memory for what the caller waits for (kHost... below), or null
+    int host_stamp;    // names this pass there
     float* logits_out;
     int acc_sim;
     long long* trace;  // optional [n_stages][kTraceEntries][gridDim.x] device timestamps (ns) and cycle counts, or null
@@ -112,6 +114,11 @@ struct PassParams {
     int off_bars, off_misc, off_psum, off_reg_a;
     int xs_bytes;      // bytes of the activation window (as few windows per stage as leave the ring 20 slots)
 };
+
+// Words of host_out: the accept block or the last row's token, the last row's margin, the error words, the pass's stamp
+constexpr int kHostMargin = 12, kHostErr = 16, kHostStamp = 24;
+
+__device__ __forceinline__ int pass_token(const PassParams& p, int m) { return p.tokens ? __ldcg(p.tokens + m) : p.inline_tokens[m]; }
 
 constexpr int kTraceEntries = 12;  // per stage and CTA: 0-7 consumer side, 8-10 producer side (first / last copy issued, stall cycles), 11 descriptor read
 constexpr int kSegK = 256;     // inputs per ring item (8 column blocks of 32; the last item of a row may hold fewer)
@@ -1465,17 +1472,27 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
                     p.argmax_out[m] = i;
                     if (p.margin_out) p.margin_out[m] = v - sc;
                     g[m] = i;
+                    if (p.host_out && m == M - 1) reinterpret_cast<float*>(p.host_out)[kHostMargin] = v - sc;
                 }
             }
             consumers_sync();
             if (tid == 0) {
-                if (p.accept_out && p.row_tokens) {
+                int* h = p.host_out;
+                if (p.accept_out) {
                     // greedy verification (Section 1): drafted token j+1 is accepted while it equals M's argmax of row j
                     int a = 0;
-                    while (a < M - 1 && p.row_tokens[a + 1] == g[a]) ++a;
-                    p.accept_out[0] = a;
-                    for (int j = 0; j < a; ++j) p.accept_out[1 + j] = p.row_tokens[j + 1];
-                    p.accept_out[1 + a] = g[a];
+                    while (a < M - 1 && pass_token(p, a + 1) == g[a]) ++a;
+                    for (int j = 0; j <= a + 1; ++j) {
+                        const int v = j == 0 ? a : (j <= a ? pass_token(p, j) : g[a]);
+                        p.accept_out[j] = v;
+                        if (h) h[j] = v;
+                    }
+                } else if (h) {
+                    h[0] = g[M - 1];
+                }
+                if (h) {  // every CTA has arrived here, so whoever gave up waiting has said so
+                    for (int j = 0; j < 8; ++j) h[kHostErr + j] = *(static_cast<volatile int*>(p.err) + j);
+                    h[kHostStamp] = p.host_stamp;
                 }
                 *p.fin_counter = 0u;
             }
@@ -2092,7 +2109,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
             const int d = p.d_model;
             for (int i = blockIdx.x * kPassConsumers + threadIdx.x; i < M * d; i += gridDim.x * kPassConsumers) {
                 const int m = i / d, e = i - m * d;
-                int t = __ldcg(p.tokens + m);
+                int t = pass_token(p, m);
                 t = min(max(t, 0), p.vocab - 1);
                 const float v = __bfloat162float(p.embed[(size_t)t * d + e]);
                 if (LL) ll_store(p.xl + i, __float_as_uint(v), p.pass_tag);
