@@ -12,7 +12,7 @@
 
 #include "../../include/asd.h"
 #include "common.cuh"
-#include "gemv.cuh"
+#include "gemv.h"
 #include "pass.cuh"
 #include "prefill.h"
 #include "sample.h"
@@ -22,26 +22,13 @@ namespace asd {
 constexpr int kPrefillRows = kPassMaxRows;  // prompt rows per pass of the chunked prefill
 constexpr size_t kAlign = 256;
 constexpr int kMaxGemvGrid = 1024;
+constexpr size_t kGemvErrOffset = 128;  // the fused GEMV's error words in the first 256 bytes of its scratch
 constexpr int kPinnedPass = 64;  // word of the pinned block at which a pass leaves its result
 constexpr size_t kPinnedOut = 256 * 1024;  // larger results of inspection calls go straight to the caller's memory
 constexpr long long kShortWaitCycles = 2000000LL;  // ASD_DEBUG_SHORT_WAITS: about a millisecond per wait
 
 static size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
-static cudaError_t launch_gemv(int M, int epi, bool norm, const GemvParams& p, int grid, size_t smem, cudaStream_t s) {
-    switch (M) {
-        case 1: return launch_gemv_m1(epi, norm, p, grid, smem, s);
-        case 2: return launch_gemv_m2(epi, norm, p, grid, smem, s);
-        case 3: return launch_gemv_m3(epi, norm, p, grid, smem, s);
-        case 4: return launch_gemv_m4(epi, norm, p, grid, smem, s);
-        case 5: return launch_gemv_m5(epi, norm, p, grid, smem, s);
-        case 6: return launch_gemv_m6(epi, norm, p, grid, smem, s);
-        case 7: return launch_gemv_m7(epi, norm, p, grid, smem, s);
-        case 8: return launch_gemv_m8(epi, norm, p, grid, smem, s);
-        case 9: return launch_gemv_m9(epi, norm, p, grid, smem, s);
-    }
-    return cudaErrorInvalidValue;
-}
 static cudaError_t launch_pass(int M, const PassParams& p, int grid, size_t smem, cudaStream_t s) {
     switch (M) {
         case 1: return launch_pass_m1(p, grid, smem, s);
@@ -86,6 +73,7 @@ static cudaError_t device_info(DeviceInfo** out) {
         if ((e = configure_m8(d.max_smem)) != cudaSuccess) return e;
         if ((e = configure_m9(d.max_smem)) != cudaSuccess) return e;
         if ((e = configure_m16(d.max_smem)) != cudaSuccess) return e;
+        if ((e = configure_gemv(d.max_smem)) != cudaSuccess) return e;
         if ((e = configure_prefill(d.max_smem)) != cudaSuccess) return e;
         d.ready = true;
     }
@@ -108,36 +96,6 @@ static bool gemv_accepts(const DeviceInfo& dv, int M, int n_rows, int n_in, bool
         }
     }
     return false;
-}
-
-// The plan of one launch (shared memory returned). Sub-items per group: the split that leaves the warps least unequal,
-// counted in segments of the longest warp; a finer split has to gain a twentieth, because each costs an epilogue addition.
-// Windows of the activations: as few as kGemvSmem holds, of equal length, beginning at multiples of the runs of all
-// sub-items. The split does not depend on M.
-// kGemvSmem is half of the SM's 256 KB although a block may have 227: the weights in flight take lines of what is left as L1
-// cache (five rows of 13760 inputs: one window and 170 KB 43-59 us, depending on how much is in flight).
-constexpr size_t kGemvSmem = 128 * 1024;
-static size_t plan_gemv(const DeviceInfo& dv, int M, int n_rows, int n_in, GemvParams* p) {
-    const int n_seg = (n_in + kGemvSeg - 1) / kGemvSeg, n_run = (n_seg + kGemvRun - 1) / kGemvRun;
-    p->max_rows = 0;
-    for (int b = 0; b < dv.num_sms; ++b) p->max_rows = std::max(p->max_rows, gemv_row(n_rows, dv.num_sms, b + 1) - gemv_row(n_rows, dv.num_sms, b));
-    p->n_blk = (p->max_rows + kGemvBlockRows - 1) / kGemvBlockRows;
-    if (p->n_blk > 1) p->max_rows = (p->max_rows + p->n_blk - 1) / p->n_blk + 2;  // block boundaries are even
-    const int groups = (p->max_rows + 15) / 16;
-    auto longest = [&](int s) { return (groups * s + kGemvWarps - 1) / kGemvWarps * ((n_run + s - 1) / s); };
-    p->split = 1;
-    for (int s = 2; s <= 16 && s <= n_run && groups * s <= kGemvMaxSub; ++s)
-        if (20 * longest(s) < 19 * longest(p->split)) p->split = s;
-    p->max_sub = groups * p->split;
-    const size_t fixed = (size_t)gemv_fixed_smem(M, p->max_sub, p->max_rows);
-    const size_t room = kGemvSmem > fixed ? (kGemvSmem - fixed) / M / 2 : 0;
-    const int most = room > (size_t)kGemvPad ? (int)((room - kGemvPad) / kGemvSeg) : 0, unit = p->split * kGemvRun;
-    p->win_segs = n_seg;
-    if (n_seg > most) {
-        const int unit_most = std::max(most / unit, 1) * unit, n_win = (n_seg + unit_most - 1) / unit_most;
-        p->win_segs = ((n_seg + n_win - 1) / n_win + unit - 1) / unit * unit;
-    }
-    return fixed + (size_t)M * (p->win_segs * kGemvSeg + kGemvPad) * 2;
 }
 
 // Shared-memory plan of the persistent pass kernel for M rows: ring slots, barriers, reduction scratch,
@@ -1651,19 +1609,18 @@ extern "C" int asd_fused_gemv(void* cuda_stream, int32_t M, int32_t n_in, int32_
     if (device_info(&dv) != cudaSuccess) return ASD_ERR_CUDA;
     GemvParams p{};
     p.W = reinterpret_cast<const __nv_bfloat16*>(W);
-    p.n_rows = n_rows;
-    p.n_in = n_in;
+    p.M = M, p.n_rows = n_rows, p.n_in = n_in;
     p.x = x;
     p.gain = reinterpret_cast<const __nv_bfloat16*>(gain);
     p.eps = eps;
     p.out = out;
     p.cos_out = cosv;
     p.counter = reinterpret_cast<unsigned*>(scratch);
+    p.err = reinterpret_cast<int*>(static_cast<unsigned char*>(scratch) + kGemvErrOffset);
     p.partials = reinterpret_cast<float*>(static_cast<unsigned char*>(scratch) + 256);
     int ctas;
     if (!gemv_accepts(*dv, M, n_rows, n_in, gain != nullptr, &ctas)) return ASD_ERR_ARG;
-    const size_t smem = plan_gemv(*dv, M, n_rows, n_in, &p);
-    if (launch_gemv(M, epilogue, gain != nullptr, p, dv->num_sms, smem, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
+    if (launch_gemv(p, epilogue, gain != nullptr, dv->max_smem, dv->num_sms, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return ASD_ERR_CUDA;
     return ASD_OK;
 }
@@ -1740,16 +1697,15 @@ extern "C" int asd_fused_gemv_static(void* cuda_stream, int32_t M, int32_t n_in,
     if (epilogue == ASD_EPI_RESIDUAL && cudaMemsetAsync(scratch, 0, 256, s) != cudaSuccess) return ASD_ERR_CUDA;
     GemvParams p{};
     p.W = reinterpret_cast<const __nv_bfloat16*>(W);
-    p.n_rows = n_rows;
-    p.n_in = n_in;
+    p.M = M, p.n_rows = n_rows, p.n_in = n_in;
     p.x = x;
     p.gain = reinterpret_cast<const __nv_bfloat16*>(gain);
     p.eps = eps;
     p.out = out;
     p.cos_out = cosv;
     p.counter = reinterpret_cast<unsigned*>(scratch);
+    p.err = reinterpret_cast<int*>(scratch + kGemvErrOffset);
     p.partials = reinterpret_cast<float*>(scratch + 256);
-    const size_t smem = plan_gemv(*dv, M, n_rows, n_in, &p);
-    if (launch_gemv(M, epilogue, gain != nullptr, p, dv->num_sms, smem, s) != cudaSuccess) return ASD_ERR_CUDA;
+    if (launch_gemv(p, epilogue, gain != nullptr, dv->max_smem, dv->num_sms, s) != cudaSuccess) return ASD_ERR_CUDA;
     return ASD_OK;
 }

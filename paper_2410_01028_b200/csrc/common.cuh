@@ -8,35 +8,12 @@ namespace asd {
 
 constexpr int kMaxRows = 9;        // rows of the stand-alone fused GEMV: max draft length 8, plus the last accepted token
 constexpr int kPassMaxRows = 16;   // rows of one pass of the persistent kernel (prefill feeds the prompt 16 rows at a time)
-constexpr int kGemvThreads = 512;  // 16 warps per CTA, one CTA per SM
-constexpr int kGemvWarps = kGemvThreads / 32;
 constexpr int kAttnChunk = 128;    // keys per attention work item; chunks are aligned to absolute positions
-
-enum Epilogue : int { kEpiPlain = 0, kEpiSwiglu = 1, kEpiResidual = 2 };
-
-// Parameter block of the fused RMSNorm -> GEMV -> epilogue kernel.
-struct GemvParams {
-    const __nv_bfloat16* W;  // [n_rows, n_in]
-    int n_rows, n_in;
-    const void* x;              // gain ? float [M, n_in] : bf16 [M, n_in]
-    const __nv_bfloat16* gain;  // [n_in] or null
-    float eps;
-    int win_segs;   // segments of the inputs whose activations are in shared memory at a time
-    int n_blk;              // blocks of rows of a CTA
-    int max_sub, max_rows;  // most sub-items and weight rows of a block
-    int split;  // sub-items per group of 16 weight rows
-    // plain / swiglu / residual
-    void* out;
-    float* cos_out;   // residual: [M]
-    float* partials;  // [gridDim.x][kMaxRows][4] cross-CTA partial results
-    unsigned* counter;  // zero before launch; reset by the last CTA
-};
 
 struct PassParams;
 
 // launchers, one translation unit per row count (inst.cu compiled with -DASD_M=1..9)
 #define ASD_DECLARE_LAUNCHERS(M)                                                                                 \
-    cudaError_t launch_gemv_m##M(int epi, bool norm, const GemvParams& p, int grid, size_t smem, cudaStream_t s); \
     cudaError_t launch_pass_m##M(const PassParams& p, int grid, size_t smem, cudaStream_t s);                    \
     cudaError_t configure_m##M(int max_smem);
 ASD_DECLARE_LAUNCHERS(1)

@@ -70,3 +70,20 @@ def test_rows_of_partial_groups_equal_those_of_nine_rows(M, n_in, n_rows):
     full, _ = _run(9, n_in, n_rows, 0, True, x, W, gain, None)  # compared with the oracle above
     part, _ = _run(M, n_in, n_rows, 0, True, x, W, gain, None)
     assert np.array_equal(part, full[:M])
+
+
+# the stream's own edges: pieces of 1024 and (from 4096 inputs, where three fit the ring) 2048 inputs, sums kept in registers over
+# 4096, one to four units of 32 inputs per warp, rows of one to three groups of 16, and activations in windows of multiples of 4096
+# inputs (nine rows of 13768). Bounds: sums of at most 13768 products in fp32 (1e-5 of the output scale, as above); rows equal
+# whatever the pieces and windows.
+@pytest.mark.parametrize("n_in", [512, 520, 1024, 1032, 4096, 4104, 8192, 13768])
+@pytest.mark.parametrize("n_rows", [148, 2 * 148 * 16 + 6])
+def test_pieces_epochs_and_windows(n_in, n_rows):
+    x = synth.make_array_f32((9, n_in), seed=n_in, stream=1)
+    W = synth.make_matrix_bf16((n_rows, n_in), seed=n_rows, stream=2, std=0.05)
+    full, _ = _run(9, n_in, n_rows, 0, False, x, W, None, None)
+    ref, _ = oracle.fused_matvec(x, W, epilogue=0, gain=None, res=None)
+    assert np.all(np.abs(full - ref) <= 1e-5 * np.abs(ref).max())
+    for M in (1, 4, 5):
+        part, _ = _run(M, n_in, n_rows, 0, False, x, W, None, None)
+        assert np.array_equal(part, full[:M]), M
