@@ -20,7 +20,9 @@
 // scoreboards with the products. Launch after launch over matrices that L2 does not hold,
 // us before -> now: 1 row 2048 -> 6144 9.6 -> 7.7, 4096 -> 22016 SwiGLU 36.8 -> 31.7 (5.7 TB/s), 8192 -> 24576 69.3 -> 63.7 (6.3 TB/s);
 // 5 rows 1024 -> 12000 11.6 -> 9.1, 13760 -> 5120 residual 36.2 -> 32.7; 9 rows 2056 -> 6145 16.0 -> 12.9, 11008 -> 4096 residual 32.6 -> 26.6,
-// 13760 -> 5120 44.8 -> 38.5, 4096 -> 22016 44.8 -> 43.2; 26 shapes of one to nine rows: none slower.
+// 13760 -> 5120 44.8 -> 38.5, 4096 -> 22016 44.8 -> 43.2; 26 shapes of one to nine rows: none slower. Behind an RMSNorm, 32 shapes of one and
+// five rows: 1.01 to 1.5 times as fast but for five rows of more than 11000 inputs (11008 -> 4096 30.2 -> 31.4, 13760 -> 5120 44.2 -> 44.7, 22016 ->
+// 8192 79.7 -> 90.2), whose norm reads the rows twice with eight warps where it had sixteen.
 #include <math.h>
 
 #include <algorithm>
@@ -97,10 +99,11 @@ __device__ __forceinline__ void gemv_walk(const GemvParams& p, int row0, int row
 
 // RMSNorm of the activation rows into the window of inputs w0 .. w1, by the multiplying warps: R rows of up to U x 1024 inputs at a
 // time are read once, all loads in flight together, and normalised from registers; what lies behind, and every window after
-// the first, is read again from L2. Thread t adds the squares of inputs 4 t + 1024 u whatever R and U.
-template <int R, int U>
+// the first, is read twice, 8 to 16 loads of a thread at a time. Thread t adds the squares of inputs
+// 4 t + 1024 u in this order whatever R and U.
+template <int R, int U, bool kTail>
 __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs, float* red, bool first, int w0, int w1) {
-    constexpr int kThreads = kGemvWarps * 32, kStep = kThreads * 4;
+    constexpr int kThreads = kGemvWarps * 32, kStep = kThreads * 4, kBatch = R == 1 ? 8 : 16 / R, kHeld = U > 0 ? U : 1;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, n_in = p.n_in;
     const float* xf = reinterpret_cast<const float*>(p.x);
     auto load = [&](int m, int i) { return *reinterpret_cast<const float4*>(xf + (size_t)m * n_in + i); };
@@ -119,15 +122,38 @@ __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs
     };
     auto gain = [&](int i) { return *reinterpret_cast<const uint2*>(p.gain + i); };
     static_assert(kGemvWarps == 8, "sums of squares of eight warps");
+    auto load_batch = [&](float4 (&a)[kBatch][R], int m0, int i, int end) {
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                a[b][r] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (m0 + r < p.M && i + kStep * b < end) a[b][r] = load(m0 + r, i + kStep * b);
+            }
+    };
+    auto fill = [&](int m0, int i, const float (&inv)[R]) {  // inputs i, i + 1024, ... of these rows
+        for (; i < w1; i += kStep * kBatch) {
+            float4 a[kBatch][R];
+            load_batch(a, m0, i, w1);
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b)
+                if (i + kStep * b < w1) {
+                    const uint2 gn = gain(i + kStep * b);
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        if (m0 + r < p.M) put(m0 + r, i + kStep * b, a[b][r], inv[r], gn);
+                }
+        }
+    };
     if (first) {  // (w0 == 0)
-        uint2 g[U];
+        uint2 g[kHeld];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             g[u] = make_uint2(0u, 0u);
             if (4 * t + kStep * u < n_in) g[u] = gain(4 * t + kStep * u);
         }
         for (int m0 = 0; m0 < p.M; m0 += R) {
-            float4 v[R][U];
+            float4 v[R][kHeld];
 #pragma unroll
             for (int r = 0; r < R; ++r)
 #pragma unroll
@@ -135,19 +161,28 @@ __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs
                     v[r][u] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (m0 + r < p.M && 4 * t + kStep * u < n_in) v[r][u] = load(m0 + r, 4 * t + kStep * u);
                 }
-            float s[R];
+            float4 ss[R];
+            auto add = [&](float4& t4, const float4& a) {
+                t4.x = fmaf(a.x, a.x, t4.x), t4.y = fmaf(a.y, a.y, t4.y), t4.z = fmaf(a.z, a.z, t4.z), t4.w = fmaf(a.w, a.w, t4.w);
+            };
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                float4 ss = make_float4(0.f, 0.f, 0.f, 0.f);
-                auto add = [&](const float4& a) {
-                    ss.x = fmaf(a.x, a.x, ss.x), ss.y = fmaf(a.y, a.y, ss.y), ss.z = fmaf(a.z, a.z, ss.z), ss.w = fmaf(a.w, a.w, ss.w);
-                };
+                ss[r] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int u = 0; u < U; ++u) add(v[r][u]);
-                if (n_in > kStep * U && m0 + r < p.M)
-                    for (int i = 4 * t + kStep * U; i < n_in; i += kStep) add(load(m0 + r, i));
-                s[r] = (ss.x + ss.y) + (ss.z + ss.w);
+                for (int u = 0; u < U; ++u) add(ss[r], v[r][u]);
             }
+            if constexpr (kTail)
+                for (int i = 4 * t + kStep * U; i < n_in; i += kStep * kBatch) {
+                    float4 a[kBatch][R];
+                    load_batch(a, m0, i, n_in);
+#pragma unroll
+                    for (int b = 0; b < kBatch; ++b)
+#pragma unroll
+                        for (int r = 0; r < R; ++r) add(ss[r], a[b][r]);
+                }
+            float s[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) s[r] = (ss[r].x + ss[r].y) + (ss[r].z + ss[r].w);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -157,23 +192,24 @@ __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs
                 if (lane == 0 && m0 + r < p.M) red[(m0 + r) * kGemvWarps + warp] = s[r];
             bar_sync(1, kThreads);
             const float inv_lane = inverse(min(m0 + min(lane, R - 1), p.M - 1));  // a row per lane: one chain of square root and division
+            float inv[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const float inv = __shfl_sync(0xffffffffu, inv_lane, r);
+                inv[r] = __shfl_sync(0xffffffffu, inv_lane, r);
                 if (m0 + r < p.M) {
 #pragma unroll
                     for (int u = 0; u < U; ++u)
-                        if (4 * t + kStep * u < w1) put(m0 + r, 4 * t + kStep * u, v[r][u], inv, g[u]);
-                    if (w1 > kStep * U)
-                        for (int i = 4 * t + kStep * U; i < w1; i += kStep) put(m0 + r, i, load(m0 + r, i), inv, gain(i));
+                        if (4 * t + kStep * u < w1) put(m0 + r, 4 * t + kStep * u, v[r][u], inv[r], g[u]);
                 }
             }
+            if constexpr (kTail) fill(m0, 4 * t + kStep * U, inv);
         }
     } else {
-        for (int m = 0; m < p.M; ++m) {
-            const float inv = inverse(m);
-#pragma unroll 4
-            for (int i = w0 + 4 * t; i < w1; i += kStep) put(m, i, load(m, i), inv, gain(i));
+        for (int m0 = 0; m0 < p.M; m0 += R) {
+            float inv[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) inv[r] = inverse(min(m0 + r, p.M - 1));
+            fill(m0, w0 + 4 * t, inv);
         }
     }
 }
@@ -228,11 +264,14 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                     return;
                 }
                 if (!first) bar_sync(1, kGemvWarps * 32);  // the window before has been read
-                if (M == 1) norm_rows<1, 8>(p, xs, red, first, w0, w1);
-                else if (M == 2) norm_rows<2, 5>(p, xs, red, first, w0, w1);
-                else if (n_in <= 3072) norm_rows<5, 3>(p, xs, red, first, w0, w1);
-                else if (n_in <= 4096) norm_rows<5, 4>(p, xs, red, first, w0, w1);
-                else norm_rows<3, 5>(p, xs, red, first, w0, w1);
+                // Without a loop over what lies behind, the kernels of up to 5120 inputs run faster as well (one row of 4096 -> 11008 SwiGLU 17.8 ->
+                // 16.2 us, nine of 2056 -> 6145 12.3 -> 11.7); five rows of 22016 -> 8192 with one load at a time 102 us, in batches 90.
+                if (M == 1) norm_rows<1, 8, true>(p, xs, red, first, w0, w1);
+                else if (n_in > 5120) norm_rows<5, 0, true>(p, xs, red, first, w0, w1);  // rows too long to hold in registers
+                else if (M == 2) norm_rows<2, 5, false>(p, xs, red, first, w0, w1);
+                else if (n_in <= 3072) norm_rows<5, 3, false>(p, xs, red, first, w0, w1);
+                else if (n_in <= 4096) norm_rows<5, 4, false>(p, xs, red, first, w0, w1);
+                else norm_rows<3, 5, false>(p, xs, red, first, w0, w1);
                 bar_sync(1, kGemvWarps * 32);
             },
             [&](int, int rows, int k0, int len, int w0) {
@@ -452,7 +491,9 @@ static size_t plan_gemv(int max_smem, int sms, GemvParams* p) {
     p->xs_ld = (p->win + 63) / 64 * 64 + 32;
     p->off_ring = (int)((p->off_xs + window_bytes(p->win) + 127) / 128 * 128);
     // The longer the pieces, the better the stream (copies of 1, 2 and 4 KB: 3.2, 5.4 and 6.2 TB/s), the shorter, the sooner it starts and
-    // the less of it is left at the end: 4 KB from 4096 inputs on, where the ring then holds three.
+    // the less of it is left at the end: 4 KB from 4096 inputs on, where the ring then holds three (two from 8192 on). us with 2 KB -> 4 KB: one row
+    // of 4096 -> 22016 33.8 -> 31.5, five of 13760 -> 5120 36.9 -> 36.1, one of 2048 -> 6144 10.0 -> 10.2, nine of 2056 -> 6145 12.3 -> 11.9 (the
+    // only one of these short rows that gains).
     for (p->seg = p->n_in >= 4096 ? 2048 : 1024;; p->seg = 1024) {
         p->pitch = (std::min(p->n_in, p->seg) + 63) / 64 * 128 + 64;
         p->stage_bytes = p->group_rows * p->pitch;
