@@ -70,13 +70,15 @@ __device__ __forceinline__ bool last_cta_arrives(unsigned* counter, int* flag_sm
 }
 
 // The order in which every role walks a CTA's rows: blocks of rows, windows of the activations, groups of at most 16 rows, epochs
-// of inputs, pieces. A role whose wait has run out walks on (every later wait returns at once), so that no barrier misses it.
+// of inputs, pieces. A warp whose wait has run out leaves (the calls return false, and so does the walk): it signals nothing any
+// more, so that whoever needs its signal leaves as well, and no ring stage, window or sums are filled again before they have
+// landed and been read.
 //   window(first_use, k0, k1)                     the activations k0 .. k1 are wanted
 //   piece(row, rows, k0, len, win0)               rows x inputs of one ring stage
 //   epoch(local_row, row, rows, k0, k1, win_end)  the sums of inputs k0 .. k1 of a group are complete; win_end: nothing else
 //                                                 reads the window
 template <class Window, class Piece, class Epoch>
-__device__ __forceinline__ void gemv_walk(const GemvParams& p, int row0, int row1, Window&& window, Piece&& piece, Epoch&& epoch) {
+__device__ __forceinline__ bool gemv_walk(const GemvParams& p, int row0, int row1, Window&& window, Piece&& piece, Epoch&& epoch) {
     for (int blk = 0; blk < p.n_blk; ++blk) {
         const int blk0 = row0 + (row1 - row0) * blk / p.n_blk / 2 * 2;
         const int rows = (blk + 1 == p.n_blk ? row1 : row0 + (row1 - row0) * (blk + 1) / p.n_blk / 2 * 2) - blk0;
@@ -84,17 +86,19 @@ __device__ __forceinline__ void gemv_walk(const GemvParams& p, int row0, int row
         if (rows <= 0) break;  // fewer pairs of rows than CTAs
         for (int w0 = 0; w0 < p.n_in; w0 += p.win) {
             const int w1 = min(p.n_in, w0 + p.win);
-            if (blk == 0 || p.win < p.n_in) window(blk + w0 == 0, w0, w1);
+            if ((blk == 0 || p.win < p.n_in) && !window(blk + w0 == 0, w0, w1)) return false;
             for (int o = 0; o < p.groups; ++o) {
                 const int r0 = 2 * (o * pairs / p.groups), n = min(rows, 2 * ((o + 1) * pairs / p.groups)) - r0;
                 for (int e0 = w0; e0 < w1; e0 += kGemvEpoch) {
                     const int e1 = min(w1, e0 + kGemvEpoch);
-                    for (int k0 = e0; k0 < e1; k0 += p.seg) piece(blk0 + r0, n, k0, min(p.seg, e1 - k0), w0);
-                    epoch(r0, blk0 + r0, n, e0, e1, o + 1 == p.groups && e1 == w1);
+                    for (int k0 = e0; k0 < e1; k0 += p.seg)
+                        if (!piece(blk0 + r0, n, k0, min(p.seg, e1 - k0), w0)) return false;
+                    if (!epoch(r0, blk0 + r0, n, e0, e1, o + 1 == p.groups && e1 == w1)) return false;
                 }
             }
         }
     }
+    return true;
 }
 
 // RMSNorm of the activation rows into the window of inputs w0 .. w1, by the multiplying warps: R rows of up to U x 1024 inputs at a
@@ -225,17 +229,23 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
     uint64_t* acc_empty = acc_full + 2;                      // [2] and have been read
     uint64_t* x_full = acc_empty + 2;                        // bf16 activations of a window landed
     int* flag = reinterpret_cast<int*>(x_full + 1);
+    volatile int* gone = flag + 1;                           // a warp of this CTA has left
     float* red = reinterpret_cast<float*>(flag + 6);         // [kMaxRows][kGemvWarps] sums of squares
     float* psum = reinterpret_cast<float*>(smem_raw + kGemvHead);  // [2][kGemvWarps][group_rows * M]
     float* tot = psum + 2 * kGemvWarps * p.group_rows * M;         // [max_rows][M], when a row has more than one epoch
     __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(smem_raw + p.off_xs);  // [M][xs_ld]
     unsigned char* ring = smem_raw + p.off_ring;
     volatile int* err = p.err;
+    auto wait = [&](uint64_t* bar, int phase, int role, int item, int slot, int tag) {
+        return mbar_wait_warp(bar, (uint32_t)(phase & 1), err, kErrGemvWait, role, item, slot, tag, gone);
+    };
+    bool ok = true;  // this warp has not left
 
     if (tid == 0) {
         for (int s = 0; s < p.n_stages; ++s) mbar_init(&full[s], 1), mbar_init(&empty[s], kGemvWarps);
         for (int b = 0; b < 2; ++b) mbar_init(&acc_full[b], kGemvWarps), mbar_init(&acc_empty[b], 2);
         mbar_init(x_full, 1);
+        *gone = 0;
         mbar_fence_init();
     }
     pdl_launch_dependents();
@@ -255,14 +265,11 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                 for (int e = 0; e < 4; ++e) acc[nb][e] = 0.f;
         };
         zero();
-        gemv_walk(
+        ok = gemv_walk(
             p, cta_row0, cta_row1,
             [&](bool first, int w0, int w1) {
-                if (!NORM) {
-                    ++n_x;
-                    mbar_wait_warp(x_full, (uint32_t)((n_x - 1) & 1), err, kErrGemvWait, 0, n_x, 0, 1);
-                    return;
-                }
+                ++n_x;
+                if (!NORM) return wait(x_full, n_x - 1, 0, n_x, 0, 1);
                 if (!first) bar_sync(1, kGemvWarps * 32);  // the window before has been read
                 // Without a loop over what lies behind, the kernels of up to 5120 inputs run faster as well (one row of 4096 -> 11008 SwiGLU 17.8 ->
                 // 16.2 us, nine of 2056 -> 6145 12.3 -> 11.7); five rows of 22016 -> 8192 with one load at a time 102 us, in batches 90.
@@ -273,9 +280,10 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                 else if (n_in <= 4096) norm_rows<5, 4, false>(p, xs, red, first, w0, w1);
                 else norm_rows<3, 5, false>(p, xs, red, first, w0, w1);
                 bar_sync(1, kGemvWarps * 32);
+                return true;
             },
             [&](int, int rows, int k0, int len, int w0) {
-                const bool landed = mbar_wait_warp(&full[s], (uint32_t)(lap & 1), err, kErrGemvWait, 0, k0, s, 2);
+                if (!wait(&full[s], lap, 0, k0, s, 2)) return false;
                 const unsigned char* st = ring + (size_t)s * p.stage_bytes + q * 16;
                 const unsigned char *wa = st + min(g, rows - 1) * p.pitch, *wb = st + min(g + 8, rows - 1) * p.pitch;
                 // Sums of 1024 inputs at a time, whatever the length of a piece; a warp's four units in pairs, each with sums of its own
@@ -312,11 +320,11 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty[s]);
                 if (++s == p.n_stages) s = 0, ++lap;
-                if (!landed) acc[0][0] = acc[0][1] = acc[0][2] = acc[0][3] = NAN;
+                return true;
             },
             [&](int, int, int rows, int, int, bool) {
                 const int b = n_epoch & 1;
-                if (n_epoch >= 2) mbar_wait_warp(&acc_empty[b], (uint32_t)((n_epoch / 2 - 1) & 1), err, kErrGemvWait, 0, n_epoch, b, 3);
+                if (n_epoch >= 2 && !wait(&acc_empty[b], n_epoch / 2 - 1, 0, n_epoch, b, 3)) return false;
                 ++n_epoch;
                 float* dst = psum + (size_t)(b * kGemvWarps + warp) * p.group_rows * M;
 #pragma unroll
@@ -329,22 +337,32 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                 zero();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_full[b]);
+                return true;
             });
+        if (!ok) {
+            *gone = 1;
+            if (NORM)  // the barriers of the windows to come
+                for (const int all = p.win < n_in ? p.n_blk * ((n_in + p.win - 1) / p.win) : 1; n_x < all; ++n_x)
+                    bar_sync(1, kGemvWarps * 32), bar_sync(1, kGemvWarps * 32);
+        }
     } else if (warp == kGemvWarps) {
         // ------------------------------------------------------------------------------------ weights -> ring
         int s = 0, lap = 0;
-        gemv_walk(
-            p, cta_row0, cta_row1, [&](bool, int, int) {},
+        ok = gemv_walk(
+            p, cta_row0, cta_row1, [&](bool, int, int) { return true; },
             [&](int row, int rows, int k0, int len, int) {
-                if (lap > 0) mbar_wait_warp(&empty[s], (uint32_t)((lap - 1) & 1), err, kErrGemvWait, 1, k0, s, 4);
+                if (lap > 0 && !wait(&empty[s], lap - 1, 1, k0, s, 4)) return false;
                 if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)(rows * len * 2));
                 __syncwarp();
                 if (lane < rows)
                     tma_load_1d(ring + (size_t)s * p.stage_bytes + lane * p.pitch, p.W + (size_t)(row + lane) * n_in + k0, (uint32_t)len * 2, &full[s]);
                 if (++s == p.n_stages) s = 0, ++lap;
+                return true;
             },
-            [&](int, int, int, int, int, bool) {});
-        // what is in flight lands before the CTA leaves, also when somebody has given up
+            [&](int, int, int, int, int, bool) { return true; });
+        if (!ok) *gone = 1;
+        // what is in flight lands before the CTA leaves, also when this warp leaves early: at most the last piece of every stage, for
+        // the ones before have been read
         for (int i = max(0, (lap - 1) * p.n_stages + s); i < lap * p.n_stages + s; ++i)
             mbar_drain(&full[i % p.n_stages], (uint32_t)((i / p.n_stages) & 1));
     } else {
@@ -362,8 +380,8 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
         };
         int blocks_left = p.n_blk;
         if (cta_row1 > cta_row0) request_x(0, min(n_in, p.win));
-        gemv_walk(
-            p, cta_row0, cta_row1, [&](bool, int, int) {}, [&](int, int, int, int, int) {},
+        ok = gemv_walk(
+            p, cta_row0, cta_row1, [&](bool, int, int) { return true; }, [&](int, int, int, int, int) { return true; },
             [&](int local, int row, int rows, int e0, int e1, bool win_end) {
                 const bool last = e1 == n_in;
                 float x0[3] = {0.f, 0.f, 0.f};
@@ -373,8 +391,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                         if (r < rows && m_first + 4 * i < M) x0[i] = out[(size_t)(m_first + 4 * i) * p.n_rows + row + r];
                 }
                 const int b = n_epoch & 1;
-                // sums that never came read as NaN
-                const float missing = mbar_wait_warp(&acc_full[b], (uint32_t)((n_epoch / 2) & 1), err, kErrGemvWait, 2, n_epoch, b, 5) ? 0.f : NAN;
+                if (!wait(&acc_full[b], n_epoch / 2, 2, n_epoch, b, 5)) return false;
                 ++n_epoch;
                 // every multiplying warp has read the window
                 if (win_end && p.win < n_in) {
@@ -395,7 +412,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                         for (int st = 1; st < kGemvWarps; st *= 2)
 #pragma unroll
                             for (int j = 0; j < kGemvWarps; j += 2 * st) w[j] += w[j + st];
-                        v[i] = w[0] + missing;
+                        v[i] = w[0];
                         if (e0 > 0) v[i] = tot[(local + r) * M + m] + v[i];
                         if (!last) tot[(local + r) * M + m] = v[i];
                     }
@@ -423,7 +440,18 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                         }
                     }
                 }
+                return true;
             });
+        if (!ok) {  // what is missing reads as NaN, and so does whatever else the CTA has written
+            *gone = 1;
+            for (int i = lane; i < (cta_row1 - cta_row0) * M; i += 32) {
+                const int m = i / (cta_row1 - cta_row0), at = cta_row0 + i - m * (cta_row1 - cta_row0);
+                if (EPI != kEpiSwiglu) out[(size_t)m * p.n_rows + at] = NAN;
+                else if (at % 2 == 0) reinterpret_cast<__nv_bfloat16*>(p.out)[(size_t)m * (p.n_rows >> 1) + (at >> 1)] = __float2bfloat16_rn(NAN);
+            }
+#pragma unroll
+            for (int i = 0; i < 3; ++i) s_loc[i][0] = s_loc[i][1] = s_loc[i][2] = NAN;
+        }
         if (n_x > 0) mbar_drain(x_full, (uint32_t)((n_x - 1) & 1));
         if (EPI == kEpiResidual) {
 #pragma unroll

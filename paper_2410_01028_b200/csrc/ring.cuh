@@ -44,16 +44,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Wait for a phase of an mbarrier. Returns false when the wait was abandoned (error word set).
+// Wait for a phase of an mbarrier. Returns false when the wait was abandoned (error word set, or the word `gone` of the CTA's own).
 // The first wait to give up also records where it was: err[1..7] = stage, ring item, slot, CTA, thread, tag, parity.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* err, int code, int stage = -1,
-                                          unsigned item = 0, int slot = -1, int tag = 0, long long budget = kWaitCycles) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* err, int code, int stage = -1, unsigned item = 0,
+                                          int slot = -1, int tag = 0, long long budget = kWaitCycles, volatile int* gone = nullptr) {
     if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     for (unsigned spin = 1;; ++spin) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((spin & 255u) != 0) continue;  // the error word lives in global memory: look at it only now and then
-        if (*err != kErrNone) return false;
+        if (*err != kErrNone || (gone && *gone)) return false;
         if (clock64() - t0 > budget) {
             if (atomicCAS(const_cast<int*>(err), kErrNone, code) == kErrNone) {
                 err[1] = stage, err[2] = (int)item, err[3] = slot, err[4] = blockIdx.x, err[5] = threadIdx.x, err[6] = tag;
@@ -66,9 +66,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 
 // The same for a whole converged warp; the result is the same in every lane.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* err, int code, int stage = -1,
-                                               unsigned item = 0, int slot = -1, int tag = 0) {
+                                               unsigned item = 0, int slot = -1, int tag = 0, volatile int* gone = nullptr) {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code, stage, item, slot, tag));
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code, stage, item, slot, tag, kWaitCycles, gone));
 }
 
 // Waits for copies or MMAs in flight before their shared or tensor memory is given back. They end by themselves whatever the

@@ -1,0 +1,73 @@
+"""A stand-alone fused product whose waits run out: its error word is set from the host, before the call or in mid-run, so
+that every wait that lasts some tens of microseconds gives up. The RMSNorm makes such waits, because its rows are read from
+pinned host memory over a busy bus. Every output is either right to the bit or NaN, in the last of nine rows as well, nothing is
+left in flight, and the next call (on a cleared word) is right."""
+import time
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ERR_WORD = 32  # of the scratch
+
+
+@pytest.mark.parametrize("M,n_in,n_rows,epi", [(9, 12000, 6001, 0),   # row 8 in the second block of columns; several windows
+                                               (5, 21000, 3000, 1), (3, 34000, 2000, 2)])
+def test_abandoned_calls_leave_right_outputs_or_nan(M, n_in, n_rows, epi):
+    import torch
+    import paper_2410_01028_b200 as asd
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(7)
+    x = torch.randn((M, n_in), generator=gen, device=dev).cpu().pin_memory()
+    W = torch.randn((n_rows, n_in), generator=gen, device=dev).mul_(0.02).to(torch.bfloat16)
+    gain = torch.ones(n_in, dtype=torch.bfloat16, device=dev)
+    hidden = torch.randn((M, n_rows), generator=gen, device=dev)
+    scratch = torch.zeros(asd.fused_gemv_scratch_bytes(), dtype=torch.uint8, device=dev)
+    words = scratch.view(torch.int32)
+
+    def outputs():
+        out = torch.zeros((M, n_rows // 2), dtype=torch.bfloat16, device=dev) if epi == 1 else hidden.clone()
+        return out, torch.zeros(M, device=dev)
+
+    def call(out, cos):
+        asd.fused_gemv(x, W, epi, out, gain=gain, cos=cos if epi == 2 else None, scratch=scratch)
+
+    want = outputs()
+    call(*want)
+    torch.cuda.synchronize()
+    assert not any(bool(torch.isnan(w).any()) for w in want) and not bool(words[:64].any())
+    word = torch.full((1,), 77, dtype=torch.int32).pin_memory()
+    side, bus = torch.cuda.Stream(), torch.cuda.Stream()
+    ballast = torch.zeros(64 << 20, dtype=torch.uint8).pin_memory()
+    ballast_dev = torch.empty(64 << 20, dtype=torch.uint8, device=dev)
+    seen = 0
+    for attempt in range(24):
+        before = attempt % 2 == 0
+        got, after = outputs(), outputs()
+        if before:
+            words[ERR_WORD] = 77
+        torch.cuda.synchronize()
+        with torch.cuda.stream(bus):
+            ballast_dev.copy_(ballast, non_blocking=True)  # more than a millisecond
+        call(*got)
+        if not before:
+            until = time.perf_counter() + 1e-6 * (10 + 20 * (attempt % 12))
+            while time.perf_counter() < until:
+                pass
+            with torch.cuda.stream(side):
+                words[ERR_WORD:ERR_WORD + 1].copy_(word, non_blocking=True)
+        torch.cuda.synchronize()
+        cut = any(bool(torch.isnan(g).any()) for g in got)
+        for g, w in zip(got, want):
+            left = torch.isnan(g)
+            assert torch.equal(g[~left], w[~left])
+        if before and cut:  # whoever gave up has cleared the word behind it
+            assert int(words[ERR_WORD]) == 0
+        else:
+            words[ERR_WORD] = 0
+        assert not bool(words[:ERR_WORD].any()) and not bool(words[ERR_WORD + 8:64].any())
+        call(*after)
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, w) for a, w in zip(after, want))
+        seen += cut
+    assert seen > 0
