@@ -274,8 +274,9 @@ int asd_gemm_bf16(void* cuda_stream, int32_t M, int32_t N, int32_t K, const uint
  *              ASD_EPI_RESIDUAL out = float [M, n_rows], updated IN PLACE: out += a (the residual add), and
  *                               cos[m] = cosine(out before, out after)  -- the summand of C_l, Section 3.2
  *   scratch  : >= asd_fused_gemv_scratch_bytes() bytes, 256-byte aligned; its first 256 bytes must be zero
- *              before the first use and are left zero by every call (unless a wait inside the kernel has run out,
- *              about two seconds: words 32 to 39 then say where, and outputs read NaN).
+ *              before the first use and are left zero by every call, but for words 33 to 39: they say where a wait
+ *              inside the kernel has run out (about two seconds), if one has. Every output is then either right
+ *              or NaN, and the next call starts anew: nothing has to be cleared.
  *   limit    : a shape counts as the work of c CTAs, c the least multiple of the SM count for which
  *              2 * M * ceil(ceil(n_rows / 2) / c) * ceil(n_in / 1024) floats (and with a gain M * n_in bf16
  *              values) fit a block's shared memory; shapes without such a c of at most 1024 are refused (ARG)

@@ -1692,8 +1692,8 @@ extern "C" int asd_fused_gemv_static(void* cuda_stream, int32_t M, int32_t n_in,
         return ASD_ERR_NOMEM;
     }
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    // the array keeps whatever the previous call left: the arrival counter, which only the residual epilogue
-    // uses, must start at zero
+    // the arrival counter, which only the residual epilogue uses, must start at zero (the error word, which every epilogue's
+    // waits look at, is left zero by every call)
     if (epilogue == ASD_EPI_RESIDUAL && cudaMemsetAsync(scratch, 0, 256, s) != cudaSuccess) return ASD_ERR_CUDA;
     GemvParams p{};
     p.W = reinterpret_cast<const __nv_bfloat16*>(W);

@@ -465,6 +465,11 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                 }
         }
     }
+    // whoever has set the error word comes here afterwards: no call leaves it set
+    if (!ok) {
+        __syncwarp();
+        if (lane == 0) *err = kErrNone;
+    }
 
     if (EPI == kEpiResidual) {
         if (last_cta_arrives(p.counter, flag)) {

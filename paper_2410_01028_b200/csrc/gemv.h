@@ -18,7 +18,7 @@ struct GemvParams {
     float* cos_out;     // residual: [M]
     float* partials;    // [gridDim.x][kMaxRows][4] cross-CTA partial results
     unsigned* counter;  // zero before launch; reset by the last CTA
-    int* err;           // 8 words: where a bounded wait has run out
+    int* err;           // 8 words: the first is set while warps whose bounded wait has run out leave, the others say where
     // the plan, filled in by launch_gemv
     int n_blk;               // blocks of rows of a CTA
     int groups, group_rows;  // groups of rows per block, and the most rows of one

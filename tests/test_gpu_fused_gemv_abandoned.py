@@ -1,7 +1,7 @@
 """A stand-alone fused product whose waits run out: its error word is set from the host, before the call or in mid-run, so
 that every wait that lasts some tens of microseconds gives up. The RMSNorm makes such waits, because its rows are read from
 pinned host memory over a busy bus. Every output is either right to the bit or NaN, in the last of nine rows as well, nothing is
-left in flight, and the next call (on a cleared word) is right."""
+left in flight or in the scratch, and the next call is right."""
 import time
 
 import pytest
