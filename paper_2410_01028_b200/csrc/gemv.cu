@@ -218,6 +218,82 @@ __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs
     }
 }
 
+// The same for R rows too long to hold in registers, from row m0 on: read twice, 12 loads of a thread in flight (8 and 20: up to 5 % and 7 %
+// slower). Eight warps are two for each scheduler, so what counts is the number of instructions: packed arithmetic, groups of exactly
+// R rows, no bounds in whole batches. (Five rows of 11008 inputs took 10 us in the loops above; L2 gives them twice in 4.5.) Same sums as above.
+template <int R>
+__device__ __forceinline__ void norm_long(const GemvParams& p, __nv_bfloat16* xs, float* red, int m0, bool first, int w0, int w1) {
+    constexpr int kThreads = kGemvWarps * 32, kStep = kThreads * 4, kBatch = 12 / R;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, n_in = p.n_in;
+    const float* x = reinterpret_cast<const float*>(p.x) + (size_t)m0 * n_in + 4 * t;
+    auto load = [&](ulonglong2 (&a)[kBatch][R], int i, int end, bool whole) {
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                a[b][r] = make_ulonglong2(0ull, 0ull);
+                if (whole || i + kStep * b + 4 * t < end) a[b][r] = *reinterpret_cast<const ulonglong2*>(x + (size_t)r * n_in + i + kStep * b);
+            }
+    };
+    auto inverse = [&](int m) {
+        const float* q = red + m * kGemvWarps;
+        return 1.0f / sqrtf((((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]))) / (float)n_in + p.eps);
+    };
+    if (first) {
+        unsigned long long ss[R][2] = {};
+        auto add = [&](int i, bool whole) {
+            ulonglong2 a[kBatch][R];
+            load(a, i, n_in, whole);
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b)
+#pragma unroll
+                for (int r = 0; r < R; ++r) ss[r][0] = ffma2(a[b][r].x, a[b][r].x, ss[r][0]), ss[r][1] = ffma2(a[b][r].y, a[b][r].y, ss[r][1]);
+        };
+        int i = 0;
+        for (; i + kStep * kBatch <= n_in; i += kStep * kBatch) add(i, true);
+        if (i < n_in) add(i, false);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            float a, b, c, d;
+            unpack2(ss[r][0], a, b);
+            unpack2(ss[r][1], c, d);
+            const float s = warp_sum((a + b) + (c + d));
+            if (lane == 0) red[(m0 + r) * kGemvWarps + warp] = s;
+        }
+        bar_sync(1, kThreads);
+    }
+    const float inv_lane = inverse(m0 + min(lane, R - 1));  // a row per lane: one chain of square root and division
+    unsigned long long inv[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float v = __shfl_sync(0xffffffffu, inv_lane, r);
+        inv[r] = pack2(v, v);
+    }
+    __nv_bfloat16* to = xs + (size_t)m0 * p.xs_ld + 4 * t - w0;
+    auto fill = [&](int i, bool whole) {
+        ulonglong2 a[kBatch][R];
+        load(a, i, w1, whole);
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            if (!whole && i + kStep * b + 4 * t >= w1) continue;
+            const uint2 g = *reinterpret_cast<const uint2*>(p.gain + 4 * t + i + kStep * b);
+            const unsigned long long g0 = bf2_to_f2(g.x), g1 = bf2_to_f2(g.y);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float lo0, hi0, lo1, hi1;
+                unpack2(fmul2(fmul2(a[b][r].x, inv[r]), g0), lo0, hi0);
+                unpack2(fmul2(fmul2(a[b][r].y, inv[r]), g1), lo1, hi1);
+                const __nv_bfloat162 y0 = __floats2bfloat162_rn(lo0, hi0), y1 = __floats2bfloat162_rn(lo1, hi1);
+                *reinterpret_cast<uint2*>(to + (size_t)r * p.xs_ld + i + kStep * b) =
+                    make_uint2(*reinterpret_cast<const uint32_t*>(&y0), *reinterpret_cast<const uint32_t*>(&y1));
+            }
+        }
+    };
+    int i = w0;
+    for (; i + kStep * kBatch <= w1; i += kStep * kBatch) fill(i, true);
+    if (i < w1) fill(i, false);
+}
+
 template <int NB, int EPI, bool NORM>
 __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_constant__ GemvParams p) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -274,7 +350,19 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                 // Without a loop over what lies behind, the kernels of up to 5120 inputs run faster as well (one row of 4096 -> 11008 SwiGLU 17.8 ->
                 // 16.2 us, nine of 2056 -> 6145 12.3 -> 11.7); five rows of 22016 -> 8192 with one load at a time 102 us, in batches 90.
                 if (M == 1) norm_rows<1, 8, true>(p, xs, red, first, w0, w1);
-                else if (n_in > 5120) norm_rows<5, 0, true>(p, xs, red, first, w0, w1);  // rows too long to hold in registers
+                else if (n_in > 5120) {  // rows too long to hold in registers, in even shares of at most five
+                    if (M == 2) norm_long<2>(p, xs, red, 0, first, w0, w1);
+                    else if (M == 3 || M == 6) {
+                        norm_long<3>(p, xs, red, 0, first, w0, w1);
+                        if (M == 6) norm_long<3>(p, xs, red, 3, first, w0, w1);
+                    } else if (M == 5) norm_long<5>(p, xs, red, 0, first, w0, w1);
+                    else {
+                        norm_long<4>(p, xs, red, 0, first, w0, w1);
+                        if (M == 7) norm_long<3>(p, xs, red, 4, first, w0, w1);
+                        if (M == 8) norm_long<4>(p, xs, red, 4, first, w0, w1);
+                        if (M == 9) norm_long<5>(p, xs, red, 4, first, w0, w1);
+                    }
+                }
                 else if (M == 2) norm_rows<2, 5, false>(p, xs, red, first, w0, w1);
                 else if (n_in <= 3072) norm_rows<5, 3, false>(p, xs, red, first, w0, w1);
                 else if (n_in <= 4096) norm_rows<5, 4, false>(p, xs, red, first, w0, w1);

@@ -133,6 +133,11 @@ __device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsign
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ unsigned long long fmul2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 // exact g / d for 0 <= g < 2^22 and 1 <= d <= 64, with magic = 2^32 / d + 1 (computed on the host)
 __device__ __forceinline__ uint32_t fast_div(uint32_t g, uint32_t magic) { return __umulhi(g, magic); }
 

@@ -1,0 +1,42 @@
+"""GPU parity of the stand-alone fused product where its variants meet: RMSNorm of rows that are held in registers or read twice, in
+groups of one to five; groups of short weight rows by a warp each; the last piece of a row; blocks of weight rows together with windows
+of activations; and activations that are not finite. Every row of a call equals the same row of a call with nine rows."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from test_gpu_fused_gemv_plans import _run
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(n_in, n_rows, epi, norm, rows, tol):
+    x = synth.make_array_f32((9, n_in), seed=n_in, stream=1)
+    W = synth.make_matrix_bf16((n_rows, n_in), seed=n_rows, stream=2, std=0.05)
+    gain = synth.make_matrix_bf16((n_in,), seed=3, stream=3, mean=1.0)
+    res = synth.make_array_f32((9, n_rows), seed=4, stream=4)
+    most = max(rows)
+    pairs = dict(W2=np.ascontiguousarray(W[1::2])) if epi == 1 else {}
+    ref, ref_cos = oracle.fused_matvec(x[:most], np.ascontiguousarray(W[0::2]) if epi == 1 else W, epilogue=epi,
+                                       gain=gain if norm else None, res=res[:most] if epi == 2 else None, **pairs)
+    full, full_cos = _run(most, n_in, n_rows, epi, norm, x, W, gain, res)
+    scale = np.abs(ref).max()
+    assert np.all(np.abs(full - ref) <= (2 ** -7 * np.abs(ref) if epi == 1 else 0) + tol * scale)
+    if epi == 2:
+        assert np.abs(full_cos - ref_cos).max() <= 1e-5 + (1e-3 if norm else 0)
+    for M in rows:
+        part, part_cos = _run(M, n_in, n_rows, epi, norm, x, W, gain, res)
+        assert np.array_equal(part, full[:M]), M
+        if epi == 2:
+            assert np.array_equal(part_cos, full_cos[:M]), M
+
+
+# Bound behind an RMSNorm: a flipped bf16 rounding of a normalised input moves one product by 2^-8 of itself, a few of thousands
+# flip (2e-3 of the output scale, as in the tests of the launch plans). Up to 5120 inputs rows are held in registers; beyond, they are read
+# in batches of 1024 x (12 / rows of a group) inputs; 12296 and 34000 inputs have activations in several windows.
+@pytest.mark.parametrize("n_in,rows", [(3080, (1, 2, 3, 5, 9)), (4096, (1, 2, 3, 5, 9)), (4104, (1, 2, 3, 5, 9)), (5120, (1, 2, 3, 5, 9)),
+                                       (5128, tuple(range(1, 10))), (6144, tuple(range(1, 10))), (9224, tuple(range(1, 10))),
+                                       (12296, tuple(range(1, 9))), (22016, (1, 2, 3, 4)), (34000, (1, 2, 3))])
+def test_norm_of_long_rows(n_in, rows):
+    _check(n_in, 297, 0, True, rows, 2e-3)
