@@ -20,9 +20,13 @@ struct GemvParams {
     unsigned* counter;  // zero before launch; reset by the last CTA
     int* err;           // 8 words: the first is set while warps whose bounded wait has run out leave, the others say where
     // the plan, filled in by launch_gemv
+    int cta_pairs, cta_more;          // pairs of rows: pairs / CTAs and the remainder
+    unsigned div_grid, div_groups;    // for divisions by the numbers of CTAs and of groups
     int n_blk;               // blocks of rows of a CTA
     int groups, group_rows;  // groups of rows per block, and the most rows of one
-    int seg;                 // inputs of a piece
+    int seg, tail;           // inputs of a piece, and how many more the last one of a row may have
+    int whole;               // a piece is whole rows, copied as one
+    int by_warp;             // a group of rows is one warp's alone
     int win;                 // inputs whose activations are in shared memory at a time
     int xs_ld;               // bf16 per activation row there
     int pitch, stage_bytes, n_stages, off_xs, off_ring;  // the ring of weight pieces

@@ -40,3 +40,18 @@ def _check(n_in, n_rows, epi, norm, rows, tol):
                                        (12296, tuple(range(1, 9))), (22016, (1, 2, 3, 4)), (34000, (1, 2, 3))])
 def test_norm_of_long_rows(n_in, rows):
     _check(n_in, 297, 0, True, rows, 2e-3)
+
+
+# Groups of 16 rows by a warp each: up to 768 inputs and from 50 weight rows per SM on (7104 weight rows: 48 per SM), one to three
+# units of 256 inputs, a ring of 8 and of 16 stages, one lap of it and several
+@pytest.mark.parametrize("n_in", [8, 248, 256, 264, 512, 520, 688, 768, 776])
+@pytest.mark.parametrize("n_rows", [7104, 7106, 148 * 130 + 7, 148 * 300])
+@pytest.mark.parametrize("epi,norm", [(0, False), (1, True), (2, False), (2, True)])
+def test_short_rows(n_in, n_rows, epi, norm):
+    _check(n_in, n_rows + (n_rows % 2 if epi == 1 else 0), epi, norm, (1, 2, 5, 8, 9), 2e-3 if norm else 1e-5)
+
+
+# The last piece of a row takes what is left up to half a piece more (1024 and, from 4096 inputs on, 2048 inputs)
+@pytest.mark.parametrize("n_in", [1032, 1536, 1544, 2056, 2560, 2568, 3080, 4104, 5632, 6152, 7168, 7176, 11008])
+def test_last_piece_of_a_row(n_in):
+    _check(n_in, 2371, 0, False, (1, 3, 5, 7, 9), 1e-5)
