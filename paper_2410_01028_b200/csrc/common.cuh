@@ -47,15 +47,6 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
 __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 
-// streaming 16-byte load of weights: read-only path, do not keep in L1
-__device__ __forceinline__ uint4 ldg_stream(const void* p) {
-    uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p));
-    return v;
-}
-
 // Programmatic dependent launch: a kernel that was launched with the attribute may start while the one before it on the
 // stream is still running (once all of that one's CTAs have asked for it or ended) and waits here for its end and its
 // writes before it reads or writes anything itself. Without the attribute both do nothing.

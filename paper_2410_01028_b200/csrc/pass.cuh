@@ -512,8 +512,8 @@ __device__ __forceinline__ void top2_merge(float& v, int& i, float& s, float ov,
 // A buffer is only overwritten by a stage that itself needed ALL outputs of a later stage than every reader's, so no
 // reader can still be waiting for the old contents (same ordering a barrier would give, carried by the data).
 // The attention stage takes part: W_qkv's epilogue leaves q and this pass's k and v as tagged words (one bf16 each), a
-// (head, chunk) item leaves its partial result as tagged words, and the group that took a head's last chunk merges the
-// head once all items of its CTA are done. q, k, v and the partial results of a layer are overwritten by the next
+// (head, chunk) item leaves its partial result as tagged words, and the warps without items merge the heads, chunk by chunk as
+// the words arrive. q, k, v and the partial results of a layer are overwritten by the next
 // layer's stages, which a CTA only reaches through W_o's stage, i.e. after every head's merged output (and with it
 // every read of q, k, v and of the partial results) exists.
 __device__ __forceinline__ void ll_store(uint2* dst, uint32_t data, uint32_t tag) {

@@ -6,7 +6,8 @@
 // at 8 mantissa bits each, which represents every fp32 probability exactly); with fewer terms the 2^-17 error of P
 // flips bf16 roundings of the attention output in about every second row.
 //
-// What bounds it: the tensor core, once two CTAs share an SM. Per 64 keys an S tile takes 384 cycles (N = 64 with both operands
+// What bounds it: the lengths of its MMAs, once two CTAs share an SM (1152 of the 1500 cycles of a tile below; the counter of active tensor
+// cycles reads less, 47 % over a launch with its folds and its partly filled second round). Per 64 keys an S tile takes 384 cycles (N = 64 with both operands
 // in shared memory is bound by the operand reads: 48 KB at 128 B per cycle) and the three P V products take 256 each; the
 // softmax of a row takes about 1400 cycles (450 for S and its maximum, 480 for the exponentials and terms of either half). P is
 // handed over in halves of 32 keys, so that the exponentials of one half run while the products of the other do, and S of the
