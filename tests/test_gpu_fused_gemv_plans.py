@@ -1,5 +1,5 @@
 """GPU parity of the stand-alone fused product over its launch plans: one to nine activation rows, fewer weight rows than SMs,
-rows that end inside a group of 16, inputs that end inside a segment of 128, activations in several windows of shared
+rows that end inside a group of 16, inputs that end inside a piece and inside a unit of 32, activations in several windows of shared
 memory, several blocks of rows per CTA; and rows that do not depend on how many rows a call has."""
 import numpy as np
 import pytest
@@ -59,8 +59,8 @@ def test_plans_match_oracle_and_rows_do_not_depend_on_M(n_in, n_rows, epi, norm)
             assert np.array_equal(part_cos, full_cos[:M]), M
 
 
-# the RMSNorm of more than five rows takes them three at a time: whole and partial groups of three, activations in one window
-# and in several
+# the RMSNorm takes rows of up to 4096 inputs five at a time and longer ones in groups of two to five: whole and partial groups,
+# activations in one window and in several
 @pytest.mark.parametrize("M", [3, 4, 6, 7])
 @pytest.mark.parametrize("n_in,n_rows", [(136, 295), (2056, 4737), (8200, 296)])
 def test_rows_of_partial_groups_equal_those_of_nine_rows(M, n_in, n_rows):

@@ -55,3 +55,45 @@ def test_short_rows(n_in, n_rows, epi, norm):
 @pytest.mark.parametrize("n_in", [1032, 1536, 1544, 2056, 2560, 2568, 3080, 4104, 5632, 6152, 7168, 7176, 11008])
 def test_last_piece_of_a_row(n_in):
     _check(n_in, 2371, 0, False, (1, 3, 5, 7, 9), 1e-5)
+
+
+# More than 256 weight rows per SM, so several blocks, each going through two windows of the activations anew
+@pytest.mark.parametrize("norm", [False, True])
+def test_blocks_of_rows_and_windows(norm):
+    import torch
+    import paper_2410_01028_b200 as asd
+    M, n_in, n_rows = 9, 11000, 38500
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    x = torch.randn((M, n_in), generator=gen, device="cuda")
+    x = x if norm else x.to(torch.bfloat16)
+    W = torch.randn((n_rows, n_in), generator=gen, device="cuda").mul_(0.05).to(torch.bfloat16)
+    gain = torch.randn(n_in, generator=gen, device="cuda").mul_(0.1).add_(1).to(torch.bfloat16)
+    scratch = torch.zeros(asd.fused_gemv_scratch_bytes(), dtype=torch.uint8, device="cuda")
+    out = torch.empty((M, n_rows), device="cuda")
+    asd.fused_gemv(x, W, asd.EPI_PLAIN, out, gain=gain if norm else None, scratch=scratch)
+    xin = x.double()
+    if norm:
+        xin = (xin * torch.rsqrt((xin * xin).mean(-1, keepdim=True) + 1e-5) * gain.double()).to(torch.bfloat16).double()
+    ref = torch.cat([xin @ w.double().T for w in W.split(4096)], 1)
+    assert (out.double() - ref).abs().max() <= (2e-3 if norm else 1e-5) * ref.abs().max()
+    few = torch.empty((2, n_rows), device="cuda")
+    asd.fused_gemv(x[:2].contiguous(), W, asd.EPI_PLAIN, few, gain=gain if norm else None, scratch=scratch)
+    assert torch.equal(few, out[:2])
+
+
+# What is not finite stays in its row of the results
+@pytest.mark.parametrize("n_in,n_rows", [(520, 8000), (2056, 300), (13768, 300)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("norm", [False, True])
+def test_rows_that_are_not_finite(n_in, n_rows, bad, norm):
+    M = 9 if n_in < 13000 else 8
+    x = synth.make_array_f32((9, n_in), seed=n_in, stream=1)
+    W = synth.make_matrix_bf16((n_rows, n_in), seed=n_rows, stream=2, std=0.05)
+    gain = synth.make_matrix_bf16((n_in,), seed=3, stream=3, mean=1.0)
+    good, _ = _run(M, n_in, n_rows, 0, norm, x, W, gain, None)
+    x[2, n_in - 3] = bad
+    got, _ = _run(M, n_in, n_rows, 0, norm, x, W, gain, None)
+    others = [m for m in range(M) if m != 2]
+    assert np.array_equal(got[others], good[others])
+    # (a row with an infinity has a root mean square of infinity: zeros, but for infinity over infinity)
+    assert np.all(np.isnan(got[2])) if norm or np.isnan(bad) else not np.any(np.isfinite(got[2]))
