@@ -25,6 +25,10 @@ constexpr int kMaxGemvGrid = 1024;
 constexpr size_t kGemvErrOffset = 128;  // the fused GEMV's error words in the first 256 bytes of its scratch
 constexpr int kPinnedPass = 64;  // word of the pinned block at which a pass leaves its result
 constexpr size_t kPinnedOut = 256 * 1024;  // larger results of inspection calls go straight to the caller's memory
+// Recorded logits of up to this many bytes are written to pinned memory by the pass itself, where asd_get_last_logits finds them: the
+// call then needs no kernel, no copy and no wait of its own (20 us of the 38 between two draft steps of the tiny decoder). 256 KB take
+// 5 us to cross PCIe beside the rest of the pass; more of them a caller who does not read them would notice.
+constexpr size_t kPinnedLogits = 256 * 1024;
 constexpr long long kShortWaitCycles = 2000000LL;  // ASD_DEBUG_SHORT_WAITS: about a millisecond per wait
 
 static size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -336,6 +340,9 @@ struct asd_ctx {
     int32_t pass_stamp = 0;   // of the last pass that was told to deliver its result
     bool delivered = false;   // the last pass was
     unsigned char* pinned_out = nullptr;
+    float* pinned_logits = nullptr;
+    double* pinned_sums = nullptr;  // copy of the sums behind C_l, written by whoever adds to them
+    bool logits_on_host = false;    // the last pass has left its logits in pinned_logits
     bool tables_current = false;   // the stage tables on the device are those of skip_attn / skip_mlp
     bool skipped_cos_nan = false;  // the cosines of the sublayers in the mask are NaN: no pass of the full model since they were set
     uint32_t bar_base = 0;      // value of the grid-barrier counter at the start of the next pass
@@ -629,7 +636,10 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     x->delivered = deliver && lm_head && x->temperature == 0.0;  // (a drawn token takes the argmax's place afterwards)
     if (x->delivered) p.host_out = x->pinned + kPinnedPass, p.host_stamp = ++x->pass_stamp;
     p.logits_out = (x->debug_logits || x->temperature > 0.0) ? x->at<float>(ly.logits) : nullptr;
+    x->logits_on_host = x->delivered && x->debug_logits && (size_t)M * c.vocab * 4 <= kPinnedLogits;
+    p.logits_host = x->logits_on_host ? x->pinned_logits : nullptr;
     p.acc_sim = acc_sim ? 1 : 0;
+    p.sim_base = x->at<double>(ly.sumcos), p.sim_host = x->pinned_sums;
     p.trace = x->trace ? x->at<long long>(ly.trace) : nullptr;
     x->last_n_stages = p.n_stages;
     p.ns = pl.ns, p.attn_groups = pl.attn_groups;
@@ -694,6 +704,7 @@ static int wait_pass(asd_ctx* x, const int* dev_src, int n, const int32_t** word
     ASD_CUDA(x, cudaStreamSynchronize(x->stream));
     const int32_t* h = x->pinned + kPinnedPass;
     if (h[kHostStamp] != x->pass_stamp) {  // a pass that was abandoned before its end
+        x->logits_on_host = false;
         const int rc = read_back(x, dev_src, n);
         return rc ? rc : fail(x, ASD_ERR_CUDA, "a pass has left no result");
     }
@@ -703,7 +714,8 @@ static int wait_pass(asd_ctx* x, const int* dev_src, int n, const int32_t** word
 
 // Small results go to pinned memory by a kernel: one launch, where copies are one transfer each with gaps between them.
 constexpr size_t kKernelOut = 64 * 1024;
-__global__ void __launch_bounds__(256) results_kernel(uint32_t* dst, const uint32_t* src0, int n0, const uint32_t* src1, int n1) {
+template <class T>
+__global__ void __launch_bounds__(256) results_kernel(T* dst, const T* src0, int n0, const T* src1, int n1) {
     for (int i = blockIdx.x * 256 + threadIdx.x; i < n0 + n1; i += gridDim.x * 256) dst[i] = i < n0 ? src0[i] : src1[i - n0];
 }
 
@@ -712,9 +724,14 @@ static int copy_out(asd_ctx* x, void* dst0, const void* src0, size_t bytes0, voi
     const size_t n0 = dst0 ? bytes0 : 0, n1 = dst1 ? bytes1 : 0;
     const bool staged = n0 + n1 <= kPinnedOut;
     if (n0 + n1 > 0 && n0 + n1 <= kKernelOut && (n0 | n1) % 4 == 0) {
-        const int words = (int)((n0 + n1) / 4);
-        results_kernel<<<(words + 255) / 256, 256, 0, x->stream>>>(reinterpret_cast<uint32_t*>(x->pinned_out), static_cast<const uint32_t*>(src0), (int)(n0 / 4),
-                                                                   static_cast<const uint32_t*>(src1), (int)(n1 / 4));
+        auto run = [&](auto unit) {
+            using T = decltype(unit);
+            const int n = (int)((n0 + n1) / sizeof(T));
+            results_kernel<T><<<(n + 255) / 256, 256, 0, x->stream>>>(reinterpret_cast<T*>(x->pinned_out), static_cast<const T*>(src0), (int)(n0 / sizeof(T)),
+                                                                      static_cast<const T*>(src1), (int)(n1 / sizeof(T)));
+        };
+        if ((n0 | n1 | (uintptr_t)src0 | (uintptr_t)src1) % 16 == 0) run(uint4{});
+        else run(uint32_t{});
         ASD_CUDA(x, cudaGetLastError());
     } else {
         if (n0) ASD_CUDA(x, cudaMemcpyAsync(staged ? x->pinned_out : dst0, src0, n0, cudaMemcpyDeviceToHost, x->stream));
@@ -832,10 +849,14 @@ extern "C" int asd_create(const asd_config* cfg, void* dev_workspace, size_t byt
         const size_t cos_bytes = align_up((size_t)2 * std::max(cfg->n_layers, 1) * kPassMaxRows * 4);
         const size_t tok_bytes = align_up(((size_t)cfg->max_seq + 64) * 4);
         unsigned char* h = nullptr;
-        if ((e = cudaHostAlloc((void**)&h, 4096 + cos_bytes + tok_bytes + kPinnedOut, cudaHostAllocDefault)) != cudaSuccess) return bail(e);
+        const size_t sum_bytes = align_up((size_t)2 * std::max(cfg->n_layers, 1) * 8);
+        if ((e = cudaHostAlloc((void**)&h, 4096 + cos_bytes + tok_bytes + kPinnedOut + kPinnedLogits + sum_bytes, cudaHostAllocDefault)) != cudaSuccess)
+            return bail(e);
         x->pinned = reinterpret_cast<int32_t*>(h);
         x->pinned_tokens = reinterpret_cast<int32_t*>(h + 4096 + cos_bytes);
         x->pinned_out = h + 4096 + cos_bytes + tok_bytes;
+        x->pinned_logits = reinterpret_cast<float*>(x->pinned_out + kPinnedOut);
+        x->pinned_sums = reinterpret_cast<double*>(x->pinned_out + kPinnedOut + kPinnedLogits);
     }
     // rotary table: angle(p, j) = p * theta^(-2j/head_dim), evaluated in double, stored as float
     {
@@ -1041,6 +1062,7 @@ extern "C" int asd_reset(asd_ctx* x) {
     x->n_sim_rows = 0;
     std::fill(x->run_attn.begin(), x->run_attn.end(), 0.0);
     std::fill(x->run_mlp.begin(), x->run_mlp.end(), 0.0);
+    std::fill_n(x->pinned_sums, (size_t)2 * std::max(x->c.n_layers, 1), 0.0);
     x->n_run_rows = 0;
     x->last_M = 0;
     x->drafted.clear();
@@ -1119,7 +1141,7 @@ static int prefill_dense(asd_ctx* x, const int32_t* dev_tokens, int n, int pos0)
                                           pcos + (size_t)(L + l) * R, s));
             x->stats.kernel_launches += 3;
         }
-        ASD_CUDA(x, launch_sumcos(pcos, R, rows, 2 * L, x->at<double>(ly.sumcos), s));
+        ASD_CUDA(x, launch_sumcos(pcos, R, rows, 2 * L, x->at<double>(ly.sumcos), x->pinned_sums, s));
         x->stats.kernel_launches += 2;
     }
     return ASD_OK;
@@ -1220,9 +1242,8 @@ extern "C" int asd_get_similarity(asd_ctx* x, float* c_attn, float* c_mlp, int32
     if (n_rows) *n_rows = (int32_t)rows;
     if (x->n_sim_rows == 0) return fail(x, ASD_ERR_STATE, "no prompt row has been processed");
     const int L = x->c.n_layers;
-    std::vector<double> h(2 * (size_t)std::max(L, 1));
-    const int rc = copy_out(x, h.data(), x->ws + x->lay.sumcos, h.size() * 8);
-    if (rc) return rc;
+    ASD_CUDA(x, cudaStreamSynchronize(x->stream));
+    const double* h = x->pinned_sums;
     for (int l = 0; l < L; ++l) {
         if (c_attn) c_attn[l] = (float)((h[l] + x->run_attn[l]) / (double)rows);
         if (c_mlp) c_mlp[l] = (float)((h[L + l] + x->run_mlp[l]) / (double)rows);
@@ -1564,7 +1585,11 @@ extern "C" int asd_get_last_logits(asd_ctx* x, int32_t* M, float* logits) {
     if (!x) return ASD_ERR_ARG;
     if (x->last_M == 0 || !x->last_has_logits) return fail(x, ASD_ERR_STATE, "no logits recorded (asd_set_debug)");
     if (M) *M = x->last_M;
-    return logits ? copy_out(x, logits, x->ws + x->lay.logits, (size_t)x->last_M * x->c.vocab * 4) : ASD_OK;
+    if (!logits) return ASD_OK;
+    const size_t bytes = (size_t)x->last_M * x->c.vocab * 4;
+    if (!x->logits_on_host) return copy_out(x, logits, x->ws + x->lay.logits, bytes);
+    memcpy(logits, x->pinned_logits, bytes);  // the call that ran the pass has waited for it
+    return ASD_OK;
 }
 
 extern "C" int asd_get_last_margins(asd_ctx* x, int32_t* M, float* margins) {

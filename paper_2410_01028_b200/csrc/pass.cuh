@@ -105,7 +105,10 @@ struct PassParams {
     int* host_out;     // pinned host memory for what the caller waits for (kHost... below), or null
     int host_stamp;    // names this pass there
     float* logits_out;
+    float* logits_host;  // pinned host memory for the same logits [M][vocab], or null
     int acc_sim;
+    const double* sim_base;  // the sums behind C_l [2][L], and their copy in pinned host memory
+    double* sim_host;
     long long* trace;  // optional [n_stages][kTraceEntries][gridDim.x] device timestamps (ns) and cycle counts, or null
     // shared-memory plan (bytes from the 1024-aligned base)
     int ns;            // ring slots
@@ -787,7 +790,8 @@ __device__ __noinline__ void epi_gateup_rows(const float* psum, int pair0, int n
 // logit, its lowest index, second-largest logit) does not depend on the order of the comparisons. lmp: this CTA's
 // block of the per-CTA results.
 template <int M>
-__device__ __noinline__ void epi_lmhead_rows(const float* psum, float* red, int pair0, int np, int S, int n_rows, float* logits_out, float* lmp) {
+__device__ __noinline__ void epi_lmhead_rows(const float* psum, float* red, int pair0, int np, int S, int n_rows, float* logits_out, float* logits_host,
+                                             float* lmp) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int copy_stride = np * 2 * M;
     constexpr int G = M < kPassConsumerWarps ? M : kPassConsumerWarps;
@@ -802,6 +806,10 @@ __device__ __noinline__ void epi_lmhead_rows(const float* psum, float* red, int 
             if (logits_out) {
                 logits_out[(size_t)m * n_rows + ra] = va;
                 if (has_b) logits_out[(size_t)m * n_rows + rb] = vb;
+            }
+            if (logits_host) {
+                logits_host[(size_t)m * n_rows + ra] = va;
+                if (has_b) logits_host[(size_t)m * n_rows + rb] = vb;
             }
             if (va > bv) {  // rows come in ascending order: an equal logit keeps the lower index
                 sv = bv, bv = va, bi = ra;
@@ -1420,6 +1428,10 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
                     p.logits_out[(size_t)m * n_rows + ra] = va;
                     if (has_b) p.logits_out[(size_t)m * n_rows + rb] = vb;
                 }
+                if (p.logits_host) {
+                    p.logits_host[(size_t)m * n_rows + ra] = va;
+                    if (has_b) p.logits_host[(size_t)m * n_rows + rb] = vb;
+                }
                 if (va > best_v[m]) {  // rows come in ascending order: an equal logit keeps the lower index
                     sec_v[m] = best_v[m];
                     best_v[m] = va;
@@ -1499,7 +1511,7 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
         else if (type == kStGateUp)
             epi_gateup_rows<M>(psum, pair0, np, S, p.t, n_rows >> 1);
         else
-            epi_lmhead_rows<M>(psum, red, pair0, np, S, n_rows, p.logits_out,
+            epi_lmhead_rows<M>(psum, red, pair0, np, S, n_rows, p.logits_out, p.logits_host,
                                p.partials + ((size_t)p.n_resid * gridDim.x + blockIdx.x) * kPassMaxRows * 4);
     }
     if (type == kStLmHead) {
@@ -1587,6 +1599,7 @@ __device__ void finish_stage(const PassParams& p, const PassSmem& sm) {
             double acc = *out.sumcos;
             for (int m = 0; m < M; ++m) acc += (double)sm.red[m];
             *out.sumcos = acc;
+            p.sim_host[out.sumcos - p.sim_base] = acc;
         }
         consumers_sync();
     }

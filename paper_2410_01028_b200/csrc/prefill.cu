@@ -526,13 +526,13 @@ __global__ void __launch_bounds__(kRowThreads) resid_norm_vec_kernel(int d, floa
     }
 }
 
-__global__ void __launch_bounds__(32) sumcos_kernel(const float* cos_rows, int stride, int n_rows, double* sumcos) {
+__global__ void __launch_bounds__(32) sumcos_kernel(const float* cos_rows, int stride, int n_rows, double* sumcos, double* host) {
     const float* c = cos_rows + (size_t)blockIdx.x * stride;
     double acc = 0.0;
     for (int r = threadIdx.x; r < n_rows; r += 32) acc += (double)c[r];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (threadIdx.x == 0) sumcos[blockIdx.x] += acc;
+    if (threadIdx.x == 0) sumcos[blockIdx.x] = host[blockIdx.x] = sumcos[blockIdx.x] + acc;
 }
 
 cudaError_t launch_embed_norm(const int* tokens, int n_rows, int d, int vocab, const __nv_bfloat16* embed, const __nv_bfloat16* gain,
@@ -551,8 +551,8 @@ cudaError_t launch_resid_norm(int n_rows, int d, float* x, const float* c, int p
     else if (nv <= 5) kernel = resid_norm_vec_kernel<5>;
     return launch_pdl(kernel, dim3(n_rows), dim3(kRowThreads), 0, s, 1, d, x, c, parts, part_stride, gain, eps, xn, cos_out);
 }
-cudaError_t launch_sumcos(const float* cos_rows, int stride, int n_rows, int n_sub, double* sumcos, cudaStream_t s) {
-    sumcos_kernel<<<n_sub, 32, 0, s>>>(cos_rows, stride, n_rows, sumcos);
+cudaError_t launch_sumcos(const float* cos_rows, int stride, int n_rows, int n_sub, double* sumcos, double* host, cudaStream_t s) {
+    sumcos_kernel<<<n_sub, 32, 0, s>>>(cos_rows, stride, n_rows, sumcos, host);
     return cudaGetLastError();
 }
 

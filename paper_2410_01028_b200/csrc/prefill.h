@@ -61,8 +61,8 @@ cudaError_t launch_embed_norm(const int* tokens, int n_rows, int d, int vocab, c
 cudaError_t launch_resid_norm(int n_rows, int d, float* x, const float* c, int parts, size_t part_stride, const __nv_bfloat16* gain, float eps, __nv_bfloat16* xn,
                               float* cos_out, cudaStream_t s);
 
-// sumcos[b] += sum over rows of cos_rows[b * stride + r], rows in a fixed order, double precision
-cudaError_t launch_sumcos(const float* cos_rows, int stride, int n_rows, int n_sub, double* sumcos, cudaStream_t s);
+// sumcos[b] += sum over rows of cos_rows[b * stride + r], rows in a fixed order, double precision; host: a copy in pinned memory
+cudaError_t launch_sumcos(const float* cos_rows, int stride, int n_rows, int n_sub, double* sumcos, double* host, cudaStream_t s);
 
 // causal attention of prompt rows [0, n_rows) at positions pos0 + r over keys 0 .. pos0 + r of the cache. Tensor maps (bf16,
 // 128-byte swizzle): the queries [rows, d_model] in boxes of 64 columns x 128 rows, the caches [max_seq, kv_dim] in boxes of
