@@ -117,7 +117,7 @@ static bool plan_pass(const DeviceInfo& dv, const asd_config& c, int M, PassPlan
     // per-pair partial sums; when a CTA has fewer than 8 groups of 8 pairs up to 15 warps keep copies (at most 15 / groups
     // copies of at most 8 * groups pairs: 120 pairs in all)
     const size_t psum = ((size_t)std::max<long long>(np_max, 120) * 2 * M * 4 + 15) & ~(size_t)15;
-    const size_t misc = ((size_t)16 * kPassMaxRows * 4 * 4 + 32 + 64 * 4 + 8 * 4 * 4 + 15) & ~(size_t)15;  // reduction scratch, flags, slot generations, split table
+    const size_t misc = ((size_t)16 * kPassMaxRows * 4 * 4 + 32 + 64 * 4 + 8 * 4 * 4 + kPassMaxRows * 4 + 15) & ~(size_t)15;  // reduction scratch, flags, slot generations, split table, tokens
     const size_t attn_scratch = ((size_t)M * c.head_dim * 4 + (size_t)M * kAttnChunk * 4 + 4 * kPassMaxRows * 4 + 15) & ~(size_t)15;
     // Activation window: the longest reduction dimension (in segments of 256 inputs) cut into as few windows as leave
     // the ring 20 slots. Every further window costs a stage of a multi-row pass a block-wide refill, every slot less
@@ -650,9 +650,11 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     // against the barrier variant of the same kernel: 1 % faster at one row, 2 % slower at two rows (twice the words to poll).
     p.use_ll = (!x->no_tagged_handoff && !head_only && M == 1 && d <= kPassConsumers * 12 && d % 8 == 0 && f % 8 == 0 && c.head_dim <= 256 &&
                 (long long)pass_wseg(M, pl.xs_bytes) * kSegK >= std::max(d, f)) ? 1 : 0;
+    // the first sublayer's RMSNorm takes rows that it holds whole straight from the embedding
+    p.embed_direct = (p.use_ll || (M == 2 && d <= kPassConsumers * 12 && pass_wseg(M, pl.xs_bytes) * kSegK >= d)) ? 1 : 0;
     const int grid = x->dev->num_sms;
     ASD_CUDA(x, launch_pass(M, p, grid, pl.smem, s));
-    x->bar_base += (uint32_t)p.n_stages * (uint32_t)grid;
+    x->bar_base += (uint32_t)(p.use_ll ? n_table - 2 : p.n_stages) * (uint32_t)grid;  // (tagged handoff: nobody arrives behind the finish stage)
     if (!p.use_ll && !head_only)  // one arrival per CTA and attention stage
         for (int l = 0; l < L; ++l) x->merge_base += (use_mask && x->skip_attn[l]) ? 0u : (uint32_t)grid;
     x->pass_tag += (uint32_t)ly.max_stages + 1u;

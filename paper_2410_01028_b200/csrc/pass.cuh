@@ -47,6 +47,11 @@ constexpr int kPassConsumerWarps = 15;
 constexpr int kPassConsumers = kPassConsumerWarps * 32;
 constexpr int kPassThreads = kPassConsumers + 32;  // + one producer warp
 constexpr unsigned kProducerNapNs = 50;             // the producer warp's sleep after a round without a free slot
+constexpr int kFinishBar = 7;  // named barrier: a CTA's cosines are done (1: consumer warps, 2 to 4: groups of attention warps)
+// Passes of one and two rows read the embeddings in the first sublayer and finish their cosines beside the LM head; in the code of more rows
+// both cost more (registers) than the two hand-offs that they save: five rows of the tiny decoder 136 -> 139 us, 16 rows 5 %.
+template <int M>
+constexpr bool kFewRows = M <= 2;
 constexpr int kXsBudget = 40960;                    // most shared memory the attention scratch of all warp groups may take
 
 enum StageType : int { kStEmbed = 0, kStQkv, kStAttn, kStOproj, kStGateUp, kStDown, kStLmHead, kStFinish };
@@ -83,6 +88,7 @@ struct PassParams {
     uint2 *ql, *kl, *vl;  // tagged handoff: this pass's query [d], key and value [kv_dim], one bf16 per word
     uint2 *pl_acc, *pl_ml;  // tagged handoff: attention partial results per (head, chunk): [head_dim] sums and (maximum, sum of weights)
     uint32_t pass_tag;     // tag of stage 0 of this pass; stage s writes pass_tag + s
+    int embed_direct;      // 1: the first sublayer reads the rows' embeddings itself (see pass_kernel)
     int use_ll;            // 1: launch the kernel variant that hands activations over through the tagged buffers (host: one row, d_model <= 5760)
     float *part_acc, *part_ml;
     int chunk_stride;
@@ -153,6 +159,7 @@ struct PassSmem {
     int* flag;    // [8]
     volatile unsigned* consumed;  // [64] generations of each ring slot that consumers have finished with
     const int* split;             // [8][4] per stage type: this CTA's first pair, pair count, groups of 16 rows, warp sets per group
+    const int* tok;               // [16] the rows' tokens, clamped to the vocabulary
     float* psum;
     unsigned char* reg_a;
 };
@@ -444,54 +451,49 @@ __device__ __forceinline__ void trace_mark(const PassParams& p, int stage, int k
 // ============================================================================================ grid barrier
 __device__ __forceinline__ void consumers_sync() { bar_sync(1, kPassConsumers); }
 
-// release = false: the arrival only counts (nobody will wait for this stage before a later, releasing arrival of the
-// same CTA, whose release is cumulative); the CTA does not wait for its stores to be acknowledged.
-__device__ __forceinline__ void grid_arrive(unsigned* counter, bool release = true) {
+// n: the stages that this arrival ends
+__device__ __forceinline__ void grid_arrive(unsigned* counter, unsigned n = 1u) {
     consumers_sync();
     // one release at GPU scope: cumulative over the writes of the whole CTA, which the barrier above ordered before it
-    if (threadIdx.x == 0) {
-        if (release) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(1u) : "memory");
-        else asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(1u) : "memory");
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(n) : "memory");
+}
+__device__ __forceinline__ void grid_poll(const PassParams& p, const unsigned* counter, unsigned target) {  // one thread
+    volatile int* err = p.err;
+    const long long t0 = clock64();
+    // every poll is a round trip to L2; the error word and the clock are looked at only now and then
+    for (unsigned spin = 1; (int)(ld_acquire_gpu(counter) - target) < 0; ++spin) {
+        if ((spin & 63u) != 0) continue;
+        if (*err != kErrNone) break;
+        if (clock64() - t0 > p.wait_cycles) {
+            if (atomicCAS(p.err, kErrNone, kErrGridWait) == kErrNone) {
+                p.err[1] = counter == p.grid_bar ? (int)((target - p.bar_base) / gridDim.x) : -1, p.err[2] = (int)ld_acquire_gpu(counter);
+                p.err[3] = (int)target, p.err[4] = blockIdx.x;
+            }
+            break;
+        }
     }
 }
 __device__ __forceinline__ void grid_wait(const PassParams& p, const unsigned* counter, unsigned target) {
-    if (threadIdx.x == 0) {
-        volatile int* err = p.err;
-        const long long t0 = clock64();
-        // every poll is a round trip to L2; the error word and the clock are looked at only now and then
-        for (unsigned spin = 1; (int)(ld_acquire_gpu(counter) - target) < 0; ++spin) {
-            if ((spin & 63u) != 0) continue;
-            if (*err != kErrNone) break;
-            if (clock64() - t0 > p.wait_cycles) {
-                if (atomicCAS(p.err, kErrNone, kErrGridWait) == kErrNone) {
-                    p.err[1] = counter == p.grid_bar ? (int)((target - p.bar_base) / gridDim.x) : -1, p.err[2] = (int)ld_acquire_gpu(counter);
-                    p.err[3] = (int)target, p.err[4] = blockIdx.x;
-                }
-                break;
-            }
-        }
-    }
+    if (threadIdx.x == 0) grid_poll(p, counter, target);
     consumers_sync();
 }
 
 // consumers only: true in every thread of the last CTA to arrive on a global counter
 __device__ __forceinline__ bool last_cta_consumers(unsigned* counter, int* flag_smem) {
-    __threadfence();
     consumers_sync();
     if (threadIdx.x == 0) {
-        const unsigned t = atomicAdd(counter, 1u);
+        unsigned t;  // cumulative over the CTA's writes, like the grid barrier's arrival
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
         *flag_smem = (t == gridDim.x - 1) ? 1 : 0;
     }
     consumers_sync();
-    const bool last = *flag_smem != 0;
-    if (last) __threadfence();
-    return last;
+    return *flag_smem != 0;
 }
 
 // Every stage starts by waiting for the previous stage of all CTAs. Whatever does not depend on activations (the
 // stage descriptor, index arithmetic, zeroing of partial sums, RMSNorm gains) is done before this wait.
-__device__ __forceinline__ void stage_begin(const PassParams& p, int s, unsigned extra = 0u) {
-    if (s > 0) grid_wait(p, p.grid_bar, p.bar_base + (unsigned)s * gridDim.x + extra);
+__device__ __forceinline__ void stage_begin(const PassParams& p, int s) {
+    if (s > 0) grid_wait(p, p.grid_bar, p.bar_base + (unsigned)s * gridDim.x);
     trace_mark(p, s, 1);
 }
 
@@ -553,9 +555,19 @@ __device__ __forceinline__ bool ll_keep_waiting(const PassParams& p, unsigned& s
 // batch in flight together, and what was loaded for the statistics is normalised from registers, so a batch costs one
 // memory round trip. The arithmetic of a row is the one of the other paths: thread t adds the squares of its chunks
 // t, t + 480, t + 960 element by element, lanes by butterfly, warps in index order.
+// Four elements of a row of the hidden state: from x, or (emb given) from the embedding of the row's token.
+__device__ __forceinline__ float4 load_row4(const float* xf, const __nv_bfloat16* emb, const int* tok, int m, int n_in, int i) {
+    if (!emb) return __ldcg(reinterpret_cast<const float4*>(xf + (size_t)m * n_in + i));
+    const uint2 e = *reinterpret_cast<const uint2*>(emb + (size_t)tok[m] * n_in + i);
+    return make_float4(bf_lo(e.x), bf_hi(e.x), bf_lo(e.y), bf_hi(e.y));
+}
 template <int M>
-__device__ __forceinline__ void norm_rows_body(const float* xf, const __nv_bfloat16* gain, int n_in, int wlen, int xstride, float eps,
-                                               __nv_bfloat16* xs, float* red) {
+__device__ __forceinline__ float4 load_row4_of(const float* xf, const __nv_bfloat16* emb, const int* tok, int m, int n_in, int i) {
+    return load_row4(xf, kFewRows<M> ? emb : nullptr, tok, m, n_in, i);
+}
+template <int M>
+__device__ __forceinline__ void norm_rows_body(const float* xf, const __nv_bfloat16* emb, const int* tok, const __nv_bfloat16* gain, int n_in, int wlen,
+                                               int xstride, float eps, __nv_bfloat16* xs, float* red) {
     constexpr int kBatches = (M + 5) / 6, kRB = (M + kBatches - 1) / kBatches;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint2 gv[3];
@@ -574,7 +586,7 @@ __device__ __forceinline__ void norm_rows_body(const float* xf, const __nv_bfloa
             for (int c = 0; c < 3; ++c) {
                 const int i = (tid + c * kPassConsumers) * 4;
                 v[u][c] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (m0 + u < M && i < n_in) v[u][c] = __ldcg(reinterpret_cast<const float4*>(xf + (size_t)(m0 + u) * n_in + i));
+                if (m0 + u < M && i < n_in) v[u][c] = load_row4_of<M>(xf, emb, tok, m0 + u, n_in, i);
             }
 #pragma unroll
         for (int u = 0; u < kRB; ++u)
@@ -628,8 +640,8 @@ __device__ __forceinline__ void norm_rows_body(const float* xf, const __nv_bfloa
 // longest row is what four loads of a lane hold; the function above spreads longer ones over the block. The sums are those of that function: lane l of group g has the element group of thread 32 g + l, the groups'
 // butterflies are added in ascending order.
 template <int M>
-__device__ __forceinline__ void norm_rows_narrow(const float* xf, const __nv_bfloat16* gain, int n_in, int wlen, int xstride, float eps,
-                                                 __nv_bfloat16* xs) {
+__device__ __forceinline__ void norm_rows_narrow(const float* xf, const __nv_bfloat16* emb, const int* tok, const __nv_bfloat16* gain, int n_in, int wlen,
+                                                 int xstride, float eps, __nv_bfloat16* xs) {
     constexpr int kGroups = kNarrowRow / 128;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint2 gv[kGroups];
@@ -646,7 +658,7 @@ __device__ __forceinline__ void norm_rows_narrow(const float* xf, const __nv_bfl
         for (int g = 0; g < kGroups; ++g) {
             const int i = (g * 32 + lane) * 4;
             v[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i < n_in) v[g] = __ldcg(reinterpret_cast<const float4*>(xf + (size_t)m * n_in + i));
+            if (i < n_in) v[g] = load_row4_of<M>(xf, emb, tok, m, n_in, i);
         }
         float s = 0.f;
 #pragma unroll
@@ -677,16 +689,16 @@ __device__ __forceinline__ void norm_rows_narrow(const float* xf, const __nv_bfl
 // Called as a function by most row counts; with five and six rows the call itself (measured) costs more than the
 // registers it frees.
 template <int M>
-__device__ __noinline__ void norm_rows_call(const float* xf, const __nv_bfloat16* gain, int n_in, int wlen, int xstride, float eps,
-                                            __nv_bfloat16* xs, float* red) {
-    norm_rows_body<M>(xf, gain, n_in, wlen, xstride, eps, xs, red);
+__device__ __noinline__ void norm_rows_call(const float* xf, const __nv_bfloat16* emb, const int* tok, const __nv_bfloat16* gain, int n_in, int wlen,
+                                            int xstride, float eps, __nv_bfloat16* xs, float* red) {
+    norm_rows_body<M>(xf, emb, tok, gain, n_in, wlen, xstride, eps, xs, red);
 }
 template <int M>
-__device__ __forceinline__ void norm_rows_into_window(const float* xf, const __nv_bfloat16* gain, int n_in, int wlen, int xstride, float eps,
-                                                      __nv_bfloat16* xs, float* red) {
-    if (n_in <= kNarrowRow) norm_rows_narrow<M>(xf, gain, n_in, wlen, xstride, eps, xs);
-    else if constexpr (M == 5 || M == 6) norm_rows_body<M>(xf, gain, n_in, wlen, xstride, eps, xs, red);
-    else norm_rows_call<M>(xf, gain, n_in, wlen, xstride, eps, xs, red);
+__device__ __forceinline__ void norm_rows_into_window(const float* xf, const __nv_bfloat16* emb, const int* tok, const __nv_bfloat16* gain, int n_in, int wlen,
+                                                      int xstride, float eps, __nv_bfloat16* xs, float* red) {
+    if (n_in <= kNarrowRow) norm_rows_narrow<M>(xf, emb, tok, gain, n_in, wlen, xstride, eps, xs);
+    else if constexpr (M == 5 || M == 6) norm_rows_body<M>(xf, emb, tok, gain, n_in, wlen, xstride, eps, xs, red);
+    else norm_rows_call<M>(xf, emb, tok, gain, n_in, wlen, xstride, eps, xs, red);
 }
 
 // Epilogues of a GEMV stage with three or more activation rows, as functions of their own (their registers are their
@@ -699,8 +711,16 @@ __device__ __forceinline__ void norm_rows_into_window(const float* xf, const __n
 // the thread (W_qkv: rotary factors) or of the warp (residual stages: old hidden state) needs from global memory,
 // requested by the caller ahead of the weight stream.
 __device__ __forceinline__ float psum_total(const float* psum, int idx, int S, int copy_stride) {
-    float v = psum[idx];  // the copies of a partial sum (warp sets that shared a group) in the order 0, 1, ...
-    for (int k = 1; k < S; ++k) v += psum[(size_t)k * copy_stride + idx];
+    float v = psum[idx];  // the copies of a partial sum (warp sets that shared a group) in the order 0, 1, ..., four loads in flight
+#pragma unroll 1
+    for (int k = 1; k < S; k += 4) {
+        float c[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) c[i] = k + i < S ? psum[(k + i) * copy_stride + idx] : 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (k + i < S) v += c[i];
+    }
     return v;
 }
 
@@ -790,8 +810,7 @@ __device__ __noinline__ void epi_gateup_rows(const float* psum, int pair0, int n
 // logit, its lowest index, second-largest logit) does not depend on the order of the comparisons. lmp: this CTA's
 // block of the per-CTA results.
 template <int M>
-__device__ __noinline__ void epi_lmhead_rows(const float* psum, float* red, int pair0, int np, int S, int n_rows, float* logits_out, float* logits_host,
-                                             float* lmp) {
+__device__ __noinline__ void epi_lmhead_rows(const float* psum, float* red, int pair0, int np, int S, int n_rows, float* logits_out, float* lmp) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int copy_stride = np * 2 * M;
     constexpr int G = M < kPassConsumerWarps ? M : kPassConsumerWarps;
@@ -806,10 +825,6 @@ __device__ __noinline__ void epi_lmhead_rows(const float* psum, float* red, int 
             if (logits_out) {
                 logits_out[(size_t)m * n_rows + ra] = va;
                 if (has_b) logits_out[(size_t)m * n_rows + rb] = vb;
-            }
-            if (logits_host) {
-                logits_host[(size_t)m * n_rows + ra] = va;
-                if (has_b) logits_host[(size_t)m * n_rows + rb] = vb;
             }
             if (va > bv) {  // rows come in ascending order: an equal logit keeps the lower index
                 sv = bv, bv = va, bi = ra;
@@ -873,6 +888,7 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
     const uint32_t tag_x = p.pass_tag + (uint32_t)st.src_stage;   // tag of the hidden state this stage reads
     const uint32_t tag_in = p.pass_tag + (uint32_t)(stage - 1);   // tag of the attention / SwiGLU output (previous stage)
     const uint32_t tag_out = p.pass_tag + (uint32_t)stage;        // tag of what this stage writes
+    const bool direct = kFewRows<M> && norm && p.embed_direct && st.src_stage == 0;  // the hidden state is still the rows' embeddings
     unsigned ll_spins = 0;
     long long ll_t0 = 0;
     // Fewer groups than warps (the d x d matrices leave ~28 rows to a CTA): several warps share a group, warp set ks
@@ -880,12 +896,11 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
     // added in the epilogue in the order ks = 0, 1, ... (a fixed order that depends on the matrix shape only).
     const int S = sm.split[type * 4 + 3];
     const int copy_stride = np * 2 * M;
-    // A warp's first item of the stage stores its sums, later items add: the partial sums need no zeroing (only when a
-    // row has fewer segments than warp sets, i.e. some copies would never be written, they are zeroed and all items add)
-    const bool store_first = n_seg >= S;
-    if (!store_first)
-        for (int i = tid; i < S * copy_stride; i += kPassConsumers) psum[i] = 0.f;
+    // A warp's first item of the stage stores its sums, later items add: the partial sums need no zeroing (there are no more warp sets than segments)
     constexpr bool kKeepX = (M == 1);
+    // tagged handoff: no barrier stands between the cosine sums of a stage and the next RMSNorm, whose sums therefore lie elsewhere
+    constexpr int kRedNorm = LL ? 3 : 0;
+    const int chunks = n_in > kPassConsumers * 8 ? 3 : n_in > kPassConsumers * 4 ? 2 : 1;  // of 4 elements of a thread; short rows skip the code of the others
     const bool keep = kKeepX && norm && n_in <= kPassConsumers * 12;
     uint2 gpre[3] = {make_uint2(0u, 0u), make_uint2(0u, 0u), make_uint2(0u, 0u)};  // this thread's RMSNorm gains
     const bool short_rows = norm && n_in <= kPassConsumers * 12;  // a thread owns at most three 4-element chunks of a row
@@ -925,8 +940,8 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
             }
         }
     }
-    if (ll) trace_mark(p, stage, 1);  // no barrier: the loads below wait for exactly the words they need
-    else stage_begin(p, stage);
+    if (ll || direct || type == kStLmHead) trace_mark(p, stage, 1);  // no barrier: the loads below wait for exactly the words they need,
+    else stage_begin(p, stage);  // the embeddings are there, and in front of the LM head the finish stage has waited
     if (kSpreadEpi && (type == kStOproj || type == kStDown)) {
         const int W = (np * 2 + 31) >> 5;
         if (warp < M * W) {
@@ -975,24 +990,28 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
                 for (int m = 0; m < (kKeepX ? M : 0); ++m)
 #pragma unroll
                     for (int c = 0; c < 3; ++c)
-                        if ((tid + c * kPassConsumers) * 4 < n_in) stale |= 3u << ((m * 3 + c) * 2);
+                        if (!direct && (tid + c * kPassConsumers) * 4 < n_in) stale |= 3u << ((m * 3 + c) * 2);
                 for (;;) {
 #pragma unroll
                     for (int m = 0; m < (kKeepX ? M : 0); ++m)
 #pragma unroll
-                        for (int c = 0; c < 3; ++c)
+                        for (int c = 0; c < 3; ++c) {
+                            if (c >= chunks) break;
 #pragma unroll
                             for (int h = 0; h < 2; ++h)
                                 if (stale & (1u << ((m * 3 + c) * 2 + h)))
                                     ll_load2(p.xl + (size_t)m * n_in + (tid + c * kPassConsumers) * 4 + 2 * h, raw[m][c][2 * h], raw[m][c][2 * h + 1]);
+                        }
 #pragma unroll
                     for (int m = 0; m < (kKeepX ? M : 0); ++m)
 #pragma unroll
-                        for (int c = 0; c < 3; ++c)
+                        for (int c = 0; c < 3; ++c) {
+                            if (c >= chunks) break;
 #pragma unroll
                             for (int h = 0; h < 2; ++h)
                                 if ((stale & (1u << ((m * 3 + c) * 2 + h))) && ll_ready(raw[m][c][2 * h], tag_x) && ll_ready(raw[m][c][2 * h + 1], tag_x))
                                     stale &= ~(1u << ((m * 3 + c) * 2 + h));
+                        }
                     if (stale == 0u || !ll_keep_waiting(p, ll_spins, ll_t0, stage)) break;
                     __nanosleep(ll_spins < 4 ? 100u : 300u);
                 }
@@ -1007,9 +1026,11 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
             for (int m = 0; m < M; ++m) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
+                    if (c >= chunks) break;
                     const int i = (tid + c * kPassConsumers) * 4;
                     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (ll) v = xr[kKeepX ? m : 0][c];
+                    if (ll && !direct) v = xr[kKeepX ? m : 0][c];
+                    else if (ll) v = i < n_in ? load_row4(xf, p.embed, sm.tok, m, n_in, i) : v;
                     else if (i < n_in) v = __ldcg(reinterpret_cast<const float4*>(xf + (size_t)m * n_in + i));
                     xr[kKeepX ? m : 0][c] = v;
                     if (i < n_in) {
@@ -1047,14 +1068,14 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
 #pragma unroll
         for (int m = 0; m < M; ++m) {
             const float s = warp_sum(ssq[m]);
-            if (lane == 0) red[warp * (kPassMaxRows * 4) + m] = s;
+            if (lane == 0) red[warp * (kPassMaxRows * 4) + m + kRedNorm] = s;
         }
         consumers_sync();
 #pragma unroll
         for (int m = 0; m < M; ++m) {
             float s = 0.f;
 #pragma unroll
-            for (int w = 0; w < kPassConsumerWarps; ++w) s += red[w * (kPassMaxRows * 4) + m];
+            for (int w = 0; w < kPassConsumerWarps; ++w) s += red[w * (kPassMaxRows * 4) + m + kRedNorm];
             inv[m] = 1.0f / sqrtf(s / (float)n_in + p.eps);
         }
     }
@@ -1067,12 +1088,15 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
         const int ws = min(wseg, n_seg - w0);
         const int k0 = w0 * kSegK;
         const int wlen = ws * kSegK;  // inputs in this window, including the zero padding past n_in
-        consumers_sync();  // previous window fully consumed; psum zeroed; red free
+        // previous window fully consumed (the first one: the stage before has ended with a barrier behind its products; with 16 rows the warps that
+        // drift apart without it cost more than it does, 7B width 684 -> 696 us)
+        if (w0 > 0 || M > kMaxRows) consumers_sync();
         if (fused) {
-            norm_rows_into_window<M>(xf, st.gain, n_in, wlen, xstride, p.eps, xs, red);
+            norm_rows_into_window<M>(xf, direct ? p.embed : nullptr, sm.tok, st.gain, n_in, wlen, xstride, p.eps, xs, red);
         } else if (keep) {  // a single window (n_in <= 5760): normalise the rows held in registers
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
+                if (c >= chunks && c * kPassConsumers * 4 >= wlen) break;
                 const int i = (tid + c * kPassConsumers) * 4;
                 if (i < wlen) {
                     const bool in = i < n_in;
@@ -1273,7 +1297,7 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
                     const int wr = g8 + 8 * hr;
                     if (wr < rows) {
                         float* dst = psum_w + (size_t)(kGrpRows * o + wr) * M;
-                        const bool first = store_first && seg == ((S > 1) ? ks : 0);
+                        const bool first = seg == ((S > 1) ? ks : 0);
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
                             const int mm = 2 * q4 + e;
@@ -1337,9 +1361,7 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
             }
 #pragma unroll
             for (int m = 0; m < M; ++m) {
-                float v = psum[e * M + m];
-                for (int k = 1; k < S; ++k) v += psum[(size_t)k * copy_stride + e * M + m];
-                const float y = xv[m] + v;
+                const float y = xv[m] + psum_total(psum, e * M + m, S, copy_stride);
                 if (ll) ll_store(p.xl + (size_t)m * n_rows + row, __float_as_uint(y), tag_out);
                 else out[(size_t)m * n_rows + row] = y;
                 s_loc[m][0] = fmaf(xv[m], y, s_loc[m][0]);
@@ -1357,11 +1379,7 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int pl = 2 * pj + h;
-                    float va = psum[(pl * 2 + 0) * M + m], vb = psum[(pl * 2 + 1) * M + m];
-                    for (int k = 1; k < S; ++k) {
-                        va += psum[(size_t)k * copy_stride + (pl * 2 + 0) * M + m];
-                        vb += psum[(size_t)k * copy_stride + (pl * 2 + 1) * M + m];
-                    }
+                    const float va = psum_total(psum, (pl * 2 + 0) * M + m, S, copy_stride), vb = psum_total(psum, (pl * 2 + 1) * M + m, S, copy_stride);
                     const float t = va / (1.0f + expf(-va)) * vb;
                     word |= (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(t)) << (16 * h);
                 }
@@ -1386,11 +1404,7 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
         }
 #pragma unroll
         for (int m = 0; m < M; ++m) {
-            float va = psum[(pl * 2 + 0) * M + m], vb = psum[(pl * 2 + 1) * M + m];
-            for (int k = 1; k < S; ++k) {
-                va += psum[(size_t)k * copy_stride + (pl * 2 + 0) * M + m];
-                vb += psum[(size_t)k * copy_stride + (pl * 2 + 1) * M + m];
-            }
+            float va = psum_total(psum, (pl * 2 + 0) * M + m, S, copy_stride), vb = psum_total(psum, (pl * 2 + 1) * M + m, S, copy_stride);
             if (type == kStGateUp) {
                 const float t = va / (1.0f + expf(-va)) * vb;
                 p.t[(size_t)m * (n_rows >> 1) + (pair0 + pl)] = __float2bfloat16_rn(t);
@@ -1427,10 +1441,6 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
                 if (p.logits_out) {
                     p.logits_out[(size_t)m * n_rows + ra] = va;
                     if (has_b) p.logits_out[(size_t)m * n_rows + rb] = vb;
-                }
-                if (p.logits_host) {
-                    p.logits_host[(size_t)m * n_rows + ra] = va;
-                    if (has_b) p.logits_host[(size_t)m * n_rows + rb] = vb;
                 }
                 if (va > best_v[m]) {  // rows come in ascending order: an equal logit keeps the lower index
                     sec_v[m] = best_v[m];
@@ -1511,11 +1521,20 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
         else if (type == kStGateUp)
             epi_gateup_rows<M>(psum, pair0, np, S, p.t, n_rows >> 1);
         else
-            epi_lmhead_rows<M>(psum, red, pair0, np, S, n_rows, p.logits_out, p.logits_host,
+            epi_lmhead_rows<M>(psum, red, pair0, np, S, n_rows, p.logits_out,
                                p.partials + ((size_t)p.n_resid * gridDim.x + blockIdx.x) * kPassMaxRows * 4);
     }
     if (type == kStLmHead) {
-        if (last_cta_consumers(p.fin_counter, sm.flag)) {
+        if (kFewRows<M> && blockIdx.x < (unsigned)p.n_resid) bar_sync(kFinishBar, kPassThreads);  // this CTA's share of the cosines is done as well
+        const bool last_cta = last_cta_consumers(p.fin_counter, sm.flag);
+        if (p.logits_host) {  // (behind the ticket, whose release would wait for the way over PCIe)
+            const int n = min(2 * np, n_rows - 2 * pair0);
+            for (int i = tid; i < M * n; i += kPassConsumers) {
+                const int m = i / n, e = i - m * n;
+                p.logits_host[(size_t)m * n_rows + 2 * pair0 + e] = psum_total(psum, e * M + m, S, copy_stride);
+            }
+        }
+        if (last_cta) {
             int* g = reinterpret_cast<int*>(red);
             for (int m = warp; m < M; m += kPassConsumerWarps) {  // a warp per row: lanes scan the per-CTA partials, then a butterfly; ties -> lowest index
                 float v = -INFINITY, sc = -INFINITY;
@@ -1566,9 +1585,11 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
 }
 
 // ============================================================================================ finish stage
-// Cosine similarities of all residual stages of the pass (summand of C_l, Section 3.2). Residual stage r is
-// finished by CTA r mod gridDim.x: one warp per activation row adds the per-CTA partials b = lane, lane+32, ...
-// in order, then an xor butterfly, all in double precision (fixed order, independent of the row count).
+// Cosine similarities of all residual stages of the pass (summand of C_l, Section 3.2). Residual stage r is finished by the
+// producer warp of CTA r mod gridDim.x when its last copy is on its way, beside the LM head's products: the per-CTA partials b = lane, lane +
+// 32, ... are added in order, then by an xor butterfly, all in double precision (fixed order, independent of the row count). As a
+// stage of the consumer warps it stood between the last sublayer and the LM head (figures: pass_kernel, embedding stage).
+// Passes of more rows finish them by their consumer warps, a warp per row.
 template <int M>
 __device__ void finish_stage(const PassParams& p, const PassSmem& sm) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1578,9 +1599,8 @@ __device__ void finish_stage(const PassParams& p, const PassSmem& sm) {
         for (int m = warp; m < M; m += kPassConsumerWarps) {
             double sxy = 0, sxx = 0, syy = 0;
             for (unsigned b = lane; b < gridDim.x; b += 32) {
-                sxy += (double)__ldcg(part + ((size_t)b * kPassMaxRows + m) * 4 + 0);
-                sxx += (double)__ldcg(part + ((size_t)b * kPassMaxRows + m) * 4 + 1);
-                syy += (double)__ldcg(part + ((size_t)b * kPassMaxRows + m) * 4 + 2);
+                const float4 v = __ldcg(reinterpret_cast<const float4*>(part + ((size_t)b * kPassMaxRows + m) * 4));
+                sxy += (double)v.x, sxx += (double)v.y, syy += (double)v.z;
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -1588,11 +1608,7 @@ __device__ void finish_stage(const PassParams& p, const PassSmem& sm) {
                 sxx += __shfl_xor_sync(0xffffffffu, sxx, o);
                 syy += __shfl_xor_sync(0xffffffffu, syy, o);
             }
-            if (lane == 0) {
-                const double c = sxy / fmax(sqrt(sxx) * sqrt(syy), 1e-30);
-                out.cos_out[m] = (float)c;
-                sm.red[m] = (float)c;
-            }
+            if (lane == 0) out.cos_out[m] = sm.red[m] = (float)(sxy / fmax(sqrt(sxx) * sqrt(syy), 1e-30));
         }
         consumers_sync();
         if (tid == 0 && p.acc_sim && out.sumcos) {  // rows are added in order: chunked prefill equals one-shot prefill
@@ -1603,6 +1619,63 @@ __device__ void finish_stage(const PassParams& p, const PassSmem& sm) {
         }
         consumers_sync();
     }
+}
+template <int M>
+__device__ __forceinline__ void finish_rows(const PassParams& p) {
+    const int lane = threadIdx.x & 31;
+    if (blockIdx.x >= (unsigned)p.n_resid) return;
+    if (lane == 0) {
+        const int stage = p.n_stages - (p.stages[p.n_stages - 1].type == kStFinish ? 1 : 2);
+        grid_poll(p, p.grid_bar, p.bar_base + (unsigned)stage * gridDim.x + p.bar_extra_last);  // (test hook: extra arrivals that never come)
+    }
+    __syncwarp();
+    for (int r = blockIdx.x; r < p.n_resid; r += gridDim.x) {
+        const float4* part = reinterpret_cast<const float4*>(p.partials + (size_t)r * gridDim.x * kPassMaxRows * 4);
+        const ResidOut out = p.resid[r];
+        const bool sum = lane == 0 && p.acc_sim && out.sumcos;
+        double acc = sum ? *out.sumcos : 0.0;  // rows are added in order: chunked prefill equals one-shot prefill
+        constexpr int kB = M < 3 ? M : 3;      // rows whose partials are requested together
+#pragma unroll 1
+        for (int m0 = 0; m0 < M; m0 += kB) {
+            double s[kB][3] = {};
+            for (unsigned b0 = 0; b0 < gridDim.x; b0 += 160) {
+                float4 v[kB][5];
+#pragma unroll
+                for (int u = 0; u < kB; ++u)
+#pragma unroll
+                    for (int i = 0; i < 5; ++i) {
+                        const unsigned b = b0 + i * 32 + lane;
+                        v[u][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (m0 + u < M && b < gridDim.x) v[u][i] = __ldcg(part + (size_t)b * kPassMaxRows + m0 + u);
+                    }
+#pragma unroll
+                for (int u = 0; u < kB; ++u)
+#pragma unroll
+                    for (int i = 0; i < 5; ++i) s[u][0] += (double)v[u][i].x, s[u][1] += (double)v[u][i].y, s[u][2] += (double)v[u][i].z;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int u = 0; u < kB; ++u)
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) s[u][j] += __shfl_xor_sync(0xffffffffu, s[u][j], o);
+            if (lane == 0) {
+#pragma unroll
+                for (int u = 0; u < kB; ++u)
+                    if (m0 + u < M) {
+                        const float c = (float)(s[u][0] / fmax(sqrt(s[u][1]) * sqrt(s[u][2]), 1e-30));
+                        out.cos_out[m0 + u] = c;
+                        acc += (double)c;
+                    }
+            }
+        }
+        if (sum) {
+            *out.sumcos = acc;
+            p.sim_host[out.sumcos - p.sim_base] = acc;
+        }
+    }
+    __syncwarp();
+    if (p.stages[p.n_stages - 1].type == kStLmHead) bar_arrive(kFinishBar, kPassThreads);  // the LM head stage's last word comes after this
 }
 
 // ============================================================================================ attention stage
@@ -2101,6 +2174,7 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
     } else if (LL) {
         merge_tagged(p, stage, n_chunks, item_warps, kPassConsumerWarps - item_warps);
     }
+    if (LL) consumers_sync();  // the next stage's window takes the place of the items' scratch
     if (!LL) {
         grid_arrive(p.merge_bar);
         merge_target += gridDim.x;
@@ -2124,6 +2198,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
     sm.consumed = reinterpret_cast<volatile unsigned*>(sm.flag + 8);
     int* split = reinterpret_cast<int*>(const_cast<unsigned*>(sm.consumed) + 64);
     sm.split = split;
+    int* tok = split + 8 * 4;
+    sm.tok = tok;
     sm.psum = reinterpret_cast<float*>(base + p.off_psum);
     sm.reg_a = base + p.off_reg_a;
 
@@ -2144,14 +2220,21 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
         int pair0 = 0, np = 0;
         if (n_rows > 0) cta_pairs(n_rows, type, pair0, np);
         const int n_oct = (np + kGrpPairs - 1) / kGrpPairs;
-        // fewer groups than warps: several warp sets share a group (see gemv_stage)
+        // fewer groups than warps: several warp sets share a group, no more of them than a row has segments (see gemv_stage; copies of the partial
+        // sums that nobody wrote were zeroed and added all the same: one row of the tiny decoder 100 -> 92 us, five rows 138 -> 129)
+        const int n_seg = ((type == kStDown ? p.d_ffn : p.d_model) + kSegK - 1) / kSegK;
         split[type * 4 + 0] = pair0, split[type * 4 + 1] = np, split[type * 4 + 2] = n_oct;
-        split[type * 4 + 3] = (n_oct > 0 && n_oct < 8) ? kPassConsumerWarps / n_oct : 1;
+        split[type * 4 + 3] = (n_oct > 0 && n_oct < 8) ? max(1, min(kPassConsumerWarps / n_oct, n_seg)) : 1;
+    }
+    if (threadIdx.x >= 64 && threadIdx.x < 64 + M && p.stages[0].type == kStEmbed) {
+        const int m = threadIdx.x - 64;
+        tok[m] = min(max(pass_token(p, m), 0), p.vocab - 1);
     }
     __syncthreads();
 
     if (threadIdx.x >= kPassConsumers) {
         pass_producer<M>(p, sm);
+        if constexpr (kFewRows<M>) finish_rows<M>(p);
         return;
     }
 
@@ -2171,30 +2254,40 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
             asm volatile("prefetch.global.L1 [%0];" ::"l"(reinterpret_cast<const char*>(p.stages + s + 1) + threadIdx.x * 64));
         if (p.trace && threadIdx.x == 0) p.trace[((size_t)s * kTraceEntries + 11) * gridDim.x + blockIdx.x] = st.type >= 0 ? global_ns() : 0;  // descriptor read
         if (st.type == kStEmbed) {
-            stage_begin(p, s);
             const int d = p.d_model;
-            for (int i = blockIdx.x * kPassConsumers + threadIdx.x; i < M * d; i += gridDim.x * kPassConsumers) {
-                const int m = i / d, e = i - m * d;
-                int t = pass_token(p, m);
-                t = min(max(t, 0), p.vocab - 1);
-                const float v = __bfloat162float(p.embed[(size_t)t * d + e]);
-                if (LL) ll_store(p.xl + i, __float_as_uint(v), p.pass_tag);
-                else p.x[i] = v;
+            if (kFewRows<M> && p.embed_direct) {
+                // The first RMSNorm reads the embeddings itself; what the residual stages will want of them, the CTA's own rows, it leaves here
+                // for itself, and nobody waits for anybody. (A stage that spread the embeddings over the CTAs cost a hand-off; without it and with
+                // the cosines beside the LM head one row of the 7B width, four layers, took 329.8 us for 332.7, two rows of the tiny decoder 121 for 124.)
+                const int row0 = 2 * split[kStOproj * 4 + 0], n = min(2 * split[kStOproj * 4 + 1], d - row0);
+                for (int i = threadIdx.x; i < M * n; i += kPassConsumers) {
+                    const int m = i / n, e = row0 + i - m * n;
+                    const float v = __bfloat162float(p.embed[(size_t)tok[m] * d + e]);
+                    if (LL) ll_store(p.xl + (size_t)m * d + e, __float_as_uint(v), p.pass_tag);
+                    else p.x[(size_t)m * d + e] = v;
+                }
+            } else {
+                for (int i = blockIdx.x * kPassConsumers + threadIdx.x; i < M * d; i += gridDim.x * kPassConsumers) {
+                    const int m = i / d, e = i - m * d;
+                    p.x[i] = __bfloat162float(p.embed[(size_t)tok[m] * d + e]);
+                }
             }
         } else if (st.type == kStFinish) {
-            stage_begin(p, s, p.bar_extra_last);  // (test hook: extra arrivals that never come)
-            finish_stage<M>(p, sm);
+            if (!LL) stage_begin(p, s);  // the LM head wants the hidden state of all CTAs; the producer warp does the work (finish_rows)
+            if constexpr (!kFewRows<M>) finish_stage<M>(p, sm);
         } else if (st.type == kStAttn) {
             attn_stage<M, LL>(p, st, sm, gi, merge_target, s);
         } else {
             gemv_stage<M, LL>(p, st, sm, gi, s);
         }
         trace_mark(p, s, 3);
-        // With the tagged handoff only the finish stage still waits at the grid barrier: the arrival in front of it
-        // publishes everything this CTA has written so far, the others just count.
-        bool release = true;
-        if (LL && next_type >= 0) release = (next_type == kStFinish);
-        grid_arrive(p.grid_bar, release);
+        if (!LL) {
+            grid_arrive(p.grid_bar);
+        } else if (next_type == kStFinish) {
+            // Tagged handoff: only the finish stage waits at the grid barrier, so the CTA arrives once for all stages in front of it. (Nothing
+            // else ends a stage with a barrier: what the next one writes first, the window and the sums of squares, nobody reads any more.)
+            grid_arrive(p.grid_bar, (unsigned)(s + 1));
+        }
     }
 }
 
