@@ -118,7 +118,7 @@ static bool plan_pass(const DeviceInfo& dv, const asd_config& c, int M, PassPlan
     // copies of at most 8 * groups pairs: 120 pairs in all)
     const size_t psum = ((size_t)std::max<long long>(np_max, 120) * 2 * M * 4 + 15) & ~(size_t)15;
     const size_t misc = ((size_t)16 * kPassMaxRows * 4 * 4 + 32 + 64 * 4 + 8 * 4 * 4 + kPassMaxRows * 4 + 15) & ~(size_t)15;  // reduction scratch, flags, slot generations, split table, tokens
-    const size_t attn_scratch = ((size_t)M * c.head_dim * 4 + (size_t)M * kAttnChunk * 4 + 4 * kPassMaxRows * 4 + 15) & ~(size_t)15;
+    const size_t attn_scratch = (size_t)attn_scratch_bytes(M, c.n_heads / c.n_kv_heads, c.head_dim);
     // Activation window: the longest reduction dimension (in segments of 256 inputs) cut into as few windows as leave
     // the ring 20 slots. Every further window costs a stage of a multi-row pass a block-wide refill, every slot less
     // costs bandwidth (one row, 7B shape: 24 slots 0.402 ms per 4 layers, 21: 0.409, 16: 0.422, 12: 0.481); 20 was the

@@ -38,6 +38,8 @@
 #pragma once
 #include <limits.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "ring.cuh"
 
@@ -47,6 +49,7 @@ constexpr int kPassConsumerWarps = 15;
 constexpr int kPassConsumers = kPassConsumerWarps * 32;
 constexpr int kPassThreads = kPassConsumers + 32;  // + one producer warp
 constexpr unsigned kProducerNapNs = 50;             // the producer warp's sleep after a round without a free slot
+constexpr int kAttnDoneBar = 8;  // named barriers 8 to 10: a group of attention warps has read its value tile
 constexpr int kFinishBar = 7;  // named barrier: a CTA's cosines are done (1: consumer warps, 2 to 4: groups of attention warps)
 // Passes of one and two rows read the embeddings in the first sublayer and finish their cosines beside the LM head; in the code of more rows
 // both cost more (registers) than the two hand-offs that they save: five rows of the tiny decoder 136 -> 139 us, 16 rows 5 %.
@@ -1691,32 +1694,45 @@ struct TileAddr {
     }
 };
 
-// Merging the chunks of a head: a chunk with maximum m_c moves the running maximum to max(m, m_c), scales what has been added so
-// far by exp(old - new maximum) and comes in with exp(m_c - new). These factors are the same for every output dimension: lane i
-// works out those of chunk i of 32 (the running maximum by a scan over the lanes) and hands them round.
-struct MergeFactors {
-    float s_old, s_new, sum;
-    // ml: (maximum, sum of weights) of this lane's chunk, -inf past the last one; mx: the running maximum, moved on
-    __device__ __forceinline__ MergeFactors(float2 ml, float& mx) : sum(ml.y) {
-        const int lane = threadIdx.x & 31;
-        float m = ml.x;
-#pragma unroll
-        for (int o = 1; o < 32; o *= 2) {
-            const float t = __shfl_up_sync(0xffffffffu, m, o);
-            if (lane >= o) m = fmaxf(m, t);
-        }
-        m = fmaxf(m, mx);
-        float before = __shfl_up_sync(0xffffffffu, m, 1);
-        if (lane == 0) before = mx;
-        s_old = expf(before - m), s_new = expf(ml.x - m);
-        mx = __shfl_sync(0xffffffffu, m, 31);
-    }
-    __device__ __forceinline__ void of(int i, float& so, float& sn, float& s) const {
-        so = __shfl_sync(0xffffffffu, s_old, i), sn = __shfl_sync(0xffffffffu, s_new, i), s = __shfl_sync(0xffffffffu, sum, i);
-    }
-};
+// Four 8x8 matrices of bf16 from shared memory, a row address per lane; the second form hands out their transposes.
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+// A * B alone: the sum of 16 products starts from zero
+__device__ __forceinline__ void mma_bf16_zero(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
 
-// HD: the head size when the code is compiled for it (loops and divisions by it are then fixed), 0: p.head_dim.
+// Shared memory of a group of warps: the queries of eight columns [column][head_dim] and their probabilities as three bf16 terms
+// [term][column][128 keys], rows 16 bytes longer than they are (the eight rows of a matrix then lie in different banks), then the warps' maxima and sums.
+constexpr int kAttnCols = 8;  // (row, head of the group) pairs per step: the N of m16n8k16
+constexpr int kAttnPRow = kAttnChunk * 2 + 16;
+__host__ __device__ inline int attn_cols(int M, int group) { return M * group < kAttnCols ? M * group : kAttnCols; }
+__host__ __device__ inline int attn_scratch_bytes(int M, int group, int hd) {
+    return attn_cols(M, group) * (2 * hd + 16 + 3 * kAttnPRow) + 2 * 4 * kAttnCols * 4;
+}
+
+// Work items (kv head, 128-key chunk) of this CTA on the tensor cores (mma.sync m16n8k16), a group of four warps to an item. The COLUMNS of the
+// products are the (row, query head) pairs that share the item's keys, eight at a time; what a column gets does not depend on its
+// neighbours, so neither does a row's result on the row count.
+//   S^T = K Q^T: 16 keys are the rows of a step (a warp has 32 keys), both operands read with ldmatrix; every 16 products start from zero and are
+//   added on the CUDA cores.
+//   softmax statistics of the chunk in fp32, the probabilities as the exact sum of three bf16 terms (cut off at 8 bits each) to shared memory.
+//   O^T = V^T P: 16 dimensions are the rows (a warp has head_dim / 4 of them), V read transposed; every 16 products of a term start from zero as
+//   above. (One or two columns have room for their three terms in one product: a third of the steps.)
+// The order of the keys inside a block of 16 is free. Row r of a step is key r (r < 8) or 8 + ((r - 8) ^ 4): a lane then holds two keys that become
+// neighbours in P, and the eight rows of every matrix, of K as of V, have different swizzles: no bank conflicts.
+// Error: a sum of 16 products on the tensor core is nearly exact, and chains of additions are half as long as with one FMA per product.
+// What bounds it: at 8000 positions of the 7B width the K/V stream (20 us a layer), the barrier and the merge behind it (10 us); at few positions the chain of an item
+// (three barriers, about 3 us). Against fp32 FMAs fed from shared memory, heads one after the other and rows unrolled, kernel times in us (four layers of the 7B
+// width; two layers 2048 wide with 32 heads of 64 on 8): five rows on 8000 keys 595 -> 546, nine 876 -> 720, 16 rows of a prompt 683 -> 636; grouped
+// queries: one row on 8000 keys 111 -> 89, five 185 -> 140, nine 295 -> 188, 16 rows of a prompt 244 -> 211.
+// HD: the head size when the code is compiled for it, 0: p.head_dim.
 template <int M, bool LL, int HD>
 __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassSmem& sm, uint32_t gi0, int stage, int n_chunks, int first, int n_local) {
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -1729,19 +1745,27 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
     long long ll_t0 = 0;
     const int grp = warp >> 2;
     const int gt = tid & 127, glane = gt & 31, gwarp = gt >> 5;
+    const int g8 = glane >> 2, q4 = glane & 3;  // fragment coordinates: row g8 (and g8 + 8), columns 2 q4 and 2 q4 + 1
     const int bar_id = 2 + grp;
     const int group = p.n_heads / p.n_kv_heads;
+    const int n_cols = M * group;  // column c: row c % M of query head c / M of the group
     const int vec_per_row = hd / 8;
-    TileAddr ta{nhb, box_cols * 2, (box_cols * 2 == 128) ? 1 : 0};
+    const TileAddr ta{nhb, box_cols * 2, (box_cols * 2 == 128) ? 1 : 0};
 
-    // per-group scratch in region A
-    const size_t scratch_bytes = ((size_t)M * hd * 4 + (size_t)M * kAttnChunk * 4 + 4 * kPassMaxRows * 4 + 16 + 15) & ~(size_t)15;
-    unsigned char* base = sm.reg_a + (size_t)grp * scratch_bytes;
-    float* qs = reinterpret_cast<float*>(base);   // [M][hd]
-    float* Ps = qs + M * hd;                       // [M][128]
-    float* red = Ps + M * kAttnChunk;              // [4][kPassMaxRows]
+    const int q_row = 2 * hd + 16, ct_max = attn_cols(M, group);
+    unsigned char* qs = sm.reg_a + (size_t)grp * attn_scratch_bytes(M, group, hd);
+    unsigned char* ps = qs + ct_max * q_row;
+    float* red = reinterpret_cast<float*>(ps + 3 * ct_max * kAttnPRow);  // [4][8] maxima, then [4][8] sums
+    const uint32_t ring_addr = smem_u32(sm.ring);
 
-    int q_head = -1;   // head whose queries are in qs
+    // matrix rows that this lane addresses: of K (matrix bit 0: rows 8-15, bit 1: second half of 16 dimensions), of V (bit 0: second
+    // half of 16 dimensions, bit 1: keys 8-15 of P's order), of Q and P (a column; the matrices follow one another along the row)
+    const int mi = glane & 7, mat = glane >> 3;
+    const int k_key = (mat & 1) ? 8 + (mi ^ 4) : mi;
+    const int v_pos = (mat >> 1) * 8 + mi, v_key = (v_pos & 1) ? 8 + ((v_pos >> 1) ^ 4) : v_pos >> 1;
+    const int k_swz = ta.swz ? (k_key & 7) : 0, v_swz = ta.swz ? (v_key & 7) : 0;
+
+    int q_kvh = -1;  // kv head whose queries are in qs
     for (int j = grp; j < n_local; j += p.attn_groups) {
         const int idx = first + j;
         const int kvh = idx / n_chunks, chunk = idx - kvh * n_chunks;
@@ -1749,11 +1773,11 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
         const int last_pos = p.pos0 + M - 1;
         const int n_valid = min(kAttnChunk, last_pos + 1 - key0);
         const uint32_t gk = gi0 + (uint32_t)(j * 2 * tile_slots), gv = gk + tile_slots;
-        auto slot_ptr = [&](uint32_t g) -> unsigned char* {
+        auto slot_off = [&](uint32_t g) -> uint32_t {
             int slot;
             uint32_t gen;
             ring_locate(p, g, slot, gen);
-            return sm.ring + (size_t)slot * kSlotBytes;
+            return (uint32_t)slot * kSlotBytes;
         };
         // the boxes of a tile: every warp waits for all of them, a lane each
         auto wait_tile = [&](uint32_t g0, int tag) {
@@ -1766,42 +1790,22 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
                 ring_release(p, sm, g0 + (uint32_t)gt);
             }
         };
-
-        // ---- K tile: wait for the boxes, then overwrite the rows this pass has just written (the producer may
-        //      have copied the tile before the QKV stage of this pass stored them)
-        constexpr int kQPer = LL ? 1 : (M * 64 + 127) / 128;  // four elements per load, head_dim <= 256
-        uint2 qreg[kQPer];
-        if (!LL) {
-#pragma unroll
-            for (int u = 0; u < kQPer; ++u) {  // the first head's queries are requested before waiting for the tile
-                const int i = (gt + u * 128) * 4;
-                const int m = i / hd, e = i - m * hd;
-                qreg[u] = make_uint2(0u, 0u);
-                if (i < M * hd && q_head != kvh * group)
-                    qreg[u] = __ldcg(reinterpret_cast<const uint2*>(p.q + (size_t)m * p.d_model + (size_t)(kvh * group) * hd + e));
-            }
-        }
-        auto put_q = [&](int i, const uint2& v) { *reinterpret_cast<float4*>(qs + i) = make_float4(bf_lo(v.x), bf_hi(v.x), bf_lo(v.y), bf_hi(v.y)); };
-        // tagged handoff (one row): first look at this thread's words of q and of the fresh k and v; stale ones are asked for again where they are used
-        constexpr int kLLPer = LL ? 2 : 1;  // head_dim <= 256: at most two elements per thread
-        unsigned long long qraw[kLLPer] = {}, kraw[kLLPer] = {}, vraw[kLLPer] = {};
-        const bool has_fresh = LL && key0 <= p.pos0 && p.pos0 < key0 + kAttnChunk;
+        // The rows that this pass has just written: the producer may have copied the tile before the QKV stage of this pass stored them. They are
+        // requested before the waits, so patching the tiles costs no round trip.
+        const int fresh0 = max(p.pos0, key0), fresh1 = min(last_pos, key0 + kAttnChunk - 1);
+        const int n_fresh = fresh1 - fresh0 + 1;
+        constexpr int kFreshPer = LL ? 1 : (M * (HD ? HD : 256) / 8 + 127) / 128;
+        uint4 kpre[kFreshPer], vpre[kFreshPer];
+        constexpr int kLLPer = LL && (HD == 0 || HD == 256) ? 2 : 1;  // tagged handoff: one word per element
+        unsigned long long kraw[kLLPer] = {}, vraw[kLLPer] = {};
+        const bool has_fresh = n_fresh > 0;
         if (LL) {
 #pragma unroll
             for (int u = 0; u < kLLPer; ++u) {
                 const int e = gt + u * 128;
-                if (e < hd) {
-                    if (q_head != kvh * group) qraw[u] = ll_load1(p.ql + (size_t)(kvh * group) * hd + e);
-                    if (has_fresh) kraw[u] = ll_load1(p.kl + (size_t)kvh * hd + e), vraw[u] = ll_load1(p.vl + (size_t)kvh * hd + e);
-                }
+                if (has_fresh && e < hd) kraw[u] = ll_load1(p.kl + (size_t)kvh * hd + e), vraw[u] = ll_load1(p.vl + (size_t)kvh * hd + e);
             }
-        }
-        const int fresh0 = max(p.pos0, key0), fresh1 = min(last_pos, key0 + kAttnChunk - 1);
-        const int n_fresh = fresh1 - fresh0 + 1;
-        // the fresh K and V rows are requested here too, so patching the tiles later costs no round trip
-        constexpr int kFreshPer = LL ? 1 : (M * 32 + 127) / 128;  // head_dim <= 256: at most 32 vectors per row
-        uint4 kpre[kFreshPer], vpre[kFreshPer];
-        if (!LL) {
+        } else {
 #pragma unroll
             for (int u = 0; u < kFreshPer; ++u) {
                 const int i = gt + u * 128;
@@ -1814,249 +1818,298 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
                 }
             }
         }
-        auto patch = [&](uint32_t g0, const uint4 (&rows)[kFreshPer]) {  // over whatever the producer copied
+        auto patch = [&](uint32_t g0, const uint4 (&rows)[kFreshPer], const uint2* src, unsigned long long (&raw)[kLLPer]) {
+            if (LL) {
 #pragma unroll
-            for (int u = 0; u < kFreshPer; ++u) {
-                const int i = gt + u * 128;
-                if (i < n_fresh * vec_per_row) {
+                for (int u = 0; u < kLLPer; ++u) {
+                    const int e = gt + u * 128;
+                    if (e < hd) {
+                        while (!ll_ready(raw[u], tag_in) && ll_keep_waiting(p, ll_spins, ll_t0, stage)) raw[u] = ll_load1(src + (size_t)kvh * hd + e);
+                        int sit, off;
+                        ta.locate(p.pos0 - key0, e >> 3, sit, off);
+                        *reinterpret_cast<unsigned short*>(sm.ring + slot_off(g0 + sit) + off + (e & 7) * 2) = (unsigned short)raw[u];
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < kFreshPer; ++u) {
+                    const int i = gt + u * 128;
+                    if (i < n_fresh * vec_per_row) {
+                        const int fr = i / vec_per_row, c = i - fr * vec_per_row;
+                        int sit, off;
+                        ta.locate(fresh0 + fr - key0, c, sit, off);
+                        *reinterpret_cast<uint4*>(sm.ring + slot_off(g0 + sit) + off) = rows[u];
+                    }
+                }
+            }
+        };
+
+        for (int c0 = 0; c0 < n_cols; c0 += kAttnCols) {  // eight columns at a time
+            const int ct = min(kAttnCols, n_cols - c0);
+            if (q_kvh != kvh || n_cols > kAttnCols) {
+                // queries of these columns (nobody reads the ones before any more: the group has met at a barrier behind their scores)
+                if (LL) {
+                    for (int i0 = gt; i0 < ct * hd; i0 += 2 * 128) {
+                        unsigned long long raw[2] = {};
+                        const uint2* src = p.ql + (size_t)(kvh * group + c0) * hd;
+#pragma unroll
+                        for (int u = 0; u < 2; ++u)
+                            if (i0 + u * 128 < ct * hd) raw[u] = ll_load1(src + i0 + u * 128);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const int i = i0 + u * 128;
+                            if (i < ct * hd) {
+                                while (!ll_ready(raw[u], tag_in) && ll_keep_waiting(p, ll_spins, ll_t0, stage)) raw[u] = ll_load1(src + i);
+                                const int c = i / hd;
+                                *reinterpret_cast<unsigned short*>(qs + c * q_row + (i - c * hd) * 2) = (unsigned short)raw[u];
+                            }
+                        }
+                    }
+                } else {
+                    for (int i = gt; i < ct * vec_per_row; i += 128) {
+                        const int c = i / vec_per_row, v = i - c * vec_per_row;
+                        const int g = (c0 + c) / M, m = (c0 + c) - g * M;
+                        *reinterpret_cast<uint4*>(qs + c * q_row + v * 16) =
+                            __ldcg(reinterpret_cast<const uint4*>(p.q + (size_t)m * p.d_model + (size_t)(kvh * group + g) * hd) + v);
+                    }
+                }
+            }
+            if (c0 == 0) {
+                wait_tile(gk, M * 1000 + j);
+                if (has_fresh) patch(gk, kpre, p.kl, kraw);
+            }
+            bar_sync(bar_id, 128);  // queries and patched keys are there
+            if (j == 0 && c0 == 0) trace_mark(p, stage, 2);  // attention timeline: 2 = inputs staged, 4 = softmax done, 5 = P V done, 6 = value tile released, 7 = merged
+
+            // ---- scores: keys 32 gwarp + 16 t + {g8, 8 + (g8 ^ 4)} of columns 2 q4, 2 q4 + 1 to a lane
+            float s[2][4] = {};
+            {
+                const uint32_t q_addr = smem_u32(qs) + min(mi, ct - 1) * q_row + mat * 16;
+                const uint32_t k_row = (uint32_t)(((gwarp & 1) * 32 + k_key) * ta.row_bytes);
+                const uint32_t tile0 = gk + (uint32_t)((gwarp >> 1) * nhb);
+#pragma unroll 1  // (unrolled, here and in P V: five rows on 8000 keys 546 -> 559 us, the instruction caches)
+                for (int hb = 0; hb < (HD ? (HD + 63) / 64 : nhb); ++hb) {
+                    const uint32_t k_addr = ring_addr + slot_off(tile0 + hb) + k_row;
+#pragma unroll
+                    for (int ks = 0; ks < 4; ks += 2) {  // two steps of 16 dimensions
+                        if (!HD && ks * 16 >= hd) break;
+                        uint32_t q[4];
+                        ldmatrix4(q, q_addr + (uint32_t)((hb * 4 + ks) * 32));
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            uint32_t a[4];
+                            float d[4];
+                            ldmatrix4(a, k_addr + (uint32_t)(t * 16 * ta.row_bytes) + (uint32_t)(((ks * 2 + (mat >> 1)) ^ k_swz) << 4));
+                            mma_bf16_zero(d, a, q[0], q[1]);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) s[t][e] += d[e];
+                            if (HD || (ks + 1) * 16 < hd) {
+                                ldmatrix4(a, k_addr + (uint32_t)(t * 16 * ta.row_bytes) + (uint32_t)(((ks * 2 + 2 + (mat >> 1)) ^ k_swz) << 4));
+                                mma_bf16_zero(d, a, q[2], q[3]);
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) s[t][e] += d[e];
+                            }
+                        }
+                    }
+                }
+            }
+            // ---- softmax statistics of the chunk; the row at position pos0 + m sees keys <= pos0 + m
+            const int my_key = key0 + gwarp * 32 + g8, other = 8 + (g8 ^ 4) - g8;
+            float mx[2] = {-INFINITY, -INFINITY}, sum[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int pos = p.pos0 + (c0 + 2 * q4 + e) % M;
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float& v = s[t][e + 2 * h];
+                        v = my_key + t * 16 + h * other <= pos ? v * p.attn_scale : -INFINITY;
+                        mx[e] = fmaxf(mx[e], v);
+                    }
+#pragma unroll
+                for (int o = 4; o < 32; o *= 2) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], o));
+            }
+            if (glane < 4) *reinterpret_cast<float2*>(red + gwarp * kAttnCols + 2 * q4) = make_float2(mx[0], mx[1]);
+            bar_sync(bar_id, 128);
+            if (c0 + kAttnCols >= n_cols) release_tile(gk);  // K tile no longer needed: hand its slots back to the producer
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const float2 r = *reinterpret_cast<const float2*>(red + w * kAttnCols + 2 * q4);
+                mx[0] = fmaxf(mx[0], r.x), mx[1] = fmaxf(mx[1], r.y);
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                sum[e] = 0.f;
+                if (e >= ct) break;  // a single column
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float& v = s[i >> 1][e + 2 * (i & 1)];
+                    v = v == -INFINITY ? 0.f : expf(v - mx[e]);
+                }
+                sum[e] = (s[0][e] + s[0][e + 2]) + (s[1][e] + s[1][e + 2]);
+                if (2 * q4 + e < ct) {
+                    unsigned char* dst = ps + (2 * q4 + e) * kAttnPRow + (gwarp * 32 + 2 * g8) * 2;
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        float a = s[t][e], b = s[t][e + 2];
+#pragma unroll
+                        for (int term = 0; term < 3; ++term) {
+                            const uint32_t w = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);  // the upper halves
+                            *reinterpret_cast<uint32_t*>(dst + term * ct_max * kAttnPRow + t * 32) = w;
+                            a -= bf_lo(w), b -= bf_hi(w);  // exact
+                        }
+                    }
+                }
+#pragma unroll
+                for (int o = 4; o < 32; o *= 2) sum[e] += __shfl_xor_sync(0xffffffffu, sum[e], o);
+            }
+            if (glane < 4) *reinterpret_cast<float2*>(red + 4 * kAttnCols + gwarp * kAttnCols + 2 * q4) = make_float2(sum[0], sum[1]);
+            const int n_steps = (n_valid + 15) >> 4;  // blocks of 16 keys
+            if (c0 == 0) {  // V tile: wait and patch once per item
+                wait_tile(gv, M * 1000 + 500 + j);
+                if (has_fresh) patch(gv, vpre, p.vl, vraw);
+                // the probabilities behind the last key are zero, and so are the values that they meet
+                for (int i = gt; i < (n_steps * 16 - n_valid) * vec_per_row; i += 128) {
                     const int fr = i / vec_per_row, c = i - fr * vec_per_row;
                     int sit, off;
-                    ta.locate(fresh0 + fr - key0, c, sit, off);
-                    *reinterpret_cast<uint4*>(slot_ptr(g0 + sit) + off) = rows[u];
+                    ta.locate(n_valid + fr, c, sit, off);
+                    *reinterpret_cast<uint4*>(sm.ring + slot_off(gv + sit) + off) = make_uint4(0u, 0u, 0u, 0u);
                 }
             }
-        };
-        // tagged handoff: this pass's key or value, element by element from the tagged words
-        auto patch_tagged = [&](uint32_t g0, const uint2* src, unsigned long long (&raw)[kLLPer]) {
-#pragma unroll
-            for (int u = 0; u < kLLPer; ++u) {
-                const int e = gt + u * 128;
-                if (e < hd) {
-                    while (!ll_ready(raw[u], tag_in) && ll_keep_waiting(p, ll_spins, ll_t0, stage)) raw[u] = ll_load1(src + (size_t)kvh * hd + e);
-                    int sit, off;
-                    ta.locate(p.pos0 - key0, e >> 3, sit, off);
-                    *reinterpret_cast<unsigned short*>(slot_ptr(g0 + sit) + off + (e & 7) * 2) = (unsigned short)raw[u];
-                }
+            bar_sync(bar_id, 128);
+            if (gt < ct) {
+                const float m = fmaxf(fmaxf(red[gt], red[kAttnCols + gt]), fmaxf(red[2 * kAttnCols + gt], red[3 * kAttnCols + gt]));
+                const float* r = red + 4 * kAttnCols + gt;
+                const float l = ((r[0] + r[kAttnCols]) + r[2 * kAttnCols]) + r[3 * kAttnCols];
+                const int g = (c0 + gt) / M, row = (c0 + gt) - g * M;
+                const size_t at = (size_t)(kvh * group + g) * p.chunk_stride + chunk;
+                if (LL) ll_store(p.pl_ml + at * 2, __float_as_uint(m), tag_out), ll_store(p.pl_ml + at * 2 + 1, __float_as_uint(l), tag_out);
+                else *reinterpret_cast<float2*>(p.part_ml + (at * kPassMaxRows + row) * 2) = make_float2(m, l);
             }
-        };
-        wait_tile(gk, M * 1000 + j);
-        if (!LL) patch(gk, kpre);
-        else if (has_fresh) patch_tagged(gk, p.kl, kraw);
-        for (int g = 0; g < group; ++g) {
-            const int head = kvh * group + g;
-            bar_sync(bar_id, 128);  // patched tile visible; previous head's Ps / qs consumed
-            if (LL) {
-                if (q_head != head) {
+            if (j == 0 && c0 == 0) trace_mark(p, stage, 4);
+            // ---- P V: dimensions 16 mt + {g8, g8 + 8} of columns 2 q4, 2 q4 + 1 to a lane, two such blocks side by side from 128 dimensions on.
+            //      One or two columns: the terms are columns of one product. Either way the sums of a term over the blocks of 16 keys are added
+            //      in order, then hi + (mid + lo).
+            const int tiles = hd >= 64 ? hd / 64 : 1;
+            auto products = [&](auto packed) {
+                constexpr bool kPacked = decltype(packed)::value;
+                constexpr int kTiles = HD == 64 || M <= 2 ? 1 : 2;  // (one and two rows: their registers)
+                constexpr int kTerms = kPacked ? 1 : 3;
+                const uint32_t p_addr = smem_u32(ps) + min(mi, (kPacked ? 3 : 1) * ct - 1) * kAttnPRow + mat * 16;
+#pragma unroll 1
+                for (int mt0 = gwarp * tiles; mt0 < (gwarp + 1) * tiles && mt0 * 16 < hd; mt0 += kTiles) {
+                    const int nt = HD >= 64 ? kTiles : min(kTiles, tiles);
+                    uint32_t v_addr[kTiles];
 #pragma unroll
-                    for (int u = 0; u < kLLPer; ++u) {
-                        const int e = gt + u * 128;
-                        if (e < hd) {
-                            if (g > 0) qraw[u] = ll_load1(p.ql + (size_t)head * hd + e);
-                            while (!ll_ready(qraw[u], tag_in) && ll_keep_waiting(p, ll_spins, ll_t0, stage)) qraw[u] = ll_load1(p.ql + (size_t)head * hd + e);
-                            qs[e] = __uint_as_float((uint32_t)qraw[u] << 16);
+                    for (int w = 0; w < kTiles; ++w) {
+                        const int c = (mt0 + w) * 2 + (mat & 1);  // 16-byte chunk of the head
+                        v_addr[w] = ring_addr + (uint32_t)(v_key * ta.row_bytes) + (uint32_t)(((nhb > 1 ? c & 7 : c) ^ v_swz) << 4);
+                    }
+                    const int hb = nhb > 1 ? mt0 >> 2 : 0;  // (both blocks lie in one box)
+                    float acc[kTiles][kTerms][4] = {};
+#pragma unroll 1
+                    for (int kk = 0; kk < kAttnChunk / 16; kk += 2) {
+                        if (kk >= n_steps) break;
+                        uint32_t b[kTerms][4];
+#pragma unroll
+                        for (int term = 0; term < kTerms; ++term) ldmatrix4(b[term], p_addr + (uint32_t)(term * ct_max * kAttnPRow + kk * 32));
+                        const uint32_t box = slot_off(gv + (uint32_t)((kk >> 2) * nhb + hb)) + (uint32_t)((kk & 3) * 16 * ta.row_bytes);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            if (kk + u >= n_steps) break;
+#pragma unroll
+                            for (int w = 0; w < kTiles; ++w) {
+                                if (w >= nt) break;
+                                uint32_t a[4];
+                                ldmatrix4_trans(a, v_addr[w] + box + (uint32_t)(u * 16 * ta.row_bytes));
+#pragma unroll
+                                for (int term = 0; term < kTerms; ++term) {
+                                    float d[4];
+                                    mma_bf16_zero(d, a, b[term][2 * u], b[term][2 * u + 1]);
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) acc[w][term][e] += d[e];
+                                }
+                            }
                         }
                     }
-                }
-            } else if (q_head != head) {
 #pragma unroll
-                for (int u = 0; u < kQPer; ++u) {
-                    const int i = (gt + u * 128) * 4;
-                    const int m = i / hd, e = i - m * hd;
-                    if (i < M * hd) put_q(i, g == 0 ? qreg[u] : __ldcg(reinterpret_cast<const uint2*>(p.q + (size_t)m * p.d_model + (size_t)head * hd + e)));
-                }
-            }
-            q_head = head;
-            bar_sync(bar_id, 128);
-
-            if (j == 0 && g == 0) trace_mark(p, stage, 2);  // attention timeline: 2 = inputs staged, 4 = softmax done, 5 = P V done, 6 = value tile released, 7 = merged
-            // ---- scores: thread t owns key key0 + t in the end. A score is the sum of four partial sums (16-byte chunk parity x
-            //      half of the chunk), added in a fixed order. The four lanes of a quad take one of them each, for four keys
-            //      (keys 8 apart, so that the eight quads of a warp read rows of eight different swizzles), and exchange them
-            //      afterwards: a query element that comes from shared memory then serves four keys instead of one.
-            float sc[M];
-            {
-                float sp[M][4];  // [row][key of the quad]
+                    for (int w = 0; w < kTiles; ++w)
 #pragma unroll
-                for (int m = 0; m < M; ++m) sp[m][0] = sp[m][1] = sp[m][2] = sp[m][3] = 0.f;
-                const int par = (glane >> 1) & 1, half = glane & 1, kq = glane >> 2;  // key of the quad: 32 gwarp + 8 i + kq
-                const int rg = (gwarp * 32) / kBoxKeys, rr = (gwarp * 32) % kBoxKeys + kq;  // (rr + 8 i) & 7 == kq
-                auto chunk_pair = [&](const unsigned char* krow, const float* qrow, int cc0) {
-                    const int cc = cc0 + par;
-                    const unsigned char* kp = krow + ((ta.swz ? (cc ^ kq) : cc) << 4);
-                    uint2 kv[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) kv[i] = *reinterpret_cast<const uint2*>(kp + i * 8 * ta.row_bytes);
-#pragma unroll
-                    for (int m = 0; m < M; ++m) {
-                        const float4 qv = *reinterpret_cast<const float4*>(qrow + m * hd + cc0 * 8);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            float a = sp[m][i];
-                            a = fmaf(qv.x, bf_lo(kv[i].x), a);
-                            a = fmaf(qv.y, bf_hi(kv[i].x), a);
-                            a = fmaf(qv.z, bf_lo(kv[i].y), a);
-                            a = fmaf(qv.w, bf_hi(kv[i].y), a);
-                            sp[m][i] = a;
-                        }
-                    }
-                };
-#pragma unroll 1
-                for (int hb = 0; hb < nhb; ++hb) {
-                    const unsigned char* krow = slot_ptr(gk + rg * nhb + hb) + rr * ta.row_bytes + half * 8;
-                    const float* qrow = qs + (hb * 8 + par) * 8 + half * 4;
-                    if (HD >= 64) {
-#pragma unroll
-                        for (int cc0 = 0; cc0 < 8; cc0 += 2) chunk_pair(krow, qrow, cc0);
-                    } else {
-                        for (int cc0 = 0; cc0 < box_cols / 8; cc0 += 2) chunk_pair(krow, qrow, cc0);  // an even number: head_dim >= 16
-                    }
-                }
-                const int home = ((glane & 7) << 2) | (glane >> 3);  // the lane that ends up with this lane's key
-#pragma unroll
-                for (int m = 0; m < M; ++m) {
-                    const float b0 = __shfl_xor_sync(0xffffffffu, half ? sp[m][0] : sp[m][1], 1), b1 = __shfl_xor_sync(0xffffffffu, half ? sp[m][2] : sp[m][3], 1);
-                    const float t0 = (half ? sp[m][1] : sp[m][0]) + b0, t1 = (half ? sp[m][3] : sp[m][2]) + b1;  // keys half, half + 2
-                    const float c = __shfl_xor_sync(0xffffffffu, par ? t0 : t1, 2);
-                    sc[m] = __shfl_sync(0xffffffffu, (par ? t1 : t0) + c, home);
-                }
-            }
-            // ---- chunk-local softmax statistics; the row at position pos0+m sees keys <= pos0+m
-            const int key = key0 + gt;
-            float cmax[M];
-#pragma unroll
-            for (int m = 0; m < M; ++m) {
-                const bool ok = key <= p.pos0 + m;
-                sc[m] = ok ? sc[m] * p.attn_scale : -INFINITY;
-                const float v = warp_max(sc[m]);
-                if (glane == 0) red[gwarp * kPassMaxRows + m] = v;
-            }
-            bar_sync(bar_id, 128);
-            if (g == group - 1) release_tile(gk);  // K tile no longer needed: hand its slots back to the producer
-#pragma unroll
-            for (int m = 0; m < M; ++m)
-                cmax[m] = fmaxf(fmaxf(red[0 * kPassMaxRows + m], red[1 * kPassMaxRows + m]),
-                                fmaxf(red[2 * kPassMaxRows + m], red[3 * kPassMaxRows + m]));
-            bar_sync(bar_id, 128);
-#pragma unroll
-            for (int m = 0; m < M; ++m) {
-                const float pe = (sc[m] == -INFINITY) ? 0.f : expf(sc[m] - cmax[m]);
-                Ps[m * kAttnChunk + gt] = pe;
-                const float v = warp_sum(pe);
-                if (glane == 0) red[gwarp * kPassMaxRows + m] = v;
-            }
-            if (g == 0) {  // V tile: wait and patch once per item
-                wait_tile(gv, M * 1000 + 500 + j);
-                if (!LL) patch(gv, vpre);
-                else if (has_fresh) patch_tagged(gv, p.vl, vraw);
-            }
-            bar_sync(bar_id, 128);
-            if (gt < M) {
-                const float l = ((red[0 * kPassMaxRows + gt] + red[1 * kPassMaxRows + gt]) + red[2 * kPassMaxRows + gt]) + red[3 * kPassMaxRows + gt];
-                if (LL) ll_store(p.pl_ml + ((size_t)head * p.chunk_stride + chunk) * 2 + 1, __float_as_uint(l), tag_out);
-                else p.part_ml[(((size_t)head * p.chunk_stride + chunk) * kPassMaxRows + gt) * 2 + 1] = l;
-            }
-            if (gt == 0) {
-#pragma unroll
-                for (int m = 0; m < M; ++m) {
-                    if (LL) ll_store(p.pl_ml + ((size_t)head * p.chunk_stride + chunk) * 2 + 0, __float_as_uint(cmax[m]), tag_out);
-                    else p.part_ml[(((size_t)head * p.chunk_stride + chunk) * kPassMaxRows + m) * 2 + 0] = cmax[m];
-                }
-            }
-            if (j == 0 && g == 0) trace_mark(p, stage, 4);
-            // ---- P V: thread (c, kg) owns the 8 output dimensions of 16-byte chunk c for the keys kg, kg + 8, ... (one
-            //      16-byte read per key); the eight key groups of a chunk sit in neighbouring lanes and are added in pairs
-            //      (lanes 1, 2, 4 apart). Up to six rows share one sweep over the keys (more rows: two or more sweeps).
-            //      Probabilities past n_valid are zero and the tile rows behind them hold finite cache contents.
-            {
-                constexpr int kRowBatch = M <= 6 ? M : (M <= 12 ? (M + 1) / 2 : 4);
-                const int kg = gt & 7;
-                const int n_steps = (n_valid + 7) >> 3;  // keys kg + 8 i, i < n_steps
-                for (int c0 = 0; c0 < (hd >> 3); c0 += 16) {  // every lane runs the loop (the sums below are warp-wide)
-                    const bool active = c0 + (gt >> 3) < (hd >> 3);
-                    const int c = active ? c0 + (gt >> 3) : 0;
-                    const int hb = (nhb > 1) ? (c >> 3) : 0, cc = (nhb > 1) ? (c & 7) : c;
-                    const int coff = (ta.swz ? (cc ^ kg) : cc) << 4;  // key & 7 == kg for every key of this thread
-#pragma unroll 1
-                    for (int m0 = 0; m0 < M; m0 += kRowBatch) {
-                        float acc[kRowBatch][8];
-#pragma unroll
-                        for (int u = 0; u < kRowBatch; ++u)
-#pragma unroll
-                            for (int d8 = 0; d8 < 8; ++d8) acc[u][d8] = 0.f;
-#pragma unroll 1
-                        for (int b = 0; b < kAttnChunk / kBoxKeys; ++b) {  // the two boxes of 64 keys
-                            const unsigned char* vb = slot_ptr(gv + b * nhb + hb) + kg * ta.row_bytes + coff;
-                            const float* pb = Ps + m0 * kAttnChunk + b * kBoxKeys + kg;
-                            auto step = [&](int i) {
-                                const uint4 vv = *reinterpret_cast<const uint4*>(vb + i * 8 * ta.row_bytes);
-                                const float vf[8] = {bf_lo(vv.x), bf_hi(vv.x), bf_lo(vv.y), bf_hi(vv.y), bf_lo(vv.z), bf_hi(vv.z), bf_lo(vv.w), bf_hi(vv.w)};
-#pragma unroll
-                                for (int u = 0; u < kRowBatch; ++u)
-                                    if (m0 + u < M) {
-                                        const float pw = pb[u * kAttnChunk + i * 8];
-#pragma unroll
-                                        for (int d8 = 0; d8 < 8; ++d8) acc[u][d8] = fmaf(pw, vf[d8], acc[u][d8]);
-                                    }
-                            };
-                            const int n = n_steps - b * (kBoxKeys / 8);
-                            if (n >= kBoxKeys / 8) {
-#pragma unroll (M <= 4 ? 4 : 2)
-                                for (int i = 0; i < kBoxKeys / 8; ++i) step(i);
+                        for (int e = 0; e < 4; ++e) {
+                            const int col = 2 * q4 + (e & 1), dim = (mt0 + w) * 16 + g8 + (e >> 1) * 8;
+                            float o;
+                            if constexpr (kPacked) {  // the terms of a column are 1 or 2 columns apart
+                                const float next = __shfl_down_sync(0xffffffffu, acc[w][0][e], 1), after = __shfl_down_sync(0xffffffffu, acc[w][0][e], 2);
+                                o = ct == 1 ? acc[w][0][e] + (acc[w][0][e | 1] + next) : acc[w][0][e] + (next + after);
                             } else {
-#pragma unroll 1
-                                for (int i = 0; i < n; ++i) step(i);
+                                o = acc[w][0][e] + (acc[w][1][e] + acc[w][2][e]);
+                            }
+                            if (w < nt && col < ct) {
+                                const int g = (c0 + col) / M, m = (c0 + col) - g * M;
+                                const size_t at = (size_t)(kvh * group + g) * p.chunk_stride + chunk;
+                                if (LL) ll_store(p.pl_acc + at * hd + dim, __float_as_uint(o), tag_out);
+                                else p.part_acc[(at * kPassMaxRows + m) * hd + dim] = o;
                             }
                         }
-#pragma unroll
-                        for (int u = 0; u < kRowBatch; ++u)
-                            if (m0 + u < M) {
-                                // sums over the eight lanes, every lane left with the dimension of its number
-                                float r4[4], r2[2];
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) {
-                                    const float b = __shfl_xor_sync(0xffffffffu, (kg & 1) ? acc[u][2 * i] : acc[u][2 * i + 1], 1);
-                                    r4[i] = ((kg & 1) ? acc[u][2 * i + 1] : acc[u][2 * i]) + b;
-                                }
-#pragma unroll
-                                for (int i = 0; i < 2; ++i) {
-                                    const float b = __shfl_xor_sync(0xffffffffu, (kg & 2) ? r4[2 * i] : r4[2 * i + 1], 2);
-                                    r2[i] = ((kg & 2) ? r4[2 * i + 1] : r4[2 * i]) + b;
-                                }
-                                const float b = __shfl_xor_sync(0xffffffffu, (kg & 4) ? r2[0] : r2[1], 4);
-                                const float sum = ((kg & 4) ? r2[1] : r2[0]) + b;
-                                if (active) {
-                                    if (LL) ll_store(p.pl_acc + ((size_t)head * p.chunk_stride + chunk) * hd + c * 8 + kg, __float_as_uint(sum), tag_out);
-                                    else p.part_acc[(((size_t)head * p.chunk_stride + chunk) * kPassMaxRows + m0 + u) * hd + c * 8 + kg] = sum;
-                                }
-                            }
-                    }
                 }
-            }
+            };
+            if (M <= 2 && n_cols <= 2) products(std::true_type{});
+            else products(std::false_type{});
         }
+        q_kvh = kvh;
         if (j == 0) trace_mark(p, stage, 5);
-        bar_sync(bar_id, 128);
-        release_tile(gv);
+        // the first warp hands the value tile back when all four have read it
+        if (gwarp == 0) {
+            bar_sync(kAttnDoneBar + grp, 128);
+            release_tile(gv);
+        } else {
+            bar_arrive(kAttnDoneBar + grp, 128);
+        }
         if (j == 0) trace_mark(p, stage, 6);
     }
 }
 
-// Merging the chunks of a head, 32 output dimensions (a lane each) and one row at a time: `unit` of n_heads * rows * parts. The
-// chunks are merged in ascending order with explicit roundings, so the arithmetic is the same in every instantiation.
+// Merging the chunks of a head, 32 output dimensions and one row at a time: `unit` of n_heads * rows * parts. A lane has four dimensions of every
+// fourth chunk (with one dimension of every chunk the chain of additions and shuffles was four times as long).
 struct MergeUnit {
-    int head, m, e;
+    int head, m, e, sub;
     bool act;
     __device__ __forceinline__ MergeUnit(int unit, int rows, int hd) {
         const int parts = (hd + 31) >> 5, lane = threadIdx.x & 31;
         const int hm = unit / parts;
-        head = hm / rows, m = hm - head * rows, e = (unit - hm * parts) * 32 + lane;
+        head = hm / rows, m = hm - head * rows, e = (unit - hm * parts) * 32 + (lane & 7) * 4, sub = lane >> 3;
         act = e < hd;
     }
 };
-// two neighbouring lanes' results as one word of two bf16, in the even lane
-__device__ __forceinline__ uint32_t merged_pair(float acc, float l) {
-    const uint32_t ob = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(__fdiv_rn(acc, l)));
-    return ob | (__shfl_down_sync(0xffffffffu, ob, 1) << 16);
-}
+// The running maximum, sum of weights and sums of a merge. 32 chunks come in at a time: lane i works out the weight exp(m_i - maximum) of
+// chunk i, every lane adds the partial results of its chunks in ascending order, and the four lanes of a dimension are added in the end. The
+// same arithmetic in every instantiation.
+struct Merge {
+    float mx = -INFINITY, l = 0.f, w;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    // ml: (maximum, sum of weights) of this lane's chunk, -inf past the last one
+    __device__ __forceinline__ void begin(float2 ml) {
+        const float m = fmaxf(mx, warp_max(ml.x)), s = expf(mx - m);
+        mx = m, w = expf(ml.x - m);
+        l = __fmaf_rn(l, s, warp_sum(__fmul_rn(w, ml.y)));
+        acc = make_float4(__fmul_rn(acc.x, s), __fmul_rn(acc.y, s), __fmul_rn(acc.z, s), __fmul_rn(acc.w, s));
+    }
+    __device__ __forceinline__ void add(int i, const float4& v) {  // chunk i of the 32 (another one for every lane >> 3)
+        const float f = __shfl_sync(0xffffffffu, w, i);
+        acc = make_float4(__fmaf_rn(f, v.x, acc.x), __fmaf_rn(f, v.y, acc.y), __fmaf_rn(f, v.z, acc.z), __fmaf_rn(f, v.w, acc.w));
+    }
+    // the four dimensions as two words of two bf16, in every lane
+    __device__ __forceinline__ uint2 result() const {
+        auto of = [&](float v) {
+            v += __shfl_xor_sync(0xffffffffu, v, 8);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(__fdiv_rn(v, l)));
+        };
+        const uint32_t a = of(acc.x), b = of(acc.y), c = of(acc.z), d = of(acc.w);
+        return make_uint2(a | (b << 16), c | (d << 16));
+    }
+};
 
 // Tagged handoff: the warps without attention items merge. They ask for the chunks' (maximum, sum of weights) until the tags are
 // this stage's, then for the sums of 16 chunks at a time. Nobody who produces a partial result ever waits for a merge, so the
@@ -2072,7 +2125,8 @@ __device__ __forceinline__ void merge_tagged(const PassParams& p, int stage, int
     for (int u = blockIdx.x + warp * gridDim.x; u < units; u += n_warps * gridDim.x) {
         const MergeUnit mu(u, 1, hd);
         const size_t chunk0 = (size_t)mu.head * p.chunk_stride;
-        float mx = -INFINITY, l = 0.f, acc = 0.f;
+        Merge mg;
+#pragma unroll 1
         for (int c0 = 0; c0 < n_chunks; c0 += 32) {
             unsigned long long rm = 0, rl = 0;
             bool stale_ml = c0 + lane < n_chunks;
@@ -2085,79 +2139,75 @@ __device__ __forceinline__ void merge_tagged(const PassParams& p, int stage, int
                 if (!__all_sync(0xffffffffu, ll_keep_waiting(p, spins, t0, stage))) break;
                 __nanosleep(100u);
             }
-            const MergeFactors mf(c0 + lane < n_chunks ? make_float2(__uint_as_float((uint32_t)rm), __uint_as_float((uint32_t)rl)) : make_float2(-INFINITY, 0.f), mx);
+            mg.begin(c0 + lane < n_chunks ? make_float2(__uint_as_float((uint32_t)rm), __uint_as_float((uint32_t)rl)) : make_float2(-INFINITY, 0.f));
 #pragma unroll 1
             for (int c1 = 0; c1 < 32 && c0 + c1 < n_chunks; c1 += 16) {
-                unsigned long long ra[16] = {};
+                unsigned long long ra[4][4] = {};
                 unsigned stale = 0u;
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    if (mu.act && c0 + c1 + i < n_chunks) stale |= 1u << i;
+                for (int i = 0; i < 4; ++i)
+                    if (mu.act && c0 + c1 + 4 * i + mu.sub < n_chunks) stale |= 1u << i;
                 for (;;) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (stale & (1u << i)) ra[i] = ll_load1(p.pl_acc + (chunk0 + c0 + c1 + i) * hd + mu.e);
+                    for (int i = 0; i < 4; ++i)
+                        if (stale & (1u << i)) {
+                            const uint2* src = p.pl_acc + (chunk0 + c0 + c1 + 4 * i + mu.sub) * hd + mu.e;
+                            ll_load2(src, ra[i][0], ra[i][1]);
+                            ll_load2(src + 2, ra[i][2], ra[i][3]);
+                        }
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if ((stale & (1u << i)) && ll_ready(ra[i], tag_out)) stale &= ~(1u << i);
+                    for (int i = 0; i < 4; ++i)
+                        if ((stale & (1u << i)) && ll_ready(ra[i][0], tag_out) && ll_ready(ra[i][1], tag_out) && ll_ready(ra[i][2], tag_out) && ll_ready(ra[i][3], tag_out))
+                            stale &= ~(1u << i);
                     if (!__any_sync(0xffffffffu, stale != 0u)) break;
                     if (!__all_sync(0xffffffffu, ll_keep_waiting(p, spins, t0, stage))) break;
                     __nanosleep(100u);
                 }
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    if (c0 + c1 + i < n_chunks) {
-                        float s_old, s_new, cl;
-                        mf.of(c1 + i, s_old, s_new, cl);
-                        acc = __fmaf_rn(acc, s_old, __fmul_rn(__uint_as_float((uint32_t)ra[i]), s_new));
-                        l = __fmaf_rn(l, s_old, __fmul_rn(cl, s_new));
-                    }
-                }
+                for (int i = 0; i < 4; ++i)  // (chunks past the last one weigh nothing)
+                    mg.add(c1 + 4 * i + mu.sub, make_float4(__uint_as_float((uint32_t)ra[i][0]), __uint_as_float((uint32_t)ra[i][1]), __uint_as_float((uint32_t)ra[i][2]),
+                                                            __uint_as_float((uint32_t)ra[i][3])));
             }
         }
-        const uint32_t pair = merged_pair(acc, l);
-        if (mu.act && (lane & 1) == 0) ll_store(p.al + (((size_t)mu.head * hd + mu.e) >> 1), pair, tag_out);
+        const uint2 out = mg.result();
+        if (mu.act && mu.sub < 2) ll_store(p.al + (((size_t)mu.head * hd + mu.e) >> 1) + mu.sub, mu.sub ? out.y : out.x, tag_out);
     }
 }
 
 // Without tags: behind a grid barrier of its own the heads and rows are dealt to all warps of the grid. (Merged by the group whose
 // report completed a head, five rows cost 4 us behind the last item at five chunks and 29 us at 65: 32 of the 148 CTAs, and
-// in each a chain of 18 trips to L2. Attention stage of five rows 17.2 -> 13.3 us at 512 positions of the 7B shape, 91 -> 58 us at 8192,
-// where the shorter items below have a share; two and three rows at 512 positions cost the same either way.)
+// in each a chain of 18 trips to L2. Two and three rows at 512 positions cost the same either way.)
 template <int M>
 __device__ __forceinline__ void merge_all(const PassParams& p) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, hd = p.head_dim;
     const int units = p.n_heads * M * ((hd + 31) >> 5);
+#pragma unroll 1
     for (int u = blockIdx.x + warp * gridDim.x; u < units; u += kPassConsumerWarps * gridDim.x) {
         const MergeUnit mu(u, M, hd);
-        const int nc = (p.pos0 + mu.m) / kAttnChunk + 1, e = mu.act ? mu.e : 0;
-        float mx = -INFINITY, l = 0.f, acc = 0.f;
+        const int nc = (p.pos0 + mu.m) / kAttnChunk + 1;
+        const size_t row0 = (size_t)mu.head * p.chunk_stride * kPassMaxRows + mu.m;
+        const float* src = p.part_acc + (row0 + (size_t)mu.sub * kPassMaxRows) * hd + (mu.act ? mu.e : 0);
+        Merge mg;
+#pragma unroll 1
         for (int c0 = 0; c0 < nc; c0 += 32) {
-            const size_t row0 = ((size_t)mu.head * p.chunk_stride + c0) * kPassMaxRows + mu.m;
-            float pa[32];
+            const float2 ml = c0 + lane < nc ? __ldcg(reinterpret_cast<const float2*>(p.part_ml + (row0 + (size_t)(c0 + lane) * kPassMaxRows) * 2))
+                                             : make_float2(-INFINITY, 0.f);
+            float4 pa[8];
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                pa[i] = 0.f;
-                if ((i < 16 || c0 + 16 < nc) && c0 + i < nc) pa[i] = __ldcg(p.part_acc + (row0 + (size_t)i * kPassMaxRows) * hd + e);
+            for (int i = 0; i < 8; ++i) {
+                pa[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (c0 + 4 * i + mu.sub < nc) pa[i] = __ldcg(reinterpret_cast<const float4*>(src + (size_t)(c0 + 4 * i) * kPassMaxRows * hd));
             }
-            const MergeFactors mf(c0 + lane < nc ? __ldcg(reinterpret_cast<const float2*>(p.part_ml + (row0 + (size_t)lane * kPassMaxRows) * 2))
-                                                 : make_float2(-INFINITY, 0.f), mx);
+            mg.begin(ml);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                if (c0 + i < nc) {
-                    float s_old, s_new, cl;
-                    mf.of(i, s_old, s_new, cl);
-                    acc = __fmaf_rn(acc, s_old, __fmul_rn(pa[i], s_new));
-                    l = __fmaf_rn(l, s_old, __fmul_rn(cl, s_new));
-                }
-            }
+            for (int i = 0; i < 8; ++i) mg.add(4 * i + mu.sub, pa[i]);  // (chunks past the last one weigh nothing)
         }
-        const uint32_t pair = merged_pair(acc, l);
-        if (mu.act && (lane & 1) == 0) *reinterpret_cast<uint32_t*>(p.a + (size_t)mu.m * p.d_model + (size_t)mu.head * hd + mu.e) = pair;
+        const uint2 out = mg.result();
+        if (mu.act && mu.sub == 0) *reinterpret_cast<uint2*>(p.a + (size_t)mu.m * p.d_model + (size_t)mu.head * hd + mu.e) = out;
     }
 }
 
-template <int M, bool LL>
+template <int M, bool LL, int HD>
 __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassSmem& sm, uint32_t& gi, unsigned& merge_target, int stage) {
     const int warp = threadIdx.x >> 5;
     int n_chunks, first;
@@ -2168,9 +2218,7 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
     else stage_begin(p, stage);      // all consumer warps, also those without attention work
     const int item_warps = 4 * p.attn_groups;
     if (warp < item_warps) {
-        if (p.head_dim == 128) attn_items<M, LL, 128>(p, st, sm, gi0, stage, n_chunks, first, n_local);
-        else if (p.head_dim == 64) attn_items<M, LL, 64>(p, st, sm, gi0, stage, n_chunks, first, n_local);
-        else attn_items<M, LL, 0>(p, st, sm, gi0, stage, n_chunks, first, n_local);
+        attn_items<M, LL, HD>(p, st, sm, gi0, stage, n_chunks, first, n_local);
     } else if (LL) {
         merge_tagged(p, stage, n_chunks, item_warps, kPassConsumerWarps - item_warps);
     }
@@ -2185,7 +2233,9 @@ __device__ void attn_stage(const PassParams& p, const StageDesc& st, const PassS
 }
 
 // ============================================================================================ the kernel
-template <int M, bool LL>
+// HD: the head size that attention is compiled for, 0: any. (A kernel each: the code of a pass is larger than the instruction caches, and code in
+// between that does not run costs as well.)
+template <int M, bool LL, int HD>
 __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_constant__ PassParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -2276,7 +2326,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
             if (!LL) stage_begin(p, s);  // the LM head wants the hidden state of all CTAs; the producer warp does the work (finish_rows)
             if constexpr (!kFewRows<M>) finish_stage<M>(p, sm);
         } else if (st.type == kStAttn) {
-            attn_stage<M, LL>(p, st, sm, gi, merge_target, s);
+            attn_stage<M, LL, HD>(p, st, sm, gi, merge_target, s);
         } else {
             gemv_stage<M, LL>(p, st, sm, gi, s);
         }
