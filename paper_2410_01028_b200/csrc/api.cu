@@ -117,7 +117,7 @@ static bool plan_pass(const DeviceInfo& dv, const asd_config& c, int M, PassPlan
     // per-pair partial sums; when a CTA has fewer than 8 groups of 8 pairs up to 15 warps keep copies (at most 15 / groups
     // copies of at most 8 * groups pairs: 120 pairs in all)
     const size_t psum = ((size_t)std::max<long long>(np_max, 120) * 2 * M * 4 + 15) & ~(size_t)15;
-    const size_t misc = ((size_t)16 * kPassMaxRows * 4 * 4 + 32 + 64 * 4 + 8 * 4 * 4 + kPassMaxRows * 4 + 15) & ~(size_t)15;  // reduction scratch, flags, slot generations, split table, tokens
+    const size_t misc = ((size_t)16 * kPassMaxRows * 4 * 4 + 32 + 64 * 4 + 8 * 4 * 4 + kPassMaxRows * 4 + 8 * 16 * 2 + 15) & ~(size_t)15;  // reduction scratch, flags, slot generations, split table, tokens, warp sets
     const size_t attn_scratch = (size_t)attn_scratch_bytes(M, c.n_heads / c.n_kv_heads, c.head_dim);
     // Activation window: the longest reduction dimension (in segments of 256 inputs) cut into as few windows as leave
     // the ring 20 slots. Every further window costs a stage of a multi-row pass a block-wide refill, every slot less
@@ -600,7 +600,7 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     p.hd_shift = 0;
     if ((c.head_dim & (c.head_dim - 1)) == 0)
         while ((1 << p.hd_shift) < c.head_dim) ++p.hd_shift;
-    p.eps = c.rms_eps;
+    p.eps = c.rms_eps, p.inv_d = 1.0f / (float)d;
     p.attn_scale = 1.0f / sqrtf((float)c.head_dim);
     p.rope_cos = x->at<float>(ly.rope_cos);
     p.rope_sin = x->at<float>(ly.rope_sin);
@@ -629,7 +629,7 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     const int table = head_only ? 2 : (use_mask ? 1 : 0);
     p.stages = x->at<StageDesc>(ly.stage_tab) + (size_t)table * ly.max_stages;
     const int n_table = head_only ? 2 : (use_mask ? x->n_stages_draft : x->n_stages_full);
-    p.n_stages = lm_head ? n_table : n_table - 1;
+    p.n_stages = lm_head ? n_table : n_table - 1, p.finish_stage = n_table - 2;
     p.argmax_out = dev_argmax_out ? dev_argmax_out : x->at<int>(ly.argmax);
     p.margin_out = reinterpret_cast<float*>(x->at<int>(ly.argmax) + 32);  // second half of the argmax block
     p.accept_out = accept ? x->at<int>(ly.accept) : nullptr;
@@ -654,7 +654,7 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     p.embed_direct = (p.use_ll || (M == 2 && d <= kPassConsumers * 12 && pass_wseg(M, pl.xs_bytes) * kSegK >= d)) ? 1 : 0;
     const int grid = x->dev->num_sms;
     ASD_CUDA(x, launch_pass(M, p, grid, pl.smem, s));
-    x->bar_base += (uint32_t)(p.use_ll ? n_table - 2 : p.n_stages) * (uint32_t)grid;  // (tagged handoff: nobody arrives behind the finish stage)
+    x->bar_base += (uint32_t)(p.use_ll ? p.finish_stage : p.n_stages) * (uint32_t)grid;  // (tagged handoff: nobody arrives behind the finish stage)
     if (!p.use_ll && !head_only)  // one arrival per CTA and attention stage
         for (int l = 0; l < L; ++l) x->merge_base += (use_mask && x->skip_attn[l]) ? 0u : (uint32_t)grid;
     x->pass_tag += (uint32_t)ly.max_stages + 1u;

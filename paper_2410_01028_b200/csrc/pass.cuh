@@ -83,7 +83,7 @@ struct PassParams {
     const __nv_bfloat16* embed;
     int d_model, vocab, kv_dim, head_dim, n_heads, n_kv_heads, d_ffn;
     int hd_shift;  // log2(head_dim) when head_dim is a power of two, else 0 (divisions instead of shifts)
-    float eps, attn_scale;
+    float eps, inv_d, attn_scale;  // inv_d: 1 / d_model
     const float *rope_cos, *rope_sin;
     float* x;
     __nv_bfloat16 *q, *a, *t;
@@ -107,7 +107,7 @@ struct PassParams {
     long long wait_cycles;    // cycle budget of every bounded wait of the pass
     int* err;
     const StageDesc* stages;
-    int n_stages;
+    int n_stages, finish_stage;  // finish_stage: index of the finish stage; the LM head may follow it
     int* argmax_out;
     float* margin_out;  // [M] top-1 minus top-2 logit of every row (the confidence that ends a draft run early), or null
     int* accept_out;   // greedy verification: accepted drafts, then the tokens (null: none)
@@ -162,6 +162,7 @@ struct PassSmem {
     int* flag;    // [8]
     volatile unsigned* consumed;  // [64] generations of each ring slot that consumers have finished with
     const int* split;             // [8][4] per stage type: this CTA's first pair, pair count, groups of 16 rows, warp sets per group
+    const unsigned short* warp_set;  // [8][16] per stage type and warp: warp set | first group << 8 (divisions that a stage would start with)
     const int* tok;               // [16] the rows' tokens, clamped to the vocabulary
     float* psum;
     unsigned char* reg_a;
@@ -241,21 +242,14 @@ __device__ __forceinline__ bool ring_spin_consumed(const PassParams& p, const Pa
     }
 }
 
-// consumer: wait until ring item g has landed; returns the slot
-__device__ __forceinline__ int ring_wait_full(const PassParams& p, const PassSmem& sm, uint32_t g, int stage, int tag) {
-    int slot;
-    uint32_t gen;
-    ring_locate(p, g, slot, gen);
-    if (gen > 0 && !ring_spin_consumed(p, sm, slot, gen, kErrFullWait, stage, g, tag)) return slot;
+// consumer: wait until ring item g has landed in its slot
+__device__ __forceinline__ void ring_wait_full(const PassParams& p, const PassSmem& sm, uint32_t g, int slot, uint32_t gen, int stage, int tag) {
+    if (gen > 0 && !ring_spin_consumed(p, sm, slot, gen, kErrFullWait, stage, g, tag)) return;
     mbar_wait(&sm.full[slot], gen & 1, p.err, kErrFullWait, stage, g, slot, tag, p.wait_cycles);
-    return slot;
 }
-// consumer: one thread, after all readers of the slot are done (warp or group barrier before the call)
-__device__ __forceinline__ void ring_release(const PassParams& p, const PassSmem& sm, uint32_t g) {
-    int slot;
-    uint32_t gen;
-    ring_locate(p, g, slot, gen);
-    __threadfence_block();  // the readers' shared-memory loads are ordered before the slot is handed back
+// consumer: one thread, after all readers of the slot are done (warp or group barrier before the call, which with the arrival's
+// release orders their loads before the slot is handed back)
+__device__ __forceinline__ void ring_release(const PassSmem& sm, int slot, uint32_t gen) {
     sm.consumed[slot] = gen + 1;
     mbar_arrive(&sm.empty[slot]);
 }
@@ -570,7 +564,7 @@ __device__ __forceinline__ float4 load_row4_of(const float* xf, const __nv_bfloa
 }
 template <int M>
 __device__ __forceinline__ void norm_rows_body(const float* xf, const __nv_bfloat16* emb, const int* tok, const __nv_bfloat16* gain, int n_in, int wlen,
-                                               int xstride, float eps, __nv_bfloat16* xs, float* red) {
+                                               int xstride, float inv_d, float eps, __nv_bfloat16* xs, float* red) {
     constexpr int kBatches = (M + 5) / 6, kRB = (M + kBatches - 1) / kBatches;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint2 gv[3];
@@ -616,7 +610,7 @@ __device__ __forceinline__ void norm_rows_body(const float* xf, const __nv_bfloa
                 float s = 0.f;
 #pragma unroll
                 for (int w = 0; w < kPassConsumerWarps; ++w) s += red[w * (kPassMaxRows * 4) + m];
-                const float inv = 1.0f / sqrtf(s / (float)n_in + eps);
+                const float inv = __frsqrt_rn(fmaf(s, inv_d, eps));
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     const int i = (tid + c * kPassConsumers) * 4;
@@ -644,7 +638,7 @@ __device__ __forceinline__ void norm_rows_body(const float* xf, const __nv_bfloa
 // butterflies are added in ascending order.
 template <int M>
 __device__ __forceinline__ void norm_rows_narrow(const float* xf, const __nv_bfloat16* emb, const int* tok, const __nv_bfloat16* gain, int n_in, int wlen,
-                                                 int xstride, float eps, __nv_bfloat16* xs) {
+                                                 int xstride, float inv_d, float eps, __nv_bfloat16* xs) {
     constexpr int kGroups = kNarrowRow / 128;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint2 gv[kGroups];
@@ -673,7 +667,7 @@ __device__ __forceinline__ void norm_rows_narrow(const float* xf, const __nv_bfl
             q = fmaf(v[g].w, v[g].w, q);
             s += warp_sum(q);
         }
-        const float inv = 1.0f / sqrtf(s / (float)n_in + eps);
+        const float inv = __frsqrt_rn(fmaf(s, inv_d, eps));
 #pragma unroll
         for (int g = 0; g < kGroups; ++g) {
             const int i = (g * 32 + lane) * 4;
@@ -693,15 +687,15 @@ __device__ __forceinline__ void norm_rows_narrow(const float* xf, const __nv_bfl
 // registers it frees.
 template <int M>
 __device__ __noinline__ void norm_rows_call(const float* xf, const __nv_bfloat16* emb, const int* tok, const __nv_bfloat16* gain, int n_in, int wlen,
-                                            int xstride, float eps, __nv_bfloat16* xs, float* red) {
-    norm_rows_body<M>(xf, emb, tok, gain, n_in, wlen, xstride, eps, xs, red);
+                                            int xstride, float inv_d, float eps, __nv_bfloat16* xs, float* red) {
+    norm_rows_body<M>(xf, emb, tok, gain, n_in, wlen, xstride, inv_d, eps, xs, red);
 }
 template <int M>
 __device__ __forceinline__ void norm_rows_into_window(const float* xf, const __nv_bfloat16* emb, const int* tok, const __nv_bfloat16* gain, int n_in, int wlen,
-                                                      int xstride, float eps, __nv_bfloat16* xs, float* red) {
-    if (n_in <= kNarrowRow) norm_rows_narrow<M>(xf, emb, tok, gain, n_in, wlen, xstride, eps, xs);
-    else if constexpr (M == 5 || M == 6) norm_rows_body<M>(xf, emb, tok, gain, n_in, wlen, xstride, eps, xs, red);
-    else norm_rows_call<M>(xf, emb, tok, gain, n_in, wlen, xstride, eps, xs, red);
+                                                      int xstride, float inv_d, float eps, __nv_bfloat16* xs, float* red) {
+    if (n_in <= kNarrowRow) norm_rows_narrow<M>(xf, emb, tok, gain, n_in, wlen, xstride, inv_d, eps, xs);
+    else if constexpr (M == 5 || M == 6) norm_rows_body<M>(xf, emb, tok, gain, n_in, wlen, xstride, inv_d, eps, xs, red);
+    else norm_rows_call<M>(xf, emb, tok, gain, n_in, wlen, xstride, inv_d, eps, xs, red);
 }
 
 // Epilogues of a GEMV stage with three or more activation rows, as functions of their own (their registers are their
@@ -901,10 +895,11 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
     const int copy_stride = np * 2 * M;
     // A warp's first item of the stage stores its sums, later items add: the partial sums need no zeroing (there are no more warp sets than segments)
     constexpr bool kKeepX = (M == 1);
+    constexpr int kOpBlocks = M > 8 ? 2 : 4;  // column blocks of an item whose operands are in registers at a time
     // tagged handoff: no barrier stands between the cosine sums of a stage and the next RMSNorm, whose sums therefore lie elsewhere
     constexpr int kRedNorm = LL ? 3 : 0;
     const int chunks = n_in > kPassConsumers * 8 ? 3 : n_in > kPassConsumers * 4 ? 2 : 1;  // of 4 elements of a thread; short rows skip the code of the others
-    const bool keep = kKeepX && norm && n_in <= kPassConsumers * 12;
+    const bool keep = kKeepX && norm && (LL || n_in <= kPassConsumers * 12);
     uint2 gpre[3] = {make_uint2(0u, 0u), make_uint2(0u, 0u), make_uint2(0u, 0u)};  // this thread's RMSNorm gains
     const bool short_rows = norm && n_in <= kPassConsumers * 12;  // a thread owns at most three 4-element chunks of a row
     if (short_rows) {
@@ -1079,7 +1074,7 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
             float s = 0.f;
 #pragma unroll
             for (int w = 0; w < kPassConsumerWarps; ++w) s += red[w * (kPassMaxRows * 4) + m + kRedNorm];
-            inv[m] = 1.0f / sqrtf(s / (float)n_in + p.eps);
+            inv[m] = __frsqrt_rn(fmaf(s, p.inv_d, p.eps));
         }
     }
     trace_mark(p, stage, 6);
@@ -1095,7 +1090,7 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
         // drift apart without it cost more than it does, 7B width 684 -> 696 us)
         if (w0 > 0 || M > kMaxRows) consumers_sync();
         if (fused) {
-            norm_rows_into_window<M>(xf, direct ? p.embed : nullptr, sm.tok, st.gain, n_in, wlen, xstride, p.eps, xs, red);
+            norm_rows_into_window<M>(xf, direct ? p.embed : nullptr, sm.tok, st.gain, n_in, wlen, xstride, p.inv_d, p.eps, xs, red);
         } else if (keep) {  // a single window (n_in <= 5760): normalise the rows held in registers
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -1213,13 +1208,14 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
         // step covers 16 weight rows and nothing of the tile is wasted on padding rows.
         const __nv_bfloat16* xa = xs + (size_t)min(g8, M - 1) * xstride + q4 * 8;
         const __nv_bfloat16* xb2 = xs + (size_t)min(g8 + 8, M - 1) * xstride + q4 * 8;
-        const int ks = (S > 1) ? warp / n_oct : 0;                 // which copy of the partial sums this warp adds into
-        const int o_first = (S > 1) ? ((ks < S) ? warp - ks * n_oct : n_oct) : warp;
+        const int set = sm.warp_set[type * 16 + warp];
+        const int ks = set & 0xFF, o_first = set >> 8;             // which copy of the partial sums this warp adds into, and its first group
         const int o_step = (S > 1) ? n_oct : kPassConsumerWarps;  // S > 1: exactly one group per warp
         float* psum_w = psum + (size_t)ks * copy_stride;
         // this warp set's segments of the window: ks, ks + S, ... (one remainder per window instead of one per segment)
         int seg_first = w0;
-        if (S > 1) {
+        if (S > 1) seg_first += ks;
+        if (S > 1 && w0 > 0) {
             const int r = w0 % S;
             seg_first = w0 + (ks >= r ? ks - r : ks + S - r);
         }
@@ -1229,7 +1225,10 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
                 const uint32_t g = gi + (uint32_t)(seg * n_oct + o);
                 const int rows = 2 * min(kGrpPairs, np - kGrpPairs * o);
                 const long long tw0 = p.trace ? clock64() : 0;
-                const int slot = ring_wait_full(p, sm, g, stage, M * 1000 + seg);
+                int slot;
+                uint32_t gen;
+                ring_locate(p, g, slot, gen);
+                ring_wait_full(p, sm, g, slot, gen, stage, M * 1000 + seg);
                 const long long tw1 = p.trace ? clock64() : 0;
                 const unsigned char* sl = sm.ring + (size_t)slot * kSlotBytes + g8 * 64 + q4 * 16;
                 const int blk = rows * 64;
@@ -1241,24 +1240,24 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
                 for (int a = 0; a < 4; ++a) acc[a][0] = acc[a][1] = acc[a][2] = acc[a][3] = 0.f;
 #pragma unroll
                 for (int a = 0; a < (M > 8 ? 4 : 1); ++a) acc2[a][0] = acc2[a][1] = acc2[a][2] = acc2[a][3] = 0.f;
-                // Operands of four column blocks in registers, then 8 steps; twice per full item. Lanes whose weight row lies
+                // Operands of four column blocks in registers, two with more than eight rows (16 rows, 2048 wide: 213 -> 195 us, they spilled), then two steps for each block. Lanes whose weight row lies
                 // beyond the item's rows, or whose activation row beyond M, read whatever follows in the slot / the last
                 // activation row: every output element depends on its own weight row and activation row only, and the
                 // outputs of such rows are never stored. Only column blocks past the end of a ragged last segment must
                 // contribute nothing and are replaced by zeros.
                 if (nblk == kSegBlocks) {
+#pragma unroll (M > 8 ? 1 : kSegBlocks / kOpBlocks)
+                    for (int h = 0; h < kSegBlocks / kOpBlocks; ++h) {
+                        uint4 wlo[kOpBlocks], whi[kOpBlocks], xv[kOpBlocks], xv2[M > 8 ? kOpBlocks : 1];
 #pragma unroll
-                    for (int h = 0; h < kSegBlocks / 4; ++h) {
-                        uint4 wlo[4], whi[4], xv[4], xv2[M > 8 ? 4 : 1];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            wlo[j] = *reinterpret_cast<const uint4*>(sl + (h * 4 + j) * blk);
-                            whi[j] = *reinterpret_cast<const uint4*>(sl + (h * 4 + j) * blk + 8 * 64);
-                            xv[j] = *reinterpret_cast<const uint4*>(xa + sg * kSegK + (h * 4 + j) * 32);
-                            if (M > 8) xv2[j] = *reinterpret_cast<const uint4*>(xb2 + sg * kSegK + (h * 4 + j) * 32);
+                        for (int j = 0; j < kOpBlocks; ++j) {
+                            wlo[j] = *reinterpret_cast<const uint4*>(sl + (h * kOpBlocks + j) * blk);
+                            whi[j] = *reinterpret_cast<const uint4*>(sl + (h * kOpBlocks + j) * blk + 8 * 64);
+                            xv[j] = *reinterpret_cast<const uint4*>(xa + sg * kSegK + (h * kOpBlocks + j) * 32);
+                            if (M > 8) xv2[j] = *reinterpret_cast<const uint4*>(xb2 + sg * kSegK + (h * kOpBlocks + j) * 32);
                         }
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
+                        for (int j = 0; j < kOpBlocks; ++j) {
                             mma_bf16_16816(acc[(j & 1) * 2 + 0], wlo[j].x, whi[j].x, wlo[j].y, whi[j].y, xv[j].x, xv[j].y);
                             mma_bf16_16816(acc[(j & 1) * 2 + 1], wlo[j].z, whi[j].z, wlo[j].w, whi[j].w, xv[j].z, xv[j].w);
                             if (M > 8) {
@@ -1269,18 +1268,18 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
                     }
                 } else {
 #pragma unroll 1
-                    for (int h = 0; h * 4 < nblk; ++h) {
-                        uint4 wlo[4], whi[4], xv[4], xv2[M > 8 ? 4 : 1];
+                    for (int h = 0; h * kOpBlocks < nblk; ++h) {
+                        uint4 wlo[kOpBlocks], whi[kOpBlocks], xv[kOpBlocks], xv2[M > 8 ? kOpBlocks : 1];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const bool inb = h * 4 + j < nblk;
-                            wlo[j] = inb ? *reinterpret_cast<const uint4*>(sl + (h * 4 + j) * blk) : make_uint4(0u, 0u, 0u, 0u);
-                            whi[j] = inb ? *reinterpret_cast<const uint4*>(sl + (h * 4 + j) * blk + 8 * 64) : make_uint4(0u, 0u, 0u, 0u);
-                            xv[j] = *reinterpret_cast<const uint4*>(xa + sg * kSegK + (h * 4 + j) * 32);
-                            if (M > 8) xv2[j] = *reinterpret_cast<const uint4*>(xb2 + sg * kSegK + (h * 4 + j) * 32);
+                        for (int j = 0; j < kOpBlocks; ++j) {
+                            const bool inb = h * kOpBlocks + j < nblk;
+                            wlo[j] = inb ? *reinterpret_cast<const uint4*>(sl + (h * kOpBlocks + j) * blk) : make_uint4(0u, 0u, 0u, 0u);
+                            whi[j] = inb ? *reinterpret_cast<const uint4*>(sl + (h * kOpBlocks + j) * blk + 8 * 64) : make_uint4(0u, 0u, 0u, 0u);
+                            xv[j] = *reinterpret_cast<const uint4*>(xa + sg * kSegK + (h * kOpBlocks + j) * 32);
+                            if (M > 8) xv2[j] = *reinterpret_cast<const uint4*>(xb2 + sg * kSegK + (h * kOpBlocks + j) * 32);
                         }
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
+                        for (int j = 0; j < kOpBlocks; ++j) {
                             mma_bf16_16816(acc[(j & 1) * 2 + 0], wlo[j].x, whi[j].x, wlo[j].y, whi[j].y, xv[j].x, xv[j].y);
                             mma_bf16_16816(acc[(j & 1) * 2 + 1], wlo[j].z, whi[j].z, wlo[j].w, whi[j].w, xv[j].z, xv[j].w);
                             if (M > 8) {
@@ -1291,7 +1290,7 @@ __device__ void gemv_stage(const PassParams& p, const StageDesc& st, const PassS
                     }
                 }
                 __syncwarp();
-                if (lane == 0) ring_release(p, sm, g);
+                if (lane == 0) ring_release(sm, slot, gen);
                 // c[0], c[1]: weight row g8 of the group, activation rows 2*q4 and 2*q4 + 1; c[2], c[3]: weight row g8 + 8.
                 // Local weight row 16*o + r is row (r & 1) of local pair 8*o + r/2. Segments are added in ascending
                 // order, always by this lane.
@@ -1628,8 +1627,7 @@ __device__ __forceinline__ void finish_rows(const PassParams& p) {
     const int lane = threadIdx.x & 31;
     if (blockIdx.x >= (unsigned)p.n_resid) return;
     if (lane == 0) {
-        const int stage = p.n_stages - (p.stages[p.n_stages - 1].type == kStFinish ? 1 : 2);
-        grid_poll(p, p.grid_bar, p.bar_base + (unsigned)stage * gridDim.x + p.bar_extra_last);  // (test hook: extra arrivals that never come)
+        grid_poll(p, p.grid_bar, p.bar_base + (unsigned)p.finish_stage * gridDim.x + p.bar_extra_last);  // (test hook: extra arrivals that never come)
     }
     __syncwarp();
     for (int r = blockIdx.x; r < p.n_resid; r += gridDim.x) {
@@ -1678,7 +1676,7 @@ __device__ __forceinline__ void finish_rows(const PassParams& p) {
         }
     }
     __syncwarp();
-    if (p.stages[p.n_stages - 1].type == kStLmHead) bar_arrive(kFinishBar, kPassThreads);  // the LM head stage's last word comes after this
+    if (p.finish_stage + 1 < p.n_stages) bar_arrive(kFinishBar, kPassThreads);  // the LM head stage's last word comes after this
 }
 
 // ============================================================================================ attention stage
@@ -1781,13 +1779,21 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
         };
         // the boxes of a tile: every warp waits for all of them, a lane each
         auto wait_tile = [&](uint32_t g0, int tag) {
-            if (glane < tile_slots) ring_wait_full(p, sm, g0 + (uint32_t)glane, stage, tag);
+            if (glane < tile_slots) {
+                int slot;
+                uint32_t gen;
+                ring_locate(p, g0 + (uint32_t)glane, slot, gen);
+                ring_wait_full(p, sm, g0 + (uint32_t)glane, slot, gen, stage, tag);
+            }
             __syncwarp();
         };
         auto release_tile = [&](uint32_t g0) {  // behind a barrier of the group
             if (gt < tile_slots) {
                 fence_proxy_async_smem();
-                ring_release(p, sm, g0 + (uint32_t)gt);
+                int slot;
+                uint32_t gen;
+                ring_locate(p, g0 + (uint32_t)gt, slot, gen);
+                ring_release(sm, slot, gen);
             }
         };
         // The rows that this pass has just written: the producer may have copied the tile before the QKV stage of this pass stored them. They are
@@ -2250,6 +2256,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
     sm.split = split;
     int* tok = split + 8 * 4;
     sm.tok = tok;
+    unsigned short* warp_set = reinterpret_cast<unsigned short*>(tok + kPassMaxRows);
+    sm.warp_set = warp_set;
     sm.psum = reinterpret_cast<float*>(base + p.off_psum);
     sm.reg_a = base + p.off_reg_a;
 
@@ -2275,6 +2283,11 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
         const int n_seg = ((type == kStDown ? p.d_ffn : p.d_model) + kSegK - 1) / kSegK;
         split[type * 4 + 0] = pair0, split[type * 4 + 1] = np, split[type * 4 + 2] = n_oct;
         split[type * 4 + 3] = (n_oct > 0 && n_oct < 8) ? max(1, min(kPassConsumerWarps / n_oct, n_seg)) : 1;
+        const int S = split[type * 4 + 3];
+        for (int w = 0; w < kPassConsumerWarps; ++w) {  // S > 1: exactly one group per warp
+            const int ks = S > 1 ? w / n_oct : 0;
+            warp_set[type * 16 + w] = (unsigned short)(ks | (S > 1 ? (ks < S ? w - ks * n_oct : n_oct) : w) << 8);
+        }
     }
     if (threadIdx.x >= 64 && threadIdx.x < 64 + M && p.stages[0].type == kStEmbed) {
         const int m = threadIdx.x - 64;
@@ -2298,7 +2311,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
     for (int s = 0; s < p.n_stages; ++s) {
         trace_mark(p, s, 0);
         const StageDesc st = p.stages[s];  // static: read before waiting for the previous stage
-        const int next_type = (s + 1 < p.n_stages) ? p.stages[s + 1].type : -1;  // (read now: at the end of the stage it would be a round trip)
         // the next descriptor is requested now so that reading it at the next stage boundary hits L1
         if (threadIdx.x < 2 && s + 1 < p.n_stages)
             asm volatile("prefetch.global.L1 [%0];" ::"l"(reinterpret_cast<const char*>(p.stages + s + 1) + threadIdx.x * 64));
@@ -2333,7 +2345,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
         trace_mark(p, s, 3);
         if (!LL) {
             grid_arrive(p.grid_bar);
-        } else if (next_type == kStFinish) {
+        } else if (s + 1 == p.finish_stage) {
             // Tagged handoff: only the finish stage waits at the grid barrier, so the CTA arrives once for all stages in front of it. (Nothing
             // else ends a stage with a barrier: what the next one writes first, the window and the sums of squares, nobody reads any more.)
             grid_arrive(p.grid_bar, (unsigned)(s + 1));
