@@ -101,8 +101,9 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 // ============================================================================================ the GEMM
 // Persistent units (CG = 1: one SM; CG = 2: a cluster of two SMs) walk the 128 * CG x BN tiles of the product, row tiles
 // fastest. Warp 0 is the TMA producer, warp 1 issues the MMAs and owns the tensor-memory allocation,
-// warps 2-5 are the epilogue (warp w reads lanes 32 * (w % 4) .. + 31 of tensor memory, the quarter its position in the
-// warp group gives it access to). The accumulator is double-buffered in tensor memory (2 x BN columns), so the epilogue
+// warps 2-9 are the epilogue (warp w reads lanes 32 * (w % 4) .. + 31 of tensor memory, the quarter its position in the
+// warp group gives it access to, and every second 32 columns: with four warps the epilogue of the last tile, which nothing covers, was longer:
+// gate/up of 512 rows of the 7B width 68.4 -> 64.4 us in the prompt's chain, of 1023 rows 2048 wide 41.3 -> 37.0). The accumulator is double-buffered in tensor memory (2 x BN columns), so the epilogue
 // of a tile runs while the MMAs of the next tile are already filling the other buffer. Barriers: full[s] (TMA bytes landed
 // in stage s), empty[s] (the MMAs reading stage s have finished: tcgen05.commit), acc_full[b] (all MMAs of the tile in
 // buffer b have finished), acc_empty[b] (the epilogue warps have read buffer b). Ragged edges: TMA fills out-of-range
@@ -125,7 +126,8 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 // consumer adds them up (fp32 output), the number of parts the reduction dimension is cut into by the time they take
 // over the rounds (gemm_plan.h). Cutting the tiles of a last round with an exchange of the parts through L2 inside the
 // kernel (last arriver adds) was measured: 8-10 us per exchange, more than the part of a round it saves.
-constexpr int kGemmThreads = 192;
+constexpr int kGemmEpiWarps = 8;
+constexpr int kGemmThreads = 64 + 32 * kGemmEpiWarps;
 static int g_gemm_ctas = 148;  // persistent CTAs per launch: the SM count of the device (set by configure_prefill)
 
 // BN = 0: the width is a parameter of the launch (a multiple of 32).
@@ -192,7 +194,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 4 * CG);
+            mbar_init(&acc_empty[b], kGemmEpiWarps * CG);
         }
         mbar_init(drained, 1);
         *abandoned = 0;
@@ -292,7 +294,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             if (!ok && lane == 0) give_up();
         }
     } else {
-        const int quarter = warp & 3;
+        const int quarter = warp & 3, first = (warp - 2) / 4 * 32;  // two warps for each quarter take every second 32 columns
         bool ok = true;
         GemmItem it;
         for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
@@ -305,7 +307,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             if (!ok) break;
             const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * Cfg::kAccStride);
             const int n_cols = min(bn, N - n0);
-            for (int c = 0; c < n_cols; c += 32) {
+            for (int c = first; c < n_cols; c += 32 * (kGemmEpiWarps / 4)) {
                 float v[32];
                 tmem_ld32(acc + c, v);
                 if (row < M) gemm_epilogue(ep, row, n0 + c, N, v, it.part);
