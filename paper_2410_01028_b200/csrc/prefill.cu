@@ -143,16 +143,19 @@ struct GemmCfg {
 
 // The work of one launch: items (tile, part of the reduction dimension), tiles fastest, dealt round robin to the units.
 struct GemmWork {
-    int m_tiles, tiles, parts, bn;
+    int m_tiles, tiles, parts, bn, wide, narrow;  // (see GemmPlan; tiles: all of them)
 };
 struct GemmItem {
-    int tile, part, kb0, kb1;
+    int part, kb0, kb1;
+    int m, n0, width;  // row of tiles, first column and columns
 };
 // item `local` of unit `unit`; false when there is none
 __device__ __forceinline__ bool gemm_item(const GemmWork& w, int num_kb, int unit, int n_units, int local, GemmItem& it) {
     const int item = unit + local * n_units;
     if (item >= w.tiles * w.parts) return false;
-    it.tile = item % w.tiles, it.part = item / w.tiles;
+    const int tile = item % w.tiles, col = tile / w.m_tiles;  // row tiles vary fastest: units that run together share their weight tile (read once from HBM, then from L2)
+    it.part = item / w.tiles, it.m = tile - col * w.m_tiles;
+    it.n0 = min(col, w.wide) * w.bn + max(col - w.wide, 0) * w.narrow, it.width = col < w.wide ? w.bn : w.narrow;
     it.kb0 = it.part * num_kb / w.parts, it.kb1 = (it.part + 1) * num_kb / w.parts;
     return true;
 }
@@ -225,7 +228,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (warp == 0 && ep.w_static) {
         GemmItem it;
         if (gemm_item(work, num_kb, unit, n_units, 0, it))
-            for (; ahead < kStages && it.kb0 + ahead < it.kb1; ++ahead) load_w(ahead, it.kb0 + ahead, it.tile / work.m_tiles * bn + rank * (bn / CG));
+            for (; ahead < kStages && it.kb0 + ahead < it.kb1; ++ahead) load_w(ahead, it.kb0 + ahead, it.n0 + rank * (it.width / CG));
     }
     pdl_wait();  // everything above overlaps the end of the kernel in front
 
@@ -235,8 +238,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         bool ok = true;
         GemmItem it;
         for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
-            // row tiles vary fastest: units that run together share their weight tile (read once from HBM, then from L2)
-            const int m0 = (it.tile % work.m_tiles * CG + rank) * kGemmBM, n0 = it.tile / work.m_tiles * bn + rank * (bn / CG);
+            const int m0 = (it.m * CG + rank) * kGemmBM, n0 = it.n0 + rank * (it.width / CG);
             for (int kb = it.kb0; kb < it.kb1; ++kb) {
                 if (lap > 0) ok = mbar_wait_warp(&empty[s], (uint32_t)((lap - 1) & 1), err, kErrGemmWait, 0, issued, s, 1);
                 if (!ok) break;
@@ -257,7 +259,6 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         }
     } else if (warp == 1) {
         if (rank == 0) {
-            const uint32_t idesc = umma_idesc_bf16(kGemmBM * CG, bn);
             const uint32_t base_addr = smem_u32(base);
             int s = 0, lap = 0;  // ring position of the next k-block
             bool ok = true;
@@ -268,7 +269,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 if (local >= 2) ok = mbar_wait_warp(&acc_empty[buf], (uint32_t)((local / 2 - 1) & 1), err, kErrGemmWait, 3, local, buf, 4);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t tmem_d = tmem + (uint32_t)(buf * Cfg::kAccStride);
+                const uint32_t tmem_d = tmem + (uint32_t)(buf * Cfg::kAccStride), idesc = umma_idesc_bf16(kGemmBM * CG, it.width);
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     ok = mbar_wait_warp(&full[s], (uint32_t)(lap & 1), err, kErrGemmWait, 1, kb, s, 2);
                     if (!ok) break;
@@ -299,14 +300,14 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         GemmItem it;
         for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
             const int buf = local & 1;
-            const int m0 = (it.tile % work.m_tiles * CG + rank) * kGemmBM, n0 = it.tile / work.m_tiles * bn;
+            const int m0 = (it.m * CG + rank) * kGemmBM, n0 = it.n0;
             const int row = m0 + quarter * 32 + lane;
             ok = mbar_wait(&acc_full[buf], (uint32_t)((local / 2) & 1), err, kErrGemmWait, 2, local, buf, 3) && *err == kErrNone;
             ok = __all_sync(0xffffffffu, ok);  // tensor-memory loads are warp-wide
             tc_fence_after();
             if (!ok) break;
             const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * Cfg::kAccStride);
-            const int n_cols = min(bn, N - n0);
+            const int n_cols = min(it.width, N - n0);
             for (int c = first; c < n_cols; c += 32 * (kGemmEpiWarps / 4)) {
                 float v[32];
                 tmem_ld32(acc + c, v);
@@ -355,7 +356,7 @@ GemmPlan plan_gemm(int M, int N, int K, int max_parts) { return plan_gemm(M, N, 
 
 cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmPlan& p, const GemmEpi& ep, cudaStream_t s) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
-    const GemmWork w{p.m_tiles, p.tiles, p.parts, p.bn};
+    const GemmWork w{p.m_tiles, p.items, p.parts, p.bn, p.wide, p.narrow};
     if (p.cg == 1) return launch_gemm<0, 1>(tm_a, tm_w, M, N, K, w, ep, s);
     if (p.bn == 256) return launch_gemm<256, 2>(tm_a, tm_w, M, N, K, w, ep, s);
     if (p.bn == 224) return launch_gemm<224, 2>(tm_a, tm_w, M, N, K, w, ep, s);
