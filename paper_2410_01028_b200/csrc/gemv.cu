@@ -64,16 +64,14 @@ __device__ __forceinline__ void mma_zero(float (&d)[4], uint32_t a0, uint32_t a1
 
 // Signal arrival of this CTA; returns true in every thread of the last CTA to arrive.
 __device__ __forceinline__ bool last_cta_arrives(unsigned* counter, int* flag_smem) {
-    __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned t = atomicAdd(counter, 1u);
+        unsigned t;  // one release and acquire at GPU scope, cumulative over the CTA's writes, which the barrier has ordered before it
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
         *flag_smem = (t == gridDim.x - 1) ? 1 : 0;
     }
     __syncthreads();
-    const bool last = *flag_smem != 0;
-    if (last) __threadfence();
-    return last;
+    return *flag_smem != 0;
 }
 
 // The order in which every role walks a CTA's rows: blocks of rows, windows of the activations, groups of at most 16 rows, epochs
@@ -141,37 +139,36 @@ private:
 // thread at a time. Thread t adds the squares of inputs 4 t + 1024 u in this order whatever R and U.
 template <int R, int U, bool kTail>
 __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs, float* red, bool first, int w0, int w1) {
-    constexpr int kThreads = kGemvWarps * 32, kStep = kThreads * 4, kBatch = R == 1 ? 8 : 16 / R, kHeld = U > 0 ? U : 1;
+    constexpr int kThreads = kGemvWarps * 32, kStep = kThreads * 4, kBatch = R == 1 ? 8 : R > 5 ? 2 : 16 / R, kHeld = U > 0 ? U : 1;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, n_in = p.n_in;
     const float* xf = reinterpret_cast<const float*>(p.x);
-    auto load = [&](int m, int i) { return *reinterpret_cast<const float4*>(xf + (size_t)m * n_in + i); };
+    auto load = [&](int m, int i) { return *reinterpret_cast<const ulonglong2*>(xf + (size_t)m * n_in + i); };
     auto inverse = [&](int m) {  // of the row's root mean square
         const float* r = red + m * kGemvWarps;
         const float s = ((r[0] + r[1]) + (r[2] + r[3])) + ((r[4] + r[5]) + (r[6] + r[7]));
         return 1.0f / sqrtf(s / (float)n_in + p.eps);
     };
-    auto put = [&](int m, int i, const float4& a, float inv, const uint2& gn) {
-        uint2 o;
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(a.x * inv * bf_lo(gn.x), a.y * inv * bf_hi(gn.x));
-        const __nv_bfloat162 hi = __floats2bfloat162_rn(a.z * inv * bf_lo(gn.y), a.w * inv * bf_hi(gn.y));
-        o.x = *reinterpret_cast<const uint32_t*>(&lo);
-        o.y = *reinterpret_cast<const uint32_t*>(&hi);
-        *reinterpret_cast<uint2*>(xs + (size_t)m * p.xs_ld + (i - w0)) = o;
+    auto put = [&](int m, int i, const ulonglong2& a, unsigned long long inv, const uint2& gn) {
+        float lo0, hi0, lo1, hi1;
+        unpack2(fmul2(fmul2(a.x, inv), bf2_to_f2(gn.x)), lo0, hi0);
+        unpack2(fmul2(fmul2(a.y, inv), bf2_to_f2(gn.y)), lo1, hi1);
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(lo0, hi0), hi = __floats2bfloat162_rn(lo1, hi1);
+        *reinterpret_cast<uint2*>(xs + (size_t)m * p.xs_ld + (i - w0)) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
     };
     auto gain = [&](int i) { return *reinterpret_cast<const uint2*>(p.gain + i); };
     static_assert(kGemvWarps == 8, "sums of squares of eight warps");
-    auto load_batch = [&](float4 (&a)[kBatch][R], int m0, int i, int end) {
+    auto load_batch = [&](ulonglong2 (&a)[kBatch][R], int m0, int i, int end) {
 #pragma unroll
         for (int b = 0; b < kBatch; ++b)
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                a[b][r] = make_float4(0.f, 0.f, 0.f, 0.f);
+                a[b][r] = make_ulonglong2(0ull, 0ull);
                 if (m0 + r < p.M && i + kStep * b < end) a[b][r] = load(m0 + r, i + kStep * b);
             }
     };
-    auto fill = [&](int m0, int i, const float (&inv)[R]) {  // inputs i, i + 1024, ... of these rows
+    auto fill = [&](int m0, int i, const unsigned long long (&inv)[R]) {  // inputs i, i + 1024, ... of these rows
         for (; i < w1; i += kStep * kBatch) {
-            float4 a[kBatch][R];
+            ulonglong2 a[kBatch][R];
             load_batch(a, m0, i, w1);
 #pragma unroll
             for (int b = 0; b < kBatch; ++b)
@@ -191,27 +188,23 @@ __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs
             if (4 * t + kStep * u < n_in) g[u] = gain(4 * t + kStep * u);
         }
         for (int m0 = 0; m0 < p.M; m0 += R) {
-            float4 v[R][kHeld];
+            ulonglong2 v[R][kHeld];
 #pragma unroll
             for (int r = 0; r < R; ++r)
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    v[r][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[r][u] = make_ulonglong2(0ull, 0ull);
                     if (m0 + r < p.M && 4 * t + kStep * u < n_in) v[r][u] = load(m0 + r, 4 * t + kStep * u);
                 }
-            float4 ss[R];
-            auto add = [&](float4& t4, const float4& a) {
-                t4.x = fmaf(a.x, a.x, t4.x), t4.y = fmaf(a.y, a.y, t4.y), t4.z = fmaf(a.z, a.z, t4.z), t4.w = fmaf(a.w, a.w, t4.w);
-            };
+            unsigned long long ss[R][2] = {};
+            auto add = [&](unsigned long long (&q)[2], const ulonglong2& a) { q[0] = ffma2(a.x, a.x, q[0]), q[1] = ffma2(a.y, a.y, q[1]); };
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                ss[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int r = 0; r < R; ++r)
 #pragma unroll
                 for (int u = 0; u < U; ++u) add(ss[r], v[r][u]);
-            }
             if constexpr (kTail)
                 for (int i = 4 * t + kStep * U; i < n_in; i += kStep * kBatch) {
-                    float4 a[kBatch][R];
+                    ulonglong2 a[kBatch][R];
                     load_batch(a, m0, i, n_in);
 #pragma unroll
                     for (int b = 0; b < kBatch; ++b)
@@ -220,7 +213,12 @@ __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs
                 }
             float s[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) s[r] = (ss[r].x + ss[r].y) + (ss[r].z + ss[r].w);
+            for (int r = 0; r < R; ++r) {
+                float a, b, c, d;
+                unpack2(ss[r][0], a, b);
+                unpack2(ss[r][1], c, d);
+                s[r] = (a + b) + (c + d);
+            }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -230,10 +228,11 @@ __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs
                 if (lane == 0 && m0 + r < p.M) red[(m0 + r) * kGemvWarps + warp] = s[r];
             bar_sync(1, kThreads);
             const float inv_lane = inverse(min(m0 + min(lane, R - 1), p.M - 1));  // a row per lane: one chain of square root and division
-            float inv[R];
+            unsigned long long inv[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                inv[r] = __shfl_sync(0xffffffffu, inv_lane, r);
+                const float f = __shfl_sync(0xffffffffu, inv_lane, r);
+                inv[r] = pack2(f, f);
                 if (m0 + r < p.M) {
 #pragma unroll
                     for (int u = 0; u < U; ++u)
@@ -244,9 +243,12 @@ __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs
         }
     } else {
         for (int m0 = 0; m0 < p.M; m0 += R) {
-            float inv[R];
+            unsigned long long inv[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) inv[r] = inverse(min(m0 + r, p.M - 1));
+            for (int r = 0; r < R; ++r) {
+                const float f = inverse(min(m0 + r, p.M - 1));
+                inv[r] = pack2(f, f);
+            }
             fill(m0, w0 + 4 * t, inv);
         }
     }
@@ -418,8 +420,9 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
             ++n_x;
             if (!NORM) return wait(x_full, n_x - 1, 0, n_x, 0, 1);
             if (!first) bar_sync(1, kGemvWarps * 32);  // the window before has been read
-            // Registers hold 15 to 20 groups of four inputs of a thread, 8 of one row: rows of up to 3072 inputs five at a time, 4096 five, 5120 three
-            // or two. Behind one row only is there a loop over what does not fit (nine rows of 2056 -> 6145 with one 12.3 us, without 11.7).
+            // Registers hold 15 to 27 groups of four inputs of a thread, 8 of one row: rows of up to 3072 inputs all together, 4096 five at a time, 5120 three
+            // or two. (Six to nine rows of up to 3072 in two batches, the second one's loads behind the first one's sums: 6 rows of 2048 -> 6144 8.6 us for 8.4, 7 of
+            // 3000 -> 9000 13.0 for 12.4.) Behind one row only is there a loop over what does not fit (nine rows of 2056 -> 6145 with one 12.3 us, without 11.7).
             if (BY_WARP) {  // (at most 768 inputs)
                 if (M == 1) norm_rows<1, 1, false>(p, xs, red, first, w0, w1);
                 else norm_rows<5, 1, false>(p, xs, red, first, w0, w1);
@@ -437,7 +440,8 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                     if (M == 9) norm_long<5>(p, xs, red, 4, first, w0, w1);
                 }
             } else if (M == 2) norm_rows<2, 5, false>(p, xs, red, first, w0, w1);
-            else if (n_in <= 3072) norm_rows<5, 3, false>(p, xs, red, first, w0, w1);
+            else if (n_in <= 3072 && M <= 5) norm_rows<5, 3, false>(p, xs, red, first, w0, w1);
+            else if (n_in <= 3072) norm_rows<9, 3, false>(p, xs, red, first, w0, w1);
             else if (n_in <= 4096) norm_rows<5, 4, false>(p, xs, red, first, w0, w1);
             else norm_rows<3, 5, false>(p, xs, red, first, w0, w1);
             bar_sync(1, kGemvWarps * 32);
