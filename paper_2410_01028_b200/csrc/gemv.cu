@@ -420,9 +420,10 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
             ++n_x;
             if (!NORM) return wait(x_full, n_x - 1, 0, n_x, 0, 1);
             if (!first) bar_sync(1, kGemvWarps * 32);  // the window before has been read
-            // Registers hold 15 to 27 groups of four inputs of a thread, 8 of one row: rows of up to 3072 inputs all together, 4096 five at a time, 5120 three
-            // or two. (Six to nine rows of up to 3072 in two batches, the second one's loads behind the first one's sums: 6 rows of 2048 -> 6144 8.6 us for 8.4, 7 of
-            // 3000 -> 9000 13.0 for 12.4.) Behind one row only is there a loop over what does not fit (nine rows of 2056 -> 6145 with one 12.3 us, without 11.7).
+            // Registers hold 15 to 24 groups of four inputs of a thread, 8 of one row: six to eight rows of up to 3072 inputs all together, others of them five at a time,
+            // 4096 five, 5120 three or two. (Six to eight rows in two batches, the second one's loads behind the first one's sums: 6 rows of 2048 -> 6144 8.6 us for
+            // 8.4, 7 of 3000 -> 9000 13.0 for 12.4; nine together 2504 -> 1564 7.7 for 7.5.) Behind one row only is there a loop over what does not fit (nine
+            // rows of 2056 -> 6145 with one 12.3 us, without 11.7).
             if (BY_WARP) {  // (at most 768 inputs)
                 if (M == 1) norm_rows<1, 1, false>(p, xs, red, first, w0, w1);
                 else norm_rows<5, 1, false>(p, xs, red, first, w0, w1);
@@ -440,8 +441,8 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const __grid_cons
                     if (M == 9) norm_long<5>(p, xs, red, 4, first, w0, w1);
                 }
             } else if (M == 2) norm_rows<2, 5, false>(p, xs, red, first, w0, w1);
-            else if (n_in <= 3072 && M <= 5) norm_rows<5, 3, false>(p, xs, red, first, w0, w1);
-            else if (n_in <= 3072) norm_rows<9, 3, false>(p, xs, red, first, w0, w1);
+            else if (n_in <= 3072 && (M <= 5 || M == 9)) norm_rows<5, 3, false>(p, xs, red, first, w0, w1);
+            else if (n_in <= 3072) norm_rows<8, 3, false>(p, xs, red, first, w0, w1);
             else if (n_in <= 4096) norm_rows<5, 4, false>(p, xs, red, first, w0, w1);
             else norm_rows<3, 5, false>(p, xs, red, first, w0, w1);
             bar_sync(1, kGemvWarps * 32);
