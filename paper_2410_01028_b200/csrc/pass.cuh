@@ -611,19 +611,17 @@ __device__ __forceinline__ void norm_rows_body(const float* xf, const __nv_bfloa
 #pragma unroll
                 for (int w = 0; w < kPassConsumerWarps; ++w) s += red[w * (kPassMaxRows * 4) + m];
                 const float inv = __frsqrt_rn(fmaf(s, inv_d, eps));
+                const unsigned long long inv2 = pack2(inv, inv);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     const int i = (tid + c * kPassConsumers) * 4;
-                    if (i < wlen) {
-                        uint2 o = make_uint2(0u, 0u);
-                        if (i < n_in) {
-                            const float g0 = bf_lo(gv[c].x), g1 = bf_hi(gv[c].x), g2 = bf_lo(gv[c].y), g3 = bf_hi(gv[c].y);
-                            __nv_bfloat162 lo = __floats2bfloat162_rn(v[u][c].x * inv * g0, v[u][c].y * inv * g1);
-                            __nv_bfloat162 hi = __floats2bfloat162_rn(v[u][c].z * inv * g2, v[u][c].w * inv * g3);
-                            o.x = *reinterpret_cast<uint32_t*>(&lo);
-                            o.y = *reinterpret_cast<uint32_t*>(&hi);
-                        }
-                        *reinterpret_cast<uint2*>(xs + (size_t)m * xstride + i) = o;
+                    if (i < wlen) {  // (past n_in everything is zero)
+                        float a0, a1, a2, a3;
+                        unpack2(fmul2(fmul2(pack2(v[u][c].x, v[u][c].y), inv2), bf2_to_f2(gv[c].x)), a0, a1);
+                        unpack2(fmul2(fmul2(pack2(v[u][c].z, v[u][c].w), inv2), bf2_to_f2(gv[c].y)), a2, a3);
+                        const __nv_bfloat162 lo = __floats2bfloat162_rn(a0, a1), hi = __floats2bfloat162_rn(a2, a3);
+                        *reinterpret_cast<uint2*>(xs + (size_t)m * xstride + i) =
+                            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
                     }
                 }
             }
