@@ -102,63 +102,6 @@ static bool gemv_accepts(const DeviceInfo& dv, int M, int n_rows, int n_in, bool
     return false;
 }
 
-// Shared-memory plan of the persistent pass kernel for M rows: ring slots, barriers, reduction scratch,
-// per-pair partial sums, activation window / attention scratch.
-struct PassPlan {
-    int ns, attn_groups, off_bars, off_misc, off_psum, off_reg_a, xs_bytes;
-    size_t smem;
-};
-
-static bool plan_pass(const DeviceInfo& dv, const asd_config& c, int M, PassPlan* pl) {
-    const int kvd = c.n_kv_heads * c.head_dim;
-    const long long max_rows = std::max<long long>(std::max(c.vocab, 2 * c.d_ffn), std::max(c.d_model + 2 * kvd, c.d_model));
-    const long long np_max = ((max_rows + 1) / 2 + dv.num_sms - 1) / dv.num_sms + 2;
-    if ((max_rows + 1) / 2 * dv.num_sms >= (1LL << 31)) return false;  // the kernel splits a matrix's pairs over the CTAs in 32-bit arithmetic
-    // per-pair partial sums; when a CTA has fewer than 8 groups of 8 pairs up to 15 warps keep copies (at most 15 / groups
-    // copies of at most 8 * groups pairs: 120 pairs in all)
-    const size_t psum = ((size_t)std::max<long long>(np_max, 120) * 2 * M * 4 + 15) & ~(size_t)15;
-    const size_t misc = ((size_t)16 * kPassMaxRows * 4 * 4 + 32 + 64 * 4 + 8 * 4 * 4 + kPassMaxRows * 4 + 8 * 16 * 2 + 15) & ~(size_t)15;  // reduction scratch, flags, slot generations, split table, tokens, warp sets
-    const size_t attn_scratch = (size_t)attn_scratch_bytes(M, c.n_heads / c.n_kv_heads, c.head_dim);
-    // Activation window: the longest reduction dimension (in segments of 256 inputs) cut into as few windows as leave
-    // the ring 20 slots. Every further window costs a stage of a multi-row pass a block-wide refill, every slot less
-    // costs bandwidth (one row, 7B shape: 24 slots 0.402 ms per 4 layers, 21: 0.409, 16: 0.422, 12: 0.481); 20 was the
-    // best trade for three and four rows (measured again with 22 and 24 after the kernel had changed: four and five rows
-    // 0.7 % slower). Windows do not get shorter than a row of d_model while that leaves 16 slots: the RMSNorm stages want
-    // their rows whole (six to nine rows: 1-2.5 % faster than with W_d's row cut into equal parts). One row always fits whole.
-    const size_t seg_max = ((size_t)std::max(c.d_model, c.d_ffn) + kSegK - 1) / kSegK;
-    const size_t seg_norm = ((size_t)c.d_model + kSegK - 1) / kSegK;  // the RMSNorm stages want their rows whole in the window
-    const long long fixed = 1024 + (long long)(psum + misc) + 2 * 64 * 8;
-    size_t wseg_plan = seg_max;
-    auto leaves_ring = [&](size_t wseg, long long slots) {
-        const size_t bytes = (size_t)M * (wseg * kSegK + kXsPad) * 2;
-        return (long long)dv.max_smem - fixed - (long long)((bytes + 15) & ~(size_t)15) >= slots * kSlotBytes;
-    };
-    for (size_t nw = 1; nw <= seg_max; ++nw) {
-        wseg_plan = (seg_max + nw - 1) / nw;
-        if (leaves_ring(wseg_plan, 20)) break;
-    }
-    // not shorter than a row of d_model while the ring keeps 16 slots: the RMSNorm stages want their rows whole
-    if (wseg_plan < seg_norm && leaves_ring(seg_norm, 16)) wseg_plan = seg_norm;
-    const int xs_bytes = (int)((size_t)M * (wseg_plan * kSegK + kXsPad) * 2);
-    const size_t xs = (size_t)M * ((size_t)pass_wseg(M, xs_bytes) * kSegK + kXsPad) * 2;
-    // up to three groups of four warps work on attention items, as many as their scratch fits the window's bytes
-    const int groups_by_scratch = (int)std::max<size_t>(1, std::min<size_t>(3, (size_t)kXsBudget / attn_scratch));
-    const size_t reg_a = (std::max(xs, groups_by_scratch * attn_scratch) + 15) & ~(size_t)15;
-    const long long avail = (long long)dv.max_smem - 1024 - (long long)(psum + misc + reg_a) - 2 * 64 * 8;
-    int ns = (int)std::min<long long>(64, avail / kSlotBytes);
-    const int tile_slots = (kAttnChunk / kBoxKeys) * std::max(1, c.head_dim / 64);
-    if (ns < 2 * tile_slots || ns < 8) return false;
-    pl->ns = ns;
-    pl->xs_bytes = xs_bytes;
-    pl->attn_groups = std::max(1, std::min(groups_by_scratch, ns / (2 * tile_slots)));
-    pl->off_bars = ns * kSlotBytes;
-    pl->off_misc = pl->off_bars + 2 * 64 * 8;
-    pl->off_psum = pl->off_misc + (int)misc;
-    pl->off_reg_a = pl->off_psum + (int)psum;
-    pl->smem = (size_t)pl->off_reg_a + reg_a + 1024;
-    return pl->smem <= (size_t)dv.max_smem;
-}
-
 // ---------------------------------------------------------------- workspace layout
 struct Layout {
     size_t embed, lm_head, final_norm, layers, layer_stride;
@@ -581,7 +524,7 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     if (M < 1 || (M > kMaxRows && M != kPassMaxRows)) return fail(x, ASD_ERR_ARG, "row count out of range");
     if ((long long)pos0 + M > c.max_seq) return fail(x, ASD_ERR_OVERFLOW, "pass would exceed max_seq positions");
     PassPlan pl;
-    if (!plan_pass(*x->dev, c, M, &pl)) return fail(x, ASD_ERR_ARG, "decoder shape does not fit the pass kernel's shared-memory plan");
+    if (!plan_pass(x->dev->num_sms, x->dev->max_smem, c, M, &pl)) return fail(x, ASD_ERR_ARG, "decoder shape does not fit the pass kernel's shared-memory plan");
 
     float* cosv = x->at<float>(ly.cosv);
     // NaN = skipped. A pass of the full model writes every sublayer's entry of its rows, a draft pass those of the kept
@@ -842,7 +785,7 @@ extern "C" int asd_create(const asd_config* cfg, void* dev_workspace, size_t byt
     if (e != cudaSuccess) return bail(e);
     {
         PassPlan pl;
-        if (!plan_pass(*x->dev, *cfg, kPassMaxRows, &pl) || !plan_pass(*x->dev, *cfg, 1, &pl)) {
+        if (!plan_pass(x->dev->num_sms, x->dev->max_smem, *cfg, kPassMaxRows, &pl) || !plan_pass(x->dev->num_sms, x->dev->max_smem, *cfg, 1, &pl)) {
             delete x;
             return ASD_ERR_ARG;
         }

@@ -7,8 +7,6 @@
 namespace asd {
 
 constexpr int kMaxRows = 9;        // rows of the stand-alone fused GEMV: max draft length 8, plus the last accepted token
-constexpr int kPassMaxRows = 16;   // rows of one pass of the persistent kernel (prefill feeds the prompt 16 rows at a time)
-constexpr int kAttnChunk = 128;    // keys per attention work item; chunks are aligned to absolute positions
 
 struct PassParams;
 

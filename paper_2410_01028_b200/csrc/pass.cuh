@@ -41,6 +41,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "pass_plan.h"
 #include "ring.cuh"
 
 namespace asd {
@@ -55,7 +56,6 @@ constexpr int kFinishBar = 7;  // named barrier: a CTA's cosines are done (1: co
 // both cost more (registers) than the two hand-offs that they save: five rows of the tiny decoder 136 -> 139 us, 16 rows 5 %.
 template <int M>
 constexpr bool kFewRows = M <= 2;
-constexpr int kXsBudget = 40960;                    // most shared memory the attention scratch of all warp groups may take
 
 enum StageType : int { kStEmbed = 0, kStQkv, kStAttn, kStOproj, kStGateUp, kStDown, kStLmHead, kStFinish };
 
@@ -133,19 +133,10 @@ constexpr int kHostMargin = 12, kHostErr = 16, kHostStamp = 24;
 __device__ __forceinline__ int pass_token(const PassParams& p, int m) { return p.tokens ? __ldcg(p.tokens + m) : p.inline_tokens[m]; }
 
 constexpr int kTraceEntries = 12;  // per stage and CTA: 0-7 consumer side, 8-10 producer side (first / last copy issued, stall cycles), 11 descriptor read
-constexpr int kSegK = 256;     // inputs per ring item (8 column blocks of 32; the last item of a row may hold fewer)
-constexpr int kBoxKeys = 64;   // keys per K/V box (one ring slot)
 constexpr int kGrpPairs = 8;   // pairs of weight rows per ring item: 16 rows, the M of one m16n8k16 tensor-core step
 constexpr int kGrpRows = 2 * kGrpPairs;
 constexpr int kSegBlocks = kSegK / 32;  // column blocks of 32 inputs per full segment
 constexpr int kNarrowRow = 512;  // rows up to this length are normalised by a warp each (passes of several rows)
-constexpr int kXsPad = 32;     // bf16 elements of padding per activation row (64 bytes: conflict-free 16-byte reads)
-
-// 256-input segments whose activations (M rows, bf16, padded rows) fit the shared-memory window
-__host__ __device__ inline int pass_wseg(int M, int xs_bytes) {
-    const int w = (xs_bytes / M - kXsPad * 2) / (kSegK * 2);
-    return w < 1 ? 1 : w;
-}
 
 // D (16x8, fp32) += A (16x16, bf16, row) * B (16x8, bf16, col): one warp-wide tensor-core step
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
@@ -160,7 +151,7 @@ struct PassSmem {
     uint64_t *full, *empty;
     float* red;   // [16][kPassMaxRows*4]
     int* flag;    // [8]
-    volatile unsigned* consumed;  // [64] generations of each ring slot that consumers have finished with
+    volatile unsigned* consumed;  // [kMaxSlots] generations of each ring slot that consumers have finished with
     const int* split;             // [8][4] per stage type: this CTA's first pair, pair count, groups of 16 rows, warp sets per group
     const unsigned short* warp_set;  // [8][16] per stage type and warp: warp set | first group << 8 (divisions that a stage would start with)
     const int* tok;               // [16] the rows' tokens, clamped to the vocabulary
@@ -1704,15 +1695,6 @@ __device__ __forceinline__ void mma_bf16_zero(float (&d)[4], const uint32_t (&a)
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 
-// Shared memory of a group of warps: the queries of eight columns [column][head_dim] and their probabilities as three bf16 terms
-// [term][column][128 keys], rows 16 bytes longer than they are (the eight rows of a matrix then lie in different banks), then the warps' maxima and sums.
-constexpr int kAttnCols = 8;  // (row, head of the group) pairs per step: the N of m16n8k16
-constexpr int kAttnPRow = kAttnChunk * 2 + 16;
-__host__ __device__ inline int attn_cols(int M, int group) { return M * group < kAttnCols ? M * group : kAttnCols; }
-__host__ __device__ inline int attn_scratch_bytes(int M, int group, int hd) {
-    return attn_cols(M, group) * (2 * hd + 16 + 3 * kAttnPRow) + 2 * 4 * kAttnCols * 4;
-}
-
 // Work items (kv head, 128-key chunk) of this CTA on the tensor cores (mma.sync m16n8k16), a group of four warps to an item. The COLUMNS of the
 // products are the (row, query head) pairs that share the item's keys, eight at a time; what a column gets does not depend on its
 // neighbours, so neither does a row's result on the row count.
@@ -2250,7 +2232,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
     sm.red = reinterpret_cast<float*>(base + p.off_misc);
     sm.flag = reinterpret_cast<int*>(sm.red + 16 * kPassMaxRows * 4);
     sm.consumed = reinterpret_cast<volatile unsigned*>(sm.flag + 8);
-    int* split = reinterpret_cast<int*>(const_cast<unsigned*>(sm.consumed) + 64);
+    int* split = reinterpret_cast<int*>(const_cast<unsigned*>(sm.consumed) + kMaxSlots);
     sm.split = split;
     int* tok = split + 8 * 4;
     sm.tok = tok;

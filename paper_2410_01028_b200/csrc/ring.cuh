@@ -10,7 +10,6 @@
 
 namespace asd {
 
-constexpr int kSlotBytes = 8192;             // one ring slot: 8 weight rows x 512 bf16 inputs, or one 64-key K/V box
 constexpr long long kWaitCycles = 4000000000LL;  // default budget of one wait: ~2 s at 2 GHz
 
 enum DeviceError : int {
