@@ -478,10 +478,11 @@ __device__ __forceinline__ bool last_cta_consumers(unsigned* counter, int* flag_
     return *flag_smem != 0;
 }
 
-// Every stage starts by waiting for the previous stage of all CTAs. Whatever does not depend on activations (the
-// stage descriptor, index arithmetic, zeroing of partial sums, RMSNorm gains) is done before this wait.
-__device__ __forceinline__ void stage_begin(const PassParams& p, int s) {
-    if (s > 0) grid_wait(p, p.grid_bar, p.bar_base + (unsigned)s * gridDim.x);
+// A stage of a pass without tags starts by waiting for the previous stage of all CTAs, but for the first RMSNorm where it reads the
+// embeddings itself and the LM head, in front of which the finish stage has waited. Whatever does not depend on activations (the
+// stage descriptor, index arithmetic, RMSNorm gains) is done before this wait. extra: arrivals beyond the grid's (test hook).
+__device__ __forceinline__ void stage_begin(const PassParams& p, int s, unsigned extra = 0u) {
+    if (s > 0) grid_wait(p, p.grid_bar, p.bar_base + (unsigned)s * gridDim.x + extra);
     trace_mark(p, s, 1);
 }
 
@@ -2315,7 +2316,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
                 }
             }
         } else if (st.type == kStFinish) {
-            if (!LL) stage_begin(p, s);  // the LM head wants the hidden state of all CTAs; the producer warp does the work (finish_rows)
+            // The LM head wants the hidden state of all CTAs. The cosines of one and two rows are the producer warp's work (finish_rows), those of
+            // more rows the consumer warps'. (The test hook's wait is this one: the arrivals behind it would end the producer's.)
+            if (!LL) stage_begin(p, s, p.bar_extra_last);
             if constexpr (!kFewRows<M>) finish_stage<M>(p, sm);
         } else if (st.type == kStAttn) {
             attn_stage<M, LL, HD>(p, st, sm, gi, merge_target, s);
