@@ -579,8 +579,8 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     x->delivered = deliver && lm_head && x->temperature == 0.0;  // (a drawn token takes the argmax's place afterwards)
     if (x->delivered) p.host_out = x->pinned + kPinnedPass, p.host_stamp = ++x->pass_stamp;
     p.logits_out = (x->debug_logits || x->temperature > 0.0) ? x->at<float>(ly.logits) : nullptr;
-    x->logits_on_host = x->delivered && x->debug_logits && (size_t)M * c.vocab * 4 <= kPinnedLogits;
-    p.logits_host = x->logits_on_host ? x->pinned_logits : nullptr;
+    const bool logits_on_host = x->delivered && x->debug_logits && (size_t)M * c.vocab * 4 <= kPinnedLogits;
+    p.logits_host = logits_on_host ? x->pinned_logits : nullptr;
     p.acc_sim = acc_sim ? 1 : 0;
     p.sim_base = x->at<double>(ly.sumcos), p.sim_host = x->pinned_sums;
     p.trace = x->trace ? x->at<long long>(ly.trace) : nullptr;
@@ -613,6 +613,7 @@ static int run_pass(asd_ctx* x, int M, int pos0, const int* dev_tokens, bool use
     }
     if (lm_head) bytes += 2.0 * (double)c.vocab * d;
     x->last_has_logits = lm_head && x->debug_logits;
+    x->logits_on_host = logits_on_host;  // (behind the launch, like the row count: a pass that was not launched leaves the one before in place)
     x->last_had_lm_head = lm_head;
     x->last_M = M;
     if (bytes_out) *bytes_out = bytes;
