@@ -2297,6 +2297,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
             asm volatile("prefetch.global.L1 [%0];" ::"l"(reinterpret_cast<const char*>(p.stages + s + 1) + threadIdx.x * 64));
         if (p.trace && threadIdx.x == 0) p.trace[((size_t)s * kTraceEntries + 11) * gridDim.x + blockIdx.x] = st.type >= 0 ? global_ns() : 0;  // descriptor read
         if (st.type == kStEmbed) {
+            trace_mark(p, s, 1);  // (nothing to wait for)
             const int d = p.d_model;
             if (kFewRows<M> && p.embed_direct) {
                 // The first RMSNorm reads the embeddings itself; what the residual stages will want of them, the CTA's own rows, it leaves here
@@ -2319,6 +2320,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(const __grid_cons
             // The LM head wants the hidden state of all CTAs. The cosines of one and two rows are the producer warp's work (finish_rows), those of
             // more rows the consumer warps'. (The test hook's wait is this one: the arrivals behind it would end the producer's.)
             if (!LL) stage_begin(p, s, p.bar_extra_last);
+            else trace_mark(p, s, 1);
             if constexpr (!kFewRows<M>) finish_stage<M>(p, sm);
         } else if (st.type == kStAttn) {
             attn_stage<M, LL, HD>(p, st, sm, gi, merge_target, s);
