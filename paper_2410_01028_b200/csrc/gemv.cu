@@ -139,7 +139,7 @@ private:
 // thread at a time. Thread t adds the squares of inputs 4 t + 1024 u in this order whatever R and U.
 template <int R, int U, bool kTail>
 __device__ __forceinline__ void norm_rows(const GemvParams& p, __nv_bfloat16* xs, float* red, bool first, int w0, int w1) {
-    constexpr int kThreads = kGemvWarps * 32, kStep = kThreads * 4, kBatch = R == 1 ? 8 : R > 5 ? 2 : 16 / R, kHeld = U > 0 ? U : 1;
+    constexpr int kThreads = kGemvWarps * 32, kStep = kThreads * 4, kBatch = R == 1 ? 8 : 16 / R, kHeld = U > 0 ? U : 1;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, n_in = p.n_in;
     const float* xf = reinterpret_cast<const float*>(p.x);
     auto load = [&](int m, int i) { return *reinterpret_cast<const ulonglong2*>(xf + (size_t)m * n_in + i); };

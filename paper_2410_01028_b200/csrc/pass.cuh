@@ -244,18 +244,6 @@ __device__ __forceinline__ void ring_release(const PassSmem& sm, int slot, uint3
     sm.consumed[slot] = gen + 1;
     mbar_arrive(&sm.empty[slot]);
 }
-// producer: wait until the slot of ring item g may be overwritten; returns the slot
-__device__ __forceinline__ int ring_acquire(const PassParams& p, const PassSmem& sm, uint32_t g, int stage, int tag) {
-    int slot;
-    uint32_t gen;
-    ring_locate(p, g, slot, gen);
-    if (gen > 0) {
-        if (!ring_spin_consumed(p, sm, slot, gen, kErrEmptyWait, stage, g, tag)) return slot;
-        mbar_wait(&sm.empty[slot], (gen - 1) & 1, p.err, kErrEmptyWait, stage, g, slot, tag, p.wait_cycles);
-    }
-    return slot;
-}
-
 __device__ __forceinline__ long long global_ns() {
     long long t;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -1614,6 +1602,7 @@ __device__ void finish_stage(const PassParams& p, const PassSmem& sm) {
 }
 template <int M>
 __device__ __forceinline__ void finish_rows(const PassParams& p) {
+    static_assert(kFewRows<M>, "the partials of all rows are requested together");
     const int lane = threadIdx.x & 31;
     if (blockIdx.x >= (unsigned)p.n_resid) return;
     if (lane == 0) {
@@ -1625,39 +1614,34 @@ __device__ __forceinline__ void finish_rows(const PassParams& p) {
         const ResidOut out = p.resid[r];
         const bool sum = lane == 0 && p.acc_sim && out.sumcos;
         double acc = sum ? *out.sumcos : 0.0;  // rows are added in order: chunked prefill equals one-shot prefill
-        constexpr int kB = M < 3 ? M : 3;      // rows whose partials are requested together
-#pragma unroll 1
-        for (int m0 = 0; m0 < M; m0 += kB) {
-            double s[kB][3] = {};
-            for (unsigned b0 = 0; b0 < gridDim.x; b0 += 160) {
-                float4 v[kB][5];
+        double s[M][3] = {};
+        for (unsigned b0 = 0; b0 < gridDim.x; b0 += 160) {
+            float4 v[M][5];
 #pragma unroll
-                for (int u = 0; u < kB; ++u)
+            for (int m = 0; m < M; ++m)
 #pragma unroll
-                    for (int i = 0; i < 5; ++i) {
-                        const unsigned b = b0 + i * 32 + lane;
-                        v[u][i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (m0 + u < M && b < gridDim.x) v[u][i] = __ldcg(part + (size_t)b * kPassMaxRows + m0 + u);
-                    }
+                for (int i = 0; i < 5; ++i) {
+                    const unsigned b = b0 + i * 32 + lane;
+                    v[m][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (b < gridDim.x) v[m][i] = __ldcg(part + (size_t)b * kPassMaxRows + m);
+                }
 #pragma unroll
-                for (int u = 0; u < kB; ++u)
+            for (int m = 0; m < M; ++m)
 #pragma unroll
-                    for (int i = 0; i < 5; ++i) s[u][0] += (double)v[u][i].x, s[u][1] += (double)v[u][i].y, s[u][2] += (double)v[u][i].z;
-            }
+                for (int i = 0; i < 5; ++i) s[m][0] += (double)v[m][i].x, s[m][1] += (double)v[m][i].y, s[m][2] += (double)v[m][i].z;
+        }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
+        for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-                for (int u = 0; u < kB; ++u)
+            for (int m = 0; m < M; ++m)
 #pragma unroll
-                    for (int j = 0; j < 3; ++j) s[u][j] += __shfl_xor_sync(0xffffffffu, s[u][j], o);
-            if (lane == 0) {
+                for (int j = 0; j < 3; ++j) s[m][j] += __shfl_xor_sync(0xffffffffu, s[m][j], o);
+        if (lane == 0) {
 #pragma unroll
-                for (int u = 0; u < kB; ++u)
-                    if (m0 + u < M) {
-                        const float c = (float)(s[u][0] / fmax(sqrt(s[u][1]) * sqrt(s[u][2]), 1e-30));
-                        out.cos_out[m0 + u] = c;
-                        acc += (double)c;
-                    }
+            for (int m = 0; m < M; ++m) {
+                const float c = (float)(s[m][0] / fmax(sqrt(s[m][1]) * sqrt(s[m][2]), 1e-30));
+                out.cos_out[m] = c;
+                acc += (double)c;
             }
         }
         if (sum) {
@@ -1711,14 +1695,13 @@ __device__ __forceinline__ void mma_bf16_zero(float (&d)[4], const uint32_t (&a)
 // (three barriers, about 3 us). Against fp32 FMAs fed from shared memory, heads one after the other and rows unrolled, kernel times in us (four layers of the 7B
 // width; two layers 2048 wide with 32 heads of 64 on 8): five rows on 8000 keys 595 -> 546, nine 876 -> 720, 16 rows of a prompt 683 -> 636; grouped
 // queries: one row on 8000 keys 111 -> 89, five 185 -> 140, nine 295 -> 188, 16 rows of a prompt 244 -> 211.
-// HD: the head size when the code is compiled for it, 0: p.head_dim.
+// HD: the head size when the code is compiled for it, 0: p.head_dim, 16 or 32 (a box of K or V is narrower than 128 bytes then, and not swizzled).
 template <int M, bool LL, int HD>
 __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassSmem& sm, uint32_t gi0, int stage, int n_chunks, int first, int n_local) {
     const int tid = threadIdx.x, warp = tid >> 5;
     const int hd = HD ? HD : p.head_dim;
-    const int nhb = hd > 64 ? hd / 64 : 1;
-    const int box_cols = hd > 64 ? 64 : hd;
-    const int tile_slots = (kAttnChunk / kBoxKeys) * nhb;
+    constexpr int nhb = HD > 64 ? HD / 64 : 1;
+    constexpr int tile_slots = (kAttnChunk / kBoxKeys) * nhb;
     const uint32_t tag_in = p.pass_tag + (uint32_t)(stage - 1), tag_out = p.pass_tag + (uint32_t)stage;  // W_qkv's stage precedes this one
     unsigned ll_spins = 0;
     long long ll_t0 = 0;
@@ -1729,7 +1712,7 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
     const int group = p.n_heads / p.n_kv_heads;
     const int n_cols = M * group;  // column c: row c % M of query head c / M of the group
     const int vec_per_row = hd / 8;
-    const TileAddr ta{nhb, box_cols * 2, (box_cols * 2 == 128) ? 1 : 0};
+    const TileAddr ta{nhb, HD ? 128 : hd * 2, HD ? 1 : 0};
 
     const int q_row = 2 * hd + 16, ct_max = attn_cols(M, group);
     unsigned char* qs = sm.reg_a + (size_t)grp * attn_scratch_bytes(M, group, hd);
@@ -1781,9 +1764,9 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
         // requested before the waits, so patching the tiles costs no round trip.
         const int fresh0 = max(p.pos0, key0), fresh1 = min(last_pos, key0 + kAttnChunk - 1);
         const int n_fresh = fresh1 - fresh0 + 1;
-        constexpr int kFreshPer = LL ? 1 : (M * (HD ? HD : 256) / 8 + 127) / 128;
+        constexpr int kFreshPer = LL ? 1 : (M * (HD ? HD : 32) / 8 + 127) / 128;
         uint4 kpre[kFreshPer], vpre[kFreshPer];
-        constexpr int kLLPer = LL && (HD == 0 || HD == 256) ? 2 : 1;  // tagged handoff: one word per element
+        constexpr int kLLPer = LL && HD == 256 ? 2 : 1;  // tagged handoff: one word per element
         unsigned long long kraw[kLLPer] = {}, vraw[kLLPer] = {};
         const bool has_fresh = n_fresh > 0;
         if (LL) {
@@ -1875,7 +1858,7 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
                 const uint32_t k_row = (uint32_t)(((gwarp & 1) * 32 + k_key) * ta.row_bytes);
                 const uint32_t tile0 = gk + (uint32_t)((gwarp >> 1) * nhb);
 #pragma unroll 1  // (unrolled, here and in P V: five rows on 8000 keys 546 -> 559 us, the instruction caches)
-                for (int hb = 0; hb < (HD ? (HD + 63) / 64 : nhb); ++hb) {
+                for (int hb = 0; hb < nhb; ++hb) {
                     const uint32_t k_addr = ring_addr + slot_off(tile0 + hb) + k_row;
 #pragma unroll
                     for (int ks = 0; ks < 4; ks += 2) {  // two steps of 16 dimensions
@@ -1978,15 +1961,14 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
             // ---- P V: dimensions 16 mt + {g8, g8 + 8} of columns 2 q4, 2 q4 + 1 to a lane, two such blocks side by side from 128 dimensions on.
             //      One or two columns: the terms are columns of one product. Either way the sums of a term over the blocks of 16 keys are added
             //      in order, then hi + (mid + lo).
-            const int tiles = hd >= 64 ? hd / 64 : 1;
+            constexpr int kBlocks = HD >= 64 ? HD / 64 : 1;  // of a warp
             auto products = [&](auto packed) {
                 constexpr bool kPacked = decltype(packed)::value;
-                constexpr int kTiles = HD == 64 || M <= 2 ? 1 : 2;  // (one and two rows: their registers)
+                constexpr int kTiles = kBlocks == 1 || M <= 2 ? 1 : 2;  // (one and two rows: their registers)
                 constexpr int kTerms = kPacked ? 1 : 3;
                 const uint32_t p_addr = smem_u32(ps) + min(mi, (kPacked ? 3 : 1) * ct - 1) * kAttnPRow + mat * 16;
 #pragma unroll 1
-                for (int mt0 = gwarp * tiles; mt0 < (gwarp + 1) * tiles && mt0 * 16 < hd; mt0 += kTiles) {
-                    const int nt = HD >= 64 ? kTiles : min(kTiles, tiles);
+                for (int mt0 = gwarp * kBlocks; mt0 < (gwarp + 1) * kBlocks && mt0 * 16 < hd; mt0 += kTiles) {
                     uint32_t v_addr[kTiles];
 #pragma unroll
                     for (int w = 0; w < kTiles; ++w) {
@@ -2007,7 +1989,6 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
                             if (kk + u >= n_steps) break;
 #pragma unroll
                             for (int w = 0; w < kTiles; ++w) {
-                                if (w >= nt) break;
                                 uint32_t a[4];
                                 ldmatrix4_trans(a, v_addr[w] + box + (uint32_t)(u * 16 * ta.row_bytes));
 #pragma unroll
@@ -2032,7 +2013,7 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
                             } else {
                                 o = acc[w][0][e] + (acc[w][1][e] + acc[w][2][e]);
                             }
-                            if (w < nt && col < ct) {
+                            if (col < ct) {
                                 const int g = (c0 + col) / M, m = (c0 + col) - g * M;
                                 const size_t at = (size_t)(kvh * group + g) * p.chunk_stride + chunk;
                                 if (LL) ll_store(p.pl_acc + at * hd + dim, __float_as_uint(o), tag_out);
