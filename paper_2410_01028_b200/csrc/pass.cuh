@@ -89,7 +89,7 @@ struct PassParams {
     __nv_bfloat16 *q, *a, *t;
     uint2 *xl, *al, *tl;  // tagged handoff (one-row passes): hidden state [d], attention output [d/2], SwiGLU output [f/2] as (value, tag) words
     uint2 *ql, *kl, *vl;  // tagged handoff: this pass's query [d], key and value [kv_dim], one bf16 per word
-    uint2 *pl_acc, *pl_ml;  // tagged handoff: attention partial results per (head, chunk): [head_dim] sums and (maximum, sum of weights)
+    uint2 *pl_acc, *pl_ml;  // tagged handoff: attention partial results per (head, chunk): [head_dim] sums and (maximum before the scale, sum of weights)
     uint32_t pass_tag;     // tag of stage 0 of this pass; stage s writes pass_tag + s
     int embed_direct;      // 1: the first sublayer reads the rows' embeddings itself (see pass_kernel)
     int use_ll;            // 1: launch the kernel variant that hands activations over through the tagged buffers (host: one row, d_model <= 5760)
@@ -1683,14 +1683,19 @@ __device__ __forceinline__ void mma_bf16_zero(float (&d)[4], const uint32_t (&a)
 // Work items (kv head, 128-key chunk) of this CTA on the tensor cores (mma.sync m16n8k16), a group of four warps to an item. The COLUMNS of the
 // products are the (row, query head) pairs that share the item's keys, eight at a time; what a column gets does not depend on its
 // neighbours, so neither does a row's result on the row count.
-//   S^T = K Q^T: 16 keys are the rows of a step (a warp has 32 keys), both operands read with ldmatrix; every 16 products start from zero and are
-//   added on the CUDA cores.
-//   softmax statistics of the chunk in fp32, the probabilities as the exact sum of three bf16 terms (cut off at 8 bits each) to shared memory.
+//   S^T = K Q^T: 16 keys are the rows of a step (a warp has 32 keys), both operands read with ldmatrix; every 16 products start from zero, and the sums
+//   of a score are added on the CUDA cores, from heads of 128 on as a tree.
+//   softmax statistics of the chunk in fp32, the scale behind the difference from the maximum, the probabilities as the exact sum of three bf16 terms (cut off at 8 bits each) to shared memory.
 //   O^T = V^T P: 16 dimensions are the rows (a warp has head_dim / 4 of them), V read transposed; every 16 products of a term start from zero as
 //   above. (One or two columns have room for their three terms in one product: a third of the steps.)
 // The order of the keys inside a block of 16 is free. Row r of a step is key r (r < 8) or 8 + ((r - 8) ^ 4): a lane then holds two keys that become
 // neighbours in P, and the eight rows of every matrix, of K as of V, have different swizzles: no bank conflicts.
-// Error: a sum of 16 products on the tensor core is nearly exact, and chains of additions are half as long as with one FMA per product.
+// Error: the tensor core cuts off what lies below the last bits of its sum (on average 0.2 2^-24 of a score), and every addition behind it rounds. The
+// tree, and the scale behind the subtraction, keep a score within what four chains of FMAs gave: two keys with equal scores, errors in 2^-24 of the
+// score, heads of 128 and 256: FMAs 0.56 and 0.55, sums added one after the other 0.79 and 0.98, this 0.47 and 0.52. Attention of one to nine
+// rows on up to 8000 positions, heads of 64 and 128 (error of the fp32 output, 2^-24): 2.06, 2.07, 1.74; heads of 128 of a 40-head decoder 3.57,
+// 4.31, 3.31. Heads of up to 64 have four sums at most, in a chain. The tree costs 0-1.5 % with heads of 128 (16 rows of the 7B width, four layers,
+// 590 -> 598 us, five rows 404.5 -> 405.2), 0-3 % with 256.
 // What bounds it: at 8000 positions of the 7B width the K/V stream (20 us a layer), the barrier and the merge behind it (10 us); at few positions the chain of an item
 // (three barriers, about 3 us). Against fp32 FMAs fed from shared memory, heads one after the other and rows unrolled, kernel times in us (four layers of the 7B
 // width; two layers 2048 wide with 32 heads of 64 on 8): five rows on 8000 keys 595 -> 546, nine 876 -> 720, 16 rows of a prompt 683 -> 636; grouped
@@ -1854,12 +1859,14 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
             // ---- scores: keys 32 gwarp + 16 t + {g8, 8 + (g8 ^ 4)} of columns 2 q4, 2 q4 + 1 to a lane
             float s[2][4] = {};
             {
+                float s_odd[2][4] = {};  // (heads of 256: boxes 1 and 3, or 0 and 2 where s has those)
                 const uint32_t q_addr = smem_u32(qs) + min(mi, ct - 1) * q_row + mat * 16;
                 const uint32_t k_row = (uint32_t)(((gwarp & 1) * 32 + k_key) * ta.row_bytes);
                 const uint32_t tile0 = gk + (uint32_t)((gwarp >> 1) * nhb);
 #pragma unroll 1  // (unrolled, here and in P V: five rows on 8000 keys 546 -> 559 us, the instruction caches)
                 for (int hb = 0; hb < nhb; ++hb) {
                     const uint32_t k_addr = ring_addr + slot_off(tile0 + hb) + k_row;
+                    float box[2][4];
 #pragma unroll
                     for (int ks = 0; ks < 4; ks += 2) {  // two steps of 16 dimensions
                         if (!HD && ks * 16 >= hd) break;
@@ -1871,16 +1878,35 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
                             float d[4];
                             ldmatrix4(a, k_addr + (uint32_t)(t * 16 * ta.row_bytes) + (uint32_t)(((ks * 2 + (mat >> 1)) ^ k_swz) << 4));
                             mma_bf16_zero(d, a, q[0], q[1]);
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) s[t][e] += d[e];
-                            if (HD || (ks + 1) * 16 < hd) {
-                                ldmatrix4(a, k_addr + (uint32_t)(t * 16 * ta.row_bytes) + (uint32_t)(((ks * 2 + 2 + (mat >> 1)) ^ k_swz) << 4));
-                                mma_bf16_zero(d, a, q[2], q[3]);
+                            if (HD <= 64) {
 #pragma unroll
                                 for (int e = 0; e < 4; ++e) s[t][e] += d[e];
                             }
+                            if (HD || (ks + 1) * 16 < hd) {
+                                float d2[4];
+                                ldmatrix4(a, k_addr + (uint32_t)(t * 16 * ta.row_bytes) + (uint32_t)(((ks * 2 + 2 + (mat >> 1)) ^ k_swz) << 4));
+                                mma_bf16_zero(d2, a, q[2], q[3]);
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    if (HD <= 64) {
+                                        s[t][e] += d2[e];
+                                    } else if (ks == 0) {
+                                        box[t][e] = d[e] + d2[e];
+                                    } else {
+                                        const float sum = s[t][e] + (box[t][e] + (d[e] + d2[e]));
+                                        if (HD == 256) s[t][e] = s_odd[t][e], s_odd[t][e] = sum;
+                                        else s[t][e] = sum;
+                                    }
+                                }
+                            }
                         }
                     }
+                }
+                if (HD == 256) {
+#pragma unroll
+                    for (int t = 0; t < 2; ++t)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) s[t][e] += s_odd[t][e];
                 }
             }
             // ---- softmax statistics of the chunk; the row at position pos0 + m sees keys <= pos0 + m
@@ -1894,7 +1920,7 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         float& v = s[t][e + 2 * h];
-                        v = my_key + t * 16 + h * other <= pos ? v * p.attn_scale : -INFINITY;
+                        v = my_key + t * 16 + h * other <= pos ? v : -INFINITY;
                         mx[e] = fmaxf(mx[e], v);
                     }
 #pragma unroll
@@ -1915,7 +1941,7 @@ __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassS
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     float& v = s[i >> 1][e + 2 * (i & 1)];
-                    v = v == -INFINITY ? 0.f : expf(v - mx[e]);
+                    v = v == -INFINITY ? 0.f : expf((v - mx[e]) * p.attn_scale);
                 }
                 sum[e] = (s[0][e] + s[0][e + 2]) + (s[1][e] + s[1][e + 2]);
                 if (2 * q4 + e < ct) {
@@ -2056,10 +2082,10 @@ struct MergeUnit {
 struct Merge {
     float mx = -INFINITY, l = 0.f, w;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    // ml: (maximum, sum of weights) of this lane's chunk, -inf past the last one
-    __device__ __forceinline__ void begin(float2 ml) {
-        const float m = fmaxf(mx, warp_max(ml.x)), s = expf(mx - m);
-        mx = m, w = expf(ml.x - m);
+    // ml: (maximum before scaling, sum of weights) of this lane's chunk, -inf past the last one
+    __device__ __forceinline__ void begin(float2 ml, float scale) {
+        const float m = fmaxf(mx, warp_max(ml.x)), s = expf((mx - m) * scale);
+        mx = m, w = expf((ml.x - m) * scale);
         l = __fmaf_rn(l, s, warp_sum(__fmul_rn(w, ml.y)));
         acc = make_float4(__fmul_rn(acc.x, s), __fmul_rn(acc.y, s), __fmul_rn(acc.z, s), __fmul_rn(acc.w, s));
     }
@@ -2107,7 +2133,7 @@ __device__ __forceinline__ void merge_tagged(const PassParams& p, int stage, int
                 if (!__all_sync(0xffffffffu, ll_keep_waiting(p, spins, t0, stage))) break;
                 __nanosleep(100u);
             }
-            mg.begin(c0 + lane < n_chunks ? make_float2(__uint_as_float((uint32_t)rm), __uint_as_float((uint32_t)rl)) : make_float2(-INFINITY, 0.f));
+            mg.begin(c0 + lane < n_chunks ? make_float2(__uint_as_float((uint32_t)rm), __uint_as_float((uint32_t)rl)) : make_float2(-INFINITY, 0.f), p.attn_scale);
 #pragma unroll 1
             for (int c1 = 0; c1 < 32 && c0 + c1 < n_chunks; c1 += 16) {
                 unsigned long long ra[4][4] = {};
@@ -2166,7 +2192,7 @@ __device__ __forceinline__ void merge_all(const PassParams& p) {
                 pa[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (c0 + 4 * i + mu.sub < nc) pa[i] = __ldcg(reinterpret_cast<const float4*>(src + (size_t)(c0 + 4 * i) * kPassMaxRows * hd));
             }
-            mg.begin(ml);
+            mg.begin(ml, p.attn_scale);
 #pragma unroll
             for (int i = 0; i < 8; ++i) mg.add(4 * i + mu.sub, pa[i]);  // (chunks past the last one weigh nothing)
         }
