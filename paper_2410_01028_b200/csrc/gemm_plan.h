@@ -58,9 +58,13 @@ inline GemmPlan plan_gemm(int M, int N, int K, int max_parts, int sms) {
     // Pair tiles over several rounds: the units of the last rounds have columns to spare, so tiles there are narrower, as narrow as
     // still cover the product in these rounds. A tile of bn - 32 columns takes 34 ns less for each 64 elements of the reduction, but no tile less than
     // its operands' way from L2, and the copies fetch bn columns of W either way: bn - 64 at least.
-    // 1023 x 11008 x 2048 37.9 -> 37.2 us, 512 x 22016 x 4096 71.0 -> 70.0, a prompt of 1023 rows 2048 wide, four layers, 667 -> 658; 511 x 12288 x 4096 the same.
+    // Only where rows of A and W are whole multiples of 64 bytes and rows of C of 32: otherwise the copies (a memory sector more for every 128 bytes
+    // and tile) or the stores (word by word) are what bounds a round, and more tiles or a shorter one behind a longer epilogue do not pay. With narrow
+    // tiles against without, in turn, 192 products of 33 to 2048 rows and 1024 to 22016 columns for each kind, K from 1024 on: K % 32 == 0 and N % 8
+    // == 0 2.8-2.9 % faster on average and none slower; K an odd multiple of 8 0.4 % slower (one in four more than 1 %, 6 % at worst), of 16 1.8 %
+    // faster (1.4 % slower at worst); N odd 1.2 % faster (one in nine more than 1 % slower, 3.3 % at worst). (A product against itself: 0.5 %.)
     best.wide = best.tiles / best.m_tiles, best.narrow = best.bn, best.items = best.tiles;
-    if (best.cg == 2 && best.parts == 1) {
+    if (best.cg == 2 && best.parts == 1 && K % 32 == 0 && N % 8 == 0) {
         const int units = sms / 2, rounds = (best.tiles + units - 1) / units;
         const int cols = (int)((long long)rounds * units / best.m_tiles);  // tiles of a row of tiles that these rounds hold
         int saved = 0;

@@ -18,7 +18,7 @@ MARGIN = 1e-2        # token ids must agree wherever the oracle's top-2 logit ga
 MASK_MARGIN = 1e-3   # skip masks must agree wherever |C_l - alpha| exceeds this
 
 
-GemmPlan = collections.namedtuple("GemmPlan", "bn cg m_tiles tiles parts")
+GemmPlan = collections.namedtuple("GemmPlan", "bn cg m_tiles tiles parts wide narrow items")
 
 
 @functools.lru_cache(None)
@@ -29,14 +29,14 @@ def _plan_lib():
         with open(src, "w") as f:
             f.write('#include "gemm_plan.h"\nextern "C" void plan(int m, int n, int k, int parts, int sms, int* o) {\n'
                     "    const asd::GemmPlan p = asd::plan_gemm(m, n, k, parts, sms);\n"
-                    "    o[0] = p.bn, o[1] = p.cg, o[2] = p.m_tiles, o[3] = p.tiles, o[4] = p.parts;\n}\n")
+                    "    o[0] = p.bn, o[1] = p.cg, o[2] = p.m_tiles, o[3] = p.tiles, o[4] = p.parts, o[5] = p.wide, o[6] = p.narrow, o[7] = p.items;\n}\n")
         subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", csrc, "-o", lib, src], check=True)
         return ctypes.CDLL(lib)
 
 
 def gemm_plan(M, N, K, max_parts=1, sms=148):
     """The library's own rule for the tiles and parts of a dense product, built from its header."""
-    out = (ctypes.c_int * 5)()
+    out = (ctypes.c_int * 8)()
     _plan_lib().plan(M, N, K, max_parts, sms, out)
     return GemmPlan(*out)
 
