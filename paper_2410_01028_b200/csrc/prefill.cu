@@ -103,7 +103,9 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 // fastest. Warp 0 is the TMA producer, warp 1 issues the MMAs and owns the tensor-memory allocation,
 // warps 2-9 are the epilogue (warp w reads lanes 32 * (w % 4) .. + 31 of tensor memory, the quarter its position in the
 // warp group gives it access to, and every second 32 columns: with four warps the epilogue of the last tile, which nothing covers, was longer:
-// gate/up of 512 rows of the 7B width 68.4 -> 64.4 us in the prompt's chain, of 1023 rows 2048 wide 41.3 -> 37.0). The accumulator is double-buffered in tensor memory (2 x BN columns), so the epilogue
+// gate/up of 512 rows of the 7B width 68.4 -> 64.4 us in the prompt's chain, of 1023 rows 2048 wide 41.3 -> 37.0). Four warps where a tile has 32
+// columns, and where rows of C are no multiple of 32 bytes: their stores bound the tile, and eight warps get in each other's way (pair tiles, 150 products
+// with N odd: 1-3 % slower with eight than with four; N an odd multiple of 4: 1 %). The accumulator is double-buffered in tensor memory (2 x BN columns), so the epilogue
 // of a tile runs while the MMAs of the next tile are already filling the other buffer. Barriers: full[s] (TMA bytes landed
 // in stage s), empty[s] (the MMAs reading stage s have finished: tcgen05.commit), acc_full[b] (all MMAs of the tile in
 // buffer b have finished), acc_empty[b] (the epilogue warps have read buffer b). Ragged edges: TMA fills out-of-range
@@ -126,8 +128,7 @@ __device__ __forceinline__ void epi_qkv(const GemmEpi& ep, int row, int col0, in
 // consumer adds them up (fp32 output), the number of parts the reduction dimension is cut into by the time they take
 // over the rounds (gemm_plan.h). Cutting the tiles of a last round with an exchange of the parts through L2 inside the
 // kernel (last arriver adds) was measured: 8-10 us per exchange, more than the part of a round it saves.
-constexpr int kGemmEpiWarps = 8;
-constexpr int kGemmThreads = 64 + 32 * kGemmEpiWarps;
+constexpr int kGemmThreads = 64 + 32 * 8;  // at most (see launch_gemm_tn)
 static int g_gemm_ctas = 148;  // persistent CTAs per launch: the SM count of the device (set by configure_prefill)
 
 // BN = 0: the width is a parameter of the launch (a multiple of 32).
@@ -197,7 +198,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], kGemmEpiWarps * CG);
+            mbar_init(&acc_empty[b], (blockDim.x / 32 - 2) * CG);
         }
         mbar_init(drained, 1);
         *abandoned = 0;
@@ -295,7 +296,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             if (!ok && lane == 0) give_up();
         }
     } else {
-        const int quarter = warp & 3, first = (warp - 2) / 4 * 32;  // two warps for each quarter take every second 32 columns
+        const int quarter = warp & 3, first = (warp - 2) / 4 * 32, step = blockDim.x > 192 ? 64 : 32;  // two warps for each quarter take every second 32 columns
         bool ok = true;
         GemmItem it;
         for (int local = 0; ok && gemm_item(work, num_kb, unit, n_units, local, it); ++local) {
@@ -308,7 +309,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             if (!ok) break;
             const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * Cfg::kAccStride);
             const int n_cols = min(it.width, N - n0);
-            for (int c = first; c < n_cols; c += 32 * (kGemmEpiWarps / 4)) {
+            for (int c = first; c < n_cols; c += step) {
                 float v[32];
                 tmem_ld32(acc + c, v);
                 if (row < M) gemm_epilogue(ep, row, n0 + c, N, v, it.part);
@@ -346,10 +347,10 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 }
 
 template <int BN, int CG>
-static cudaError_t launch_gemm(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmWork& w, const GemmEpi& ep,
+static cudaError_t launch_gemm(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmWork& w, const GemmEpi& ep, int epi_warps,
                                cudaStream_t s) {
     const dim3 grid((unsigned)(std::min(g_gemm_ctas / CG, w.tiles * w.parts) * CG));
-    return launch_pdl(gemm_tn_kernel<BN, CG>, grid, dim3(kGemmThreads), GemmCfg<BN, CG>::kSmem, s, CG, tm_a, tm_w, M, N, K, w, ep);
+    return launch_pdl(gemm_tn_kernel<BN, CG>, grid, dim3(64 + 32 * epi_warps), GemmCfg<BN, CG>::kSmem, s, CG, tm_a, tm_w, M, N, K, w, ep);
 }
 
 GemmPlan plan_gemm(int M, int N, int K, int max_parts) { return plan_gemm(M, N, K, max_parts, g_gemm_ctas); }
@@ -357,10 +358,11 @@ GemmPlan plan_gemm(int M, int N, int K, int max_parts) { return plan_gemm(M, N, 
 cudaError_t launch_gemm_tn(const CUtensorMap& tm_a, const CUtensorMap& tm_w, int M, int N, int K, const GemmPlan& p, const GemmEpi& ep, cudaStream_t s) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
     const GemmWork w{p.m_tiles, p.items, p.parts, p.bn, p.wide, p.narrow};
-    if (p.cg == 1) return launch_gemm<0, 1>(tm_a, tm_w, M, N, K, w, ep, s);
-    if (p.bn == 256) return launch_gemm<256, 2>(tm_a, tm_w, M, N, K, w, ep, s);
-    if (p.bn == 224) return launch_gemm<224, 2>(tm_a, tm_w, M, N, K, w, ep, s);
-    return launch_gemm<192, 2>(tm_a, tm_w, M, N, K, w, ep, s);
+    const int epi_warps = p.bn == 32 || (ep.mode == kGemmF32 && (ep.ldc & 7) != 0) ? 4 : 8;
+    if (p.cg == 1) return launch_gemm<0, 1>(tm_a, tm_w, M, N, K, w, ep, epi_warps, s);
+    if (p.bn == 256) return launch_gemm<256, 2>(tm_a, tm_w, M, N, K, w, ep, epi_warps, s);
+    if (p.bn == 224) return launch_gemm<224, 2>(tm_a, tm_w, M, N, K, w, ep, epi_warps, s);
+    return launch_gemm<192, 2>(tm_a, tm_w, M, N, K, w, ep, epi_warps, s);
 }
 
 // The status words of a product on its own, cleared by a kernel whose launch overlaps the end of the kernel in front and under
