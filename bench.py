@@ -95,7 +95,7 @@ def measured_traffic_ratio():
         return None
     rec = dict(line.strip().split("=", 1) for line in open(path) if "=" in line and not line.startswith("#"))
     h = hashlib.sha256()
-    for name in ("pass.cuh", "ring.cuh", "common.cuh"):
+    for name in ("pass.cuh", "pass_plan.h", "ring.cuh", "common.cuh"):
         with open(os.path.join(ROOT, "paper_2410_01028_b200", "csrc", name), "rb") as fh:
             h.update(fh.read())
     if rec.get("sources_sha256") != h.hexdigest():

@@ -223,9 +223,11 @@ int asd_get_last_cosines(asd_ctx* ctx, int32_t* M, float* cos_attn, float* cos_m
 /* Top-2 logit gap (largest minus second-largest logit; 0 when two tokens tie) of every row of the last pass that
  * ran the LM head, margins[M]. margins may be NULL to query M. Errors: STATE if no such pass has run. */
 int asd_get_last_margins(asd_ctx* ctx, int32_t* M, float* margins);
-/* Logits [M][vocab] of the last pass; only recorded while bit 0 of asd_set_debug's flags is set. */
+/* Logits [M][vocab] of the last pass; only recorded while bit 0 of asd_set_debug's flags is set. Up to 256 KB of a greedy pass are
+ * in host memory already when the call that ran it returns; the call then only copies them. */
 int asd_get_last_logits(asd_ctx* ctx, int32_t* M, float* logits);
-/* Debug flags: bit 0 = record the logits of every pass; bit 1 = record a per-stage device timeline.
+/* Debug flags: bit 0 = record the logits of every pass (a greedy pass with up to 256 KB of them also sends them to the host as it ends,
+ * 2-5 us, whether they are asked for or not); bit 1 = record a per-stage device timeline.
  * Two more bits exercise the error path of the bounded device waits without hanging anything.
  * ASD_DEBUG_SHORT_WAITS: every wait of the pass kernel (ring slots, grid barrier) gives up after about a
  * millisecond instead of about two seconds. ASD_DEBUG_MISSING_ARRIVAL: the grid barrier in front of the stage
@@ -242,9 +244,10 @@ int asd_set_debug(asd_ctx* ctx, int32_t flags);
  * timestamps in ns of every CTA: 0 = stage entered, 1 = inputs of the stage ready (previous stage finished on
  * all CTAs), 2 = weight streaming done, 3 = stage left. Entries 4 and 5 are SM cycles that the CTA's first
  * consumer warp spent waiting for ring slots and working on them; entries 6 and 7 are timestamps of a GEMV stage
- * after the RMSNorm statistics and after the first activation window is in shared memory. Entries 8-10 are the
+ * after the RMSNorm statistics and after the first activation window is in shared memory (entries 2 and 4 to 7 are
+ * left as they were by stages that have nothing of the kind). Entries 8-10 are the
  * producer's: timestamps of its first and last copy of the stage, and the SM cycles it waited for free ring
- * slots in between (one of its lanes); entry 11 is unused. Call first with ns_out = NULL for the sizes. */
+ * slots in between (one of its lanes); entry 11 is the time at which the stage descriptor had been read. Call first with ns_out = NULL for the sizes. */
 int asd_get_last_trace(asd_ctx* ctx, int32_t* n_stages, int32_t* n_ctas, int64_t* ns_out);
 /* K and V rows (bf16 patterns, n_kv_heads*head_dim each) of one layer (0-based) at one position. */
 int asd_get_kv(asd_ctx* ctx, int32_t layer, int32_t pos, uint16_t* k, uint16_t* v);

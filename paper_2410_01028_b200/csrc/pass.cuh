@@ -31,9 +31,9 @@
 // purpose: its smallest tile (64 weight rows) does not fit a 148-way row split that leaves ~28 rows of the
 // d x d matrices to a CTA, and its A operand would need the activations padded to 64+ rows in shared memory.
 //
-// Reduction order is fixed and independent of the row count M: an item's 16 steps alternate between two
-// accumulators that are added at the end, segments are added in ascending order. Attention chunks are aligned
-// to absolute positions and merged in order. Row m of a (k+1)-row verify pass is therefore bit-identical to
+// Reduction order is fixed and independent of the row count M: an item's 16 steps go round four
+// accumulators that are added in pairs at the end, segments are added in ascending order. Attention chunks are aligned
+// to absolute positions and merged in a fixed order. Row m of a (k+1)-row verify pass is therefore bit-identical to
 // a 1-row decode pass at the same position, so speculative output equals autoregressive output bit for bit.
 #pragma once
 #include <limits.h>
@@ -62,7 +62,7 @@ enum StageType : int { kStEmbed = 0, kStQkv, kStAttn, kStOproj, kStGateUp, kStDo
 struct StageDesc {
     int type, layer;
     int n_rows, n_in;
-    const unsigned char* W;             // packed weights of this stage (4 KB items, see above)
+    const unsigned char* W;             // packed weights of this stage (items of up to 8 KB, see above)
     const __nv_bfloat16* gain;
     __nv_bfloat16 *k_cache, *v_cache;   // this layer's cache [max_seq, kv_dim]
     const CUtensorMap *tm_k, *tm_v;     // tensor maps over the same
@@ -1699,7 +1699,8 @@ __device__ __forceinline__ void mma_bf16_zero(float (&d)[4], const uint32_t (&a)
 // What bounds it: at 8000 positions of the 7B width the K/V stream (20 us a layer), the barrier and the merge behind it (10 us); at few positions the chain of an item
 // (three barriers, about 3 us). Against fp32 FMAs fed from shared memory, heads one after the other and rows unrolled, kernel times in us (four layers of the 7B
 // width; two layers 2048 wide with 32 heads of 64 on 8): five rows on 8000 keys 595 -> 546, nine 876 -> 720, 16 rows of a prompt 683 -> 636; grouped
-// queries: one row on 8000 keys 111 -> 89, five 185 -> 140, nine 295 -> 188, 16 rows of a prompt 244 -> 211.
+// queries: one row on 8000 keys 111 -> 89, five 185 -> 140, nine 295 -> 188, 16 rows of a prompt 244 -> 211. (As the whole pass is now: 530, 699, 598; 87, 140,
+// 182, 174.)
 // HD: the head size when the code is compiled for it, 0: p.head_dim, 16 or 32 (a box of K or V is narrower than 128 bytes then, and not swizzled).
 template <int M, bool LL, int HD>
 __device__ void attn_items(const PassParams& p, const StageDesc& st, const PassSmem& sm, uint32_t gi0, int stage, int n_chunks, int first, int n_local) {
@@ -2107,9 +2108,8 @@ struct Merge {
 
 // Tagged handoff: the warps without attention items merge. They ask for the chunks' (maximum, sum of weights) until the tags are
 // this stage's, then for the sums of 16 chunks at a time. Nobody who produces a partial result ever waits for a merge, so the
-// wait ends. (Merged by the group that took a head's last chunk after its items, a head cost 2-3 us behind the last item at
-// five chunks and 11 us at 65; here the chunks before the last one are merged while that one is still being worked on: attention
-// stage 7.9 -> 4.9 us at 512 positions of the 7B shape, 36.9 -> 25.3 us at 8192.)
+// wait ends. The chunks before the last one are merged while that one is still being worked on: at 512 positions of the 7B shape the
+// stage is 4.9 us, 1.0 of it behind the last item. (A group that merged the heads whose last chunk it had took 2-3 us there, and 11 at 65 chunks.)
 __device__ __forceinline__ void merge_tagged(const PassParams& p, int stage, int n_chunks, int warp0, int n_warps) {
     const int lane = threadIdx.x & 31, hd = p.head_dim, warp = (threadIdx.x >> 5) - warp0;
     const uint32_t tag_out = p.pass_tag + (uint32_t)stage;
@@ -2168,9 +2168,9 @@ __device__ __forceinline__ void merge_tagged(const PassParams& p, int stage, int
     }
 }
 
-// Without tags: behind a grid barrier of its own the heads and rows are dealt to all warps of the grid. (Merged by the group whose
-// report completed a head, five rows cost 4 us behind the last item at five chunks and 29 us at 65: 32 of the 148 CTAs, and
-// in each a chain of 18 trips to L2. Two and three rows at 512 positions cost the same either way.)
+// Without tags: behind a grid barrier of its own the heads and rows are dealt to all warps of the grid: 3.3 us behind the last item at 512
+// positions of the 7B shape, barriers included, of a stage of 9.2 with five rows. (Merged by the group whose report completes a head, on 32 of
+// the 148 CTAs with a chain of 18 trips to L2 in each, five rows took 4 us at five chunks and 29 at 65.)
 template <int M>
 __device__ __forceinline__ void merge_all(const PassParams& p) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, hd = p.head_dim;
